@@ -42,39 +42,31 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
-# the stages one step runs, with their mc_step_stage ids (the scan stage is two kernels, one when every
-# world fits one scan block)
-STAGES = [("pbd", 0), ("bin_scan", 1), ("bin_scatter", 2), ("deposit_x", 3), ("force_lbm", 7), ("interp_advance", 6)]
-KERNELS_PER_STEP = 7
-GRAPH_STEPS = 16   # mc_step replays graphs of 16 steps: PBD, then 15 x (previous advance + PBD), 16 x (scan (2),
-                   # scatter, deposit, force + LBM), and the last advance = 97 kernels
+# the stages one step runs, with their mc_step_stage ids
+STAGES = [("pbd", 0), ("deposit_x", 3), ("force_lbm", 7), ("interp_advance", 6)]
+KERNELS_PER_STEP = 4
+GRAPH_STEPS = 16   # mc_step replays graphs of 16 steps: PBD, then 15 x (previous advance + PBD), 16 x (deposit,
+                   # force + LBM), and the last advance = 49 kernels
 
 
 def mdf_launches(steps: int, m: int) -> int:
-    """Kernels of direct-forcing steps (always the unfused sequence): PBD (returns), bins, scan (2),
-    scatter, deposit, steric spread, moments, predicted PBD, m passes (one tile kernel each), LBM,
-    advance."""
-    return steps * (11 + m)
+    """Kernels of direct-forcing steps (always the unfused sequence): PBD (returns), bins, deposit,
+    steric spread, moments, predicted PBD, m passes (one tile kernel each), LBM, advance."""
+    return steps * (8 + m)
 
 
-def scan_kernels(specs) -> int:
-    """The bin-offset scan is one kernel when every world's bins fit one 1024-bin scan block, else two."""
-    return 1 if all((sp.H // 8) * (sp.W // 8) <= 1024 for sp in specs) else 2
-
-
-def graph_launches(steps: int, scans: int = 2) -> int:
+def graph_launches(steps: int) -> int:
     """Kernels of a run of `steps` steps: 16-step graphs, then the leftover r steps in the same fused
-    order (r PBDs, r x (scan, scatter, deposit, force + LBM), one advance; one step alone runs the
-    six stages)."""
-    per = 4 + scans   # PBD, scan, scatter, deposit, force + LBM per step, plus the last advance
+    order (r PBDs, r x (deposit, force + LBM), one advance)."""
+    per = 3   # PBD, deposit, force + LBM per step, plus the last advance
     r = steps % GRAPH_STEPS
     return (steps // GRAPH_STEPS) * (GRAPH_STEPS * per + 1) + (per * r + 1 if r else 0)
-def run_launches(steps: int, cfg: dict, scans: int) -> int:
+
+
+def run_launches(steps: int, cfg: dict) -> int:
     """Kernels of a run of `steps` steps in a launch configuration: the persistent step is one cooperative
-    launch per run; otherwise the graph sequence above (two scan kernels when the configuration asks)."""
-    if cfg.get("persistent"):
-        return 1
-    return graph_launches(steps, 2 if cfg.get("scan_kernels") == 2 else scans)
+    launch per run; otherwise the graph sequence above."""
+    return 1 if cfg.get("persistent") else graph_launches(steps)
 
 
 # k_force_lbm, the dominant kernel: per cell read f 36 + rho_x 4, write f' 36 + u 8;
@@ -423,11 +415,11 @@ def bench_batched(args, steps=None):
             "plain_per_world_graph": {"value": plain_graph, "ms_per_step": ms_graph / 16,
                                       "description": "each world's own 16-step CUDA graph, replayed world after world"},
             "plain_per_world": {"value": plain, "ms_per_step": ms_plain / plain_steps,
-                                "launches_per_step": len(worlds) * (KERNELS_PER_STEP - 2 + scan_kernels(specs)),
+                                "launches_per_step": len(worlds) * KERNELS_PER_STEP,
                                 "description": "single direct steps, world after world"},
             "batched_over_plain_graph": batched / plain_graph, "batched_over_plain": batched / plain,
             "launch_config": tuned, "config_ms_per_step": configs,
-            "gpu_launches": run_launches(steps, tuned, scan_kernels(specs)),
+            "gpu_launches": run_launches(steps, tuned),
             "clocks": clk.summary()}
 
 
@@ -713,8 +705,8 @@ def main():
                    "l2": "state 1.8 GB > L2: no flush needed" if C >= 4096 * 4096 else "state may fit in L2; per-step timing includes no flush"},
         "e2e": {"value": e2e_val, "unit": "particle-steps/s", "steps": e2e_steps,
                 "h2d_bytes_per_step": h2d / e2e_steps, "d2h_bytes_per_step": d2h / e2e_steps},
-        "gpu_launches": (mdf_launches(args.steps, args.mdf_iters) - (2 - scan_kernels([spec])) * args.steps if mdf
-                         else run_launches(args.steps, tuned, scan_kernels([spec]))),
+        "gpu_launches": (mdf_launches(args.steps, args.mdf_iters) if mdf
+                         else run_launches(args.steps, tuned)),
         "launch_config": tuned,
         "roofline": None if mdf else {
             "bound": "hbm", "kernel": "k_force_lbm", "achieved": top_gbs, "peak": hbm_peak, "unit": "GB/s",

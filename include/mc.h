@@ -225,8 +225,8 @@ mc_status mc_step_batched(mc_world* const* worlds, int n_worlds, int n_steps, vo
  *                 check reports MC_ERR_TIMEOUT (their state is then
  *                 unspecified).
  *   pbd_warps     most filaments per block of the PBD kernels: 8, 4 or 2
- *   scan_kernels  0: one bin-offset kernel when every world's bins fit one
- *                 scan block (1024 bins), else two; 2: always two
+ *   scan_kernels  0 or 2; accepted and returned, without effect (a step
+ *                 computes no bin offsets)
  *   force_kernel  0: the fused force + LBM kernel with one 32x32 tile per
  *                 block; 1: its warp-specialised persistent form (half of
  *                 each block's warps run a tile's force phase while the
@@ -275,9 +275,9 @@ mc_status mc_autotune_mode(int mode);
 mc_status mc_debug_barrier_test(unsigned extra_arrivals, int64_t timeout_ns);
 
 /* Enqueues one stage of the next step on `stream` (for per-stage timing).
- * Stages: 0 drive + PBD + elastic force + bin histogram (a1-a3), 1 bin
- * offsets (one kernel, or two when the bins span several scan blocks),
- * 2 bin scatter (a2), 3 steric deposit + x pass of
+ * Stages: 0 drive + PBD + elastic force + binning (a1-a3, a2), 1 the bin
+ * offsets and 2 the records in bin order (the sorted read-outs of a2; the
+ * step's own stages read the bins' slots and do not need them), 3 steric deposit + x pass of
  * the Gaussian filter (a4, a5), 7 y pass + steric force + spread + LBM
  * (a5-a7, one kernel, the force density handed to the collision in shared
  * memory), 6 interpolation + advance (a8).  Enqueuing stages 0, 1, 2, 3, 7, 6

@@ -1,4 +1,4 @@
-// Device code of the bead-parallel stages (a1-a3 PBD, a2 scatter, a8
+// Device code of the bead-parallel stages (a1-a3 PBD with a2's binning, a8
 // interpolation + advance), shared by the per-stage kernels (k_bead.cu) and
 // the persistent batched step (k_persist.cu).
 #pragma once
@@ -247,34 +247,67 @@ __device__ __forceinline__ float2 bead_normal(float2 out, bool has_out, float2 i
   return make_float2(-t.y, t.x);
 }
 
-// F_el = kappa (x_hat - X) / dt of one bead, its 8x8 bin (a2) and one
-// histogram atomic per group of lanes sharing a bin.  Every lane calls this.
-// With direct forcing (kMode 2) the bead's output is instead its velocity
-// U_s = U* + dl/dt, U* (the fluid's, stored in ubead by the prediction) plus
-// the PBD correction of the carried position.
-template <int kMode>
-__device__ __forceinline__ void bead_out(const WorldDev& w, const PbdConst& k, bool valid, int b, const float4 P,
-                                         float dlx, float dly, float& fmax) {
-  if (kMode == 2) {
-    if (valid) {
-      const float2 U = w.ubead[b];
-      const float2 Us = make_float2(U.x + dlx / k.dt, U.y + dly / k.dt);
-      w.ubead[b] = Us;
-      w.sus[w.bead_slot[b]] = Us;   // the MDF passes read U_s in bin order
-    }
-    return;
-  }
+// a2: lanes of one warp that share a bin take consecutive places from one
+// atomic on its count.  bin_claim starts it (valid lanes pass their bin,
+// the others a negative one of their own); bin_place returns the lane's slot.
+// Every lane calls both; two claims can be in flight before their places.
+struct BinClaim {
+  int bin, base;
+  unsigned peers;
+};
+
+__device__ __forceinline__ BinClaim bin_claim(int* counts, bool valid, int bin) {
   const int lane = threadIdx.x & 31;
-  int bin = -1 - lane;
-  if (valid) {
-    const float2 fe = make_float2(k.kappa_dt * dlx, k.kappa_dt * dly);
+  BinClaim c;
+  c.bin = valid ? bin : -1 - lane;
+  c.peers = __match_any_sync(0xffffffffu, c.bin);
+  c.base = 0;
+  if (valid && (__ffs(c.peers) - 1) == lane) c.base = atomicAdd(&counts[bin], __popc(c.peers));
+  return c;
+}
+
+__device__ __forceinline__ int bin_place(const WorldDev& w, int* counts, bool valid, const BinClaim& c) {
+  const int lane = threadIdx.x & 31;
+  const int at = __shfl_sync(0xffffffffu, c.base, __ffs(c.peers) - 1) + __popc(c.peers & ((1u << lane) - 1u));
+  if (!valid) return -1;
+  if (at < w.slot_cap) return c.bin * w.slot_cap + at;
+  return w.n_bins * w.slot_cap + atomicAdd(&counts[w.n_bins], 1);   // the bin's slots are full
+}
+
+// The bin of the bead at P.
+__device__ __forceinline__ int bead_bin_of(const float4& P, int nbx) {
+  return (cell_y(P) / kBin) * nbx + cell_x(P) / kBin;
+}
+
+// The bead's record in its slot, and the slot by bead where a later kernel
+// asks for it.
+__device__ __forceinline__ void bin_store(const WorldDev& w, int slot, int b, const float4& P, float2 fe) {
+  w.bpos[slot] = P;
+  w.brec[slot] = make_float4(fe.x, fe.y, __int_as_float(b), 0.0f);
+  if (w.bead_slot) w.bead_slot[b] = slot;
+}
+
+// With direct forcing the PBD's output for a bead is its velocity U_s =
+// U* + dl/dt, U* (the fluid's, stored in ubead by the prediction) plus the
+// PBD correction of the carried position.
+__device__ __forceinline__ void bead_out_velocity(const WorldDev& w, const PbdConst& k, int b, float dlx, float dly) {
+  const float2 U = w.ubead[b];
+  const float2 Us = make_float2(U.x + dlx / k.dt, U.y + dly / k.dt);
+  w.ubead[b] = Us;
+  w.sus[w.bead_slot[b]] = Us;   // the MDF passes read U_s by slot
+}
+
+// F_el = kappa (x_hat - X) / dt of one bead; with `fields`, kept with its
+// bin for read-out.
+__device__ __forceinline__ float2 bead_out_force(const WorldDev& w, const PbdConst& k, int b, int bin, float dlx,
+                                                 float dly, int fields, float& fmax) {
+  const float2 fe = make_float2(k.kappa_dt * dlx, k.kappa_dt * dly);
+  fmax = fmaxf(fmax, fmaxf(fabsf(fe.x), fabsf(fe.y)));
+  if (fields) {
     w.fel[b] = fe;
-    fmax = fmaxf(fmax, fmaxf(fabsf(fe.x), fabsf(fe.y)));
-    bin = (cell_y(P) / kBin) * k.nbx + cell_x(P) / kBin;
     w.bead_bin[b] = bin;
   }
-  const unsigned peers = __match_any_sync(0xffffffffu, bin);
-  if (valid && (__ffs(peers) - 1) == lane) atomicAdd(&w.bin_count[bin], __popc(peers));
+  return fe;
 }
 
 // Jacobi PBD of a filament of at most 64 beads in registers: lane l holds
@@ -282,7 +315,7 @@ __device__ __forceinline__ void bead_out(const WorldDev& w, const PbdConst& k, b
 // warp shuffles.  The same arithmetic, in the same order, as pbd_smem.
 template <bool kExt, int kMode>
 __device__ __forceinline__ float pbd_regs(const WorldDev& w, const PbdConst& k, int b0, int B, int e0, int j0,
-                                          long long t) {
+                                          long long t, int fields) {
   constexpr unsigned kAll = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int nE = B - 1, nJ = B - 2;
@@ -412,8 +445,20 @@ __device__ __forceinline__ float pbd_regs(const WorldDev& w, const PbdConst& k, 
   if (he0) w.theta[e0 + i0] = th0;
   if (he1) w.theta[e0 + i1] = th1;
   float fmax = 0.0f;
-  bead_out<kMode>(w, k, hb0, b0 + i0, P0, dlx0, dly0, fmax);
-  bead_out<kMode>(w, k, hb1, b0 + i1, P1, dlx1, dly1, fmax);
+  if (kMode == 2) {
+    if (hb0) bead_out_velocity(w, k, b0 + i0, dlx0, dly0);
+    if (hb1) bead_out_velocity(w, k, b0 + i1, dlx1, dly1);
+  } else {
+    const int bin0 = bead_bin_of(P0, k.nbx), bin1 = bead_bin_of(P1, k.nbx);
+    float2 fe0 = make_float2(0.0f, 0.0f), fe1 = fe0;
+    if (hb0) fe0 = bead_out_force(w, k, b0 + i0, bin0, dlx0, dly0, fields, fmax);
+    if (hb1) fe1 = bead_out_force(w, k, b0 + i1, bin1, dlx1, dly1, fields, fmax);
+    int* counts = step_counts(w, t);
+    const BinClaim c0 = bin_claim(counts, hb0, bin0), c1 = bin_claim(counts, hb1, bin1);
+    const int s0 = bin_place(w, counts, hb0, c0), s1 = bin_place(w, counts, hb1, c1);
+    if (hb0) bin_store(w, s0, b0 + i0, P0, fe0);
+    if (hb1) bin_store(w, s1, b0 + i1, P1, fe1);
+  }
   if (kExt && w.observe && t >= 1) {
     // behaviour descriptors (Eqs. 5, 6): squared change of the rest angles
     // and rest lengths from step t - 1 to step t
@@ -436,7 +481,7 @@ __device__ __forceinline__ float pbd_regs(const WorldDev& w, const PbdConst& k, 
 // so all corrections of a pass see the state before it.
 template <bool kExt, int kMode>
 __device__ __forceinline__ float pbd_smem(const WorldDev& w, const PbdConst& k, int b0, int B, int e0, int j0,
-                                          long long t, float* s, int maxB) {
+                                          long long t, int fields, float* s, int maxB) {
   const int lane = threadIdx.x & 31;
   const int nE = B - 1, nJ = B - 2;
   float* vx = s;
@@ -554,10 +599,21 @@ __device__ __forceinline__ float pbd_smem(const WorldDev& w, const PbdConst& k, 
   }
   for (int e = lane; e < nE; e += 32) w.theta[e0 + e] = th[e];
   float fmax = 0.0f;
-  for (int i0 = 0; i0 < B; i0 += 32) {
-    const int i = i0 + lane;
-    bead_out<kMode>(w, k, i < B, b0 + i, i < B ? P[i] : make_float4(0.0f, 0.0f, 0.0f, 0.0f), i < B ? dlx[i] : 0.0f,
-                    i < B ? dly[i] : 0.0f, fmax);
+  if (kMode == 2) {
+    for (int i = lane; i < B; i += 32) bead_out_velocity(w, k, b0 + i, dlx[i], dly[i]);
+  } else {
+    int* counts = step_counts(w, t);
+    for (int i0 = 0; i0 < B; i0 += 32) {
+      const int i = i0 + lane;
+      const bool valid = i < B;
+      const float4 p = valid ? P[i] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      const int bin = bead_bin_of(p, k.nbx);
+      const BinClaim c = bin_claim(counts, valid, bin);
+      float2 fe = make_float2(0.0f, 0.0f);
+      if (valid) fe = bead_out_force(w, k, b0 + i, bin, dlx[i], dly[i], fields, fmax);
+      const int slot = bin_place(w, counts, valid, c);
+      if (valid) bin_store(w, slot, b0 + i, p, fe);
+    }
   }
   if (kExt && w.observe && t >= 1) {
     float eb = 0.0f, ep = 0.0f;
@@ -583,7 +639,8 @@ extern __shared__ __align__(16) float pbd_dyn_smem[];
 
 template <bool kExt, int kMode, bool kSingle>
 __device__ __forceinline__ void pbd_body(const WorldDev* __restrict__ worlds, const int2* __restrict__ items,
-                                         int n_items, int maxB, unsigned blk) {
+                                         int n_items, int maxB, int off, int fields,
+                                         unsigned blk) {
   float* smem = pbd_dyn_smem;
   const int wpb = blockDim.x >> 5;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -598,12 +655,10 @@ __device__ __forceinline__ void pbd_body(const WorldDev* __restrict__ worlds, co
   const int b0 = w.fil_off[f];
   const int B = w.fil_off[f + 1] - b0;
   const int e0 = b0 - f, j0 = b0 - 2 * f;
-  // with kMode 1 the counter still holds the previous step (the scan of
-  // this step advances it)
-  const long long t = *w.t + (kMode == 1 ? 1 : 0);
+  const long long t = *w.t + off;
   const PbdConst k = pbd_const(w);
-  float fmax = B <= 64 ? pbd_regs<kExt, kMode>(w, k, b0, B, e0, j0, t)
-                       : pbd_smem<kExt, kMode>(w, k, b0, B, e0, j0, t,
+  float fmax = B <= 64 ? pbd_regs<kExt, kMode>(w, k, b0, B, e0, j0, t, fields)
+                       : pbd_smem<kExt, kMode>(w, k, b0, B, e0, j0, t, fields,
                                                smem + (size_t)warp * maxB * kPbdFloatsPerBead, maxB);
   if (kMode == 2) return;
   // largest |F_el| component of the world this step (bounds the spread's
@@ -612,43 +667,17 @@ __device__ __forceinline__ void pbd_body(const WorldDev* __restrict__ worlds, co
   if (lane == 0) atomicMax(&w.fel_max[t & 1], __float_as_uint(fmax));
 }
 
-// a2: scatter bead records into bin order.  Lanes of one warp that share a
-// bin take consecutive slots from one atomic.
-template <bool kSingle>
-__device__ __forceinline__ void bin_scatter_body(const WorldDev* __restrict__ worlds, const int2* __restrict__ items,
-                                                 const WorldDev& w1, unsigned blk) {
-  const int2 it = kSingle ? make_int2(0, (int)blk * kBeadChunk) : items[blk];
-  const WorldDev& w = kSingle ? w1 : worlds[it.x];
-  const int i = it.y + threadIdx.x;
-  const int lane = threadIdx.x & 31;
-  const bool valid = i < w.N;
-  const int bin = valid ? w.bead_bin[i] : -1 - lane;
-  // the record is loaded before the cursor atomic, so its latency overlaps
-  const float4 p = valid ? w.pos[i] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-  const float2 fe = valid ? w.fel[i] : make_float2(0.0f, 0.0f);
-  const unsigned peers = __match_any_sync(0xffffffffu, bin);
-  const int leader = __ffs(peers) - 1;
-  int base = 0;
-  if (valid && lane == leader) base = atomicAdd(&w.bin_cursor[bin], __popc(peers));
-  base = __shfl_sync(0xffffffffu, base, leader);
-  if (valid) {
-    const int slot = base + __popc(peers & ((1u << lane) - 1u));
-    w.spos[slot] = p;
-    w.srec[slot] = make_float4(fe.x, fe.y, __int_as_float(i), 0.0f);
-    if (w.bead_slot) w.bead_slot[i] = slot;   // direct forcing: U_s goes to the bead's slot
-  }
-}
-
 // a8: U_i = sum_c delta_h(c - X_i) u(c) over the 4x4 stencil, then the
 // inertia-free advance X += dt U (cell index + fraction, wrapped) and the
 // unwrapped displacement D += dt U.  Thread 0 of each world's first block
-// advances the world's step counter (no other stage kernel reads it).
+// advances the world's step counter by the inc steps of the run that this
+// advance ends (no other thread of the launch reads it).
 template <bool kExt, bool kSingle>
 __device__ __forceinline__ void interp_advance_body(const WorldDev* __restrict__ worlds,
-                                                    const int2* __restrict__ items, unsigned blk) {
+                                                    const int2* __restrict__ items, int inc, unsigned blk) {
   const int2 it = kSingle ? make_int2(0, (int)blk * kBeadChunk) : items[blk];
   const WorldDev& w = worlds[it.x];
-  if (it.y == 0 && threadIdx.x == 0) *w.t += 1;
+  if (it.y == 0 && threadIdx.x == 0) *w.t += inc;
   const int i = it.y + threadIdx.x;
   // the velocity at the bead's position at the start of the step (and, with
   // observables, the energy sampled there; every lane of the block takes

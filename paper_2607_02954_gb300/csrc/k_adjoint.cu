@@ -861,10 +861,15 @@ __global__ void __launch_bounds__(1024) k_loss_polyline(const WorldDev* __restri
   if (threadIdx.x == 0) *loss = red[0];
 }
 
-__global__ void k_set_counter(long long* t, long long v, unsigned* fel_max) {
-  *t = v;
-  fel_max[0] = 0u;
-  fel_max[1] = 0u;
+// The step counter moves to v; the slots step v accumulates into (its bin
+// counts, its F_el maximum) start at zero, the other parity's stay.
+__global__ void __launch_bounds__(256) k_set_counter(const __grid_constant__ WorldDev w, long long v) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) {
+    *w.t = v;
+    w.fel_max[v & 1] = 0u;
+  }
+  if (i <= w.n_bins) step_counts(w, v)[i] = 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -1047,7 +1052,7 @@ void launch_loss_polyline(const Plan& p, const WorldDev& h, const float2* pos0, 
 }
 
 void launch_set_counter(const WorldDev& h, long long t, cudaStream_t s) {
-  k_set_counter<<<1, 1, 0, s>>>(h.t, t, h.fel_max);
+  k_set_counter<<<(h.n_bins + 256) / 256, 256, 0, s>>>(h, t);
 }
 
 }  // namespace mc

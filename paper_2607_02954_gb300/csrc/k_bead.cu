@@ -1,5 +1,5 @@
-// Bead-parallel stages of one time step: drive + PBD + elastic force + bin
-// histogram (a1-a3), bin scatter (a2), IB interpolation + advance (a8), and
+// Bead-parallel stages of one time step: drive + PBD + elastic force +
+// binning (a1-a3), IB interpolation + advance (a8), and
 // the per-world set-up / read-out kernels.
 #include <mutex>
 
@@ -7,7 +7,7 @@
 
 namespace mc {
 
-// One warp per filament (a1 + a3 + the a2 histogram).  Bead positions enter
+// One warp per filament (a1 + a3 + a2).  Bead positions enter
 // as edge vectors v0 = min_image(X_b - X_a) plus the accumulated corrections,
 // so the corrections keep full FP32 precision whatever the magnitude of the
 // coordinates.  Filaments of at most 64 beads run in registers; longer ones
@@ -15,27 +15,17 @@ namespace mc {
 // when no filament of the launch is longer than 64 beads).
 template <bool kExt, int kMode, bool kSingle>
 __global__ void __launch_bounds__(256, 4) k_pbd(const WorldDev* __restrict__ worlds,
-                                             const int2* __restrict__ items, int n_items, int maxB) {
+                                             const int2* __restrict__ items, int n_items, int maxB, int off,
+                                             int fields) {
   pdl_trigger();
   pdl_wait();
-  pbd_body<kExt, kMode, kSingle>(worlds, items, n_items, maxB, blockIdx.x);
-}
-
-// a2: scatter bead records into bin order.  Lanes of one warp that share a
-// bin take consecutive slots from one atomic.
-template <bool kSingle>
-__global__ void __launch_bounds__(kBeadChunk) k_bin_scatter(const WorldDev* __restrict__ worlds,
-                                                            const int2* __restrict__ items,
-                                                            const __grid_constant__ WorldDev w1) {
-  pdl_trigger();
-  pdl_wait();
-  bin_scatter_body<kSingle>(worlds, items, w1, blockIdx.x);
+  pbd_body<kExt, kMode, kSingle>(worlds, items, n_items, maxB, off, fields, blockIdx.x);
 }
 
 // Spread of half of F_el + F_s at each layer point of every bead of
 // two-layer worlds, in 64-bit fixed point (bitwise independent of order).
-// Beads are read through the step's binned records, so the positions are
-// those at the start of the step even when the spread is re-run later.
+// Beads are read from the step's slots, so the positions are those at the
+// start of the step even when the spread is re-run later.
 __global__ void __launch_bounds__(kBeadChunk) k_layer_spread(const WorldDev* __restrict__ worlds,
                                                              const int2* __restrict__ items) {
   pdl_trigger();
@@ -43,12 +33,12 @@ __global__ void __launch_bounds__(kBeadChunk) k_layer_spread(const WorldDev* __r
   const int2 it = items[blockIdx.x];
   const WorldDev& w = worlds[it.x];
   if (w.layers != 2) return;
-  const int slot = it.y + threadIdx.x;
-  if (slot >= w.N) return;
+  const int i = it.y + threadIdx.x;
+  if (i >= w.N) return;
   const int W = w.W, H = w.H;
-  const float4 rec = w.srec[slot];
-  const int i = __float_as_int(rec.z);
-  const float4 p = w.spos[slot];
+  const int slot = w.bead_slot[i];
+  const float4 rec = w.brec[slot];
+  const float4 p = w.bpos[slot];
   const float2 n = w.nrm[i], fe = make_float2(rec.x, rec.y), fs = w.fs[i];
   const float hx = 0.5f * (fe.x + fs.x), hy = 0.5f * (fe.y + fs.y);
   for (int side = 0; side < 2; ++side) {
@@ -90,14 +80,13 @@ __global__ void __launch_bounds__(kCellChunk) k_layer_finish(const WorldDev* __r
 
 // a8: U_i = sum_c delta_h(c - X_i) u(c) over the 4x4 stencil, then the
 // inertia-free advance X += dt U (cell index + fraction, wrapped) and the
-// unwrapped displacement D += dt U.  Thread 0 of each world's first block
-// advances the world's step counter (no other stage kernel reads it).
+// unwrapped displacement D += dt U; the worlds' step counters move by inc.
 template <bool kExt, bool kSingle>
 __global__ void __launch_bounds__(kBeadChunk) k_interp_advance(const WorldDev* __restrict__ worlds,
-                                                               const int2* __restrict__ items) {
+                                                               const int2* __restrict__ items, int inc) {
   pdl_trigger();
   pdl_wait();
-  interp_advance_body<kExt, kSingle>(worlds, items, blockIdx.x);
+  interp_advance_body<kExt, kSingle>(worlds, items, inc, blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -216,7 +205,7 @@ void launch_pbd(const Plan& p, cudaStream_t s) {
   const bool one = p.n_worlds == 1;
   auto kern = p.any_ext ? (one ? k_pbd<true, 0, true> : k_pbd<true, 0, false>)
                         : (one ? k_pbd<false, 0, true> : k_pbd<false, 0, false>);
-  launch_pdl(kern, grid, wpb * 32, smem, s, p.d_worlds, p.d_fil_items, p.n_fil_items, mb);
+  launch_pdl(kern, grid, wpb * 32, smem, s, p.d_worlds, p.d_fil_items, p.n_fil_items, mb, 0, 1);
 }
 
 // The PBD of direct-forcing worlds (from the positions the fluid carries
@@ -228,12 +217,12 @@ void launch_pbd_mdf(const Plan& p, cudaStream_t s) {
   const size_t smem = p.max_B <= 64 ? 0 : (size_t)wpb * mb * kPbdFloatsPerBead * sizeof(float);
   const int grid = (p.n_fil_items + wpb - 1) / wpb;
   auto kern = p.n_worlds == 1 ? k_pbd<true, 2, true> : k_pbd<true, 2, false>;
-  launch_pdl(kern, grid, wpb * 32, smem, s, p.d_worlds, p.d_fil_items, p.n_fil_items, mb);
+  launch_pdl(kern, grid, wpb * 32, smem, s, p.d_worlds, p.d_fil_items, p.n_fil_items, mb, 0, 1);
 }
 
 // a8 of the previous step fused with this step's a1-a3 (plans without
-// direct-forcing worlds): the counter is advanced by this step's scan.
-void launch_advance_pbd(const Plan& p, cudaStream_t s) {
+// direct-forcing worlds), off steps after the worlds' counters.
+void launch_advance_pbd(const Plan& p, cudaStream_t s, int off, int fields) {
   if (p.n_fil_items == 0) return;
   const int mb = (p.max_B + 3) & ~3;
   const int wpb = pbd_warps_per_block(mb, p.n_fil_items, p.cfg.pbd_warps);
@@ -242,7 +231,7 @@ void launch_advance_pbd(const Plan& p, cudaStream_t s) {
   const bool one = p.n_worlds == 1;
   auto kern = p.any_ext ? (one ? k_pbd<true, 1, true> : k_pbd<true, 1, false>)
                         : (one ? k_pbd<false, 1, true> : k_pbd<false, 1, false>);
-  launch_pdl(kern, grid, wpb * 32, smem, s, p.d_worlds, p.d_fil_items, p.n_fil_items, mb);
+  launch_pdl(kern, grid, wpb * 32, smem, s, p.d_worlds, p.d_fil_items, p.n_fil_items, mb, off, fields);
 }
 
 // Shared-memory limits set once per process, outside any stream capture: the
@@ -260,23 +249,17 @@ void kernel_setup() {
   });
 }
 
-void launch_bin_scatter(const Plan& p, cudaStream_t s) {
-  // (data moves only: the single-world path cannot change a result)
-  if (p.n_worlds == 1) launch_pdl(k_bin_scatter<true>, p.n_bead_items, kBeadChunk, 0, s, p.d_worlds, p.d_bead_items, p.h_world0);
-  else launch_pdl(k_bin_scatter<false>, p.n_bead_items, kBeadChunk, 0, s, p.d_worlds, p.d_bead_items, p.h_world0);
-}
-
 void launch_layer_spread(const Plan& p, cudaStream_t s) {
   if (!p.any_layered) return;
   k_layer_spread<<<p.n_bead_items, kBeadChunk, 0, s>>>(p.d_worlds, p.d_bead_items);
   if (p.n_cell_items) k_layer_finish<<<p.n_cell_items, kCellChunk, 0, s>>>(p.d_worlds, p.d_cell_items);
 }
 
-void launch_interp_advance(const Plan& p, cudaStream_t s) {
+void launch_interp_advance(const Plan& p, cudaStream_t s, int inc) {
   const bool one = p.n_worlds == 1;
   auto kern = p.any_ext ? (one ? k_interp_advance<true, true> : k_interp_advance<true, false>)
                         : (one ? k_interp_advance<false, true> : k_interp_advance<false, false>);
-  launch_pdl(kern, p.n_bead_items, kBeadChunk, 0, s, p.d_worlds, p.d_bead_items);
+  launch_pdl(kern, p.n_bead_items, kBeadChunk, 0, s, p.d_worlds, p.d_bead_items, inc);
 }
 
 void launch_unstream_in(const float* f0dev, float* g_dst, int H, int W, cudaStream_t s) {

@@ -1,28 +1,126 @@
-// Grid-side stages of one time step: bin offsets (a2) and the fused D2Q9 TRT
-// collide + stream (a7).  The steric and spread stages (a4-a6) are in
-// k_steric.cu, the bead stages in k_bead.cu.
-#include "grid_dev.cuh"
+// Grid-side stages of one time step: the fused D2Q9 TRT collide + stream
+// (a7), the step sequence, and the sorted read-outs of the bins (a2).  The
+// steric and spread stages (a4-a6) are in k_steric.cu, the bead stages,
+// which bin the beads, in k_bead.cu.
+#include "mc_internal.cuh"
 
 namespace mc {
 
-template <bool kSingle>
-__global__ void __launch_bounds__(256) k_scan_sums(const WorldDev* __restrict__ worlds,
-                                                   const int2* __restrict__ items, int inc_t,
-                                                   const __grid_constant__ WorldDev w1) {
-  pdl_trigger();
-  pdl_wait();
-  __shared__ ScanSmem sm;
-  scan_sums_body<kSingle>(worlds, items, inc_t, w1, blockIdx.x, sm);
+// ---------------------------------------------------------------------------
+// Sorted read-outs of a step's bins: the exclusive prefix sum of the bin
+// counts, in blocks of kScanChunk bins (k_scan_sums adds up each block,
+// k_scan_apply offsets each block by the sum of the earlier ones and scans
+// it), then the records in bin order (k_sort_records).  A step does not run
+// them: its tile kernels read each bin's slots directly.  They serve the
+// field read-outs and saved images, and k_unsort_records puts a loaded
+// image's records back into slots.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ int block_sum_256(int v, int* red) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  int t = threadIdx.x < 8 ? red[threadIdx.x] : 0;
+  if (threadIdx.x < 32) {
+    for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (threadIdx.x == 0) red[8] = t;
+  }
+  __syncthreads();
+  const int r = red[8];
+  __syncthreads();
+  return r;
 }
 
-template <bool kSingle>
-__global__ void __launch_bounds__(256) k_scan_apply(const WorldDev* __restrict__ worlds,
-                                                    const int2* __restrict__ items, int book, int inc_t,
-                                                    const __grid_constant__ WorldDev w1) {
-  pdl_trigger();
-  pdl_wait();
-  __shared__ ScanSmem sm;
-  scan_apply_body<kSingle>(worlds, items, book, inc_t, w1, blockIdx.x, sm);
+__global__ void __launch_bounds__(256) k_scan_sums(const __grid_constant__ WorldDev w, int off) {
+  __shared__ int red[9];
+  const int* counts = step_counts(w, *w.t + off);
+  const int base = (int)blockIdx.x * kScanChunk;
+  const int end = min(base + kScanChunk, w.n_bins);
+  int s = 0;
+  for (int k = base + threadIdx.x; k < end; k += blockDim.x) s += counts[k];
+  s = block_sum_256(s, red);
+  if (threadIdx.x == 0) w.chunk_sum[blockIdx.x] = s;
+}
+
+// The offsets, and in bin_cursor each bin's first place after its slots'
+// records (where k_sort_records appends the beads that found them full).
+__global__ void __launch_bounds__(256) k_scan_apply(const __grid_constant__ WorldDev w, int off) {
+  __shared__ int red[9];
+  __shared__ int warp_tot[8];
+  const int* counts = step_counts(w, *w.t + off);
+  int pre = 0;
+  for (int k = threadIdx.x; k < (int)blockIdx.x; k += blockDim.x) pre += w.chunk_sum[k];
+  pre = block_sum_256(pre, red);
+  const int n = w.n_bins;
+  const int base = (int)blockIdx.x * kScanChunk + threadIdx.x * 4;
+  int v[4];
+  int tsum = 0;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    v[j] = base + j < n ? counts[base + j] : 0;
+    tsum += v[j];
+  }
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  int incl = tsum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  if (lane == 31) warp_tot[wid] = incl;
+  __syncthreads();
+  int wbase = 0;
+  for (int k = 0; k < wid; ++k) wbase += warp_tot[k];
+  int run = pre + wbase + incl - tsum;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int k = base + j;
+    if (k < n) {
+      w.bin_off[k] = run;
+      w.bin_cursor[k] = run + min(v[j], w.slot_cap);
+      run += v[j];
+      if (k == n - 1) w.bin_off[n] = run;
+    }
+  }
+}
+
+// One warp per bin copies its slots; the last block appends the beads that
+// found their slots full.
+__global__ void __launch_bounds__(256) k_sort_records(const __grid_constant__ WorldDev w, int off) {
+  const int* counts = step_counts(w, *w.t + off);
+  if (blockIdx.x == gridDim.x - 1) {
+    const int n = counts[w.n_bins];
+    for (int k = threadIdx.x; k < n; k += blockDim.x) {
+      const int src = w.n_bins * w.slot_cap + k;
+      const float4 p = w.bpos[src];
+      const int bin = (cell_y(p) / kBin) * w.nbx + cell_x(p) / kBin;
+      const int dst = atomicAdd(&w.bin_cursor[bin], 1);
+      w.spos[dst] = p;
+      w.srec[dst] = w.brec[src];
+    }
+    return;
+  }
+  const int bin = (int)blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (bin >= w.n_bins) return;
+  const int n = min(counts[bin], w.slot_cap), dst = w.bin_off[bin];
+  for (int k = threadIdx.x & 31; k < n; k += 32) {
+    w.spos[dst + k] = w.bpos[bin * w.slot_cap + k];
+    w.srec[dst + k] = w.brec[bin * w.slot_cap + k];
+  }
+}
+
+// The inverse for the last completed step (its counts start at zero).
+__global__ void __launch_bounds__(256) k_unsort_records(const __grid_constant__ WorldDev w) {
+  int* counts = step_counts(w, *w.t - 1);
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= w.bin_off[w.n_bins]) return;
+  const float4 p = w.spos[k];
+  const int bin = (cell_y(p) / kBin) * w.nbx + cell_x(p) / kBin;
+  const int at = atomicAdd(&counts[bin], 1);
+  const int slot = at < w.slot_cap ? bin * w.slot_cap + at : w.n_bins * w.slot_cap + atomicAdd(&counts[w.n_bins], 1);
+  const float4 rec = w.srec[k];
+  w.bpos[slot] = p;
+  w.brec[slot] = rec;
+  if (w.bead_slot) w.bead_slot[__float_as_int(rec.z)] = slot;
 }
 
 // ---------------------------------------------------------------------------
@@ -38,7 +136,7 @@ __global__ void __launch_bounds__(256) k_scan_apply(const WorldDev* __restrict__
 // evaluated per opposite pair (i, opp(i)) from the even and odd parts.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kCellChunk) k_lbm(const WorldDev* __restrict__ worlds,
-                                                    const int2* __restrict__ items, int layered_only) {
+                                                    const int2* __restrict__ items, int layered_only, int off) {
   pdl_trigger();
   pdl_wait();
   const int2 it = items[blockIdx.x];
@@ -50,7 +148,7 @@ __global__ void __launch_bounds__(kCellChunk) k_lbm(const WorldDev* __restrict__
   const int y = c / W, x = c - y * W;
   const int xm = x == 0 ? W - 1 : x - 1, xp = x == W - 1 ? 0 : x + 1;
   const int ym = y == 0 ? H - 1 : y - 1, yp = y == H - 1 ? 0 : y + 1;
-  const long long t = *w.t;
+  const long long t = *w.t + off;
   const LbmConst k{w.om_p, w.om_m, w.src_p, w.src_m};
   w.u[c] = lbm_cell(w.g[t & 1], w.g[(t + 1) & 1], HW, y * W, ym * W, yp * W, x, xm, xp, w.F[c], k);
 }
@@ -58,26 +156,30 @@ __global__ void __launch_bounds__(kCellChunk) k_lbm(const WorldDev* __restrict__
 // ---------------------------------------------------------------------------
 // Launchers and the step sequence.
 // ---------------------------------------------------------------------------
-void launch_bin_scan(const Plan& p, cudaStream_t s, int inc_t) {
-  // worlds of one scan block each need no block sums: one kernel (unless
-  // the launch configuration asks for two)
-  const int book = p.one_chunk && p.cfg.scan_kernels != 2 ? 1 : 0;
-  if (p.n_worlds == 1) {   // integer work only: the single-world path cannot change a result
-    if (!book) launch_pdl(k_scan_sums<true>, p.n_scan_items, 256, 0, s, p.d_worlds, p.d_scan_items, inc_t, p.h_world0);
-    launch_pdl(k_scan_apply<true>, p.n_scan_items, 256, 0, s, p.d_worlds, p.d_scan_items, book, inc_t, p.h_world0);
-  } else {
-    if (!book) launch_pdl(k_scan_sums<false>, p.n_scan_items, 256, 0, s, p.d_worlds, p.d_scan_items, inc_t, p.h_world0);
-    launch_pdl(k_scan_apply<false>, p.n_scan_items, 256, 0, s, p.d_worlds, p.d_scan_items, book, inc_t, p.h_world0);
-  }
+void launch_sorted_offsets(const Plan& p, cudaStream_t s, int off) {
+  const WorldDev& w = p.h_world0;
+  if (w.n_chunks > 1) k_scan_sums<<<w.n_chunks, 256, 0, s>>>(w, off);
+  k_scan_apply<<<w.n_chunks, 256, 0, s>>>(w, off);
 }
 
-void launch_lbm(const Plan& p, cudaStream_t s, int layered_only) {
-  if (p.n_cell_items) k_lbm<<<p.n_cell_items, kCellChunk, 0, s>>>(p.d_worlds, p.d_cell_items, layered_only);
+void launch_sorted_records(const Plan& p, cudaStream_t s, int off) {
+  const WorldDev& w = p.h_world0;
+  if (w.N) k_sort_records<<<(w.n_bins + 7) / 8 + 1, 256, 0, s>>>(w, off);
+}
+
+void launch_slots_from_sorted(const Plan& p, cudaStream_t s) {
+  const WorldDev& w = p.h_world0;
+  if (w.N) k_unsort_records<<<(w.N + 255) / 256, 256, 0, s>>>(w);
+}
+
+void launch_lbm(const Plan& p, cudaStream_t s, int layered_only, int off) {
+  if (p.n_cell_items) k_lbm<<<p.n_cell_items, kCellChunk, 0, s>>>(p.d_worlds, p.d_cell_items, layered_only, off);
 }
 
 // n steps; in plans without direct-forcing worlds every step after the
 // first runs its PBD fused with the previous step's advance (the same
-// arithmetic, one kernel and one position round trip fewer).
+// arithmetic, one kernel and one position round trip fewer), and the worlds'
+// counters move by n at the end.
 void enqueue_steps(const Plan& p, int n, cudaStream_t s) {
   if (p.any_mdf || n < 2) {
     for (int k = 0; k < n; ++k) enqueue_step(p, s);
@@ -85,13 +187,11 @@ void enqueue_steps(const Plan& p, int n, cudaStream_t s) {
   }
   for (int k = 0; k < n; ++k) {
     if (k == 0) launch_pbd(p, s);
-    else launch_advance_pbd(p, s);   // a8 of step k - 1 + a1-a3 of step k
-    launch_bin_scan(p, s, k > 0);
-    launch_bin_scatter(p, s);
-    launch_deposit_x(p, s, 0);
-    launch_force_lbm(p, s);
+    else launch_advance_pbd(p, s, k, k == n - 1);   // a8 of step k - 1 + a1-a3 of step k
+    launch_deposit_x(p, s, 0, k);
+    launch_force_lbm(p, s, k, k == n - 1);
   }
-  launch_interp_advance(p, s);
+  launch_interp_advance(p, s, n);
 }
 
 void enqueue_step(const Plan& p, cudaStream_t s) {
@@ -101,8 +201,6 @@ void enqueue_step(const Plan& p, cudaStream_t s) {
     // unfused sequence, which gives their step bitwise)
     launch_pbd(p, s);
     launch_mdf_bins(p, s);
-    launch_bin_scan(p, s);
-    launch_bin_scatter(p, s);
     launch_deposit_x(p, s, 0);
     launch_force_spread(p, s, 0);
     launch_mdf(p, s);
@@ -110,9 +208,7 @@ void enqueue_step(const Plan& p, cudaStream_t s) {
     launch_interp_advance(p, s);
     return;
   }
-  launch_pbd(p, s);              // a1 + a3 + a2 histogram
-  launch_bin_scan(p, s);         // a2 offsets (one or two kernels)
-  launch_bin_scatter(p, s);      // a2 scatter
+  launch_pbd(p, s);              // a1 + a3 + a2
   launch_deposit_x(p, s, 0);     // a4 + x pass of a5
   launch_force_lbm(p, s);        // y pass of a5 + a6 + a7
   launch_interp_advance(p, s);   // a8

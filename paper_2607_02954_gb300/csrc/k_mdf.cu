@@ -5,12 +5,12 @@
 //
 //   k_mdf_bins      bins of X (a2) and F_el = 0, so the steric spread that
 //                   follows puts only F_s on the grid;
-//   (bins, deposit, steric spread: the penalty path's kernels)
+//   (deposit, steric spread: the penalty path's kernels)
 //   k_mdf_moments   u* = (sum_i c_i f_i + F/2) / rho and rho of every cell
 //                   (the fluid before the filament's forcing, in u);
 //   k_pbd<.., 2>    X~ = X + dt I[u*](X), PBD from X~, and each bead's
 //                   velocity U_s = I[u*](X) + (x_hat - X~)/dt (in ubead,
-//                   and in bin order in sus);
+//                   and by slot in sus);
 //   m passes of     k_mdf_pass (k_steric.cu), one per 32x32 tile, Jacobi in
 //                   u (u -> u2 -> u ...): dF_i = 2 I[rho](X_i) (U_s,i -
 //                   I[u](X_i)) for every bead whose stencil reaches the
@@ -22,15 +22,15 @@
 //   kernels, the advance reading U_s).
 // Every kernel returns at once for the worlds of a batch that couple by
 // the penalty force (and for a world's passes beyond its own m).
-#include "mc_internal.cuh"
+#include "bead_dev.cuh"
 
 namespace mc {
 
 namespace {
 
-// a2 for a direct-forcing world: the bin of every bead from X (its PBD runs
-// after the steric spread), one histogram atomic per group of lanes sharing
-// a bin, and F_el = 0 (the MDF passes accumulate the bead forces in it).
+// a2 for a direct-forcing world: every bead of X into its bin (its PBD runs
+// after the steric spread), and F_el = 0 (the MDF passes accumulate the bead
+// forces in it).
 __global__ void __launch_bounds__(kBeadChunk) k_mdf_bins(const WorldDev* __restrict__ worlds,
                                                          const int2* __restrict__ items) {
   pdl_trigger();
@@ -39,16 +39,17 @@ __global__ void __launch_bounds__(kBeadChunk) k_mdf_bins(const WorldDev* __restr
   const WorldDev& w = worlds[it.x];
   if (w.ib != 1) return;
   const int i = it.y + threadIdx.x;
-  const int lane = threadIdx.x & 31;
-  int bin = -1 - lane;
-  if (i < w.N) {
-    const float4 p = w.pos[i];
-    bin = (cell_y(p) / kBin) * w.nbx + cell_x(p) / kBin;
+  const bool valid = i < w.N;
+  int* counts = step_counts(w, *w.t);
+  const float4 p = valid ? w.pos[i] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  const int bin = bead_bin_of(p, w.nbx);
+  const BinClaim c = bin_claim(counts, valid, bin);
+  if (valid) {
     w.bead_bin[i] = bin;
     w.fel[i] = make_float2(0.0f, 0.0f);
   }
-  const unsigned peers = __match_any_sync(0xffffffffu, bin);
-  if (i < w.N && (__ffs(peers) - 1) == lane) atomicAdd(&w.bin_count[bin], __popc(peers));
+  const int slot = bin_place(w, counts, valid, c);
+  if (valid) bin_store(w, slot, i, p, make_float2(0.0f, 0.0f));
 }
 
 // u* and rho of every cell from the pulled populations and the steric F.

@@ -14,7 +14,6 @@
 // beads (register PBD), Gaussian half width 4 (sigma in (0.75, 1]); the
 // autotuner offers this path only for such plans.
 #include "bead_dev.cuh"
-#include "grid_dev.cuh"
 #include "steric_dev.cuh"
 
 namespace mc {
@@ -77,7 +76,6 @@ template <int R>
 union PersistSmem {
   ForceSmem<R> force;
   DepositSmem<R> deposit;
-  ScanSmem scan;
 };
 
 }  // namespace
@@ -91,9 +89,6 @@ struct PersistArgs {
   int n_bead_items;
   const int2* tile_items;
   int n_tile_items;
-  const int2* scan_items;
-  int n_scan_items;
-  int one_chunk;
   int n_steps;
   unsigned* bar;       // [2] barrier words, zeroed before the launch
   unsigned* status;    // set to 1 when a barrier wait ran out
@@ -111,46 +106,30 @@ __global__ void __launch_bounds__(256, kBlocks) k_step_persistent(const PersistA
   auto barrier = [&]() { return grid_barrier(a.bar, gen, target, a.timeout_ns, a.status, &s_ok); };
   bool ok = true;
   for (int s = 0; s < a.n_steps && ok; ++s) {
-    // a1-a3 (fused with the previous step's a8 after the first step)
+    // a1-a3 with the binning (fused with the previous step's a8 after the first step)
+    const int fields = s == a.n_steps - 1;
     for (unsigned b = blockIdx.x; b < (unsigned)a.n_pbd_blocks; b += gridDim.x) {
-      if (s == 0) pbd_body<kExt, 0, false>(a.worlds, a.fil_items, a.n_fil_items, 0, b);
-      else pbd_body<kExt, 1, false>(a.worlds, a.fil_items, a.n_fil_items, 0, b);
+      if (s == 0) pbd_body<kExt, 0, false>(a.worlds, a.fil_items, a.n_fil_items, 0, s, fields, b);
+      else pbd_body<kExt, 1, false>(a.worlds, a.fil_items, a.n_fil_items, 0, s, fields, b);
     }
-    if (!(ok = barrier())) break;
-    // a2 bin offsets
-    if (!a.one_chunk) {
-      for (unsigned b = blockIdx.x; b < (unsigned)a.n_scan_items; b += gridDim.x) {
-        __syncthreads();
-        scan_sums_body<false>(a.worlds, a.scan_items, s > 0, w1, b, sm.scan);
-      }
-      if (!(ok = barrier())) break;
-    }
-    for (unsigned b = blockIdx.x; b < (unsigned)a.n_scan_items; b += gridDim.x) {
-      __syncthreads();
-      scan_apply_body<false>(a.worlds, a.scan_items, a.one_chunk, s > 0, w1, b, sm.scan);
-    }
-    if (!(ok = barrier())) break;
-    // a2 scatter
-    for (unsigned b = blockIdx.x; b < (unsigned)a.n_bead_items; b += gridDim.x)
-      bin_scatter_body<false>(a.worlds, a.bead_items, w1, b);
     if (!(ok = barrier())) break;
     // a4 + x pass of a5
     for (unsigned b = blockIdx.x; b < (unsigned)a.n_tile_items; b += gridDim.x) {
       __syncthreads();
-      deposit_x_body<R, false>(a.worlds, a.tile_items, 0, w1, b, sm.deposit);
+      deposit_x_body<R, false>(a.worlds, a.tile_items, 0, s, w1, b, sm.deposit);
     }
     if (!(ok = barrier())) break;
     // y pass of a5 + a6 + a7
     for (unsigned b = blockIdx.x; b < (unsigned)a.n_tile_items; b += gridDim.x) {
       __syncthreads();
-      force_lbm_body<R, false>(a.worlds, a.tile_items, w1, b, sm.force);
+      force_lbm_body<R, false>(a.worlds, a.tile_items, s, fields, w1, b, sm.force);
     }
     if (!(ok = barrier())) break;
   }
   if (ok) {
     // a8 of the last step
     for (unsigned b = blockIdx.x; b < (unsigned)a.n_bead_items; b += gridDim.x)
-      interp_advance_body<kExt, false>(a.worlds, a.bead_items, b);
+      interp_advance_body<kExt, false>(a.worlds, a.bead_items, a.n_steps, b);
     return;
   }
   // a barrier wait ran out: flag every world of the plan
@@ -217,9 +196,6 @@ cudaError_t launch_persistent(const Plan& p, int n, cudaStream_t s) {
   a.n_bead_items = p.n_bead_items;
   a.tile_items = p.d_tile_items;
   a.n_tile_items = p.n_tile_items;
-  a.scan_items = p.d_scan_items;
-  a.n_scan_items = p.n_scan_items;
-  a.one_chunk = p.one_chunk && p.cfg.scan_kernels != 2 ? 1 : 0;
   a.n_steps = n;
   a.bar = p.d_persist_bar;
   a.status = p.d_persist_bar + 2;

@@ -18,15 +18,13 @@
 // k_force_lbm    does the same and then the LBM step (a7) of the tile's
 //                cells with F taken from shared memory: the step's path.
 //
-// Beads are sorted by 8x8-cell bins in row-major order, so the beads that
-// can reach a tile lie in a few contiguous segments of the sorted arrays,
-// one per bin row (two where the row range wraps around the periodic edge).
-// The force kernel stages grid windows and bead records in shared memory
-// with cp.async, every copy in flight at once, and lists the staged beads
-// whose stencil reaches the tile first (a block-wide compaction), so its
-// per-bead arithmetic runs on full warps.  The deposit, whose per-bead work
-// is 16 atomics, reads each record straight into registers and lets the
-// beads that miss the region drop out.
+// The step's PBD has put every bead's record into a slot of its 8x8-cell bin,
+// so the beads that can reach a tile lie in the slots of at most 8 x 8 bins.
+// The force kernel stages its grid window in shared memory with cp.async,
+// reads the bead records straight from their slots meanwhile and packs those
+// whose stencil reaches the tile (a block-wide compaction), so its per-bead
+// arithmetic runs on full warps.  The deposit, whose per-bead work is 16
+// atomics, lets the beads that miss the region drop out.
 //
 // Both kernels are compiled for each filter half width R (1..8) so that the
 // filter loops unroll with the taps in registers; a launch uses the largest R
@@ -52,18 +50,18 @@ namespace mc {
 template <int R, bool kSingle>
 __global__ void __launch_bounds__(kThreads, 8) k_deposit_x(const WorldDev* __restrict__ worlds,
                                                         const int2* __restrict__ items, int store_fields,
-                                                        const __grid_constant__ WorldDev w1) {
+                                                        int off, const __grid_constant__ WorldDev w1) {
   pdl_trigger();
   pdl_wait();
   __shared__ __align__(16) DepositSmem<R> sm;
-  deposit_x_body<R, kSingle>(worlds, items, store_fields, w1, blockIdx.x, sm);
+  deposit_x_body<R, kSingle>(worlds, items, store_fields, off, w1, blockIdx.x, sm);
 }
 
 // y pass of a5 + a6: writes F.
 template <int R>
 __global__ void __launch_bounds__(kThreads) k_force_spread(const WorldDev* __restrict__ worlds,
                                                            const int2* __restrict__ items, int store_fields,
-                                                           int after_step) {
+                                                           int off) {
   pdl_trigger();
   pdl_wait();
   __shared__ __align__(16) ForceSmem<R> sm;
@@ -72,7 +70,7 @@ __global__ void __launch_bounds__(kThreads) k_force_spread(const WorldDev* __res
   const TileBox tb = tile_box(w, it.y);
   float2* __restrict__ F_out = w.F;
   const int W = w.W;
-  const int k = force_tile<R>(sm, w, (tb.y0 / kTile) * w.ntx + tb.x0 / kTile, tb, store_fields, after_step);
+  const int k = force_tile<R>(sm, w, (tb.y0 / kTile) * w.ntx + tb.x0 / kTile, tb, store_fields, off, true);
   __syncthreads();
   force_fold(sm.wk, tb, w.ntx, w.nty);
   const float inv = pow2f(-k);
@@ -90,7 +88,7 @@ __global__ void __launch_bounds__(kThreads) k_force_spread(const WorldDev* __res
 
 template <int R, bool kSingle>
 __global__ void __launch_bounds__(kThreads, 4) k_force_lbm(const WorldDev* __restrict__ worlds,
-                                                           const int2* __restrict__ items,
+                                                           const int2* __restrict__ items, int off, int fields,
                                                            const __grid_constant__ WorldDev w1) {
   pdl_trigger();
   pdl_wait();
@@ -99,7 +97,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_force_lbm(const WorldDev* __res
   // still in L2 when the next PBD (filaments in index order) interpolates
   // them, and the last rows' x-filtered densities, which the deposit wrote
   // last, are read first
-  force_lbm_body<R, kSingle>(worlds, items, w1, gridDim.x - 1 - blockIdx.x, sm);
+  force_lbm_body<R, kSingle>(worlds, items, off, fields, w1, gridDim.x - 1 - blockIdx.x, sm);
 }
 
 // y pass of a5 + a6 + a7, warp-specialised and persistent: each block walks
@@ -128,7 +126,7 @@ constexpr int kWsFull = 3, kWsEmpty = 4;
 
 template <int R, bool kSingle>
 __global__ void __launch_bounds__(kThreads, 4) k_force_lbm_ws(const WorldDev* __restrict__ worlds,
-                                                              const int2* __restrict__ items, int n_items,
+                                                              const int2* __restrict__ items, int n_items, int off, int fields,
                                                               const __grid_constant__ WorldDev w1) {
   pdl_trigger();
   pdl_wait();
@@ -141,13 +139,13 @@ __global__ void __launch_bounds__(kThreads, 4) k_force_lbm_ws(const WorldDev* __
     const WorldDev& w = kSingle ? w1 : worlds[it.x];
     const TileBox tb = tile_box(w, it.y);
     if (force_group) {
-      prefetch_populations<kWsForce>(w, tb);
+      prefetch_populations<kWsForce>(w, tb, off);
       const int tile = (tb.y0 / kTile) * w.ntx + tb.x0 / kTile;
       int k = 40;
       if (!kSingle && w.tile_rho_max[tile] == 0.0f) {
         tile_clear<kWsForce>(sm.f.wk);   // no bead reaches the tile: F = 0 (see k_force_lbm)
       } else {
-        k = force_tile<R, kWsForce>(sm.f, w, tile, tb, 0, 0);
+        k = force_tile<R, kWsForce>(sm.f, w, tile, tb, 0, off, fields);
       }
       force_sync<kWsForce>();
       force_fold<TileWork, kWsForce>(sm.f.wk, tb, w.ntx, w.nty);
@@ -161,7 +159,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_force_lbm_ws(const WorldDev* __
       ws_bar_arrive(kWsFull);
     } else {
       const int W = w.W, H = w.H, HW = H * W;
-      const long long t = *w.t;
+      const long long t = *w.t + off;
       const float* __restrict__ src = w.g[t & 1];
       float* __restrict__ dst = w.g[(t + 1) & 1];
       float2* __restrict__ u_out = w.u;
@@ -217,7 +215,7 @@ struct MdfSmem {
   int accy[kAx * kAx];
   int list[kForceCap];
   int s_cnt;
-  int s_start[kMaxSeg], s_pre[kMaxSeg + 1];
+  Segments sg;
   float red[kWarps];
 };
 
@@ -256,10 +254,10 @@ __device__ __forceinline__ int mdf_stage_chunk(MdfSmem& sm, const WorldDev& w, c
   const int W = w.W, H = w.H, ntx = w.ntx, nty = w.nty;
   const int n = min(kForceCap, total - c0);
   for (int v = tid; v < n; v += kThreads) {
-    const int slot = seg_slot(c0 + v, sm.s_start, sm.s_pre);
-    cp_async16(&sm.sp[v], &w.spos[slot]);
+    const int slot = seg_slot(c0 + v, sm.sg);
+    cp_async16(&sm.sp[v], &w.bpos[slot]);
     cp_async8(&sm.su[v], &w.sus[slot]);
-    cp_async4(&sm.si[v], reinterpret_cast<const int*>(&w.srec[slot]) + 2);   // the record's id
+    cp_async4(&sm.si[v], reinterpret_cast<const int*>(&w.brec[slot]) + 2);   // the record's id
   }
   cp_async_wait_all();
   if (tid == 0) sm.s_cnt = 0;
@@ -282,7 +280,8 @@ __device__ __forceinline__ int mdf_stage_chunk(MdfSmem& sm, const WorldDev& w, c
         keep = keep && ry <= tb.th;
       }
     }
-    list_push(keep, pack_code(v, rx, ry), sm.list, &sm.s_cnt);
+    const int at = list_place(keep, &sm.s_cnt);
+    if (keep) sm.list[at] = pack_code(v, rx, ry);
   }
   __syncthreads();
   return sm.s_cnt;
@@ -302,7 +301,8 @@ __global__ void __launch_bounds__(kThreads) k_mdf_pass(const WorldDev* __restric
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float2* __restrict__ u_in = (pass & 1) ? w.u2 : w.u;
   float2* __restrict__ u_out = (pass & 1) ? w.u : w.u2;
-  if (warp == 0) build_segments(w, tb.x0 - 2, tb.x0 + tb.tw, tb.y0 - 2, tb.y0 + tb.th, sm.s_start, sm.s_pre, nullptr);
+  if (warp == 0)
+    build_segments(w, step_counts(w, *w.t), tb.x0 - 2, tb.x0 + tb.tw, tb.y0 - 2, tb.y0 + tb.th, sm.sg);
   // the velocity and density windows, rows y0 - 3 .. y0 + th + 2 and
   // columns x0 - 4 .. x0 + tw + 3, periodic (W, H >= 8: one wrap at most),
   // in 16-byte chunks (2 velocities or 4 densities; x0 and W are multiples
@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(kThreads) k_mdf_pass(const WorldDev* __restric
     reinterpret_cast<int4*>(sm.accy)[c] = make_int4(0, 0, 0, 0);
   }
   __syncthreads();   // segments visible (the windows land with the first chunk's wait)
-  const int total = sm.s_pre[kMaxSeg];
+  const int total = sm.sg.pre[kSegs];
   const bool one_pass = total <= kForceCap;
   // sweep 1: dF of every listed bead and their largest component
   float m = 0.0f;
@@ -430,41 +430,41 @@ void ws_setup(int sms) {
 }
 
 template <int R>
-void launch_steric(const Plan& p, cudaStream_t s, int which, int store_fields, int after_step) {
+void launch_steric(const Plan& p, cudaStream_t s, int which, int store_fields, int off, int fields = 1) {
   if (which == 0) {
     if (p.n_worlds == 1)
-      launch_pdl(k_deposit_x<R, true>, p.n_tile_items, kThreads, 0, s, p.d_worlds, p.d_tile_items, store_fields, p.h_world0);
+      launch_pdl(k_deposit_x<R, true>, p.n_tile_items, kThreads, 0, s, p.d_worlds, p.d_tile_items, store_fields, off, p.h_world0);
     else
-      launch_pdl(k_deposit_x<R, false>, p.n_tile_items, kThreads, 0, s, p.d_worlds, p.d_tile_items, store_fields, p.h_world0);
+      launch_pdl(k_deposit_x<R, false>, p.n_tile_items, kThreads, 0, s, p.d_worlds, p.d_tile_items, store_fields, off, p.h_world0);
   } else if (which == 1) {
-    k_force_spread<R><<<p.n_tile_items, kThreads, 0, s>>>(p.d_worlds, p.d_tile_items, store_fields, after_step);
+    k_force_spread<R><<<p.n_tile_items, kThreads, 0, s>>>(p.d_worlds, p.d_tile_items, store_fields, off);
   } else if (p.cfg.force_ws && !p.any_layered) {
     const int grid = std::min(p.n_tile_items, ws_grid<R>());
     if (p.n_worlds == 1)
       launch_pdl(k_force_lbm_ws<R, true>, grid, kThreads, sizeof(WsSmem<R>), s, p.d_worlds, p.d_tile_items,
-                 p.n_tile_items, p.h_world0);
+                 p.n_tile_items, off, fields, p.h_world0);
     else
       launch_pdl(k_force_lbm_ws<R, false>, grid, kThreads, sizeof(WsSmem<R>), s, p.d_worlds, p.d_tile_items,
-                 p.n_tile_items, p.h_world0);
+                 p.n_tile_items, off, fields, p.h_world0);
   } else {
     if (p.n_worlds == 1)
-      launch_pdl(k_force_lbm<R, true>, p.n_tile_items, kThreads, 0, s, p.d_worlds, p.d_tile_items, p.h_world0);
+      launch_pdl(k_force_lbm<R, true>, p.n_tile_items, kThreads, 0, s, p.d_worlds, p.d_tile_items, off, fields, p.h_world0);
     else
-      launch_pdl(k_force_lbm<R, false>, p.n_tile_items, kThreads, 0, s, p.d_worlds, p.d_tile_items, p.h_world0);
+      launch_pdl(k_force_lbm<R, false>, p.n_tile_items, kThreads, 0, s, p.d_worlds, p.d_tile_items, off, fields, p.h_world0);
   }
 }
 
-void dispatch_steric(const Plan& p, cudaStream_t s, int which, int store_fields, int after_step) {
+void dispatch_steric(const Plan& p, cudaStream_t s, int which, int store_fields, int off, int fields = 1) {
   if (!p.n_tile_items) return;
   switch (p.max_R) {
-    case 1: launch_steric<1>(p, s, which, store_fields, after_step); break;
-    case 2: launch_steric<2>(p, s, which, store_fields, after_step); break;
-    case 3: launch_steric<3>(p, s, which, store_fields, after_step); break;
-    case 4: launch_steric<4>(p, s, which, store_fields, after_step); break;
-    case 5: launch_steric<5>(p, s, which, store_fields, after_step); break;
-    case 6: launch_steric<6>(p, s, which, store_fields, after_step); break;
-    case 7: launch_steric<7>(p, s, which, store_fields, after_step); break;
-    default: launch_steric<kMaxR>(p, s, which, store_fields, after_step); break;
+    case 1: launch_steric<1>(p, s, which, store_fields, off, fields); break;
+    case 2: launch_steric<2>(p, s, which, store_fields, off, fields); break;
+    case 3: launch_steric<3>(p, s, which, store_fields, off, fields); break;
+    case 4: launch_steric<4>(p, s, which, store_fields, off, fields); break;
+    case 5: launch_steric<5>(p, s, which, store_fields, off, fields); break;
+    case 6: launch_steric<6>(p, s, which, store_fields, off, fields); break;
+    case 7: launch_steric<7>(p, s, which, store_fields, off, fields); break;
+    default: launch_steric<kMaxR>(p, s, which, store_fields, off, fields); break;
   }
 }
 
@@ -481,11 +481,13 @@ void steric_setup(int sms) {
   ws_setup<8>(sms);
 }
 
-void launch_deposit_x(const Plan& p, cudaStream_t s, int store_fields) { dispatch_steric(p, s, 0, store_fields, 0); }
+void launch_deposit_x(const Plan& p, cudaStream_t s, int store_fields, int off) {
+  dispatch_steric(p, s, 0, store_fields, off);
+}
 
 // Two-layer worlds get F from their layer points after the tile pass.
-void launch_force_spread(const Plan& p, cudaStream_t s, int store_fields, int after_step) {
-  dispatch_steric(p, s, 1, store_fields, after_step);
+void launch_force_spread(const Plan& p, cudaStream_t s, int store_fields, int off) {
+  dispatch_steric(p, s, 1, store_fields, off);
   launch_layer_spread(p, s);
 }
 
@@ -493,11 +495,11 @@ void launch_mdf_pass(const Plan& p, cudaStream_t s, int pass) {
   if (p.n_tile_items) k_mdf_pass<<<p.n_tile_items, kThreads, 0, s>>>(p.d_worlds, p.d_tile_items, pass);
 }
 
-void launch_force_lbm(const Plan& p, cudaStream_t s) {
-  dispatch_steric(p, s, 2, 0, 0);
+void launch_force_lbm(const Plan& p, cudaStream_t s, int off, int fields) {
+  dispatch_steric(p, s, 2, 0, off, fields);
   if (p.any_layered) {
     launch_layer_spread(p, s);
-    launch_lbm(p, s, 1);
+    launch_lbm(p, s, 1, off);
   }
 }
 

@@ -242,10 +242,8 @@ StoredLayout stored_layout(const mc::WorldDev& h, int n) {
 // binding the step's fields to its record (bind_step).
 void run_recorded_step(const mc::Plan& p, cudaStream_t s) {
   mc::launch_pbd(p, s);
-  mc::launch_bin_scan(p, s);
-  mc::launch_bin_scatter(p, s);
   mc::launch_deposit_x(p, s, 0);
-  mc::launch_force_spread(p, s, 1, 0);
+  mc::launch_force_spread(p, s, 1);
   mc::launch_lbm(p, s);
   mc::launch_interp_advance(p, s);
 }
@@ -259,11 +257,9 @@ mc_status mdf_recorded_step(mc_world* w, char* seg, const StepSlot& ss, int q, i
                             cudaStream_t s) {
   const mc::WorldDev& h = w->h;
   mc::launch_mdf_bins(w->plan, s);
-  mc::launch_bin_scan(w->plan, s);
-  mc::launch_bin_scatter(w->plan, s);
   mc::launch_deposit_x(w->plan, s, 0);
-  mc::launch_force_spread(w->plan, s, 0, 0);
-  mc::launch_force_spread(w->plan, s, 1, 0);
+  mc::launch_force_spread(w->plan, s, 0);
+  mc::launch_force_spread(w->plan, s, 1);
   MC_ACUDA(mc::launch_mdf_recorded(w->plan, h, reinterpret_cast<float2*>(seg + (size_t)q * ss.bytes + ss.mu), s));
   mc::launch_lbm(w->plan, s);
   mc::launch_interp_advance(w->plan, s);

@@ -154,8 +154,7 @@ mc_status build_plan(mc_world* const* ws, int n, cudaStream_t s, Plan& out) {
   p.any_mdf = false;
   p.max_mdf = 0;
   p.any_ext = false;
-  p.one_chunk = true;
-  std::vector<int2> fil, bead, tile, cell, scan;
+  std::vector<int2> fil, bead, tile, cell;
   std::vector<WorldDev> table(n);
   for (int k = 0; k < n; ++k) {
     const mc_world* w = ws[k];
@@ -166,13 +165,11 @@ mc_status build_plan(mc_world* const* ws, int n, cudaStream_t s, Plan& out) {
     p.any_mdf = p.any_mdf || w->h.ib == 1;
     p.max_mdf = std::max(p.max_mdf, w->h.mdf_iters);
     p.any_ext = p.any_ext || w->h.layers == 2 || w->h.observe || w->h.has_ldrive || w->h.ib == 1;
-    p.one_chunk = p.one_chunk && w->h.n_chunks <= 1;
     for (int f = 0; f < w->h.n_fil; ++f) fil.push_back(make_int2(k, f));
     const int nb = std::max(w->h.N, 1);
     for (int b = 0; b < nb; b += mc::kBeadChunk) bead.push_back(make_int2(k, b));
     for (int ty = 0; ty < w->h.nty; ++ty)   // tile items carry (tx, ty) packed: tx | ty << 16
       for (int tx = 0; tx < w->h.ntx; ++tx) tile.push_back(make_int2(k, tx | (ty << 16)));
-    for (int c = 0; c < w->h.n_chunks; ++c) scan.push_back(make_int2(k, c));
     const int HW = w->h.H * w->h.W;
     for (int c = 0; c < HW; c += mc::kCellChunk) cell.push_back(make_int2(k, c));
   }
@@ -182,7 +179,6 @@ mc_status build_plan(mc_world* const* ws, int n, cudaStream_t s, Plan& out) {
   const size_t o_b = L.take<int2>(bead.size());
   const size_t o_t = L.take<int2>(tile.size());
   const size_t o_c = L.take<int2>(cell.size());
-  const size_t o_s = L.take<int2>(scan.size());
   const size_t o_bar = L.take<unsigned>(4);
   std::vector<char> host(L.off);
   std::memcpy(host.data() + o_w, table.data(), n * sizeof(WorldDev));
@@ -190,7 +186,6 @@ mc_status build_plan(mc_world* const* ws, int n, cudaStream_t s, Plan& out) {
   std::memcpy(host.data() + o_b, bead.data(), bead.size() * sizeof(int2));
   if (!tile.empty()) std::memcpy(host.data() + o_t, tile.data(), tile.size() * sizeof(int2));
   std::memcpy(host.data() + o_c, cell.data(), cell.size() * sizeof(int2));
-  std::memcpy(host.data() + o_s, scan.data(), scan.size() * sizeof(int2));
   cudaError_t e = cudaMallocAsync(&p.d_mem, L.off, s);
   if (e != cudaSuccess) return fail(MC_ERR_OOM, std::string("plan allocation: ") + cudaGetErrorString(e));
   e = cudaMemcpyAsync(p.d_mem, host.data(), L.off, cudaMemcpyHostToDevice, s);
@@ -201,13 +196,11 @@ mc_status build_plan(mc_world* const* ws, int n, cudaStream_t s, Plan& out) {
   p.d_bead_items = at<int2>(p.d_mem, o_b);
   p.d_tile_items = at<int2>(p.d_mem, o_t);
   p.d_cell_items = at<int2>(p.d_mem, o_c);
-  p.d_scan_items = at<int2>(p.d_mem, o_s);
   p.d_persist_bar = at<unsigned>(p.d_mem, o_bar);
   p.n_fil_items = (int)fil.size();
   p.n_bead_items = (int)bead.size();
   p.n_tile_items = (int)tile.size();
   p.n_cell_items = (int)cell.size();
-  p.n_scan_items = (int)scan.size();
   if (n == 1) p.h_world0 = table[0];
   out = p;
   return MC_OK;
@@ -319,11 +312,18 @@ void world_sizes(WorldDev& h, int H, int W, int n_fil, int N) {
   h.nty = (H + kTile - 1) / kTile;
   h.n_tiles = h.ntx * h.nty;
   h.n_chunks = (h.n_bins + kScanChunk - 1) / kScanChunk;
+  // slots of a bin: twice the mean count and some more, at least 32 (beads
+  // of a chain are about a cell apart, so a chain crossing a bin leaves 8 to
+  // 11 in it); slot numbers stay below 2^31
+  const long long mean = ((long long)N + h.n_bins - 1) / h.n_bins;
+  const long long room = (0x7fffffffLL - N) / h.n_bins;
+  h.slot_cap = (int)std::min(std::max(32LL, (2 * mean + 24 + 7) & ~7LL), room);
 }
 
 // Places every array of a world inside one arena (256-byte aligned slices).
-// With A == nullptr only returns the arena size in bytes.
-size_t world_layout(WorldDev& h, void* A) {
+// With A == nullptr only returns its sizes.  A saved image holds the leading
+// arrays up to (not including) the step's binned beads.
+ArenaSize world_layout(WorldDev& h, void* A) {
   Layout L;
   const int N = h.N, E = h.E, J = h.J;
   const size_t HW = (size_t)h.H * h.W;
@@ -365,8 +365,18 @@ size_t world_layout(WorldDev& h, void* A) {
   const size_t o_mr = L.take<float>(df ? HW : 0);
   const size_t o_bs = L.take<int>(df ? N : 0);
   const size_t o_u2 = L.take<float2>(df ? HW : 0);
-  const size_t o_su = L.take<float2>(df ? N : 0);
-  if (!A) return L.off;
+  L.take<float2>(df ? N : 0);   // (unused: keeps the layout of saved images)
+  ArenaSize sz;
+  sz.image = L.off;
+  const size_t o_cnt = L.take<int>(2 * ((size_t)h.n_bins + 1));
+  sz.zero = L.off;
+  const size_t slots = (size_t)h.n_bins * h.slot_cap + N;
+  const size_t o_bp = L.take<float4>(slots);
+  const size_t o_br = L.take<float4>(slots);
+  const size_t o_ls = L.take<int>(h.layers == 2 ? N : 0);
+  const size_t o_su = L.take<float2>(df ? slots : 0);
+  sz.total = L.off;
+  if (!A) return sz;
   h.fil_off = at<int>(A, o_fo);
   h.pos = at<float4>(A, o_pos);
   h.disp = at<float2>(A, o_disp);
@@ -402,10 +412,13 @@ size_t world_layout(WorldDev& h, void* A) {
   h.nrm = h.layers == 2 ? at<float2>(A, o_nr) : nullptr;
   h.facc = h.layers == 2 ? at<unsigned long long>(A, o_fa) : nullptr;
   h.mrho = df ? at<float>(A, o_mr) : nullptr;
-  h.bead_slot = df ? at<int>(A, o_bs) : nullptr;
+  h.bead_slot = df ? at<int>(A, o_bs) : h.layers == 2 ? at<int>(A, o_ls) : nullptr;
+  h.bin_cnt = at<int>(A, o_cnt);
+  h.bpos = at<float4>(A, o_bp);
+  h.brec = at<float4>(A, o_br);
   h.u2 = df ? at<float2>(A, o_u2) : nullptr;
   h.sus = df ? at<float2>(A, o_su) : nullptr;
-  return L.off;
+  return sz;
 }
 
 // Plan and step helpers shared with the rollout server.
@@ -425,6 +438,7 @@ mc_world* world_clone(const mc_world* w, cudaStream_t s) {
   mc_world* c = new mc_world();
   c->h = w->h;
   c->bytes = w->bytes;
+  c->image_bytes = w->image_bytes;
   c->stream = s;
   c->t = w->t;
   c->max_B = w->max_B;
@@ -564,7 +578,9 @@ mc_status mc_world_create(const mc_world_desc* d, void* stream, mc_world** out) 
   h.has_energy = d->energy != nullptr;
   h.observe = d->observe;
 
-  w->bytes = mc::world_layout(h, nullptr);
+  const mc::ArenaSize sz = mc::world_layout(h, nullptr);
+  w->bytes = sz.total;
+  w->image_bytes = sz.image;
   cudaError_t e = world_alloc(&w->arena, w->bytes, s);
   if (e != cudaSuccess) {
     delete w;
@@ -583,7 +599,7 @@ mc_status mc_world_create(const mc_world_desc* d, void* stream, mc_world** out) 
     cudaError_t e_ = (call);                                             \
     if (e_ != cudaSuccess) return fail_free(cuda_fail(e_, #call));       \
   } while (0)
-  MC_CUDA_W(cudaMemsetAsync(A, 0, w->bytes, s));
+  MC_CUDA_W(cudaMemsetAsync(A, 0, sz.zero, s));
   const cudaMemcpyKind kind = on_host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
   auto up = [&](void* dst, const void* src, size_t n, cudaMemcpyKind k) {
     return n ? cudaMemcpyAsync(dst, src, n, k, s) : cudaSuccess;
@@ -652,9 +668,10 @@ mc_status mc_world_create(const mc_world_desc* d, void* stream, mc_world** out) 
 }
 
 // ---- checkpoint / resume --------------------------------------------------
-// Image of a world: a header, the filament offsets, then the device arena
-// byte for byte (it holds no pointers: the arrays are placed again from the
-// sizes on load).
+// Image of a world: a header, the filament offsets, then the leading arrays
+// of the device arena byte for byte (they hold no pointers: the arrays are
+// placed again from the sizes on load).  The last step's binned beads go in
+// bin order, and back into slots on load.
 namespace {
 struct SaveHeader {
   char magic[8];          // "MCWORLD1"
@@ -669,7 +686,7 @@ struct SaveHeader {
 constexpr char kSaveMagic[8] = {'M', 'C', 'W', 'O', 'R', 'L', 'D', '1'};
 
 size_t save_size(const mc_world* w) {
-  return sizeof(SaveHeader) + (size_t)(w->h.n_fil + 1) * sizeof(int) + w->bytes;
+  return sizeof(SaveHeader) + (size_t)(w->h.n_fil + 1) * sizeof(int) + w->image_bytes;
 }
 }  // namespace
 
@@ -695,12 +712,15 @@ mc_status mc_world_save(const mc_world* w, void* buf, size_t bytes, void* stream
   hd.observe = w->h.observe;
   hd.max_B = w->max_B;
   hd.t = w->t;
-  hd.arena_bytes = w->bytes;
+  hd.arena_bytes = w->image_bytes;
   hd.params = w->params;
   char* out = static_cast<char*>(buf);
   std::memcpy(out, &hd, sizeof(hd));
   std::memcpy(out + sizeof(hd), w->fil_off.data(), (size_t)(w->h.n_fil + 1) * sizeof(int));
-  MC_CUDA(cudaMemcpyAsync(out + sizeof(hd) + (size_t)(w->h.n_fil + 1) * sizeof(int), w->arena, w->bytes,
+  mc::launch_sorted_offsets(w->plan, s, -1);
+  mc::launch_sorted_records(w->plan, s, -1);
+  MC_CUDA(cudaGetLastError());
+  MC_CUDA(cudaMemcpyAsync(out + sizeof(hd) + (size_t)(w->h.n_fil + 1) * sizeof(int), w->arena, w->image_bytes,
                           cudaMemcpyDeviceToHost, s));
   MC_CUDA(cudaStreamSynchronize(s));
   return MC_OK;
@@ -739,8 +759,10 @@ mc_status mc_world_load(const void* buf, size_t bytes, void* stream, mc_world** 
   h.has_ldrive = hd.has_ldrive;
   h.has_energy = hd.has_energy;
   h.observe = hd.observe;
-  w->bytes = mc::world_layout(h, nullptr);
-  if (w->bytes != hd.arena_bytes || bytes < sizeof(hd) + fo_bytes + w->bytes) {
+  const mc::ArenaSize sz = mc::world_layout(h, nullptr);
+  w->bytes = sz.total;
+  w->image_bytes = sz.image;
+  if (w->image_bytes != hd.arena_bytes || bytes < sizeof(hd) + fo_bytes + w->image_bytes) {
     delete w;
     return fail(MC_ERR_INVALID_ARG, "world image size does not match its header");
   }
@@ -750,8 +772,10 @@ mc_status mc_world_load(const void* buf, size_t bytes, void* stream, mc_world** 
     return fail(MC_ERR_OOM, std::string("world allocation: ") + cudaGetErrorString(e));
   }
   mc::world_layout(h, w->arena);
-  e = cudaMemcpyAsync(w->arena, static_cast<const char*>(buf) + sizeof(hd) + fo_bytes, w->bytes,
-                      cudaMemcpyHostToDevice, w->stream);
+  e = cudaMemsetAsync(static_cast<char*>(w->arena) + sz.image, 0, sz.zero - sz.image, w->stream);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(w->arena, static_cast<const char*>(buf) + sizeof(hd) + fo_bytes, w->image_bytes,
+                        cudaMemcpyHostToDevice, w->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(w->stream);   // the caller may reuse the buffer at once
   if (e != cudaSuccess) {
     cudaFreeAsync(w->arena, w->stream);
@@ -765,6 +789,7 @@ mc_status mc_world_load(const void* buf, size_t bytes, void* stream, mc_world** 
     delete w;
     return st;
   }
+  mc::launch_slots_from_sorted(w->plan, w->stream);
   *out = w;
   return MC_OK;
 }
@@ -891,8 +916,8 @@ mc_status mc_step_stage(mc_world* w, int stage, void* stream) {
   const Plan& p = w->plan;
   switch (stage) {
     case 0: mc::launch_pbd(p, s); break;
-    case 1: mc::launch_bin_scan(p, s); break;
-    case 2: mc::launch_bin_scatter(p, s); break;
+    case 1: mc::launch_sorted_offsets(p, s, 0); break;
+    case 2: mc::launch_sorted_records(p, s, 0); break;
     case 3: mc::launch_deposit_x(p, s, 0); break;
     case 4: mc::launch_force_spread(p, s, 0); break;
     case 5: mc::launch_lbm(p, s); break;
@@ -963,8 +988,8 @@ mc_status mc_world_get_field(const mc_world* w, int field, void* out, int mem_ki
       // the step keeps these in shared memory only: re-run the steric
       // stages on the last step's binned beads with field output on (they
       // are deterministic, so rho_x, F and F_s are rewritten identically)
-      mc::launch_deposit_x(w->plan, s, field == MC_FIELD_RHO_S);
-      if (field == MC_FIELD_RHO_BAR) mc::launch_force_spread(w->plan, s, 1, 1);
+      mc::launch_deposit_x(w->plan, s, field == MC_FIELD_RHO_S, -1);
+      if (field == MC_FIELD_RHO_BAR) mc::launch_force_spread(w->plan, s, 1, -1);
       MC_CUDA(cudaGetLastError());
       src = field == MC_FIELD_RHO_S ? (const void*)h.rho_s : (const void*)h.rho_b;
       bytes = HW * sizeof(float);
@@ -973,15 +998,22 @@ mc_status mc_world_get_field(const mc_world* w, int field, void* out, int mem_ki
       // the step hands F from the spread to the collision in shared memory:
       // re-run the spread on the last step's binned beads (deterministic);
       // a direct-forcing step leaves its total F in device memory
-      if (h.ib != 1) mc::launch_force_spread(w->plan, s, 0, 1);
+      if (h.ib != 1) mc::launch_force_spread(w->plan, s, 0, -1);
       MC_CUDA(cudaGetLastError());
       src = h.F;
       bytes = HW * sizeof(float2);
       break;
     case MC_FIELD_U: src = h.u; bytes = HW * sizeof(float2); break;
     case MC_FIELD_BIN: src = h.bead_bin; bytes = h.N * sizeof(int); break;
-    case MC_FIELD_BIN_OFF: src = h.bin_off; bytes = (h.n_bins + 1) * sizeof(int); break;
+    case MC_FIELD_BIN_OFF:
+      mc::launch_sorted_offsets(w->plan, s, -1);
+      MC_CUDA(cudaGetLastError());
+      src = h.bin_off;
+      bytes = (h.n_bins + 1) * sizeof(int); break;
     case MC_FIELD_BIN_BEADS:   // the id word of each bin-ordered record
+      mc::launch_sorted_offsets(w->plan, s, -1);
+      mc::launch_sorted_records(w->plan, s, -1);
+      MC_CUDA(cudaGetLastError());
       if (h.N)
         MC_CUDA(cudaMemcpy2DAsync(out, sizeof(int), reinterpret_cast<const char*>(h.srec) + 2 * sizeof(float),
                                   sizeof(float4), sizeof(int), h.N, dk, s));
@@ -1035,8 +1067,7 @@ mc_status mc_world_check(const mc_world* w, void* stream) {
   MC_CUDA(cudaStreamSynchronize(s));
   if (flags & mc::kFlagTimeout)
     return fail(MC_ERR_TIMEOUT,
-                "a grid barrier of the persistent step or a wait for bulk copies ran out of time; the world's state is "
-                "unspecified");
+                "a grid barrier of the persistent step ran out of time; the world's state is unspecified");
   if (flags & mc::kFlagUnstable) return fail(MC_ERR_UNSTABLE, "bead velocity watchdog tripped (|U| > 0.5 or not finite)");
   return MC_OK;
 }

@@ -10,13 +10,14 @@
 
 namespace mc {
 
-// Beads are counting-sorted by 8x8-cell bins (row-major over the bin grid);
-// the steric kernels work on 32x32-cell tiles.  Grid sizes are multiples of
+// Beads are binned by 8x8 cells (row-major over the bin grid): a step's PBD
+// writes each bead's record into the next free slot of its bin; the steric
+// kernels work on 32x32-cell tiles.  Grid sizes are multiples of
 // 8, so bins are never ragged and ragged last tiles are at least 8 cells
 // wide.
 constexpr int kBin = 8;
 constexpr int kTile = 32;
-constexpr int kScanChunk = 1024;    // bins per block of the offset scan
+constexpr int kScanChunk = 1024;    // bins per block of the offset scan (sorted read-outs)
 constexpr int kMaxR = 8;            // Gaussian half width ceil(4 sigma) <= 8
 constexpr int kBeadChunk = 256;     // beads per block of the bead-parallel kernels
 constexpr int kCellChunk = 256;     // cells per block of the LBM kernel
@@ -31,7 +32,7 @@ constexpr int kMaxNpbd = 64;
 
 enum : unsigned {
   kFlagUnstable = 1u,   // the velocity watchdog tripped
-  kFlagTimeout = 2u     // a grid barrier of the persistent step, or a wait for bulk copies, ran out of time
+  kFlagTimeout = 2u     // a grid barrier of the persistent step ran out of time
 };
 
 // Everything the kernels need to know about one world.  Lives in device
@@ -57,12 +58,21 @@ struct WorldDev {
   float2* fs;             // [N]
   float2* ubead;          // [N]
   int* bead_bin;          // [N]
-  int* bin_count;         // [n_bins]
-  int* bin_off;           // [n_bins + 1]
-  int* bin_cursor;        // [n_bins]
-  int* chunk_sum;         // [n_chunks]
-  float4* spos;           // [N] positions in bin order
-  float4* srec;           // [N] per bead in bin order: F_el (x, y), bead id (int bits), 0
+  int* bin_count;         // [n_bins] (unused, zero: keeps the layout of saved images)
+  int* bin_off;           // [n_bins + 1] sorted read-out: exclusive prefix sum of the bin counts
+  int* bin_cursor;        // [n_bins] sorted read-out
+  int* chunk_sum;         // [n_chunks] sorted read-out
+  float4* spos;           // [N] sorted read-out: positions in bin order
+  float4* srec;           // [N] sorted read-out: the records in bin order
+  // The step's binned beads: bin b holds bin_cnt[par][b] beads, the first
+  // slot_cap of them in slots b slot_cap .. of bpos and brec; beads beyond
+  // that (bin_cnt[par][n_bins] of them in all) follow at n_bins slot_cap.
+  // The counts alternate by step parity par: the deposit of a step zeroes
+  // the other parity's for the next step.
+  int slot_cap;
+  int* bin_cnt;           // [2][n_bins + 1], the last entry of each: beads that found their bin's slots full
+  float4* bpos;           // [n_bins slot_cap + N] positions
+  float4* brec;           // [n_bins slot_cap + N] F_el (x, y), bead id (int bits), 0
   float* g[2];            // [9 * H * W] post-collision population deviations (ping-pong)
   float2* F;              // [H * W]
   float2* u;              // [H * W]
@@ -79,9 +89,9 @@ struct WorldDev {
   float layer_half;       // half distance between the layers (cells)
   int ib, mdf_iters;      // coupling (0 penalty, 1 direct forcing) and MDF passes per step
   float* mrho;            // [H * W] fluid density of the step (ib == 1)
-  int* bead_slot;         // [N] slot of each bead in the bin-ordered arrays (ib == 1, else nullptr)
+  int* bead_slot;         // [N] slot of each bead in bpos and brec (ib == 1 or layers == 2, else nullptr)
   float2* u2;             // [H * W] second velocity buffer: MDF passes alternate u -> u2 -> u (ib == 1)
-  float2* sus;            // [N] U_s in bin order (ib == 1)
+  float2* sus;            // [n_bins slot_cap + N] U_s by slot (ib == 1)
   float2* nrm;            // [N] filament unit normal at each bead (layers == 2)
   unsigned long long* facc;  // [2 H W] fixed-point spread of the layer points (layers == 2)
   const float4* ldrive;   // [E] (L0, amp, freq, phase) rest-length drive, or nullptr (static L_rest)
@@ -166,7 +176,7 @@ __device__ __forceinline__ int fix_exponent64(float bound) {
 struct LaunchCfg {
   int persistent = 0;     // 3 or 4: one cooperative launch per run of steps with that many blocks per SM (k_persist.cu)
   int pbd_warps = 8;      // most filaments (warps) per block of the PBD kernels: 8, 4 or 2
-  int scan_kernels = 0;   // 0: one scan kernel when every world fits one scan block; 2: always two
+  int scan_kernels = 0;   // 0 or 2: kept for callers that set it; a step scans nothing
   int force_ws = 0;       // 1: the warp-specialised persistent force + LBM kernel (worlds without two layers)
 };
 
@@ -187,14 +197,12 @@ struct Plan {
   bool any_mdf = false;          // some world couples by direct forcing (ib == 1)
   int max_mdf = 0;               // most MDF passes of a world
   bool any_ext = false;          // some world has two layers, observables, a rest-length drive or direct forcing
-  bool one_chunk = false;        // every world's bins fit one scan block (its offsets need no block sums)
-  int n_fil_items = 0, n_bead_items = 0, n_tile_items = 0, n_cell_items = 0, n_scan_items = 0;
+  int n_fil_items = 0, n_bead_items = 0, n_tile_items = 0, n_cell_items = 0;
   WorldDev* d_worlds = nullptr;  // [n_worlds]
   int2* d_fil_items = nullptr;   // (world, filament)
   int2* d_bead_items = nullptr;  // (world, first bead)
   int2* d_tile_items = nullptr;  // (world, tx | ty << 16), row-major over the tiles
   int2* d_cell_items = nullptr;  // (world, first cell)
-  int2* d_scan_items = nullptr;  // (world, scan chunk)
   void* d_mem = nullptr;
   unsigned* d_persist_bar = nullptr;   // [3] barrier words and status of the persistent step
   cudaGraphExec_t graph = nullptr;
@@ -211,18 +219,25 @@ void persistent_test_settings(unsigned extra_arrivals, unsigned long long timeou
 void steric_setup(int sms);   // host set-up of the tile kernels (k_steric.cu), outside any stream capture
 
 // --- stage launchers (one launch covers every world of the plan) ---------
+// A run of fused steps keeps the worlds' step counters in place until its
+// last advance: its kernels take `off`, the step's distance from the counter
+// (0 in a step of its own, -1 to re-run a stage of the completed step).
 void launch_pbd(const Plan& p, cudaStream_t s);
-void launch_bin_scan(const Plan& p, cudaStream_t s, int inc_t = 0);      // one kernel when every world fits one scan block, else two
-void launch_bin_scatter(const Plan& p, cudaStream_t s);
+// sorted read-outs (off as above): the bin offsets, then the records in bin order
+void launch_sorted_offsets(const Plan& p, cudaStream_t s, int off);
+void launch_sorted_records(const Plan& p, cudaStream_t s, int off);
+// the step's slots and counts of parity (counter - 1) & 1 from the sorted
+// records (a loaded image)
+void launch_slots_from_sorted(const Plan& p, cudaStream_t s);
 // a4 + x pass of a5; store_fields also writes rho_s of each tile
-void launch_deposit_x(const Plan& p, cudaStream_t s, int store_fields);
-// y pass of a5 + a6; store_fields also writes rho_bar of each tile;
-// after_step = 1 when re-run after the step that produced the binned beads
-void launch_force_spread(const Plan& p, cudaStream_t s, int store_fields, int after_step = 0);
-void launch_lbm(const Plan& p, cudaStream_t s, int layered_only = 0);   // layered_only: two-layer worlds only
+void launch_deposit_x(const Plan& p, cudaStream_t s, int store_fields, int off = 0);
+// y pass of a5 + a6; store_fields also writes rho_bar of each tile
+void launch_force_spread(const Plan& p, cudaStream_t s, int store_fields, int off = 0);
+void launch_lbm(const Plan& p, cudaStream_t s, int layered_only = 0, int off = 0);   // layered_only: two-layer worlds only
 void launch_layer_spread(const Plan& p, cudaStream_t s);   // two-layer worlds: F from the layer points
-void launch_force_lbm(const Plan& p, cudaStream_t s);   // y pass of a5 + a6 + a7 in one kernel
-void launch_interp_advance(const Plan& p, cudaStream_t s);
+// y pass of a5 + a6 + a7 in one kernel; fields as in launch_advance_pbd
+void launch_force_lbm(const Plan& p, cudaStream_t s, int off = 0, int fields = 1);
+void launch_interp_advance(const Plan& p, cudaStream_t s, int inc = 1);   // inc: steps the counter moves by
 // direct forcing (ib == 1 worlds; the others return at once): bins and a
 // zero F_el before the steric spread, then u*, the predicted PBD and the
 // MDF passes after it
@@ -232,8 +247,9 @@ cudaError_t launch_mdf_recorded(const Plan& p, const WorldDev& h, float2* mu, cu
 void launch_mdf_pass(const Plan& p, cudaStream_t s, int pass);   // k_steric.cu: one MDF pass (tile kernel)
 void enqueue_step(const Plan& p, cudaStream_t s);
 void enqueue_steps(const Plan& p, int n, cudaStream_t s);   // n steps, fused bead stages where possible
-void launch_advance_pbd(const Plan& p, cudaStream_t s);
-constexpr int kKernelsPerStep = 8;
+// fields = 0: a step within a run, whose per-bead fields for read-out (F_el,
+// F_s, bins) are not kept (the run's last step keeps its own)
+void launch_advance_pbd(const Plan& p, cudaStream_t s, int off, int fields);
 
 // --- adjoint (one world) ----------------------------------------------------
 void launch_adj_step(const Plan& p, const WorldDev& h, AdjDev a, const AdjMdf* m, int src_parity, cudaStream_t s);
@@ -284,7 +300,12 @@ void launch_cells_out(const WorldDev& w, int* cell, cudaStream_t s);
 
 // --- world life cycle and plans (host, mc_api.cu) -------------------------
 void world_sizes(WorldDev& h, int H, int W, int n_fil, int N);
-size_t world_layout(WorldDev& h, void* arena);
+struct ArenaSize {
+  size_t image = 0;   // bytes a saved image holds (the leading arrays)
+  size_t zero = 0;    // bytes a new world needs cleared
+  size_t total = 0;
+};
+ArenaSize world_layout(WorldDev& h, void* arena);
 mc_status plan_build(mc_world* const* ws, int n, cudaStream_t s, Plan& out);
 mc_status plan_run(Plan& p, int n_steps, cudaStream_t s);
 void plan_free(Plan& p, cudaStream_t s);
@@ -470,6 +491,11 @@ __device__ __forceinline__ void obs_add_warp(unsigned long long* acc, long long 
   if ((threadIdx.x & 31) == 0 && q != 0) atomicAdd(acc, (unsigned long long)q);
 }
 
+// A world's bin counts of step t (see WorldDev).
+__device__ __forceinline__ int* step_counts(const WorldDev& w, long long t) {
+  return w.bin_cnt + (size_t)(t & 1) * (w.n_bins + 1);
+}
+
 __device__ __forceinline__ int cell_x(const float4& p) { return __float_as_int(p.z); }
 __device__ __forceinline__ int cell_y(const float4& p) { return __float_as_int(p.w); }
 
@@ -523,6 +549,7 @@ struct mc_world {
   mc::WorldDev h{};               // device descriptor (host copy)
   void* arena = nullptr;          // one allocation holding every device array
   size_t bytes = 0;
+  size_t image_bytes = 0;         // leading part of the arena that a saved image holds
   cudaStream_t stream = nullptr;  // creation stream; the arena is freed on it
   int64_t t = 0;                  // step counter after all enqueued steps
   int max_B = 2;

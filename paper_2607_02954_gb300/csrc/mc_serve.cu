@@ -152,7 +152,7 @@ size_t footprint(int H, int W, int n_fil, int N, bool ldrive, bool energy, int l
   // arena plus this world's share of a plan (work items and table entry)
   const size_t items = (size_t)n_fil + (N / mc::kBeadChunk + 1) + h.n_tiles + (size_t)H * W / mc::kCellChunk + 1 +
                        h.n_chunks;
-  return mc::world_layout(h, nullptr) + items * sizeof(int2) + sizeof(mc::WorldDev) + 4096;
+  return mc::world_layout(h, nullptr).total + items * sizeof(int2) + sizeof(mc::WorldDev) + 4096;
 }
 
 void publish(mc_server* s, uint64_t ticket, const mc_result& r) {

@@ -4,9 +4,8 @@
 // can run its steps in several configurations that advance the worlds
 // bitwise the same (LaunchCfg): the per-stage kernels replayed from a CUDA
 // graph or one persistent cooperative launch (3 or 4 blocks per SM), the
-// number of filaments per PBD block, one or two bin-offset kernels.  Which
-// is fastest depends on the plan's shape (tile and bead counts, world
-// sizes).  The tuner measures the candidates on device copies of the plan's
+// number of filaments per PBD block.  Which is fastest depends on the plan's
+// shape (tile and bead counts, world sizes).  The tuner measures the candidates on device copies of the plan's
 // worlds (the worlds themselves do not move), coordinate by coordinate from
 // the default, keeps a candidate only when it is at least 1% faster, and
 // caches the choice per class of plan for the life of the process.
@@ -31,7 +30,7 @@ bool g_auto = true;
 // Class of a plan: what its launches cover.
 std::vector<long long> plan_key(mc_world* const* ws, int n, const Plan& p) {
   long long beads = 0, cells = 0;
-  std::vector<long long> k = {n, p.max_B, p.max_R, p.any_ext, p.any_mdf, p.any_layered, p.one_chunk,
+  std::vector<long long> k = {n, p.max_B, p.max_R, p.any_ext, p.any_mdf, p.any_layered,
                               p.n_fil_items, p.n_tile_items, p.n_bead_items};
   for (int i = 0; i < n; ++i) {
     const WorldDev& h = world_dev(ws[i]);
@@ -126,11 +125,6 @@ mc_status plan_tune(mc_world* const* ws, int n, Plan& p, cudaStream_t s, bool au
         for (int wp : {4, 2}) {
           LaunchCfg c = best;
           c.pbd_warps = wp;
-          consider(c);
-        }
-        if (cp.one_chunk && !best.persistent) {
-          LaunchCfg c = best;
-          c.scan_kernels = 2;
           consider(c);
         }
       }

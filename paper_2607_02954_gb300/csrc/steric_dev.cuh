@@ -9,7 +9,6 @@ namespace mc {
 
 namespace {
 
-constexpr int kMaxSeg = 32;
 constexpr int kThreads = 256;
 constexpr int kWarps = kThreads / 32;
 constexpr int kForceCap = 640;             // bead records staged per pass (force)
@@ -42,132 +41,82 @@ __device__ __forceinline__ void cp_async4(void* sdst, const void* gsrc) {
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
-// Bulk copies into shared memory completing on an mbarrier (the tile's bead
-// records: each bin segment is contiguous in global and in shared memory).
-__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ void mbar_init(unsigned long long* bar) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_addr(bar)) : "memory");
-  asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-}
-// (before the barrier's memory is re-initialised or used for anything else)
-__device__ __forceinline__ void mbar_inval(unsigned long long* bar) {
-  asm volatile("mbarrier.inval.shared::cta.b64 [%0];\n" ::"r"(smem_addr(bar)) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(unsigned long long* bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_addr(bar)), "r"(bytes)
-               : "memory");
-}
-// Copies `bytes` (a multiple of 16; both addresses 16-byte aligned).
-__device__ __forceinline__ void bulk_copy_g2s(void* sdst, const void* gsrc, unsigned bytes, unsigned long long* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
-               ::"r"(smem_addr(sdst)), "l"(gsrc), "r"(bytes), "r"(smem_addr(bar))
-               : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(unsigned long long* bar, unsigned parity) {
-  unsigned ok;
-  asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-               : "=r"(ok)
-               : "r"(smem_addr(bar)), "r"(parity)
-               : "memory");
-  return ok != 0;
-}
-// Waits for phase `parity` of the barrier, for at most ~2^22 polls (each
-// try_wait itself suspends for a while); a wait that runs out flags the
-// world (kFlagTimeout), waits once more as long, and returns.
-__device__ __forceinline__ void mbar_wait_bounded(unsigned long long* bar, unsigned parity, unsigned* flags) {
-  for (int round = 0; round < 2; ++round) {
-    for (int it = 0; it < (1 << 22); ++it)
-      if (mbar_try_wait(bar, parity)) return;
-    if (round == 0 && flags) atomicOr(flags, kFlagTimeout);
-  }
-}
-
 __device__ __forceinline__ int floor_div(int a, int b) { return a >= 0 ? a / b : -((b - 1 - a) / b); }
 
-// Bead segments of the bins whose cells reach the cell box
-// [x_lo, x_hi] x [y_lo, y_hi] (inclusive, unwrapped coordinates), built by
-// one warp: lane 2r + q handles part q of bin row r (a row's column range is
-// split in two where it wraps), so all bin offsets load in one round trip.
-// Fills s_start[32] and s_pre[33] (prefix of segment lengths; empty
-// segments have length 0).  With max_count non-null, also returns the
-// largest bead count of a single bin in the box.
-__device__ void build_segments(const WorldDev& w, int x_lo, int x_hi, int y_lo, int y_hi, int* s_start,
-                               int* s_pre, int* max_count) {
+// The slots of the bins whose cells reach a cell box, as one concatenated
+// list: segment e < 64 holds bin (row e / 8, column e % 8) of the box, the
+// last segment the beads of the world that found their bin's slots full
+// (none unless bins are crowded; each is tested against the tile like any
+// other).  pre[] are the prefix sums of the segments' lengths.
+constexpr int kSegs = 65;
+struct Segments {
+  int start[kSegs], pre[kSegs + 1];
+  int covered;   // beads in the covering bins, full slots or not
+  int most;      // largest bead count of one of them
+};
+
+// Builds the list for the box [x_lo, x_hi] x [y_lo, y_hi] (inclusive,
+// unwrapped coordinates; at most 8 bins a side: tile + 2 R + 3 <= 51 cells)
+// with one warp; lane l handles bins l and l + 32, so all counts load in one
+// round trip.
+__device__ void build_segments(const WorldDev& w, const int* counts, int x_lo, int x_hi, int y_lo, int y_hi,
+                               Segments& sg) {
   const int lane = threadIdx.x & 31;
-  const int nbx = w.nbx, nby = w.nby;
-  const int* bin_off = w.bin_off;
+  const int nbx = w.nbx, nby = w.nby, cap = w.slot_cap;
   int bx0 = floor_div(x_lo, kBin), bx1 = floor_div(x_hi, kBin);
   int by0 = floor_div(y_lo, kBin), by1 = floor_div(y_hi, kBin);
   if (bx1 - bx0 + 1 >= nbx) { bx0 = 0; bx1 = nbx - 1; }
   if (by1 - by0 + 1 >= nby) { by0 = 0; by1 = nby - 1; }
-  const int r = lane >> 1, q = lane & 1;
-  int lo, hi;
-  bool split;
-  if (bx0 < 0) {
-    split = true;
-    lo = q == 0 ? bx0 + nbx : 0;
-    hi = q == 0 ? nbx - 1 : bx1;
-  } else if (bx1 >= nbx) {
-    split = true;
-    lo = q == 0 ? bx0 : 0;
-    hi = q == 0 ? nbx - 1 : bx1 - nbx;
-  } else {
-    split = false;
-    lo = bx0;
-    hi = bx1;
-  }
-  const bool valid = by0 + r <= by1 && (split || q == 0);
-  // every load is issued before any is used (one memory round trip)
-  int s0 = 0, e1 = 0;
-  if (valid) {
-    const int row = wrap_once(by0 + r, nby) * nbx;
-    s0 = bin_off[row + lo];
-    e1 = bin_off[row + hi + 1];
-  }
-  // the box spans at most 8 bin columns (tile + 2 R + 3 <= 51 cells) and
-  // 16 bin rows; lane (rr, cc) = (lane / 8, lane % 8) covers 4 rows per round
-  int mlo[4], mhi[4];
-  if (max_count) {
-    const int ncol = bx1 - bx0 + 1, nrow = by1 - by0 + 1;
-    const int cc = lane & 7;
+  const int ncol = bx1 - bx0 + 1, nrow = by1 - by0 + 1;
+  const int cc = lane & 7, rr = lane >> 3;
+  int bin[2] = {0, 0}, n[2] = {0, 0};
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int rr = (lane >> 3) + 4 * k;
-      mlo[k] = 0;
-      mhi[k] = 0;
-      if (rr < nrow && cc < ncol) {
-        const int bin = wrap_once(by0 + rr, nby) * nbx + wrap_once(bx0 + cc, nbx);
-        mlo[k] = bin_off[bin];
-        mhi[k] = bin_off[bin + 1];
-      }
+  for (int h = 0; h < 2; ++h) {
+    const int r = rr + 4 * h;
+    if (cc < ncol && r < nrow) {
+      bin[h] = wrap_once(by0 + r, nby) * nbx + wrap_once(bx0 + cc, nbx);
+      n[h] = counts[bin[h]];
     }
   }
-  int incl = e1 - s0;
-  for (int o = 1; o < 32; o <<= 1) {
-    const int y = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += y;
-  }
-  s_start[lane] = s0;
-  s_pre[lane + 1] = incl;
-  if (lane == 0) s_pre[0] = 0;
-  if (max_count) {
-    int m = 0;
+  const int over = counts[w.n_bins];
+  int covered = n[0] + n[1], most = max(n[0], n[1]);
+  int incl0 = min(n[0], cap), incl1 = min(n[1], cap);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) m = max(m, mhi[k] - mlo[k]);
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if (lane == 0) *max_count = m;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y0 = __shfl_up_sync(0xffffffffu, incl0, o), y1 = __shfl_up_sync(0xffffffffu, incl1, o);
+    if (lane >= o) {
+      incl0 += y0;
+      incl1 += y1;
+    }
+  }
+  incl1 += __shfl_sync(0xffffffffu, incl0, 31);
+  sg.start[lane] = bin[0] * cap;
+  sg.start[lane + 32] = bin[1] * cap;
+  sg.pre[lane + 1] = incl0;
+  sg.pre[lane + 33] = incl1;
+  for (int o = 16; o > 0; o >>= 1) {
+    covered += __shfl_xor_sync(0xffffffffu, covered, o);
+    most = max(most, __shfl_xor_sync(0xffffffffu, most, o));
+  }
+  if (lane == 31) {
+    sg.pre[0] = 0;
+    sg.start[kSegs - 1] = w.n_bins * cap;
+    sg.pre[kSegs] = incl1 + over;
+    sg.covered = covered;
+    sg.most = most;
   }
 }
 
-// Slot of the v-th bead of the concatenated segments: the segment j with
-// s_pre[j] <= v < s_pre[j + 1] by binary search over the 33 prefix entries
-// (non-decreasing; empty segments repeat a value and are never chosen).
-__device__ __forceinline__ int seg_slot(int v, const int* s_start, const int* s_pre) {
+// Slot of the v-th bead of the list: the segment j with pre[j] <= v <
+// pre[j + 1] by binary search over the prefix entries (non-decreasing; empty
+// segments repeat a value and are never chosen).
+__device__ __forceinline__ int seg_slot(int v, const Segments& sg) {
   int j = 0;
 #pragma unroll
-  for (int step = 16; step > 0; step >>= 1)
-    if (v >= s_pre[j + step]) j += step;
-  return s_start[j] + v - s_pre[j];
+  for (int step = 32; step > 0; step >>= 1)
+    if (v >= sg.pre[j + step]) j += step;
+  if (j == kSegs - 2 && v >= sg.pre[kSegs - 1]) j = kSegs - 1;
+  return sg.start[j] + v - sg.pre[j];
 }
 
 // Periodic image of d in (-n, n) taken in [-lo, n - lo).
@@ -177,18 +126,18 @@ __device__ __forceinline__ int image_lo(int d, int n, int lo) {
   return d;
 }
 
-// Appends `code` to the block's list when `keep`; every lane of the warp
-// calls this together.  The list order depends on warp timing, which no
-// result depends on (the accumulation is in integers).
-__device__ __forceinline__ void list_push(bool keep, int code, int* list, int* s_cnt) {
+// The next place of the block's list for each lane that keeps its bead;
+// every lane of the warp calls this together.  The list order depends on
+// warp timing, which no result depends on (the accumulation is in integers).
+__device__ __forceinline__ int list_place(bool keep, int* s_cnt) {
   const unsigned m = __ballot_sync(0xffffffffu, keep);
-  if (m == 0u) return;
+  if (m == 0u) return 0;
   const int lane = threadIdx.x & 31;
   const int leader = __ffs(m) - 1;
   int base = 0;
   if (lane == leader) base = atomicAdd(s_cnt, __popc(m));
   base = __shfl_sync(0xffffffffu, base, leader);
-  if (keep) list[base + __popc(m & ((1u << lane) - 1u))] = code;
+  return base + __popc(m & ((1u << lane) - 1u));
 }
 
 // list code: staged slot v (10 bits), rx + 16 and ry + 16 (11 bits each)
@@ -253,16 +202,16 @@ struct DepTile {
 // wrapped cells.  Ends with the block synchronised.
 template <int R>
 __device__ __forceinline__ void deposit_accumulate(int* acc, const WorldDev& w, const DepTile& d, int k,
-                                                   const int* s_start, const int* s_pre) {
+                                                   const Segments& sg) {
   using G = Geo<R>;
   const int tid = threadIdx.x;
   const int W = d.W, H = d.H, wR = d.wR, x0 = d.x0, y0 = d.y0, tw = d.tw, th = d.th;
-  const int cx0 = d.cx0, oxe = d.oxe, total = d.total;
+  const int cx0 = d.cx0, oxe = d.oxe, total = sg.pre[kSegs];
   const bool full_x = d.full_x, full_y = d.full_y;
-  const float4* __restrict__ spos = w.spos;
+  const float4* __restrict__ bpos = w.bpos;
   const float scale = pow2f(k);
   // each thread deposits the beads v = tid, tid + 256, ... of the segments
-  // straight from the bin-ordered records, two loads in flight at a time;
+  // straight from their slots, two loads in flight at a time;
   // a bead whose stencil misses the region adds nothing
   auto deposit = [&](const float4 p) {
     int rx = cell_x(p) - cx0, ry = cell_y(p) - y0;
@@ -289,9 +238,9 @@ __device__ __forceinline__ void deposit_accumulate(int* acc, const WorldDev& w, 
   };
   for (int v0 = tid; v0 < total; v0 += 2 * kThreads) {
     const int v1 = v0 + kThreads;
-    const float4 p0 = spos[seg_slot(v0, s_start, s_pre)];
+    const float4 p0 = bpos[seg_slot(v0, sg)];
     float4 p1 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-    if (v1 < total) p1 = spos[seg_slot(v1, s_start, s_pre)];
+    if (v1 < total) p1 = bpos[seg_slot(v1, sg)];
     deposit(p0);
     if (v1 < total) deposit(p1);
   }
@@ -396,22 +345,23 @@ template <int R>
 struct DepositSmem {
   int acc[Geo<R>::kDY * Geo<R>::kDX];
   float tap_s[Geo<R>::kTaps];
-  int s_start[kMaxSeg], s_pre[kMaxSeg + 1], s_maxc;
+  Segments sg;
   float red[kWarps];
 };
 
 // a4 + the x pass of a5 for the tile item of block `blk` (block-uniform
-// control flow; the caller's block runs it whole).
+// control flow; the caller's block runs it whole).  It also readies the next
+// step: the other parity's counts of the tile's own bins, its overflow count
+// and its F_el-maximum slot go to zero (the previous step's; this step's
+// stay readable).
 template <int R, bool kSingle>
 __device__ __forceinline__ void deposit_x_body(const WorldDev* __restrict__ worlds, const int2* __restrict__ items,
-                                               int store_fields, const WorldDev& w1, unsigned blk,
+                                               int store_fields, int off, const WorldDev& w1, unsigned blk,
                                                DepositSmem<R>& sm) {
   using G = Geo<R>;
   int* acc = sm.acc;
   float* tap_s = sm.tap_s;
-  int* s_start = sm.s_start;
-  int* s_pre = sm.s_pre;
-  int& s_maxc = sm.s_maxc;
+  const Segments& sg = sm.sg;
   float* red = sm.red;
   const int2 it = kSingle ? single_tile_item(w1, blk) : items[blk];
   const WorldDev& w = kSingle ? w1 : worlds[it.x];
@@ -431,12 +381,22 @@ __device__ __forceinline__ void deposit_x_body(const WorldDev* __restrict__ worl
   d.full_y = w.nty == 1;
   d.cx0 = d.full_x ? 0 : d.x0;                  // region column origin
   d.oxe = d.full_x ? 4 : R + 4;                 // accumulator column of region column 0
+  const long long t = *w.t + off;
   if (warp == 0)
-    build_segments(w, d.x0 - d.wR - 2, d.x0 + d.tw + d.wR, d.y0 - 2, d.y0 + d.th, s_start, s_pre, &s_maxc);
+    build_segments(w, step_counts(w, t), d.x0 - d.wR - 2, d.x0 + d.tw + d.wR, d.y0 - 2, d.y0 + d.th, sm.sg);
+  if (warp == 2) {
+    int* next = step_counts(w, t + 1);
+    const int bx = d.x0 / kBin + (lane & 3), by = d.y0 / kBin + (lane >> 2);
+    if (lane < 16 && bx < w.nbx && by < w.nby) next[by * w.nbx + bx] = 0;
+    if (lane == 16 && d.tile == 0) {
+      next[w.n_bins] = 0;
+      w.fel_max[(t + 1) & 1] = 0u;
+    }
+  }
   if (warp == 1 && lane < G::kTaps) tap_s[lane] = padded_tap<R>(w, d.wR, lane);
   for (int c = tid; c < G::kDY * G::kDX / 4; c += kThreads) reinterpret_cast<int4*>(acc)[c] = make_int4(0, 0, 0, 0);
   __syncthreads();
-  d.total = s_pre[kMaxSeg];
+  d.total = sg.covered;
   if (d.total == 0) {
     // no bead reaches the region: rho_s, rho_x and the tile maximum are zero
     // (what the passes below give for an empty accumulator, bitwise)
@@ -451,8 +411,8 @@ __device__ __forceinline__ void deposit_x_body(const WorldDev* __restrict__ worl
     if (tid == 0) w.tile_rho_max[d.tile] = 0.0f;
     return;
   }
-  int k = fix_exponent((float)s_maxc + 1.0f);
-  deposit_accumulate<R>(acc, w, d, k, s_start, s_pre);
+  int k = fix_exponent((float)sg.most + 1.0f);
+  deposit_accumulate<R>(acc, w, d, k, sg);
   if (k < 24) {
     // dense tile: the largest accumulated sum plus the rounding of its terms
     // (half a unit per bead of the covering bins, at most one term per cell
@@ -465,7 +425,7 @@ __device__ __forceinline__ void deposit_x_body(const WorldDev* __restrict__ worl
       for (int c = tid; c < G::kDY * G::kDX / 4; c += kThreads) reinterpret_cast<int4*>(acc)[c] = make_int4(0, 0, 0, 0);
       __syncthreads();
       k = k2;
-      deposit_accumulate<R>(acc, w, d, k, s_start, s_pre);
+      deposit_accumulate<R>(acc, w, d, k, sg);
     }
   }
   deposit_xpass<R>(acc, w, d, k, tap_s, red, store_fields);
@@ -479,25 +439,22 @@ __device__ __forceinline__ void deposit_x_body(const WorldDev* __restrict__ worl
 // [0, tw + 8) (tile cell (lx, ly) at window (lx + 4, ly + 4)).  Spread
 // accumulators: tile cell (lx, ly) at (lx + 3, ly + 3), F = acc 2^-k.
 // ---------------------------------------------------------------------------
-// Inputs of one tile, staged before its compute (double-buffered by the
-// persistent kernel).
+// Inputs of one tile, staged before its compute.
 template <int R>
 struct TileIn {
   float xb[Geo<R>::kLoadRows * kWin];   // rho_x window
-  float4 sp[kForceCap];                 // bead positions of the chunk (bin order)
-  float4 sr[kForceCap];                 // their F_el (x, y) and bead id (int bits)
-  unsigned long long bar;               // completion of the chunk's bulk copies
-  int s_start[kMaxSeg], s_pre[kMaxSeg + 1];
+  Segments sg;
   float nbmax[9];                       // largest rho_s of the 3x3 tiles around
   float tap_s[Geo<R>::kTaps];
 };
 
 // Working arrays of the tile being computed.
 struct TileWork {
+  float4 sp[kForceCap];                 // listed beads: fractions, tile-relative cell (int bits)
+  float4 sr[kForceCap];                 // their F_el (x, y) and bead id (int bits)
   float win[kWin * kWin];               // rho_bar window
   int accx[kAx * kAx];                  // spread accumulators
   int accy[kAx * kAx];
-  int list[kForceCap];
   int s_cnt;
 };
 
@@ -520,30 +477,50 @@ __device__ __forceinline__ void force_sync() {
   else asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
 }
 
-// Lists the n staged beads whose stencil reaches the tile (image taken on
-// axes with several tiles), packed with their tile-relative cell.
-template <int R, int NT = kThreads>
-__device__ __forceinline__ void force_compact(const TileIn<R>& in, TileWork& wk, int n, const TileBox& tb, int W,
-                                              int H, int ntx, int nty) {
-  for (int v0 = 0; v0 < n; v0 += NT) {
-    const int v = v0 + threadIdx.x;
-    bool keep = false;
-    int rx = 0, ry = 0;
-    if (v < n) {
-      const float4 p = in.sp[v];
-      rx = cell_x(p) - tb.x0;
-      ry = cell_y(p) - tb.y0;
-      keep = true;
-      if (ntx > 1) {
-        rx = image_lo(rx, W, 2);
-        keep = rx <= tb.tw;
-      }
-      if (nty > 1) {
-        ry = image_lo(ry, H, 2);
-        keep = keep && ry <= tb.th;
-      }
+// Lists the beads c0 .. c0 + n - 1 of the tile's segments whose stencil
+// reaches the tile (image taken on axes with several tiles): each thread
+// reads records straight from their slots, two in flight, and the ones that
+// reach the tile are packed into the working arrays.
+template <int NT>
+__device__ __forceinline__ void force_list(const Segments& sg, TileWork& wk, const WorldDev& w, int c0, int n,
+                                           const TileBox& tb) {
+  const int W = w.W, H = w.H, ntx = w.ntx, nty = w.nty;
+  const float4* __restrict__ bpos = w.bpos;
+  const float4* __restrict__ brec = w.brec;
+  auto list = [&](bool keep, float4 p, const float4 rec) {
+    int rx = cell_x(p) - tb.x0, ry = cell_y(p) - tb.y0;
+    if (ntx > 1) {
+      rx = image_lo(rx, W, 2);
+      keep = keep && rx <= tb.tw;
     }
-    list_push(keep, pack_code(v, rx, ry), wk.list, &wk.s_cnt);
+    if (nty > 1) {
+      ry = image_lo(ry, H, 2);
+      keep = keep && ry <= tb.th;
+    }
+    const int at = list_place(keep, &wk.s_cnt);
+    if (keep) {
+      p.z = __int_as_float(rx);
+      p.w = __int_as_float(ry);
+      wk.sp[at] = p;
+      wk.sr[at] = rec;
+    }
+  };
+  const float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  for (int v0 = 0; v0 < n; v0 += 2 * NT) {
+    const int va = v0 + threadIdx.x, vb = va + NT;
+    float4 pa = z, ra = z, pb = z, rb = z;
+    if (va < n) {
+      const int slot = seg_slot(c0 + va, sg);
+      pa = bpos[slot];
+      ra = brec[slot];
+    }
+    if (vb < n) {
+      const int slot = seg_slot(c0 + vb, sg);
+      pb = bpos[slot];
+      rb = brec[slot];
+    }
+    list(va < n, pa, ra);
+    if (v0 + NT < n) list(vb < n, pb, rb);   // block-uniform
   }
 }
 
@@ -579,9 +556,10 @@ __device__ __forceinline__ void tile_stage_window(TileIn<R>& in, const WorldDev&
 // Stage 2 (warps 0-2, plain loads): the bead segments of the bins that reach
 // the tile, the filter taps, and the largest rho_s of the 3x3 tiles around.
 template <int R>
-__device__ __forceinline__ void tile_stage_meta(TileIn<R>& in, const WorldDev& w, const TileBox& tb) {
+__device__ __forceinline__ void tile_stage_meta(TileIn<R>& in, const WorldDev& w, const TileBox& tb, int off) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (warp == 0) build_segments(w, tb.x0 - 2, tb.x0 + tb.tw, tb.y0 - 2, tb.y0 + tb.th, in.s_start, in.s_pre, nullptr);
+  if (warp == 0)
+    build_segments(w, step_counts(w, *w.t + off), tb.x0 - 2, tb.x0 + tb.tw, tb.y0 - 2, tb.y0 + tb.th, in.sg);
   if (warp == 1 && lane < Geo<R>::kTaps) in.tap_s[lane] = padded_tap<R>(w, w.R, lane);
   // bound of the cell sums of weight * |F_el + F_s|:
   //   |F_s| <= k_rep/2 max|rho_bar(c+1) - rho_bar(c-1)| <= k_rep/2 max rho_bar
@@ -591,31 +569,6 @@ __device__ __forceinline__ void tile_stage_meta(TileIn<R>& in, const WorldDev& w
     const int tx = tb.x0 / kTile, ty = tb.y0 / kTile;
     const int ty2 = wrap_once(ty + lane / 3 - 1, w.nty), tx2 = wrap_once(tx + lane % 3 - 1, w.ntx);
     in.nbmax[lane] = w.tile_rho_max[ty2 * w.ntx + tx2];
-  }
-}
-
-// Stage 3 (after stage 2 is visible to the block): the bead records c0 ..
-// c0 + n - 1 (n > 0, in segment order) as bulk copies, one lane of warp 0
-// per segment (a bin segment is contiguous in the bin-ordered arrays and in
-// the staging arrays), after lane 0 has announced the bytes on in.bar; the
-// block then waits on in.bar.  Positions and (F_el, id) records are 16 bytes
-// each, so every copy starts and ends on 16-byte boundaries.
-static_assert(kMaxSeg == 32, "one lane of a warp per segment");
-template <int R>
-__device__ __forceinline__ void tile_stage_records(TileIn<R>& in, const WorldDev& w, int c0, int n) {
-  if (threadIdx.x >= 32) return;
-  const int lane = threadIdx.x;
-  if (lane == 0) {
-    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-    mbar_expect_tx(&in.bar, (unsigned)n * 32u);
-  }
-  __syncwarp();
-  const int lo = max(in.s_pre[lane], c0), hi = min(in.s_pre[lane + 1], c0 + n);
-  if (hi > lo) {
-    const int src = in.s_start[lane] + (lo - in.s_pre[lane]);
-    const unsigned bytes = (unsigned)(hi - lo) * 16u;
-    bulk_copy_g2s(&in.sp[lo - c0], &w.spos[src], bytes, &in.bar);
-    bulk_copy_g2s(&in.sr[lo - c0], &w.srec[src], bytes, &in.bar);
   }
 }
 
@@ -630,145 +583,134 @@ __device__ __forceinline__ void tile_clear(TileWork& wk) {
   if (threadIdx.x == 0) wk.s_cnt = 0;
 }
 
-// The y pass of a5 and a6 for one tile whose inputs have landed (all stages
-// complete and visible, accumulators cleared).  Returns k: after the caller
+// The y pass of a5: rho_bar on the window from the staged rho_x, 8 window
+// rows per thread.
+template <int R, int NT>
+__device__ __forceinline__ void tile_ypass(const TileIn<R>& in, TileWork& wk, const WorldDev& w, const TileBox& tb,
+                                           int store_fields) {
+  using G = Geo<R>;
+  const int W = w.W, tw = tb.tw, th = tb.th;
+  const int ww = tw + 8, wh = th + 8;
+  float* __restrict__ rho_b = w.rho_b;
+  float tp[G::kTaps];
+#pragma unroll
+  for (int m = 0; m < G::kTaps; ++m) tp[m] = in.tap_s[m];
+  const int nstrip = wh >> 3;
+  for (int c = threadIdx.x; c < nstrip * ww; c += NT) {
+    int s;
+    if (ww == kWin) s = c / kWin;   // full tile: constant divisor
+    else s = c / ww;
+    const int j = c - s * ww;
+    const float* src = in.xb + (8 * s) * kWin + j;
+    float v[8 + 2 * R];
+#pragma unroll
+    for (int q = 0; q < 8 + 2 * R; ++q) v[q] = src[q * kWin];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      float sacc = 0.0f;
+#pragma unroll
+      for (int m = 0; m < G::kTaps; ++m) sacc = fmaf(tp[m], v[r + m], sacc);
+      const int i = 8 * s + r;
+      wk.win[i * kWin + j] = sacc;
+      if (store_fields && i >= 4 && i < th + 4 && j >= 4 && j < tw + 4)
+        rho_b[(size_t)(tb.y0 + i - 4) * W + tb.x0 + j - 4] = sacc;
+    }
+  }
+}
+
+// a6 for the cnt listed beads: the steric force of each (kept in fs by the
+// bead's own tile when asked for) and the spread of F_el + F_s into the
+// accumulators at the given scale.
+template <int NT>
+__device__ __forceinline__ void tile_beads(TileWork& wk, const WorldDev& w, const TileBox& tb, int cnt, float scale,
+                                           bool keep_fs) {
+  const float k_rep = w.k_rep;
+  const bool layered = w.layers == 2;
+  float2* __restrict__ fs_out = w.fs;
+  for (int q = threadIdx.x; q < cnt; q += NT) {
+    const float4 p = wk.sp[q];
+    const int rx = __float_as_int(p.z), ry = __float_as_int(p.w);
+    float wx[4], wy[4];
+    peskin4(p.x, wx);
+    peskin4(p.y, wy);
+    // stencil cell a sits at window column rx + 3 + a; the central
+    // differences read one cell further on each side
+    const float* base = wk.win + (ry + 2) * kWin + rx + 2;
+    float gsx = 0.0f, gsy = 0.0f;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const float* rowm = base + b * kWin;
+      const float* row0 = rowm + kWin;
+      const float* rowp = row0 + kWin;
+      float sx = 0.0f, sy = 0.0f;
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        sx = fmaf(wx[a], row0[a + 2] - row0[a], sx);
+        sy = fmaf(wx[a], rowp[a + 1] - rowm[a + 1], sy);
+      }
+      gsx = fmaf(wy[b], sx, gsx);
+      gsy = fmaf(wy[b], sy, gsy);
+    }
+    const float Fsx = -0.5f * k_rep * gsx, Fsy = -0.5f * k_rep * gsy;
+    const float4 rec = wk.sr[q];
+    if (keep_fs && rx >= 0 && rx < tb.tw && ry >= 0 && ry < tb.th)
+      fs_out[__float_as_int(rec.z)] = make_float2(Fsx, Fsy);
+    if (layered) continue;   // two-layer worlds spread at their layer points (k_layer_spread)
+    const float Fx = (rec.x + Fsx) * scale, Fy = (rec.y + Fsy) * scale;
+    float ax[4], ay[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      ax[a] = wx[a] * Fx;
+      ay[a] = wx[a] * Fy;
+    }
+    int* bx = wk.accx + (ry + 2) * kAx + rx + 2;
+    int* by = wk.accy + (ry + 2) * kAx + rx + 2;
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+#pragma unroll
+      for (int a = 0; a < 4; ++a) {
+        atomicAdd(bx + b * kAx + a, __float2int_rn(wy[b] * ax[a]));
+        atomicAdd(by + b * kAx + a, __float2int_rn(wy[b] * ay[a]));
+      }
+    }
+  }
+}
+
+// The y pass of a5 and a6 for one tile.  Returns k: after the caller
 // synchronises the block, accx/accy hold the tile's F 2^k (before folding,
 // see force_fold).
 template <int R, int NT = kThreads>
-__device__ __forceinline__ int tile_compute(TileIn<R>& in, TileWork& wk, const WorldDev& w, int tile,
-                                            const TileBox& tb, int store_fields, int after_step) {
-  using G = Geo<R>;
-  const int W = w.W, H = w.H, ntx = w.ntx, nty = w.nty;
-  const float4* __restrict__ spos = w.spos;
-  float2* __restrict__ fs_out = w.fs;
-  float* __restrict__ rho_b = w.rho_b;
-  const float k_rep = w.k_rep;
-  const float fmax_el = __uint_as_float(w.fel_max[(*w.t - after_step) & 1]);
+__device__ __forceinline__ int force_tile(ForceSmem<R>& sm, const WorldDev& w, int tile, const TileBox& tb,
+                                          int store_fields, int off, bool keep_fs) {
+  TileIn<R>& in = sm.in;
+  TileWork& wk = sm.wk;
+  tile_stage_window<R, NT>(in, w, tb);
+  tile_stage_meta(in, w, tb, off);
+  tile_clear<NT>(wk);
+  force_sync<NT>();
+  const int total = in.sg.pre[kSegs];
+  force_list<NT>(in.sg, wk, w, 0, min(kForceCap, total), tb);
+  cp_async_wait_all();   // the window
+  const float fmax_el = __uint_as_float(w.fel_max[(*w.t + off) & 1]);
   const float rho_max = w.tile_rho_max[tile];
-  const bool layered = w.layers == 2;
-  const int x0 = tb.x0, y0 = tb.y0, tw = tb.tw, th = tb.th;
-  const int tid = threadIdx.x;
-  const int ww = tw + 8, wh = th + 8;
-  const int total = in.s_pre[kMaxSeg];
-  const int n0 = min(kForceCap, total);
   float rho_nb = in.nbmax[0];
   for (int k2 = 1; k2 < 9; ++k2) rho_nb = fmaxf(rho_nb, in.nbmax[k2]);
-  const int k = fix_exponent((fmax_el + 0.5f * k_rep * rho_nb) * rho_max * 1.0001f + 1e-30f);
+  const int k = fix_exponent((fmax_el + 0.5f * w.k_rep * rho_nb) * rho_max * 1.0001f + 1e-30f);
   const float scale = pow2f(k);
-  // list the first chunk's beads that reach the tile, then the y pass
-  force_compact<R, NT>(in, wk, n0, tb, W, H, ntx, nty);
-  if (total > 0 || store_fields) {
-    // y pass, 8 window rows per thread (only the beads' gradients and the
-    // rho_bar field read it)
-    float tp[G::kTaps];
-#pragma unroll
-    for (int m = 0; m < G::kTaps; ++m) tp[m] = in.tap_s[m];
-    const int nstrip = wh >> 3;
-    for (int c = tid; c < nstrip * ww; c += NT) {
-      int s;
-      if (ww == kWin) s = c / kWin;   // full tile: constant divisor
-      else s = c / ww;
-      const int j = c - s * ww;
-      const float* src = in.xb + (8 * s) * kWin + j;
-      float v[8 + 2 * R];
-#pragma unroll
-      for (int q = 0; q < 8 + 2 * R; ++q) v[q] = src[q * kWin];
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        float sacc = 0.0f;
-#pragma unroll
-        for (int m = 0; m < G::kTaps; ++m) sacc = fmaf(tp[m], v[r + m], sacc);
-        const int i = 8 * s + r;
-        wk.win[i * kWin + j] = sacc;
-        if (store_fields && i >= 4 && i < th + 4 && j >= 4 && j < tw + 4)
-          rho_b[(size_t)(y0 + i - 4) * W + x0 + j - 4] = sacc;
-      }
-    }
-  }
   force_sync<NT>();
-  for (int c0 = 0;;) {
-    const int cnt = wk.s_cnt;
-    for (int q = tid; q < cnt; q += NT) {
-      const int code = wk.list[q];
-      const int v = code_slot(code), rx = code_rx(code), ry = code_ry(code);
-      const float4 p = in.sp[v];
-      float wx[4], wy[4];
-      peskin4(p.x, wx);
-      peskin4(p.y, wy);
-      // stencil cell a sits at window column rx + 3 + a; the central
-      // differences read one cell further on each side
-      const float* base = wk.win + (ry + 2) * kWin + rx + 2;
-      float gsx = 0.0f, gsy = 0.0f;
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const float* rowm = base + b * kWin;
-        const float* row0 = rowm + kWin;
-        const float* rowp = row0 + kWin;
-        float sx = 0.0f, sy = 0.0f;
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-          sx = fmaf(wx[a], row0[a + 2] - row0[a], sx);
-          sy = fmaf(wx[a], rowp[a + 1] - rowm[a + 1], sy);
-        }
-        gsx = fmaf(wy[b], sx, gsx);
-        gsy = fmaf(wy[b], sy, gsy);
-      }
-      const float Fsx = -0.5f * k_rep * gsx, Fsy = -0.5f * k_rep * gsy;
-      const float4 rec = in.sr[v];
-      if (rx >= 0 && rx < tw && ry >= 0 && ry < th) fs_out[__float_as_int(rec.z)] = make_float2(Fsx, Fsy);
-      if (layered) continue;   // two-layer worlds spread at their layer points (k_layer_spread)
-      const float2 fe = make_float2(rec.x, rec.y);
-      const float Fx = (fe.x + Fsx) * scale, Fy = (fe.y + Fsy) * scale;
-      float ax[4], ay[4];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        ax[a] = wx[a] * Fx;
-        ay[a] = wx[a] * Fy;
-      }
-      int* bx = wk.accx + (ry + 2) * kAx + rx + 2;
-      int* by = wk.accy + (ry + 2) * kAx + rx + 2;
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-          atomicAdd(bx + b * kAx + a, __float2int_rn(wy[b] * ax[a]));
-          atomicAdd(by + b * kAx + a, __float2int_rn(wy[b] * ay[a]));
-        }
-      }
-    }
-    c0 += kForceCap;
-    if (c0 >= total) break;
-    force_sync<NT>();   // every thread is done with this chunk
-    if (tid == 0) wk.s_cnt = 0;
-    const int n = min(kForceCap, total - c0);
-    tile_stage_records(in, w, c0, n);
-    mbar_wait_bounded(&in.bar, (unsigned)(c0 / kForceCap) & 1u, w.flags);
+  // (only the beads' gradients and the rho_bar field read the y pass)
+  if (total > 0 || store_fields) tile_ypass<R, NT>(in, wk, w, tb, store_fields);
+  force_sync<NT>();
+  tile_beads<NT>(wk, w, tb, wk.s_cnt, scale, keep_fs);
+  for (int c0 = kForceCap; c0 < total; c0 += kForceCap) {
+    force_sync<NT>();   // every thread is done with the previous chunk
+    if (threadIdx.x == 0) wk.s_cnt = 0;
     force_sync<NT>();
-    force_compact<R, NT>(in, wk, n, tb, W, H, ntx, nty);
+    force_list<NT>(in.sg, wk, w, c0, min(kForceCap, total - c0), tb);
     force_sync<NT>();
+    tile_beads<NT>(wk, w, tb, wk.s_cnt, scale, keep_fs);
   }
   return k;   // the caller synchronises before it reads the accumulators
-}
-
-// One tile staged and computed (the non-persistent kernels).
-template <int R, int NT = kThreads>
-__device__ __forceinline__ int force_tile(ForceSmem<R>& sm, const WorldDev& w, int tile, const TileBox& tb,
-                                          int store_fields, int after_step) {
-  tile_stage_window<R, NT>(sm.in, w, tb);
-  tile_stage_meta(sm.in, w, tb);
-  tile_clear<NT>(sm.wk);
-  if (threadIdx.x == 0) mbar_init(&sm.in.bar);
-  force_sync<NT>();
-  const int n0 = min(kForceCap, sm.in.s_pre[kMaxSeg]);
-  if (n0 > 0) tile_stage_records(sm.in, w, 0, n0);
-  cp_async_wait_all();   // the window (cp.async)
-  if (n0 > 0) mbar_wait_bounded(&sm.in.bar, 0u, w.flags);
-  force_sync<NT>();
-  const int k = tile_compute<R, NT>(sm.in, sm.wk, w, tile, tb, store_fields, after_step);
-  // every thread is past its last wait on the barrier (tile_compute
-  // synchronises after each chunk's wait), so its memory can be released
-  if (threadIdx.x == 0) mbar_inval(&sm.in.bar);
-  return k;
 }
 
 // Folds the stencil cells that wrapped around an axis the tile covers whole
@@ -801,8 +743,8 @@ __device__ __forceinline__ TileBox tile_box(const WorldDev& w, int packed) {
 
 // The tile's population rows (plane i, rows y - c_iy, 128-byte segments) to L2.
 template <int NT = kThreads>
-__device__ __forceinline__ void prefetch_populations(const WorldDev& w, const TileBox& tb) {
-  const float* src = w.g[*w.t & 1];
+__device__ __forceinline__ void prefetch_populations(const WorldDev& w, const TileBox& tb, int off) {
+  const float* src = w.g[(*w.t + off) & 1];
   const int W = w.W, H = w.H;
   const size_t HW = (size_t)H * W;
   for (int c = threadIdx.x; c < 9 * kTile; c += NT) {
@@ -818,9 +760,9 @@ __device__ __forceinline__ void prefetch_populations(const WorldDev& w, const Ti
 // collides rows warp, warp + 8, ...; the first row's populations are pulled
 // before the barrier that completes the spread (pulling one row ahead in the
 // loop measured slower: register pressure).
-__device__ __forceinline__ void tile_lbm(TileWork& wk, const WorldDev& w, const TileBox& tb, int k) {
+__device__ __forceinline__ void tile_lbm(TileWork& wk, const WorldDev& w, const TileBox& tb, int k, int off) {
   const int W = w.W, H = w.H, HW = H * W;
-  const long long t = *w.t;
+  const long long t = *w.t + off;
   const float* __restrict__ src = w.g[t & 1];
   float* __restrict__ dst = w.g[(t + 1) & 1];
   float2* __restrict__ u_out = w.u;
@@ -853,12 +795,13 @@ __device__ __forceinline__ void tile_lbm(TileWork& wk, const WorldDev& w, const 
 // overlap the force phase.
 template <int R, bool kSingle>
 __device__ __forceinline__ void force_lbm_body(const WorldDev* __restrict__ worlds, const int2* __restrict__ items,
-                                               const WorldDev& w1, unsigned blk, ForceSmem<R>& sm) {
+                                               int off, int fields, const WorldDev& w1, unsigned blk,
+                                               ForceSmem<R>& sm) {
   const int2 it = kSingle ? single_tile_item(w1, blk) : items[blk];
   const WorldDev& w = kSingle ? w1 : worlds[it.x];
   const TileBox tb = tile_box(w, it.y);
   const bool layered = w.layers == 2;
-  if (!layered) prefetch_populations(w, tb);
+  if (!layered) prefetch_populations(w, tb, off);
   const int tile = (tb.y0 / kTile) * w.ntx + tb.x0 / kTile;
   int k = 40;
   if (!kSingle && !layered && w.tile_rho_max[tile] == 0.0f) {
@@ -868,10 +811,10 @@ __device__ __forceinline__ void force_lbm_body(const WorldDev* __restrict__ worl
     // such tiles.
     tile_clear(sm.wk);
   } else {
-    k = force_tile<R>(sm, w, tile, tb, 0, 0);
+    k = force_tile<R>(sm, w, tile, tb, 0, off, fields || layered);
   }
   // two-layer worlds: F_s only; their layer spread and collision follow in their own kernels
-  if (!layered) tile_lbm(sm.wk, w, tb, k);
+  if (!layered) tile_lbm(sm.wk, w, tb, k, off);
 }
 
 }  // namespace mc
