@@ -74,8 +74,8 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned& gen, unsig
 // Shared memory of the persistent kernel: one stage at a time.
 template <int R>
 union PersistSmem {
-  ForceSmem<R> force;
-  DepositSmem<R> deposit;
+  ForceSmem<R, 256> force;
+  DepositSmem<R, 256> deposit;
 };
 
 }  // namespace
@@ -116,13 +116,13 @@ __global__ void __launch_bounds__(256, kBlocks) k_step_persistent(const PersistA
     // a4 + x pass of a5
     for (unsigned b = blockIdx.x; b < (unsigned)a.n_tile_items; b += gridDim.x) {
       __syncthreads();
-      deposit_x_body<R, false>(a.worlds, a.tile_items, 0, s, w1, b, sm.deposit);
+      deposit_x_body<R, false, 256>(a.worlds, a.tile_items, 0, s, w1, b, sm.deposit);
     }
     if (!(ok = barrier())) break;
     // y pass of a5 + a6 + a7
     for (unsigned b = blockIdx.x; b < (unsigned)a.n_tile_items; b += gridDim.x) {
       __syncthreads();
-      force_lbm_body<R, false>(a.worlds, a.tile_items, s, fields, w1, b, sm.force);
+      force_lbm_body<R, false, 256>(a.worlds, a.tile_items, s, fields, w1, b, sm.force);
     }
     if (!(ok = barrier())) break;
   }

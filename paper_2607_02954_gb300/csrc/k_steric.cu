@@ -47,38 +47,58 @@
 
 namespace mc {
 
-template <int R, bool kSingle>
-__global__ void __launch_bounds__(kThreads, 8) k_deposit_x(const WorldDev* __restrict__ worlds,
+// Threads of a tile's block.  A launch with fewer tiles than the SMs hold
+// blocks of 256 leaves warps idle on every SM, so its tiles take wider
+// blocks: 1024 threads while four times as many narrow blocks would be
+// resident, 512 while twice as many would.  `regs` is the registers a thread
+// of the kernel takes: 32 (deposit) or 64 (force).  A kernel that works on
+// beads alone (the deposit, the spread without the collision) also wants one
+// bead a thread of its tiles, else its barriers cost more than the idle
+// warps (128^2, 16 tiles of 32 beads: deposit 4.6 us with 256 threads, 5.4
+// with 1024).  256^2 with 4096 beads a tile: deposit 47.7 -> 24.1 us, force +
+// LBM 53.7 -> 31.3; 512^2 with 1024 beads a tile: 17.1 -> 15.9 and, with 512
+// threads, 22.4 -> 18.9; 128^2: force + LBM 7.9 -> 7.3.  A tile's sums are
+// integers or per-cell, so the width changes no result.
+static int tile_threads(const Plan& p, int sms, int regs, bool beads_only) {
+  const long long room = (long long)sms * (65536 / (regs * 256));   // blocks of 256 resident at once
+  const long long tiles = p.n_tile_items;
+  for (int nt : {1024, 512})
+    if (tiles * (nt / 256) <= room && (!beads_only || p.beads >= tiles * nt)) return nt;
+  return 256;
+}
+
+template <int R, bool kSingle, int NT>
+__global__ void __launch_bounds__(NT, 2048 / NT) k_deposit_x(const WorldDev* __restrict__ worlds,
                                                         const int2* __restrict__ items, int store_fields,
                                                         int off, const __grid_constant__ WorldDev w1) {
   pdl_trigger();
   pdl_wait();
-  __shared__ __align__(16) DepositSmem<R> sm;
-  deposit_x_body<R, kSingle>(worlds, items, store_fields, off, w1, blockIdx.x, sm);
+  __shared__ __align__(16) DepositSmem<R, NT> sm;
+  deposit_x_body<R, kSingle, NT>(worlds, items, store_fields, off, w1, blockIdx.x, sm);
 }
 
 // y pass of a5 + a6: writes F.
-template <int R>
-__global__ void __launch_bounds__(kThreads) k_force_spread(const WorldDev* __restrict__ worlds,
+template <int R, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_force_spread(const WorldDev* __restrict__ worlds,
                                                            const int2* __restrict__ items, int store_fields,
                                                            int off) {
   pdl_trigger();
   pdl_wait();
-  __shared__ __align__(16) ForceSmem<R> sm;
+  __shared__ __align__(16) ForceSmem<R, NT> sm;
   const int2 it = items[blockIdx.x];
   const WorldDev& w = worlds[it.x];
   const TileBox tb = tile_box(w, it.y);
   float2* __restrict__ F_out = w.F;
   const int W = w.W;
-  const int k = force_tile<R>(sm, w, (tb.y0 / kTile) * w.ntx + tb.x0 / kTile, tb, store_fields, off, true);
+  const int k = force_tile<R, NT>(sm, w, (tb.y0 / kTile) * w.ntx + tb.x0 / kTile, tb, store_fields, off, true);
   __syncthreads();
-  force_fold(sm.wk, tb, w.ntx, w.nty);
+  force_fold<NT>(sm.wk, tb, w.ntx, w.nty);
   const float inv = pow2f(-k);
   const int lane = threadIdx.x & 31;
   // a direct-forcing world's F holds the step's total force (steric spread
   // plus MDF passes): a re-run for the density fields leaves it
   if (store_fields && w.ib == 1) return;
-  for (int ly = threadIdx.x >> 5; ly < tb.th; ly += kWarps) {
+  for (int ly = threadIdx.x >> 5; ly < tb.th; ly += NT / 32) {
     if (lane < tb.tw) {
       const int s = (ly + 3) * kAx + lane + 3;
       F_out[(size_t)(tb.y0 + ly) * W + tb.x0 + lane] = make_float2((float)sm.wk.accx[s] * inv, (float)sm.wk.accy[s] * inv);
@@ -86,18 +106,18 @@ __global__ void __launch_bounds__(kThreads) k_force_spread(const WorldDev* __res
   }
 }
 
-template <int R, bool kSingle>
-__global__ void __launch_bounds__(kThreads, 4) k_force_lbm(const WorldDev* __restrict__ worlds,
+template <int R, bool kSingle, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_force_lbm(const WorldDev* __restrict__ worlds,
                                                            const int2* __restrict__ items, int off, int fields,
                                                            const __grid_constant__ WorldDev w1) {
   pdl_trigger();
   pdl_wait();
-  __shared__ __align__(16) ForceSmem<R> sm;
+  __shared__ __align__(16) ForceSmem<R, NT> sm;
   // tiles in reverse order: the first rows' velocities, written last, are
   // still in L2 when the next PBD (filaments in index order) interpolates
   // them, and the last rows' x-filtered densities, which the deposit wrote
   // last, are read first
-  force_lbm_body<R, kSingle>(worlds, items, off, fields, w1, gridDim.x - 1 - blockIdx.x, sm);
+  force_lbm_body<R, kSingle, NT>(worlds, items, off, fields, w1, gridDim.x - 1 - blockIdx.x, sm);
 }
 
 // y pass of a5 + a6 + a7, warp-specialised and persistent: each block walks
@@ -114,7 +134,7 @@ constexpr int kWsLbmWarps = (kThreads - kWsForce) / 32;
 
 template <int R>
 struct WsSmem {
-  ForceSmem<R> f;
+  ForceSmem<R, kWsForce> f;
   float2 Fh[kTile * kTile];   // the hand-off buffer: F of the tile being collided
 };
 
@@ -148,7 +168,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_force_lbm_ws(const WorldDev* __
         k = force_tile<R, kWsForce>(sm.f, w, tile, tb, 0, off, fields);
       }
       force_sync<kWsForce>();
-      force_fold<TileWork, kWsForce>(sm.f.wk, tb, w.ntx, w.nty);
+      force_fold<kWsForce>(sm.f.wk, tb, w.ntx, w.nty);
       if (done > 0) ws_bar_sync(kWsEmpty);   // the collision warps are done with the previous F
       const float inv = pow2f(-k);
       for (int c = threadIdx.x; c < kTile * kTile; c += kWsForce) {
@@ -204,16 +224,18 @@ __global__ void __launch_bounds__(kThreads, 4) k_force_lbm_ws(const WorldDev* __
 constexpr int kMwy = kTile + 6;   // window rows: the tile and 3 cells a side
 constexpr int kMwx = kTile + 8;   // window columns: the tile and 4 cells a side (16-byte chunks)
 
+constexpr int kMdfCap = 640;      // bead records staged per pass
+
 struct MdfSmem {
-  float4 sp[kForceCap];   // staged bead records
-  float2 su[kForceCap];   // their U_s
-  float2 df[kForceCap];   // their dF (one-pass tiles)
-  int si[kForceCap];      // their bead indices
+  float4 sp[kMdfCap];   // staged bead records
+  float2 su[kMdfCap];   // their U_s
+  float2 df[kMdfCap];   // their dF (one-pass tiles)
+  int si[kMdfCap];      // their bead indices
   float2 uw[kMwy * kMwx];   // input velocity window
   float rw[kMwy * kMwx];    // density window
   int accx[kAx * kAx];    // spread accumulators
   int accy[kAx * kAx];
-  int list[kForceCap];
+  int list[kMdfCap];
   int s_cnt;
   Segments sg;
   float red[kWarps];
@@ -252,7 +274,7 @@ __device__ __forceinline__ float2 mdf_bead_force(const MdfSmem& sm, int v, int r
 __device__ __forceinline__ int mdf_stage_chunk(MdfSmem& sm, const WorldDev& w, const TileBox& tb, int c0, int total) {
   const int tid = threadIdx.x;
   const int W = w.W, H = w.H, ntx = w.ntx, nty = w.nty;
-  const int n = min(kForceCap, total - c0);
+  const int n = min(kMdfCap, total - c0);
   for (int v = tid; v < n; v += kThreads) {
     const int slot = seg_slot(c0 + v, sm.sg);
     cp_async16(&sm.sp[v], &w.bpos[slot]);
@@ -325,10 +347,10 @@ __global__ void __launch_bounds__(kThreads) k_mdf_pass(const WorldDev* __restric
   }
   __syncthreads();   // segments visible (the windows land with the first chunk's wait)
   const int total = sm.sg.pre[kSegs];
-  const bool one_pass = total <= kForceCap;
+  const bool one_pass = total <= kMdfCap;
   // sweep 1: dF of every listed bead and their largest component
   float m = 0.0f;
-  for (int c0 = 0; c0 < total; c0 += kForceCap) {
+  for (int c0 = 0; c0 < total; c0 += kMdfCap) {
     if (c0 > 0) __syncthreads();   // the previous chunk is no longer read
     const int cnt = mdf_stage_chunk(sm, w, tb, c0, total);
     for (int q = tid; q < cnt; q += kThreads) {
@@ -340,12 +362,12 @@ __global__ void __launch_bounds__(kThreads) k_mdf_pass(const WorldDev* __restric
     }
   }
   if (total == 0) cp_async_wait_all();
-  m = block_max(m, sm.red);   // also orders the df writes before sweep 2
+  m = block_max<kThreads>(m, sm.red);   // also orders the df writes before sweep 2
   const int k = fix_exponent(m * w.tile_rho_max[tile] * 1.0001f + 1e-30f);
   const float scale = pow2f(k);
   // sweep 2: the spread, and F_el += dF on the bead's own tile
   float2* __restrict__ fel = w.fel;
-  for (int c0 = 0; c0 < total; c0 += kForceCap) {
+  for (int c0 = 0; c0 < total; c0 += kMdfCap) {
     int cnt = sm.s_cnt;
     if (!one_pass) {
       __syncthreads();
@@ -381,7 +403,7 @@ __global__ void __launch_bounds__(kThreads) k_mdf_pass(const WorldDev* __restric
     }
   }
   __syncthreads();
-  force_fold(sm, tb, ntx, nty);
+  force_fold<kThreads>(sm, tb, ntx, nty);
   const float inv = pow2f(-k);
   // the warp's rows warp, warp + 8, ...: every F load in flight at once
   float2* __restrict__ Fg = w.F;
@@ -413,6 +435,7 @@ namespace {
 // Blocks of the warp-specialised force + LBM kernel: as many as fit on every
 // SM at once (set up outside any stream capture by steric_setup).
 int g_ws_grid[kMaxR + 1] = {};
+int g_sms = 1;   // (steric_setup)
 
 template <int R>
 int ws_grid() {
@@ -429,15 +452,34 @@ void ws_setup(int sms) {
   g_ws_grid[R] = (per > 0 ? per : 1) * sms;
 }
 
+template <int R, int NT>
+void launch_deposit(const Plan& p, cudaStream_t s, int store_fields, int off) {
+  launch_pdl(p.n_worlds == 1 ? k_deposit_x<R, true, NT> : k_deposit_x<R, false, NT>, p.n_tile_items, NT, 0, s,
+             p.d_worlds, p.d_tile_items, store_fields, off, p.h_world0);
+}
+
+template <int R, int NT>
+void launch_spread(const Plan& p, cudaStream_t s, int store_fields, int off) {
+  k_force_spread<R, NT><<<p.n_tile_items, NT, 0, s>>>(p.d_worlds, p.d_tile_items, store_fields, off);
+}
+
+template <int R, int NT>
+void launch_fused(const Plan& p, cudaStream_t s, int off, int fields) {
+  launch_pdl(p.n_worlds == 1 ? k_force_lbm<R, true, NT> : k_force_lbm<R, false, NT>, p.n_tile_items, NT, 0, s,
+             p.d_worlds, p.d_tile_items, off, fields, p.h_world0);
+}
+
 template <int R>
-void launch_steric(const Plan& p, cudaStream_t s, int which, int store_fields, int off, int fields = 1) {
+void launch_steric(const Plan& p, cudaStream_t s, int which, int store_fields, int off, int fields) {
+  const int nt = tile_threads(p, g_sms, which == 0 ? 32 : 64, which != 2);
   if (which == 0) {
-    if (p.n_worlds == 1)
-      launch_pdl(k_deposit_x<R, true>, p.n_tile_items, kThreads, 0, s, p.d_worlds, p.d_tile_items, store_fields, off, p.h_world0);
-    else
-      launch_pdl(k_deposit_x<R, false>, p.n_tile_items, kThreads, 0, s, p.d_worlds, p.d_tile_items, store_fields, off, p.h_world0);
+    if (nt == 1024) launch_deposit<R, 1024>(p, s, store_fields, off);
+    else if (nt == 512) launch_deposit<R, 512>(p, s, store_fields, off);
+    else launch_deposit<R, 256>(p, s, store_fields, off);
   } else if (which == 1) {
-    k_force_spread<R><<<p.n_tile_items, kThreads, 0, s>>>(p.d_worlds, p.d_tile_items, store_fields, off);
+    if (nt == 1024) launch_spread<R, 1024>(p, s, store_fields, off);
+    else if (nt == 512) launch_spread<R, 512>(p, s, store_fields, off);
+    else launch_spread<R, 256>(p, s, store_fields, off);
   } else if (p.cfg.force_ws && !p.any_layered) {
     const int grid = std::min(p.n_tile_items, ws_grid<R>());
     if (p.n_worlds == 1)
@@ -447,10 +489,9 @@ void launch_steric(const Plan& p, cudaStream_t s, int which, int store_fields, i
       launch_pdl(k_force_lbm_ws<R, false>, grid, kThreads, sizeof(WsSmem<R>), s, p.d_worlds, p.d_tile_items,
                  p.n_tile_items, off, fields, p.h_world0);
   } else {
-    if (p.n_worlds == 1)
-      launch_pdl(k_force_lbm<R, true>, p.n_tile_items, kThreads, 0, s, p.d_worlds, p.d_tile_items, off, fields, p.h_world0);
-    else
-      launch_pdl(k_force_lbm<R, false>, p.n_tile_items, kThreads, 0, s, p.d_worlds, p.d_tile_items, off, fields, p.h_world0);
+    if (nt == 1024) launch_fused<R, 1024>(p, s, off, fields);
+    else if (nt == 512) launch_fused<R, 512>(p, s, off, fields);
+    else launch_fused<R, 256>(p, s, off, fields);
   }
 }
 
@@ -471,6 +512,7 @@ void dispatch_steric(const Plan& p, cudaStream_t s, int which, int store_fields,
 }  // namespace
 
 void steric_setup(int sms) {
+  g_sms = sms;
   ws_setup<1>(sms);
   ws_setup<2>(sms);
   ws_setup<3>(sms);

@@ -160,6 +160,7 @@ mc_status build_plan(mc_world* const* ws, int n, cudaStream_t s, Plan& out) {
     const mc_world* w = ws[k];
     table[k] = w->h;
     p.max_B = std::max(p.max_B, w->max_B);
+    p.beads += w->h.N;
     p.max_R = std::max(p.max_R, w->h.R);
     p.any_layered = p.any_layered || w->h.layers == 2;
     p.any_mdf = p.any_mdf || w->h.ib == 1;

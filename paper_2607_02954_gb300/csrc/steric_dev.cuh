@@ -9,9 +9,8 @@ namespace mc {
 
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 256;              // threads of a tile's block (the narrowest, see tile_threads)
 constexpr int kWarps = kThreads / 32;
-constexpr int kForceCap = 640;             // bead records staged per pass (force)
 constexpr int kAx = kTile + 6;             // force accumulator edge: the tile and 3 halo cells a side
 constexpr int kWin = kTile + 8;            // rho_bar window edge: the tile and 4 cells a side
 __constant__ int kLbmCy[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};   // D2Q9 lattice velocities, y components
@@ -146,13 +145,13 @@ __device__ __forceinline__ int code_slot(int c) { return c & 1023; }
 __device__ __forceinline__ int code_rx(int c) { return ((c >> 10) & 2047) - 16; }
 __device__ __forceinline__ int code_ry(int c) { return (c >> 21) - 16; }
 
-template <typename T>
+template <int NT, typename T>
 __device__ __forceinline__ T block_max(T v, T* red) {
   for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
   T m = red[0];
-  for (int k = 1; k < kWarps; ++k) m = max(m, red[k]);
+  for (int k = 1; k < NT / 32; ++k) m = max(m, red[k]);
   __syncthreads();
   return m;
 }
@@ -200,7 +199,7 @@ struct DepTile {
 
 // Deposits the tile's beads at scale 2^k into acc (zeroed) and folds the
 // wrapped cells.  Ends with the block synchronised.
-template <int R>
+template <int R, int NT>
 __device__ __forceinline__ void deposit_accumulate(int* acc, const WorldDev& w, const DepTile& d, int k,
                                                    const Segments& sg) {
   using G = Geo<R>;
@@ -210,7 +209,7 @@ __device__ __forceinline__ void deposit_accumulate(int* acc, const WorldDev& w, 
   const bool full_x = d.full_x, full_y = d.full_y;
   const float4* __restrict__ bpos = w.bpos;
   const float scale = pow2f(k);
-  // each thread deposits the beads v = tid, tid + 256, ... of the segments
+  // each thread deposits the beads v = tid, tid + NT, ... of the segments
   // straight from their slots, two loads in flight at a time;
   // a bead whose stencil misses the region adds nothing
   auto deposit = [&](const float4 p) {
@@ -236,8 +235,8 @@ __device__ __forceinline__ void deposit_accumulate(int* acc, const WorldDev& w, 
       for (int a = 0; a < 4; ++a) atomicAdd(base + b * G::kDX + a, __float2int_rn(wx[a] * sy));
     }
   };
-  for (int v0 = tid; v0 < total; v0 += 2 * kThreads) {
-    const int v1 = v0 + kThreads;
+  for (int v0 = tid; v0 < total; v0 += 2 * NT) {
+    const int v1 = v0 + NT;
     const float4 p0 = bpos[seg_slot(v0, sg)];
     float4 p1 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     if (v1 < total) p1 = bpos[seg_slot(v1, sg)];
@@ -247,7 +246,7 @@ __device__ __forceinline__ void deposit_accumulate(int* acc, const WorldDev& w, 
   __syncthreads();
   if (full_x || full_y) {
     // fold the stencil cells that wrapped around an axis the region covers whole
-    for (int c = tid; c < G::kDY * G::kDX; c += kThreads) {
+    for (int c = tid; c < G::kDY * G::kDX; c += NT) {
       const int ly = c / G::kDX - 3, lx = c % G::kDX - oxe;
       const bool out_y = ly < 0 || ly >= th;
       const bool out_x = full_x && (lx < 0 || lx >= W);
@@ -264,7 +263,7 @@ __device__ __forceinline__ void deposit_accumulate(int* acc, const WorldDev& w, 
 
 // The x pass of the accumulated sums at scale 2^k, rho_s when asked for,
 // and the tile's bound (see k_deposit_x).
-template <int R>
+template <int R, int NT>
 __device__ __forceinline__ void deposit_xpass(const int* acc, const WorldDev& w, const DepTile& d, int k,
                                               const float* tap_s, float* red, int store_fields) {
   using G = Geo<R>;
@@ -312,7 +311,7 @@ __device__ __forceinline__ void deposit_xpass(const int* acc, const WorldDev& w,
         *reinterpret_cast<float4*>(rho_s_out + c) = make_float4(v[R] * inv, v[R + 1] * inv, v[R + 2] * inv, v[R + 3] * inv);
     }
   } else {
-    for (int c = tid; c < th * kTile; c += kThreads) {
+    for (int c = tid; c < th * kTile; c += NT) {
       const int ly = c >> 5, lx = c & 31;
       if (lx < tw) {
         const float v = (float)acc[(ly + 3) * G::kDX + col0 + lx];
@@ -320,7 +319,7 @@ __device__ __forceinline__ void deposit_xpass(const int* acc, const WorldDev& w,
         if (store_fields) rho_s_out[(size_t)(y0 + ly) * W + x0 + lx] = v * inv;
       }
     }
-    for (int c = tid; c < th * tw; c += kThreads) {
+    for (int c = tid; c < th * tw; c += NT) {
       const int ly = c / tw, lx = c - ly * tw;
       const int* r = acc + (ly + 3) * G::kDX + oxe;
       float sacc = 0.0f;
@@ -329,7 +328,7 @@ __device__ __forceinline__ void deposit_xpass(const int* acc, const WorldDev& w,
       rho_x[(size_t)(y0 + ly) * W + x0 + lx] = sacc;
     }
   }
-  vmax = block_max(vmax, red);
+  vmax = block_max<NT>(vmax, red);
   // Stored bound of the tile's cell sums of the kernel weights, used for
   // the fixed-point scales of the spread: the largest deposited sum plus the
   // largest rounding its terms can hide (half a unit per bead of the
@@ -341,12 +340,12 @@ __device__ __forceinline__ void deposit_xpass(const int* acc, const WorldDev& w,
 }
 
 // Shared memory of the deposit of one tile.
-template <int R>
+template <int R, int NT>
 struct DepositSmem {
   int acc[Geo<R>::kDY * Geo<R>::kDX];
   float tap_s[Geo<R>::kTaps];
   Segments sg;
-  float red[kWarps];
+  float red[NT / 32];
 };
 
 // a4 + the x pass of a5 for the tile item of block `blk` (block-uniform
@@ -354,10 +353,10 @@ struct DepositSmem {
 // step: the other parity's counts of the tile's own bins, its overflow count
 // and its F_el-maximum slot go to zero (the previous step's; this step's
 // stay readable).
-template <int R, bool kSingle>
+template <int R, bool kSingle, int NT>
 __device__ __forceinline__ void deposit_x_body(const WorldDev* __restrict__ worlds, const int2* __restrict__ items,
                                                int store_fields, int off, const WorldDev& w1, unsigned blk,
-                                               DepositSmem<R>& sm) {
+                                               DepositSmem<R, NT>& sm) {
   using G = Geo<R>;
   int* acc = sm.acc;
   float* tap_s = sm.tap_s;
@@ -394,7 +393,7 @@ __device__ __forceinline__ void deposit_x_body(const WorldDev* __restrict__ worl
     }
   }
   if (warp == 1 && lane < G::kTaps) tap_s[lane] = padded_tap<R>(w, d.wR, lane);
-  for (int c = tid; c < G::kDY * G::kDX / 4; c += kThreads) reinterpret_cast<int4*>(acc)[c] = make_int4(0, 0, 0, 0);
+  for (int c = tid; c < G::kDY * G::kDX / 4; c += NT) reinterpret_cast<int4*>(acc)[c] = make_int4(0, 0, 0, 0);
   __syncthreads();
   d.total = sg.covered;
   if (d.total == 0) {
@@ -412,23 +411,23 @@ __device__ __forceinline__ void deposit_x_body(const WorldDev* __restrict__ worl
     return;
   }
   int k = fix_exponent((float)sg.most + 1.0f);
-  deposit_accumulate<R>(acc, w, d, k, sg);
+  deposit_accumulate<R, NT>(acc, w, d, k, sg);
   if (k < 24) {
     // dense tile: the largest accumulated sum plus the rounding of its terms
     // (half a unit per bead of the covering bins, at most one term per cell
     // each) bounds every sum; deposit again at the scale that bound gives
     int m = 0;
-    for (int c = tid; c < G::kDY * G::kDX; c += kThreads) m = max(m, acc[c]);
-    m = block_max(m, reinterpret_cast<int*>(red));
+    for (int c = tid; c < G::kDY * G::kDX; c += NT) m = max(m, acc[c]);
+    m = block_max<NT>(m, reinterpret_cast<int*>(red));
     const int k2 = fix_exponent(((float)m + 0.5f * (float)d.total) * pow2f(-k) * 1.0001f);
     if (k2 > k) {
-      for (int c = tid; c < G::kDY * G::kDX / 4; c += kThreads) reinterpret_cast<int4*>(acc)[c] = make_int4(0, 0, 0, 0);
+      for (int c = tid; c < G::kDY * G::kDX / 4; c += NT) reinterpret_cast<int4*>(acc)[c] = make_int4(0, 0, 0, 0);
       __syncthreads();
       k = k2;
-      deposit_accumulate<R>(acc, w, d, k, sg);
+      deposit_accumulate<R, NT>(acc, w, d, k, sg);
     }
   }
-  deposit_xpass<R>(acc, w, d, k, tap_s, red, store_fields);
+  deposit_xpass<R, NT>(acc, w, d, k, tap_s, red, store_fields);
 }
 
 // ---------------------------------------------------------------------------
@@ -448,20 +447,26 @@ struct TileIn {
   float tap_s[Geo<R>::kTaps];
 };
 
+// Beads listed per pass by a block of NT threads.
+template <int NT>
+constexpr int kForceCap = 5 * NT / 2;
+
 // Working arrays of the tile being computed.
+template <int NT>
 struct TileWork {
-  float4 sp[kForceCap];                 // listed beads: fractions, tile-relative cell (int bits)
-  float4 sr[kForceCap];                 // their F_el (x, y) and bead id (int bits)
+  static constexpr int kCap = kForceCap<NT < kThreads ? kThreads : NT>;
+  float4 sp[kCap];                      // listed beads: fractions, tile-relative cell (int bits)
+  float4 sr[kCap];                      // their F_el (x, y) and bead id (int bits)
   float win[kWin * kWin];               // rho_bar window
   int accx[kAx * kAx];                  // spread accumulators
   int accy[kAx * kAx];
   int s_cnt;
 };
 
-template <int R>
+template <int R, int NT>
 struct ForceSmem {
   TileIn<R> in;
-  TileWork wk;
+  TileWork<NT> wk;
 };
 
 struct TileBox {
@@ -469,11 +474,11 @@ struct TileBox {
 };
 
 // Barrier of the NT threads that run a tile's force phase: the whole block
-// (NT == kThreads), or warps 0 .. NT/32 - 1 on named barrier 1 (the
+// (NT >= kThreads), or warps 0 .. NT/32 - 1 on named barrier 1 (the
 // warp-specialised kernel, whose other warps collide).
 template <int NT>
 __device__ __forceinline__ void force_sync() {
-  if (NT == kThreads) __syncthreads();
+  if (NT >= kThreads) __syncthreads();
   else asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory");
 }
 
@@ -482,7 +487,7 @@ __device__ __forceinline__ void force_sync() {
 // reads records straight from their slots, two in flight, and the ones that
 // reach the tile are packed into the working arrays.
 template <int NT>
-__device__ __forceinline__ void force_list(const Segments& sg, TileWork& wk, const WorldDev& w, int c0, int n,
+__device__ __forceinline__ void force_list(const Segments& sg, TileWork<NT>& wk, const WorldDev& w, int c0, int n,
                                            const TileBox& tb) {
   const int W = w.W, H = w.H, ntx = w.ntx, nty = w.nty;
   const float4* __restrict__ bpos = w.bpos;
@@ -528,7 +533,7 @@ __device__ __forceinline__ void force_list(const Segments& sg, TileWork& wk, con
 // columns [x0 - 4, x0 + tw + 4) in 16-byte cp.async chunks (independent of
 // the beads).  A 4-column chunk never straddles the periodic edge (x0 and W
 // are multiples of 8); rows reach at most 4 + R <= 12 cells outside the axis.
-template <int R, int NT = kThreads>
+template <int R, int NT>
 __device__ __forceinline__ void tile_stage_window(TileIn<R>& in, const WorldDev& w, const TileBox& tb) {
   const int W = w.W, H = w.H, tid = threadIdx.x;
   const float* __restrict__ rho_x = w.rho_x;
@@ -574,8 +579,8 @@ __device__ __forceinline__ void tile_stage_meta(TileIn<R>& in, const WorldDev& w
 
 // Zeroes the spread accumulators and the list count (before the barrier
 // that precedes tile_compute).
-template <int NT = kThreads>
-__device__ __forceinline__ void tile_clear(TileWork& wk) {
+template <int NT>
+__device__ __forceinline__ void tile_clear(TileWork<NT>& wk) {
   for (int c = threadIdx.x; c < kAx * kAx / 4; c += NT) {
     reinterpret_cast<int4*>(wk.accx)[c] = make_int4(0, 0, 0, 0);
     reinterpret_cast<int4*>(wk.accy)[c] = make_int4(0, 0, 0, 0);
@@ -586,7 +591,7 @@ __device__ __forceinline__ void tile_clear(TileWork& wk) {
 // The y pass of a5: rho_bar on the window from the staged rho_x, 8 window
 // rows per thread.
 template <int R, int NT>
-__device__ __forceinline__ void tile_ypass(const TileIn<R>& in, TileWork& wk, const WorldDev& w, const TileBox& tb,
+__device__ __forceinline__ void tile_ypass(const TileIn<R>& in, TileWork<NT>& wk, const WorldDev& w, const TileBox& tb,
                                            int store_fields) {
   using G = Geo<R>;
   const int W = w.W, tw = tb.tw, th = tb.th;
@@ -622,7 +627,7 @@ __device__ __forceinline__ void tile_ypass(const TileIn<R>& in, TileWork& wk, co
 // bead's own tile when asked for) and the spread of F_el + F_s into the
 // accumulators at the given scale.
 template <int NT>
-__device__ __forceinline__ void tile_beads(TileWork& wk, const WorldDev& w, const TileBox& tb, int cnt, float scale,
+__device__ __forceinline__ void tile_beads(TileWork<NT>& wk, const WorldDev& w, const TileBox& tb, int cnt, float scale,
                                            bool keep_fs) {
   const float k_rep = w.k_rep;
   const bool layered = w.layers == 2;
@@ -679,17 +684,18 @@ __device__ __forceinline__ void tile_beads(TileWork& wk, const WorldDev& w, cons
 // The y pass of a5 and a6 for one tile.  Returns k: after the caller
 // synchronises the block, accx/accy hold the tile's F 2^k (before folding,
 // see force_fold).
-template <int R, int NT = kThreads>
-__device__ __forceinline__ int force_tile(ForceSmem<R>& sm, const WorldDev& w, int tile, const TileBox& tb,
+template <int R, int NT>
+__device__ __forceinline__ int force_tile(ForceSmem<R, NT>& sm, const WorldDev& w, int tile, const TileBox& tb,
                                           int store_fields, int off, bool keep_fs) {
+  constexpr int kCap = TileWork<NT>::kCap;
   TileIn<R>& in = sm.in;
-  TileWork& wk = sm.wk;
+  TileWork<NT>& wk = sm.wk;
   tile_stage_window<R, NT>(in, w, tb);
   tile_stage_meta(in, w, tb, off);
   tile_clear<NT>(wk);
   force_sync<NT>();
   const int total = in.sg.pre[kSegs];
-  force_list<NT>(in.sg, wk, w, 0, min(kForceCap, total), tb);
+  force_list<NT>(in.sg, wk, w, 0, min(kCap, total), tb);
   cp_async_wait_all();   // the window
   const float fmax_el = __uint_as_float(w.fel_max[(*w.t + off) & 1]);
   const float rho_max = w.tile_rho_max[tile];
@@ -702,11 +708,11 @@ __device__ __forceinline__ int force_tile(ForceSmem<R>& sm, const WorldDev& w, i
   if (total > 0 || store_fields) tile_ypass<R, NT>(in, wk, w, tb, store_fields);
   force_sync<NT>();
   tile_beads<NT>(wk, w, tb, wk.s_cnt, scale, keep_fs);
-  for (int c0 = kForceCap; c0 < total; c0 += kForceCap) {
+  for (int c0 = kCap; c0 < total; c0 += kCap) {
     force_sync<NT>();   // every thread is done with the previous chunk
     if (threadIdx.x == 0) wk.s_cnt = 0;
     force_sync<NT>();
-    force_list<NT>(in.sg, wk, w, c0, min(kForceCap, total - c0), tb);
+    force_list<NT>(in.sg, wk, w, c0, min(kCap, total - c0), tb);
     force_sync<NT>();
     tile_beads<NT>(wk, w, tb, wk.s_cnt, scale, keep_fs);
   }
@@ -715,7 +721,7 @@ __device__ __forceinline__ int force_tile(ForceSmem<R>& sm, const WorldDev& w, i
 
 // Folds the stencil cells that wrapped around an axis the tile covers whole
 // (one tile on that axis); call after the block has synchronised.
-template <class Work, int NT = kThreads>
+template <int NT, class Work>
 __device__ __forceinline__ void force_fold(Work& wk, const TileBox& tb, int ntx, int nty) {
   if (ntx > 1 && nty > 1) return;
   const bool fx = ntx == 1, fy = nty == 1;
@@ -742,7 +748,7 @@ __device__ __forceinline__ TileBox tile_box(const WorldDev& w, int packed) {
 }
 
 // The tile's population rows (plane i, rows y - c_iy, 128-byte segments) to L2.
-template <int NT = kThreads>
+template <int NT>
 __device__ __forceinline__ void prefetch_populations(const WorldDev& w, const TileBox& tb, int off) {
   const float* src = w.g[(*w.t + off) & 1];
   const int W = w.W, H = w.H;
@@ -757,10 +763,11 @@ __device__ __forceinline__ void prefetch_populations(const WorldDev& w, const Ti
 }
 
 // a7 on the tile's cells with F = acc 2^-k from shared memory.  Each warp
-// collides rows warp, warp + 8, ...; the first row's populations are pulled
+// collides rows warp, warp + NT / 32, ...; the first row's populations are pulled
 // before the barrier that completes the spread (pulling one row ahead in the
 // loop measured slower: register pressure).
-__device__ __forceinline__ void tile_lbm(TileWork& wk, const WorldDev& w, const TileBox& tb, int k, int off) {
+template <int NT>
+__device__ __forceinline__ void tile_lbm(TileWork<NT>& wk, const WorldDev& w, const TileBox& tb, int k, int off) {
   const int W = w.W, H = w.H, HW = H * W;
   const long long t = *w.t + off;
   const float* __restrict__ src = w.g[t & 1];
@@ -776,15 +783,15 @@ __device__ __forceinline__ void tile_lbm(TileWork& wk, const WorldDev& w, const 
   int y = tb.y0 + warp;
   if (active) lbm_pull(src, HW, y * W, (y == 0 ? H - 1 : y - 1) * W, (y == H - 1 ? 0 : y + 1) * W, x, xm, xp, q);
   __syncthreads();
-  force_fold(wk, tb, w.ntx, w.nty);
+  force_fold<NT>(wk, tb, w.ntx, w.nty);
   if (!active) return;
-  for (int ly = warp; ly < tb.th; ly += kWarps) {
+  for (int ly = warp; ly < tb.th; ly += NT / 32) {
     if (ly != warp)
       lbm_pull(src, HW, y * W, (y == 0 ? H - 1 : y - 1) * W, (y == H - 1 ? 0 : y + 1) * W, x, xm, xp, q);
     const int s = (ly + 3) * kAx + lane + 3;
     const float2 F = make_float2((float)wk.accx[s] * inv, (float)wk.accy[s] * inv);
     u_out[(size_t)y * W + x] = lbm_collide(q, dst, HW, y * W + x, F, kc);
-    y += kWarps;
+    y += NT / 32;
   }
 }
 
@@ -793,15 +800,15 @@ __device__ __forceinline__ void tile_lbm(TileWork& wk, const WorldDev& w, const 
 // followed by k_lbm, without F's round trip through HBM).  The tile's
 // population rows are prefetched into L2 on entry, so their DRAM reads
 // overlap the force phase.
-template <int R, bool kSingle>
+template <int R, bool kSingle, int NT>
 __device__ __forceinline__ void force_lbm_body(const WorldDev* __restrict__ worlds, const int2* __restrict__ items,
                                                int off, int fields, const WorldDev& w1, unsigned blk,
-                                               ForceSmem<R>& sm) {
+                                               ForceSmem<R, NT>& sm) {
   const int2 it = kSingle ? single_tile_item(w1, blk) : items[blk];
   const WorldDev& w = kSingle ? w1 : worlds[it.x];
   const TileBox tb = tile_box(w, it.y);
   const bool layered = w.layers == 2;
-  if (!layered) prefetch_populations(w, tb, off);
+  if (!layered) prefetch_populations<NT>(w, tb, off);
   const int tile = (tb.y0 / kTile) * w.ntx + tb.x0 / kTile;
   int k = 40;
   if (!kSingle && !layered && w.tile_rho_max[tile] == 0.0f) {
@@ -809,12 +816,12 @@ __device__ __forceinline__ void force_lbm_body(const WorldDev* __restrict__ worl
     // exactly then), so it owns no bead and the spread has no term on it:
     // F = 0, as the force pass would give.  Sparse batched worlds have many
     // such tiles.
-    tile_clear(sm.wk);
+    tile_clear<NT>(sm.wk);
   } else {
-    k = force_tile<R>(sm, w, tile, tb, 0, off, fields || layered);
+    k = force_tile<R, NT>(sm, w, tile, tb, 0, off, fields || layered);
   }
   // two-layer worlds: F_s only; their layer spread and collision follow in their own kernels
-  if (!layered) tile_lbm(sm.wk, w, tb, k, off);
+  if (!layered) tile_lbm<NT>(sm.wk, w, tb, k, off);
 }
 
 }  // namespace mc

@@ -113,3 +113,41 @@ def test_rewind_to_either_parity_starts_from_empty_bins(n):
     for k in want:
         assert np.array_equal(want[k], got[k]), k
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("H,W,n_fil,B", [(96, 64, 80, 64), (256, 256, 1024, 64), (416, 704, 2288, 64), (640, 648, 2580, 64),
+                                         (480, 1288, 300, 24)])
+def test_wide_tile_blocks_equal_the_narrow_ones(H, W, n_fil, B):
+    """Worlds on both sides of the lines where a tile's block gets wider (few
+    tiles, many beads a tile) against the persistent step, whose tiles always
+    take 256 threads: bitwise the same, and one step against the oracle."""
+    from paper_2607_02954_gb300 import set_launch_config
+    rng = np.random.default_rng(H + W)
+    f = np.arange(n_fil)
+    per_row = W // B
+    x, y = [], []
+    rows = -(-n_fil // per_row)
+    x0, y0 = (f % per_row) * B + rng.uniform(0, 0.5, n_fil), (f // per_row) * H / rows + rng.uniform(0, 0.5, n_fil)
+    x = np.mod(x0[:, None] + np.arange(B)[None], W).astype(np.float32).ravel()
+    y = np.mod(np.repeat(y0, B), H).astype(np.float32)
+    x[x >= W] = 0
+    y[y >= H] = 0
+    J = n_fil * (B - 2)
+    spec = synth._world("wide", H, W, [B] * n_fil, x, y, np.zeros(n_fil * (B - 1), np.float32),
+                        rng.normal(0, 0.1, J), np.full(J, 0.2), np.full(J, 0.01), rng.uniform(0, 1, J),
+                        params=synth.Params(k_rep=0.1))
+    a, b = World(spec), World(spec)
+    set_launch_config([b], persistent=4)
+    for w in (a, b):
+        w.step(3)
+    want, got = a.state(fluid=True), b.state(fluid=True)
+    for k in want:
+        assert np.array_equal(want[k], got[k]), k
+    for k in ("fel", "fs", "rho_s", "rho_bar", "force"):
+        assert np.array_equal(a.field(k), b.field(k)), k
+    ow = O.World(spec)
+    _, rec = O.step(ow, ow.initial_state(), record=True)
+    c = World(spec)
+    c.step(1)
+    assert_field("rho_s", c.field("rho_s"), t2n(rec["rho_s"]), 1e-5)
+    assert_field("u", c.field("u"), np.moveaxis(t2n(rec["u"]), 0, -1), 1e-5)
