@@ -119,8 +119,6 @@ __device__ __forceinline__ float2 layer_velocity(const WorldDev& w, const float4
   return make_float2(Ux, Uy);
 }
 
-constexpr double kLayerScale = 1099511627776.0;   // 2^40: fixed point of the layer spread
-
 // The energy field sampled at p with the interpolation kernel.
 __device__ __forceinline__ float energy_sample(const WorldDev& w, const float4 q) {
   const int W = w.W, H = w.H;
@@ -187,14 +185,6 @@ __device__ __forceinline__ PbdConst pbd_const(const WorldDev& w) {
   k.H = w.H;
   k.nbx = w.nbx;
   return k;
-}
-
-// Edge vector min_image(X_b - X_a) from cell indices and fractions.
-__device__ __forceinline__ float2 edge_vec(const float4 pa, const float4 pb, int W, int H) {
-  int dcx = cell_x(pb) - cell_x(pa), dcy = cell_y(pb) - cell_y(pa);
-  if (2 * dcx > W) dcx -= W; else if (2 * dcx < -W) dcx += W;
-  if (2 * dcy > H) dcy -= H; else if (2 * dcy < -H) dcy += H;
-  return make_float2((float)dcx + (pb.x - pa.x), (float)dcy + (pb.y - pa.y));
 }
 
 // The per-edge factors of the position pass: sc = (l - L)/l = 1 - L/l with

@@ -41,24 +41,22 @@ __global__ void __launch_bounds__(kBeadChunk) k_layer_spread(const WorldDev* __r
   const float4 p = w.bpos[slot];
   const float2 n = w.nrm[i], fe = make_float2(rec.x, rec.y), fs = w.fs[i];
   const float hx = 0.5f * (fe.x + fs.x), hy = 0.5f * (fe.y + fs.y);
-  for (int side = 0; side < 2; ++side) {
-    int cx, cy;
-    float fx, fy;
-    layer_cell(p, n, side ? -w.layer_half : w.layer_half, W, H, cx, cy, fx, fy);
-    float wx[4], wy[4];
-    peskin4(fx, wx);
-    peskin4(fy, wy);
+  const int b = threadIdx.x & 3;
+  int cx, cy;
+  float fx, fy;
+  layer_cell(p, n, (threadIdx.x & 4) ? -w.layer_half : w.layer_half, W, H, cx, cy, fx, fy);
+  float wx[4], wy[4];
+  peskin4(fx, wx);
+  peskin4(fy, wy);
+  const float wyb = (b & 2) ? ((b & 1) ? wy[3] : wy[2]) : ((b & 1) ? wy[1] : wy[0]);
+  unsigned long long* row = w.facc + 2 * (size_t)wrap_once(cy - 1 + b, H) * W;
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      unsigned long long* row = w.facc + 2 * (size_t)wrap_once(cy - 1 + b, H) * W;
-#pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        const float g = wx[a] * wy[b];
-        unsigned long long* c = row + 2 * wrap_once(cx - 1 + a, W);
-        atomicAdd(c, (unsigned long long)__double2ll_rn((double)(g * hx) * kLayerScale));
-        atomicAdd(c + 1, (unsigned long long)__double2ll_rn((double)(g * hy) * kLayerScale));
-      }
-    }
+  for (int a = 0; a < 4; ++a) {
+    const float g = wx[a] * wyb;
+    unsigned long long* c = row + 2 * wrap_once(cx - 1 + a, W);
+    // (the scale is a power of two: the products are exact)
+    atomicAdd(c, (unsigned long long)__float2ll_rn(g * hx * kLayerScale));
+    atomicAdd(c + 1, (unsigned long long)__float2ll_rn(g * hy * kLayerScale));
   }
 }
 
@@ -72,10 +70,7 @@ __global__ void __launch_bounds__(kCellChunk) k_layer_finish(const WorldDev* __r
   if (w.layers != 2) return;
   const int c = it.y + threadIdx.x;
   if (c >= w.H * w.W) return;
-  const long long ax = (long long)w.facc[2 * c], ay = (long long)w.facc[2 * c + 1];
-  w.F[c] = make_float2((float)((double)ax / kLayerScale), (float)((double)ay / kLayerScale));
-  w.facc[2 * c] = 0ull;
-  w.facc[2 * c + 1] = 0ull;
+  w.F[c] = layer_force(w, c);
 }
 
 // a8: U_i = sum_c delta_h(c - X_i) u(c) over the 4x4 stencil, then the

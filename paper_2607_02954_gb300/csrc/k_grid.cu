@@ -150,7 +150,9 @@ __global__ void __launch_bounds__(kCellChunk) k_lbm(const WorldDev* __restrict__
   const int ym = y == 0 ? H - 1 : y - 1, yp = y == H - 1 ? 0 : y + 1;
   const long long t = *w.t + off;
   const LbmConst k{w.om_p, w.om_m, w.src_p, w.src_m};
-  w.u[c] = lbm_cell(w.g[t & 1], w.g[(t + 1) & 1], HW, y * W, ym * W, yp * W, x, xm, xp, w.F[c], k);
+  // (layered_only follows the layer spread directly: its F needs no round trip through memory)
+  const float2 F = layered_only ? layer_force(w, c) : w.F[c];
+  w.u[c] = lbm_cell(w.g[t & 1], w.g[(t + 1) & 1], HW, y * W, ym * W, yp * W, x, xm, xp, F, k);
 }
 
 // ---------------------------------------------------------------------------

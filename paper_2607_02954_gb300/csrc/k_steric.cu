@@ -540,7 +540,7 @@ void launch_mdf_pass(const Plan& p, cudaStream_t s, int pass) {
 void launch_force_lbm(const Plan& p, cudaStream_t s, int off, int fields) {
   dispatch_steric(p, s, 2, 0, off, fields);
   if (p.any_layered) {
-    launch_layer_spread(p, s);
+    launch_layer_spread(p, s, false);
     launch_lbm(p, s, 1, off);
   }
 }

@@ -235,7 +235,9 @@ void launch_deposit_x(const Plan& p, cudaStream_t s, int store_fields, int off =
 // y pass of a5 + a6; store_fields also writes rho_bar of each tile
 void launch_force_spread(const Plan& p, cudaStream_t s, int store_fields, int off = 0);
 void launch_lbm(const Plan& p, cudaStream_t s, int layered_only = 0, int off = 0);   // layered_only: two-layer worlds only
-void launch_layer_spread(const Plan& p, cudaStream_t s);   // two-layer worlds: F from the layer points
+// two-layer worlds: the spread from the layer points; finish: F from it (else
+// the following launch_lbm with layered_only takes it from the accumulator)
+void launch_layer_spread(const Plan& p, cudaStream_t s, bool finish = true);
 // y pass of a5 + a6 + a7 in one kernel; fields as in launch_advance_pbd
 void launch_force_lbm(const Plan& p, cudaStream_t s, int off = 0, int fields = 1);
 void launch_interp_advance(const Plan& p, cudaStream_t s, int inc = 1);   // inc: steps the counter moves by
@@ -499,6 +501,24 @@ __device__ __forceinline__ int* step_counts(const WorldDev& w, long long t) {
 
 __device__ __forceinline__ int cell_x(const float4& p) { return __float_as_int(p.z); }
 __device__ __forceinline__ int cell_y(const float4& p) { return __float_as_int(p.w); }
+
+// Edge vector min_image(X_b - X_a) from cell indices and fractions.
+__device__ __forceinline__ float2 edge_vec(const float4 pa, const float4 pb, int W, int H) {
+  int dcx = cell_x(pb) - cell_x(pa), dcy = cell_y(pb) - cell_y(pa);
+  if (2 * dcx > W) dcx -= W; else if (2 * dcx < -W) dcx += W;
+  if (2 * dcy > H) dcy -= H; else if (2 * dcy < -H) dcy += H;
+  return make_float2((float)dcx + (pb.x - pa.x), (float)dcy + (pb.y - pa.y));
+}
+
+// The layer spread of cell c out of its fixed point, the accumulator cleared
+// for the next step.
+constexpr float kLayerScale = 1099511627776.0f;   // 2^40
+__device__ __forceinline__ float2 layer_force(const WorldDev& w, int c) {
+  ulonglong2* acc = reinterpret_cast<ulonglong2*>(w.facc) + c;   // (two words a cell, 256-byte aligned)
+  const ulonglong2 v = *acc;
+  *acc = make_ulonglong2(0ull, 0ull);
+  return make_float2((float)(long long)v.x * (1.0f / kLayerScale), (float)(long long)v.y * (1.0f / kLayerScale));
+}
 
 // Cell and fraction of the point X + d n for X = (cell, fraction) in p.
 __device__ __forceinline__ void layer_cell(const float4 p, float2 n, float d, int W, int H, int& cx, int& cy,
