@@ -302,7 +302,7 @@ __device__ __forceinline__ float2 bead_out_force(const WorldDev& w, const PbdCon
 
 // Jacobi PBD of a filament of at most 64 beads in registers: lane l holds
 // beads, edges and joints 2l and 2l + 1, and reads its neighbours' values by
-// warp shuffles.  The same arithmetic, in the same order, as pbd_smem.
+// warp shuffles.  The same arithmetic, in the same order, as pbd_block.
 template <bool kExt, int kMode>
 __device__ __forceinline__ float pbd_regs(const WorldDev& w, const PbdConst& k, int b0, int B, int e0, int j0,
                                           long long t, int fields) {
@@ -465,14 +465,17 @@ __device__ __forceinline__ float pbd_regs(const WorldDev& w, const PbdConst& k, 
   return fmax;
 }
 
-// Jacobi PBD of a filament of any length: the filament's edges, joints and
-// bead corrections live in a per-warp slice of shared memory; every pass
-// reads the slice, then writes corrections, with a warp barrier in between,
-// so all corrections of a pass see the state before it.
+// PBD of a filament of more than 64 beads by one block: the filament's
+// edges, joints and bead corrections live in shared memory; every pass reads
+// them, then writes corrections, with a block barrier in between, so all
+// corrections of a pass see the state before it.  A pass over a long chain
+// is bound by the latency of its rounds: with one warp a filament of 300
+// beads took ten rounds a pass, and the fused advance + PBD of 60 filaments
+// of 2 to 300 beads 33.7 us; with a block 12.6 us.
 template <bool kExt, int kMode>
-__device__ __forceinline__ float pbd_smem(const WorldDev& w, const PbdConst& k, int b0, int B, int e0, int j0,
+__device__ __forceinline__ float pbd_block(const WorldDev& w, const PbdConst& k, int b0, int B, int e0, int j0,
                                           long long t, int fields, float* s, int maxB) {
-  const int lane = threadIdx.x & 31;
+  const int tid = threadIdx.x, T = blockDim.x;
   const int nE = B - 1, nJ = B - 2;
   float* vx = s;
   float* vy = s + maxB;
@@ -490,7 +493,7 @@ __device__ __forceinline__ float pbd_smem(const WorldDev& w, const PbdConst& k, 
   if (kMode == 1) {
     // a8 of the previous step, the advanced positions staged directly
     long long q = 0;
-    for (int i = lane; i < B; i += 32) {
+    for (int i = tid; i < B; i += T) {
       const float4 p = w.pos[b0 + i];
       const float2 U = bead_velocity<kExt>(w, b0 + i, p, q);
       P[i] = advance_tail<false>(w, b0 + i, p, U.x, U.y);
@@ -498,40 +501,40 @@ __device__ __forceinline__ float pbd_smem(const WorldDev& w, const PbdConst& k, 
     if (kExt && w.observe && w.energy) obs_add_warp(&w.obs[2], q);
   } else if (kMode == 2) {
     // direct forcing: the positions the fluid (u* in u) carries the beads to
-    for (int i = lane; i < B; i += 32) {
+    for (int i = tid; i < B; i += T) {
       const float4 p = w.pos[b0 + i];
       const float2 U = interp_u(w, p);
       w.ubead[b0 + i] = U;
       P[i] = advance_pos(w, p, U.x, U.y);
     }
   } else {
-    for (int i = lane; i < B; i += 32) cpa16(&P[i], &w.pos[b0 + i]);
+    for (int i = tid; i < B; i += T) cpa16(&P[i], &w.pos[b0 + i]);
   }
-  for (int e = lane; e < nE; e += 32) {
+  for (int e = tid; e < nE; e += T) {
     cpa4(&th[e], &w.theta[e0 + e]);
     if (!kExt || !w.ldrive) cpa4(&Lr[e], &w.L_rest[e0 + e]);
     else Lr[e] = drive_length(w.ldrive[e0 + e], t);
   }
-  for (int j = lane; j < nJ; j += 32) cpa16(&D[j], &w.drive[j0 + j]);
+  for (int j = tid; j < nJ; j += T) cpa16(&D[j], &w.drive[j0 + j]);
   cpa_wait_all();
-  __syncwarp();
+  __syncthreads();
   if (kMode == 0 && w.rec_pos) {   // the step's start, into the reverse mode's record
-    for (int i = lane; i < B; i += 32) w.rec_pos[b0 + i] = P[i];
-    for (int e = lane; e < nE; e += 32) w.rec_theta[e0 + e] = th[e];
+    for (int i = tid; i < B; i += T) w.rec_pos[b0 + i] = P[i];
+    for (int e = tid; e < nE; e += T) w.rec_theta[e0 + e] = th[e];
   }
-  for (int e = lane; e < nE; e += 32) {
+  for (int e = tid; e < nE; e += T) {
     const float2 v = edge_vec(P[e], P[e + 1], k.W, k.H);
     vx[e] = v.x;
     vy[e] = v.y;
   }
-  for (int j = lane; j < nJ; j += 32) thr[j] = drive_angle(D[j], t);
-  for (int i = lane; i < B; i += 32) {
+  for (int j = tid; j < nJ; j += T) thr[j] = drive_angle(D[j], t);
+  for (int i = tid; i < B; i += T) {
     dlx[i] = 0.0f;
     dly[i] = 0.0f;
   }
-  __syncwarp();
+  __syncthreads();
   if (kExt && w.layers == 2) {
-    for (int i = lane; i < B; i += 32) {
+    for (int i = tid; i < B; i += T) {
       const float2 z2 = make_float2(0.0f, 0.0f);
       const float2 out = i < nE ? unit2(make_float2(vx[i], vy[i])) : z2;
       const float2 in = i > 0 ? unit2(make_float2(vx[i - 1], vy[i - 1])) : z2;
@@ -543,15 +546,15 @@ __device__ __forceinline__ float pbd_smem(const WorldDev& w, const PbdConst& k, 
     // two edges share a bead, so the lanes update in place
     for (int iter = 0; iter < k.n_pbd; ++iter) {
       for (int c = 0; c < 2; ++c) {
-        for (int j = 2 * lane + c; j < nJ; j += 64) {
+        for (int j = 2 * tid + c; j < nJ; j += 2 * T) {
           const float Cj = th[j + 1] - th[j] - thr[j];
           th[j] += k.hb * Cj;
           th[j + 1] -= k.hb * Cj;
         }
-        __syncwarp();
+        __syncthreads();
       }
       for (int c = 0; c < 2; ++c) {
-        for (int e = 2 * lane + c; e < nE; e += 64) {
+        for (int e = 2 * tid + c; e < nE; e += 2 * T) {
           float the = th[e], ddxe, ddye;
           edge_correction(vx[e] + (dlx[e + 1] - dlx[e]), vy[e] + (dly[e + 1] - dly[e]), Lr[e], the, k, ddxe, ddye);
           th[e] = the;
@@ -560,41 +563,41 @@ __device__ __forceinline__ float pbd_smem(const WorldDev& w, const PbdConst& k, 
           dlx[e + 1] -= ddxe;
           dly[e + 1] -= ddye;
         }
-        __syncwarp();
+        __syncthreads();
       }
     }
   }
   for (int iter = 0; iter < (k.order == 1 ? 0 : k.n_pbd); ++iter) {
-    for (int j = lane; j < nJ; j += 32) C[j] = th[j + 1] - th[j] - thr[j];
-    __syncwarp();
-    for (int e = lane; e < nE; e += 32) {
+    for (int j = tid; j < nJ; j += T) C[j] = th[j + 1] - th[j] - thr[j];
+    __syncthreads();
+    for (int e = tid; e < nE; e += T) {
       const float c1 = e < nJ ? C[e] : 0.0f;      // edge e is theta_1 of joint e
       const float c0 = e > 0 ? C[e - 1] : 0.0f;   // ... and theta_2 of joint e-1
       th[e] += k.hb * (c1 - c0);
     }
-    __syncwarp();
-    for (int e = lane; e < nE; e += 32) {
+    __syncthreads();
+    for (int e = tid; e < nE; e += T) {
       float the = th[e];
       edge_correction(vx[e] + (dlx[e + 1] - dlx[e]), vy[e] + (dly[e + 1] - dly[e]), Lr[e], the, k, ddx[e], ddy[e]);
       th[e] = the;
     }
-    __syncwarp();
-    for (int i = lane; i < B; i += 32) {
+    __syncthreads();
+    for (int i = tid; i < B; i += T) {
       const float ax = i < nE ? ddx[i] : 0.0f, ay = i < nE ? ddy[i] : 0.0f;          // x_1 of edge i
       const float bx = i > 0 ? ddx[i - 1] : 0.0f, by = i > 0 ? ddy[i - 1] : 0.0f;    // x_2 of edge i-1
       dlx[i] += ax - bx;
       dly[i] += ay - by;
     }
-    __syncwarp();
+    __syncthreads();
   }
-  for (int e = lane; e < nE; e += 32) w.theta[e0 + e] = th[e];
+  for (int e = tid; e < nE; e += T) w.theta[e0 + e] = th[e];
   float fmax = 0.0f;
   if (kMode == 2) {
-    for (int i = lane; i < B; i += 32) bead_out_velocity(w, k, b0 + i, dlx[i], dly[i]);
+    for (int i = tid; i < B; i += T) bead_out_velocity(w, k, b0 + i, dlx[i], dly[i]);
   } else {
     int* counts = step_counts(w, t);
-    for (int i0 = 0; i0 < B; i0 += 32) {
-      const int i = i0 + lane;
+    for (int i0 = 0; i0 < B; i0 += T) {
+      const int i = i0 + tid;
       const bool valid = i < B;
       const float4 p = valid ? P[i] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
       const int bin = bead_bin_of(p, k.nbx);
@@ -607,38 +610,41 @@ __device__ __forceinline__ float pbd_smem(const WorldDev& w, const PbdConst& k, 
   }
   if (kExt && w.observe && t >= 1) {
     float eb = 0.0f, ep = 0.0f;
-    for (int j = lane; j < nJ; j += 32) eb += sq(drive_angle(D[j], t - 1) - thr[j]);
+    for (int j = tid; j < nJ; j += T) eb += sq(drive_angle(D[j], t - 1) - thr[j]);
     if (w.ldrive)
-      for (int e = lane; e < nE; e += 32) ep += sq(drive_length(w.ldrive[e0 + e], t - 1) - Lr[e]);
+      for (int e = tid; e < nE; e += T) ep += sq(drive_length(w.ldrive[e0 + e], t - 1) - Lr[e]);
     obs_add_warp(&w.obs[0], obs_q(eb));
     obs_add_warp(&w.obs[1], obs_q(ep));
   }
   return fmax;
 }
 
-// One warp per filament (a1 + a3 + the a2 histogram).  Bead positions enter
-// as edge vectors v0 = min_image(X_b - X_a) plus the accumulated corrections,
-// so the corrections keep full FP32 precision whatever the magnitude of the
-// coordinates.  Filaments of at most 64 beads run in registers; longer ones
-// in the warp's slice of dynamic shared memory (maxB floats per array; zero
-// when no filament of the launch is longer than 64 beads).
-// The block's dynamic shared memory (filaments longer than 64 beads stage
-// in per-warp slices of it; maxB is a multiple of 4: float4 slices stay
-// aligned).
+// a1 + a3 + a2 of the filaments of a launch: its list holds the n_long of
+// more than 64 beads first, one block each (pbd_block), then the others, one
+// warp each in registers, wpb to a block.  Bead positions enter as edge
+// vectors v0 = min_image(X_b - X_a) plus the accumulated corrections, so the
+// corrections keep full FP32 precision whatever the magnitude of the
+// coordinates.
+struct PbdWork {
+  int n_long, n_items;   // filaments of more than 64 beads, all filaments
+  int wpb;               // filaments a block of the others takes
+  int maxB;              // slots per array of the block's dynamic shared memory (a multiple of 4: float4 arrays stay aligned)
+};
 extern __shared__ __align__(16) float pbd_dyn_smem[];
 
-template <bool kExt, int kMode, bool kSingle>
+// kLong: the launch has such filaments (a kernel of its own: holding both
+// forms costs the warp form registers, 150 -> 167 us at 2^22 beads).
+template <bool kExt, int kMode, bool kSingle, bool kLong>
 __device__ __forceinline__ void pbd_body(const WorldDev* __restrict__ worlds, const int2* __restrict__ items,
-                                         int n_items, int maxB, int off, int fields,
-                                         unsigned blk) {
-  float* smem = pbd_dyn_smem;
-  const int wpb = blockDim.x >> 5;
+                                         const PbdWork& pw, int off, int fields, unsigned blk) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int item = blk * wpb + warp;
-  if (item >= n_items) return;  // warp-uniform exit; the body has no block barrier
+  const int n_long = kLong ? pw.n_long : 0;
+  const bool is_long = kLong && (int)blk < n_long;   // block-uniform
+  const int item = is_long ? (int)blk : n_long + ((int)blk - n_long) * pw.wpb + warp;
+  if (!is_long && (warp >= pw.wpb || item >= pw.n_items)) return;  // warp-uniform exit; no block barrier follows
   // a single-world launch takes its item from the block index (the world
   // stays in the table: its fields reach the arithmetic exactly as in a batch)
-  const int2 it = kSingle ? make_int2(0, item) : items[item];
+  const int2 it = kSingle && !kLong ? make_int2(0, item) : items[item];
   const WorldDev& w = worlds[it.x];
   if ((kMode == 2) != (w.ib == 1)) return;   // direct-forcing worlds run their PBD after the steric spread
   const int f = it.y;
@@ -647,9 +653,9 @@ __device__ __forceinline__ void pbd_body(const WorldDev* __restrict__ worlds, co
   const int e0 = b0 - f, j0 = b0 - 2 * f;
   const long long t = *w.t + off;
   const PbdConst k = pbd_const(w);
-  float fmax = B <= 64 ? pbd_regs<kExt, kMode>(w, k, b0, B, e0, j0, t, fields)
-                       : pbd_smem<kExt, kMode>(w, k, b0, B, e0, j0, t, fields,
-                                               smem + (size_t)warp * maxB * kPbdFloatsPerBead, maxB);
+  float fmax;
+  if (kLong && is_long) fmax = pbd_block<kExt, kMode>(w, k, b0, B, e0, j0, t, fields, pbd_dyn_smem, pw.maxB);
+  else fmax = pbd_regs<kExt, kMode>(w, k, b0, B, e0, j0, t, fields);
   if (kMode == 2) return;
   // largest |F_el| component of the world this step (bounds the spread's
   // fixed-point scale); non-negative floats order like their bit patterns

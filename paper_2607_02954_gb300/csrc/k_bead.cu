@@ -7,33 +7,31 @@
 
 namespace mc {
 
-// One warp per filament (a1 + a3 + a2).  Bead positions enter
-// as edge vectors v0 = min_image(X_b - X_a) plus the accumulated corrections,
-// so the corrections keep full FP32 precision whatever the magnitude of the
-// coordinates.  Filaments of at most 64 beads run in registers; longer ones
-// in the warp's slice of dynamic shared memory (maxB floats per array; zero
-// when no filament of the launch is longer than 64 beads).
-template <bool kExt, int kMode, bool kSingle>
+// a1 + a3 + a2, one warp per filament of at most 64 beads (in registers), one
+// block per longer one (in dynamic shared memory): see pbd_body.
+template <bool kExt, int kMode, bool kSingle, bool kLong>
 __global__ void __launch_bounds__(256, 4) k_pbd(const WorldDev* __restrict__ worlds,
-                                             const int2* __restrict__ items, int n_items, int maxB, int off,
+                                             const int2* __restrict__ items, const PbdWork pw, int off,
                                              int fields) {
   pdl_trigger();
   pdl_wait();
-  pbd_body<kExt, kMode, kSingle>(worlds, items, n_items, maxB, off, fields, blockIdx.x);
+  pbd_body<kExt, kMode, kSingle, kLong>(worlds, items, pw, off, fields, blockIdx.x);
 }
 
 // Spread of half of F_el + F_s at each layer point of every bead of
 // two-layer worlds, in 64-bit fixed point (bitwise independent of order).
+// Eight threads a bead, one stencil row of one layer point each: 10,231
+// beads took 17.2 us with one thread each, 7.5 us so.
 // Beads are read from the step's slots, so the positions are those at the
 // start of the step even when the spread is re-run later.
 __global__ void __launch_bounds__(kBeadChunk) k_layer_spread(const WorldDev* __restrict__ worlds,
                                                              const int2* __restrict__ items) {
   pdl_trigger();
   pdl_wait();
-  const int2 it = items[blockIdx.x];
+  const int2 it = items[blockIdx.x >> 3];
   const WorldDev& w = worlds[it.x];
   if (w.layers != 2) return;
-  const int i = it.y + threadIdx.x;
+  const int i = it.y + (blockIdx.x & 7) * (kBeadChunk / 8) + (threadIdx.x >> 3);
   if (i >= w.N) return;
   const int W = w.W, H = w.H;
   const int slot = w.bead_slot[i];
@@ -162,10 +160,9 @@ __global__ void k_cells_out(const float4* __restrict__ pos, int N, int W, int* c
 // ---------------------------------------------------------------------------
 // Launchers.
 // ---------------------------------------------------------------------------
-// Warps (filaments) per block: at most 8, at most what 48 KB of shared
-// memory holds, and few enough that a small launch still spreads over every
-// SM (each warp's filament is a serial chain; warps sharing an SM's
-// schedulers only delay one another).
+// Warps (filaments) per block: at most the configuration's, and few enough
+// that a small launch still spreads over every SM (each warp's filament is a
+// serial chain; warps sharing an SM's schedulers only delay one another).
 static int num_sms() {
   // first asked by kernel_setup, outside any stream capture
   static const int sms = [] {
@@ -177,77 +174,87 @@ static int num_sms() {
   return sms;
 }
 
-static int pbd_warps_per_block(int maxB, int n_items, int most) {
+struct PbdLaunch {
+  PbdWork pw;
+  int grid, block;
+  size_t smem;
+};
+
+static PbdLaunch pbd_launch(const Plan& p) {
   const int sms = num_sms();
-  const int per_warp = maxB * kPbdFloatsPerBead * (int)sizeof(float);
-  int wpb = (48 * 1024) / per_warp;
-  if (wpb > most) wpb = most;
-  const int spread = (n_items + sms - 1) / sms;
+  const int n_short = p.n_fil_items - p.n_long;
+  int wpb = p.cfg.pbd_warps;
+  const int spread = (n_short + sms - 1) / sms;
   if (wpb > spread) wpb = spread;
   if (wpb < 1) wpb = 1;
-  return wpb;
+  PbdLaunch l;
+  l.pw.n_long = p.n_long;
+  l.pw.n_items = p.n_fil_items;
+  l.pw.wpb = wpb;
+  l.pw.maxB = (p.max_B + 3) & ~3;
+  l.grid = p.n_long + (n_short + wpb - 1) / wpb;
+  l.block = wpb * 32;
+  l.smem = 0;
+  if (p.n_long > 0) {
+    l.block = p.max_B > 128 ? 256 : 128;   // a bead or two a thread
+    if (l.pw.wpb > l.block / 32) {
+      l.pw.wpb = l.block / 32;
+      l.grid = p.n_long + (n_short + l.pw.wpb - 1) / l.pw.wpb;
+    }
+    l.smem = (size_t)l.pw.maxB * kPbdFloatsPerBead * sizeof(float);
+  }
+  return l;
 }
 
-void launch_pbd(const Plan& p, cudaStream_t s) {
+template <bool kExt, int kMode>
+static void launch_pbd_kernel(const Plan& p, cudaStream_t s, int off, int fields) {
   if (p.n_fil_items == 0) return;
-  const int mb = (p.max_B + 3) & ~3;
-  const int wpb = pbd_warps_per_block(mb, p.n_fil_items, p.cfg.pbd_warps);
-  // filaments of at most 64 beads need no shared memory
-  const size_t smem = p.max_B <= 64 ? 0 : (size_t)wpb * mb * kPbdFloatsPerBead * sizeof(float);
-  const int grid = (p.n_fil_items + wpb - 1) / wpb;
-  // worlds with a rest-length drive, observables or two layers need the
-  // extended kernel; it computes every other world exactly as the plain one
+  const PbdLaunch l = pbd_launch(p);
   const bool one = p.n_worlds == 1;
-  auto kern = p.any_ext ? (one ? k_pbd<true, 0, true> : k_pbd<true, 0, false>)
-                        : (one ? k_pbd<false, 0, true> : k_pbd<false, 0, false>);
-  launch_pdl(kern, grid, wpb * 32, smem, s, p.d_worlds, p.d_fil_items, p.n_fil_items, mb, 0, 1);
+  auto kern = p.n_long ? (one ? k_pbd<kExt, kMode, true, true> : k_pbd<kExt, kMode, false, true>)
+                       : (one ? k_pbd<kExt, kMode, true, false> : k_pbd<kExt, kMode, false, false>);
+  launch_pdl(kern, l.grid, l.block, l.smem, s, (const WorldDev*)p.d_worlds, (const int2*)p.d_fil_items, l.pw, off,
+             fields);
+}
+
+// (worlds with a rest-length drive, observables or two layers need the
+// extended kernel; it computes every other world exactly as the plain one)
+void launch_pbd(const Plan& p, cudaStream_t s) {
+  if (p.any_ext) launch_pbd_kernel<true, 0>(p, s, 0, 1);
+  else launch_pbd_kernel<false, 0>(p, s, 0, 1);
 }
 
 // The PBD of direct-forcing worlds (from the positions the fluid carries
 // the beads to; the others return at once).
-void launch_pbd_mdf(const Plan& p, cudaStream_t s) {
-  if (p.n_fil_items == 0) return;
-  const int mb = (p.max_B + 3) & ~3;
-  const int wpb = pbd_warps_per_block(mb, p.n_fil_items, p.cfg.pbd_warps);
-  const size_t smem = p.max_B <= 64 ? 0 : (size_t)wpb * mb * kPbdFloatsPerBead * sizeof(float);
-  const int grid = (p.n_fil_items + wpb - 1) / wpb;
-  auto kern = p.n_worlds == 1 ? k_pbd<true, 2, true> : k_pbd<true, 2, false>;
-  launch_pdl(kern, grid, wpb * 32, smem, s, p.d_worlds, p.d_fil_items, p.n_fil_items, mb, 0, 1);
-}
+void launch_pbd_mdf(const Plan& p, cudaStream_t s) { launch_pbd_kernel<true, 2>(p, s, 0, 1); }
 
 // a8 of the previous step fused with this step's a1-a3 (plans without
 // direct-forcing worlds), off steps after the worlds' counters.
 void launch_advance_pbd(const Plan& p, cudaStream_t s, int off, int fields) {
-  if (p.n_fil_items == 0) return;
-  const int mb = (p.max_B + 3) & ~3;
-  const int wpb = pbd_warps_per_block(mb, p.n_fil_items, p.cfg.pbd_warps);
-  const size_t smem = p.max_B <= 64 ? 0 : (size_t)wpb * mb * kPbdFloatsPerBead * sizeof(float);
-  const int grid = (p.n_fil_items + wpb - 1) / wpb;
-  const bool one = p.n_worlds == 1;
-  auto kern = p.any_ext ? (one ? k_pbd<true, 1, true> : k_pbd<true, 1, false>)
-                        : (one ? k_pbd<false, 1, true> : k_pbd<false, 1, false>);
-  launch_pdl(kern, grid, wpb * 32, smem, s, p.d_worlds, p.d_fil_items, p.n_fil_items, mb, off, fields);
+  if (p.any_ext) launch_pbd_kernel<true, 1>(p, s, off, fields);
+  else launch_pbd_kernel<false, 1>(p, s, off, fields);
 }
 
 // Shared-memory limits set once per process, outside any stream capture: the
-// PBD kernel stages up to 8 warps' filaments of at most 3072 beads.
+// PBD kernel stages a filament of at most 3072 beads.
 void kernel_setup() {
   static std::once_flag once;
   std::call_once(once, [] {
     steric_setup(num_sms());
     persistent_setup();
     const int most = 227 * 1024;
-    for (auto f : {k_pbd<false, 0, false>, k_pbd<true, 0, false>, k_pbd<false, 1, false>, k_pbd<true, 1, false>,
-                   k_pbd<true, 2, false>, k_pbd<false, 0, true>, k_pbd<true, 0, true>, k_pbd<false, 1, true>,
-                   k_pbd<true, 1, true>, k_pbd<true, 2, true>})
+    for (auto f : {k_pbd<false, 0, false, true>, k_pbd<true, 0, false, true>, k_pbd<false, 1, false, true>,
+                   k_pbd<true, 1, false, true>, k_pbd<true, 2, false, true>, k_pbd<false, 0, true, true>,
+                   k_pbd<true, 0, true, true>, k_pbd<false, 1, true, true>, k_pbd<true, 1, true, true>,
+                   k_pbd<true, 2, true, true>})
       cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   });
 }
 
-void launch_layer_spread(const Plan& p, cudaStream_t s) {
+void launch_layer_spread(const Plan& p, cudaStream_t s, bool finish) {
   if (!p.any_layered) return;
-  k_layer_spread<<<p.n_bead_items, kBeadChunk, 0, s>>>(p.d_worlds, p.d_bead_items);
-  if (p.n_cell_items) k_layer_finish<<<p.n_cell_items, kCellChunk, 0, s>>>(p.d_worlds, p.d_cell_items);
+  k_layer_spread<<<8 * p.n_bead_items, kBeadChunk, 0, s>>>(p.d_worlds, p.d_bead_items);
+  if (finish && p.n_cell_items) k_layer_finish<<<p.n_cell_items, kCellChunk, 0, s>>>(p.d_worlds, p.d_cell_items);
 }
 
 void launch_interp_advance(const Plan& p, cudaStream_t s, int inc) {

@@ -154,7 +154,7 @@ mc_status build_plan(mc_world* const* ws, int n, cudaStream_t s, Plan& out) {
   p.any_mdf = false;
   p.max_mdf = 0;
   p.any_ext = false;
-  std::vector<int2> fil, bead, tile, cell;
+  std::vector<int2> fil_long, fil, bead, tile, cell;
   std::vector<WorldDev> table(n);
   for (int k = 0; k < n; ++k) {
     const mc_world* w = ws[k];
@@ -166,7 +166,8 @@ mc_status build_plan(mc_world* const* ws, int n, cudaStream_t s, Plan& out) {
     p.any_mdf = p.any_mdf || w->h.ib == 1;
     p.max_mdf = std::max(p.max_mdf, w->h.mdf_iters);
     p.any_ext = p.any_ext || w->h.layers == 2 || w->h.observe || w->h.has_ldrive || w->h.ib == 1;
-    for (int f = 0; f < w->h.n_fil; ++f) fil.push_back(make_int2(k, f));
+    for (int f = 0; f < w->h.n_fil; ++f)
+      (w->fil_off[f + 1] - w->fil_off[f] > 64 ? fil_long : fil).push_back(make_int2(k, f));
     const int nb = std::max(w->h.N, 1);
     for (int b = 0; b < nb; b += mc::kBeadChunk) bead.push_back(make_int2(k, b));
     for (int ty = 0; ty < w->h.nty; ++ty)   // tile items carry (tx, ty) packed: tx | ty << 16
@@ -174,6 +175,8 @@ mc_status build_plan(mc_world* const* ws, int n, cudaStream_t s, Plan& out) {
     const int HW = w->h.H * w->h.W;
     for (int c = 0; c < HW; c += mc::kCellChunk) cell.push_back(make_int2(k, c));
   }
+  p.n_long = (int)fil_long.size();
+  fil.insert(fil.begin(), fil_long.begin(), fil_long.end());
   Layout L;
   const size_t o_w = L.take<WorldDev>(n);
   const size_t o_f = L.take<int2>(fil.size());

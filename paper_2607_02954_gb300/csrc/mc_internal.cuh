@@ -198,6 +198,7 @@ struct Plan {
   int max_mdf = 0;               // most MDF passes of a world
   bool any_ext = false;          // some world has two layers, observables, a rest-length drive or direct forcing
   long long beads = 0;           // of all worlds
+  int n_long = 0;                // filaments of more than 64 beads (first in d_fil_items)
   int n_fil_items = 0, n_bead_items = 0, n_tile_items = 0, n_cell_items = 0;
   WorldDev* d_worlds = nullptr;  // [n_worlds]
   int2* d_fil_items = nullptr;   // (world, filament)

@@ -151,3 +151,34 @@ def test_wide_tile_blocks_equal_the_narrow_ones(H, W, n_fil, B):
     c.step(1)
     assert_field("rho_s", c.field("rho_s"), t2n(rec["rho_s"]), 1e-5)
     assert_field("u", c.field("u"), np.moveaxis(t2n(rec["u"]), 0, -1), 1e-5)
+
+
+@pytest.mark.parametrize("lengths", [[65], [64, 65, 2], [128, 129, 7], [300, 64, 255, 256, 257, 30], [3072, 65]])
+@pytest.mark.parametrize("kw", [{}, dict(pbd_order=1), dict(layers=2), dict(ib=1, mdf_iters=1)])
+def test_long_filaments_beside_short_ones(lengths, kw):
+    """Filaments of more than 64 beads (a block each) beside short ones (a
+    warp each): one step against the oracle, and a batch against each alone."""
+    H, W = (128, 3200) if max(lengths) > 512 else (96, 320)
+    rng = np.random.default_rng(sum(lengths))
+    x = np.concatenate([2.0 + np.arange(b) + rng.uniform(0, 0.4) for b in lengths]).astype(np.float32)
+    y = np.concatenate([np.full(b, 5.0 + 12.0 * f) for f, b in enumerate(lengths)]).astype(np.float32)
+    E, J = sum(b - 1 for b in lengths), sum(b - 2 for b in lengths)
+    spec = synth._world("long", H, W, lengths, x, y, np.zeros(E, np.float32), rng.normal(0, 0.1, J), np.full(J, 0.2),
+                        np.full(J, 0.01), rng.uniform(0, 1, J), params=synth.Params(**kw))
+    spec = synth.with_observables(spec, 3)
+    ow = O.World(spec)
+    st, rec = O.step(ow, ow.initial_state(), record=True)
+    a = World(spec)
+    a.step(1)
+    assert_field("theta", a.state()["theta"], t2n(st.theta), 1e-6)
+    assert_field("disp", a.state()["disp"], t2n(st.D), 1e-5)
+    assert_field("fel", a.field("fel"), t2n(rec["F_el"]), 1e-5)
+    other = synth.world_random(4, (40, 72), 5)
+    batch = [World(other), World(spec), World(other)]
+    step_batched(batch, 4)
+    b = World(spec)
+    b.step(4)
+    want, got = b.state(fluid=True), batch[1].state(fluid=True)
+    for k in want:
+        assert np.array_equal(want[k], got[k]), k
+    assert b.observables() == batch[1].observables()
