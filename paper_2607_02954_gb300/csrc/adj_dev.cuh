@@ -40,6 +40,13 @@ struct Stencil {
   int ix[4], iy[4];   // wrapped column / row-start indices
 };
 
+// v[b] for b in 0 .. 3 without an indexed (local memory) access.
+template <typename T>
+__device__ __forceinline__ T pick4(const T v[4], int b) {
+  const T lo = (b & 1) ? v[1] : v[0], hi = (b & 1) ? v[3] : v[2];
+  return (b & 2) ? hi : lo;
+}
+
 // The stencil of the two-layer point X + d n of bead p (the forward's
 // layer_cell: cell and fraction of the shifted point).
 __device__ __forceinline__ Stencil make_layer_stencil(const float4& p, float2 n, float d, int W, int H) {

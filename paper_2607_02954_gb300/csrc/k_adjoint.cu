@@ -33,10 +33,12 @@ __device__ __forceinline__ int ubar_exponent(const WorldDev& w, const AdjDev& a)
   return fix_exponent64((float)w.N * __uint_as_float(a.amax[a.par]));
 }
 
+// (Four threads a bead, each one row of the stencil: the kernel is a chain
+// of a few loads and the atomics, bound by latency at a few thousand beads.)
 __global__ void __launch_bounds__(256) k_adj_spread_u(const WorldDev* __restrict__ wd, AdjDev a) {
   const WorldDev& w = *wd;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (a.setup && i == 0) {
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 2, b = threadIdx.x & 3;
+  if (a.setup && i == 0 && b == 0) {
     // the bounds this step's kernels produce: of Q (k_adj_lbm) and of the
     // next reversed step's u_bar (k_adj_pbd; this step's u_bar reads slot
     // a.par).  (The step's counter comes with a.t_step: the world's own
@@ -49,15 +51,15 @@ __global__ void __launch_bounds__(256) k_adj_spread_u(const WorldDev* __restrict
   const float2 xb = a.adjX[i];
   const float ux = w.dt * xb.x * scale, uy = w.dt * xb.y * scale;
   auto spread = [&](const Stencil& s, float h) {
+    const float wy = pick4(s.wy, b);
+    const int row = pick4(s.iy, b);
 #pragma unroll
-    for (int b = 0; b < 4; ++b)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const float wgt = s.wx[c] * s.wy[b] * h;
-        unsigned long long* g = &a.ubar[2 * (s.iy[b] + s.ix[c])];
-        atomicAdd(g, fx64(wgt * ux));
-        atomicAdd(g + 1, fx64(wgt * uy));
-      }
+    for (int c = 0; c < 4; ++c) {
+      const float wgt = s.wx[c] * wy * h;
+      unsigned long long* g = &a.ubar[2 * (row + s.ix[c])];
+      atomicAdd(g, fx64(wgt * ux));
+      atomicAdd(g + 1, fx64(wgt * uy));
+    }
   };
   if (w.layers == 2) {
     // U = (I[u](X + d n) + I[u](X - d n)) / 2
@@ -210,14 +212,18 @@ __device__ __forceinline__ int q_exponent(const WorldDev& w, const AdjDev& a) {
   return fix_exponent64((float)w.N * __uint_as_float(a.amax[2]));
 }
 
+// Four threads a bead: each gathers and scatters one row of the stencil, the
+// rows' sums added in a fixed order.
 __global__ void __launch_bounds__(256) k_adj_bead_a(const WorldDev* __restrict__ wd, AdjDev a) {
   const WorldDev& w = *wd;
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= w.N) return;
+  const int at = (blockIdx.x * blockDim.x + threadIdx.x) >> 2, b = threadIdx.x & 3;
+  const bool valid = at < w.N;
+  const int i = valid ? at : w.N - 1;   // (every lane takes part in the row sums)
   const float qscale = pow2f(q_exponent(w, a));
   const float4 p = w.pos[i];
   const Stencil s = make_stencil(p, w.W, w.H);
-  const float2 xb = a.adjX[i];
+  // (read by all four threads before the first writes it: rows() synchronises them)
+  const float2 xb = valid ? a.adjX[i] : make_float2(0.0f, 0.0f);
   // direct forcing: the advance does not read u, and the steric spread
   // carries F_s alone (the MDF passes' own adjoints are k_adj_mdf.cu's)
   const bool df = w.ib == 1;
@@ -226,21 +232,30 @@ __global__ void __launch_bounds__(256) k_adj_bead_a(const WorldDev* __restrict__
   const float Ftx = fe.x + fs.x, Fty = fe.y + fs.y;
   // over the stencil st (weights scaled by h): the force's adjoint and the
   // position gradient of u.U_bar + F_bar.Ftot
+  auto rows = [](float v) {
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    return v + __shfl_xor_sync(0xffffffffu, v, 2);
+  };
   auto gather = [&](const Stencil& st, float h, float& ftbx, float& ftby, float& gx, float& gy) {
+    const float wy = pick4(st.wy, b), dy = pick4(st.dy, b);
+    const int row = pick4(st.iy, b);
+    float fx = 0.0f, fy = 0.0f, px = 0.0f, py = 0.0f;
 #pragma unroll
-    for (int b = 0; b < 4; ++b)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int k = st.iy[b] + st.ix[c];
-        const float2 u = w.u[k];
-        const float2 fb = a.Fbar[k];
-        const float wgt = st.wx[c] * st.wy[b] * h;
-        ftbx = fmaf(wgt, fb.x, ftbx);
-        ftby = fmaf(wgt, fb.y, ftby);
-        const float q = (u.x * Ubx + u.y * Uby + fb.x * Ftx + fb.y * Fty) * h;
-        gx = fmaf(st.dx[c] * st.wy[b], q, gx);
-        gy = fmaf(st.wx[c] * st.dy[b], q, gy);
-      }
+    for (int c = 0; c < 4; ++c) {
+      const int k = row + st.ix[c];
+      const float2 u = w.u[k];
+      const float2 fb = a.Fbar[k];
+      const float wgt = st.wx[c] * wy * h;
+      fx = fmaf(wgt, fb.x, fx);
+      fy = fmaf(wgt, fb.y, fy);
+      const float q = (u.x * Ubx + u.y * Uby + fb.x * Ftx + fb.y * Fty) * h;
+      px = fmaf(st.dx[c] * wy, q, px);
+      py = fmaf(st.wx[c] * dy, q, py);
+    }
+    ftbx += rows(fx);
+    ftby += rows(fy);
+    gx += rows(px);
+    gy += rows(py);
   };
   float ftbx = 0.0f, ftby = 0.0f, gx = 0.0f, gy = 0.0f;
   if (w.layers == 2) {
@@ -252,26 +267,29 @@ __global__ void __launch_bounds__(256) k_adj_bead_a(const WorldDev* __restrict__
     gather(make_layer_stencil(p, n, -w.layer_half, w.W, w.H), 0.5f, ftbx, ftby, gmx, gmy);
     gx = gpx + gmx;
     gy = gpy + gmy;
-    a.nbar[i] = make_float2(w.layer_half * (gpx - gmx), w.layer_half * (gpy - gmy));
+    if (valid && b == 0) a.nbar[i] = make_float2(w.layer_half * (gpx - gmx), w.layer_half * (gpy - gmy));
   } else {
     gather(s, 1.0f, ftbx, ftby, gx, gy);
   }
-  a.adjX[i] = make_float2(xb.x + gx, xb.y + gy);
-  a.fbt[i] = make_float2(ftbx, ftby);
+  if (!valid) return;
+  if (b == 0) {
+    a.adjX[i] = make_float2(xb.x + gx, xb.y + gy);
+    a.fbt[i] = make_float2(ftbx, ftby);
+  }
   const float qx = ftbx * qscale, qy = ftby * qscale;
+  const float wy = pick4(s.wy, b);
+  const int row = pick4(s.iy, b);
 #pragma unroll
-  for (int b = 0; b < 4; ++b)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const float wgt = s.wx[c] * s.wy[b];
-      unsigned long long* q = &a.Q[2 * (s.iy[b] + s.ix[c])];
-      atomicAdd(q, fx64(wgt * qx));
-      atomicAdd(q + 1, fx64(wgt * qy));
-    }
+  for (int c = 0; c < 4; ++c) {
+    const float wgt = s.wx[c] * wy;
+    unsigned long long* q = &a.Q[2 * (row + s.ix[c])];
+    atomicAdd(q, fx64(wgt * qx));
+    atomicAdd(q + 1, fx64(wgt * qy));
+  }
 }
 
 // ---------------------------------------------------------------------------
-// a6 gradient transposed and a5 transposed, one 32 x 8 strip per block:
+// a6 gradient transposed and a5 transposed, one strip of 32 columns per block:
 //   rho_bar_bar = -k_rep D^T Q with D the central difference,
 //     (D^T v)(c) = (v_x(c - e_x) - v_x(c + e_x) + v_y(c - e_y) - v_y(c + e_y))/2,
 //   then the periodic separable filter (symmetric), x pass then y pass.
@@ -280,20 +298,22 @@ __global__ void __launch_bounds__(256) k_adj_bead_a(const WorldDev* __restrict__
 // pass on the strip; the sums run in the same order as cell-wise passes over
 // the whole grid, so the result does not depend on the tiling.
 // ---------------------------------------------------------------------------
-constexpr int kBlurRows = 8;   // rows of a block's strip (32 columns): more, smaller blocks for small grids
-
+// The filter half width is compiled in (the tap loops unroll).  A block's
+// strip has 8 rows while that leaves fewer than four blocks an SM, else 16
+// (less halo a cell).
+template <int R, int kRows>
 __global__ void __launch_bounds__(256) k_adj_rho_blur(const WorldDev* __restrict__ wd, AdjDev a) {
-  constexpr int kE = kTile + 2 * kMaxR;        // column capacity of the rho_bar_bar region
-  constexpr int kER = kBlurRows + 2 * kMaxR;   // row capacity
-  constexpr int kQ = kE + 2;                   // Q window capacity
+  constexpr int kE = kTile + 2 * R;     // columns of the rho_bar_bar region
+  constexpr int kER = kRows + 2 * R;    // rows
+  constexpr int kQ = kE + 2;            // Q window columns
   __shared__ float2 q[(kER + 2) * kQ];
   __shared__ float rb[kER * kE];
   __shared__ float tm[kER * kTile];
   const WorldDev& w = *wd;
-  const int W = w.W, H = w.H, R = w.R;
+  const int W = w.W, H = w.H;
   const int ntx = (W + kTile - 1) / kTile;
-  const int x0 = (int)(blockIdx.x % ntx) * kTile, y0 = (int)(blockIdx.x / ntx) * kBlurRows;
-  const int tw = min(kTile, W - x0), th = min(kBlurRows, H - y0);
+  const int x0 = (int)(blockIdx.x % ntx) * kTile, y0 = (int)(blockIdx.x / ntx) * kRows;
+  const int tw = min(kTile, W - x0), th = min(kRows, H - y0);
   const int ew = tw + 2 * R, eh = th + 2 * R;   // region: rows y0 - R .., columns x0 - R ..
   const int qw = ew + 2, qh = eh + 2;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
@@ -303,14 +323,18 @@ __global__ void __launch_bounds__(256) k_adj_rho_blur(const WorldDev* __restrict
     int gy = y0 - R - 1 + i;
     while (gy < 0) gy += H;
     while (gy >= H) gy -= H;
-    const unsigned long long* __restrict__ row = a.Q + 2 * (size_t)gy * W;
+    const ulonglong2* __restrict__ row = reinterpret_cast<const ulonglong2*>(a.Q) + (size_t)gy * W;
     for (int j = lane; j < qw; j += 32) {
       int gx = x0 - R - 1 + j;
       while (gx < 0) gx += W;
       while (gx >= W) gx -= W;
-      q[i * kQ + j] = make_float2(fx64_value(row[2 * gx], qinv), fx64_value(row[2 * gx + 1], qinv));
+      const ulonglong2 v = row[gx];   // (Q is 256-byte aligned, two words a cell)
+      q[i * kQ + j] = make_float2(fx64_value(v.x, qinv), fx64_value(v.y, qinv));
     }
   }
+  float tp[2 * R + 1];
+#pragma unroll
+  for (int m = 0; m <= 2 * R; ++m) tp[m] = w.taps[m];
   __syncthreads();
   const float kq = -0.5f * w.k_rep;
   for (int i = warp; i < eh; i += nw) {
@@ -325,7 +349,8 @@ __global__ void __launch_bounds__(256) k_adj_rho_blur(const WorldDev* __restrict
     if (lane < tw) {
       const float* r = rb + i * kE + lane;
       float acc = 0.0f;
-      for (int m = 0; m <= 2 * R; ++m) acc = fmaf(w.taps[m], r[m], acc);
+#pragma unroll
+      for (int m = 0; m <= 2 * R; ++m) acc = fmaf(tp[m], r[m], acc);
       tm[i * kTile + lane] = acc;
     }
   }
@@ -334,9 +359,30 @@ __global__ void __launch_bounds__(256) k_adj_rho_blur(const WorldDev* __restrict
     if (lane < tw) {
       const float* r = tm + i * kTile + lane;
       float acc = 0.0f;
-      for (int m = 0; m <= 2 * R; ++m) acc = fmaf(w.taps[m], r[m * kTile], acc);
+#pragma unroll
+      for (int m = 0; m <= 2 * R; ++m) acc = fmaf(tp[m], r[m * kTile], acc);
       a.rsb[(size_t)(y0 + i) * W + x0 + lane] = acc;
     }
+  }
+}
+
+template <int R>
+static void launch_blur_r(const WorldDev& h, const WorldDev* wd, const AdjDev& a, cudaStream_t s) {
+  const int b8 = h.ntx * ((h.H + 7) / 8);
+  if (b8 < 4 * 152) k_adj_rho_blur<R, 8><<<b8, 256, 0, s>>>(wd, a);
+  else k_adj_rho_blur<R, 16><<<h.ntx * ((h.H + 15) / 16), 256, 0, s>>>(wd, a);
+}
+
+static void launch_adj_rho_blur(const WorldDev& h, const WorldDev* wd, const AdjDev& a, cudaStream_t s) {
+  switch (h.R) {
+    case 1: launch_blur_r<1>(h, wd, a, s); break;
+    case 2: launch_blur_r<2>(h, wd, a, s); break;
+    case 3: launch_blur_r<3>(h, wd, a, s); break;
+    case 4: launch_blur_r<4>(h, wd, a, s); break;
+    case 5: launch_blur_r<5>(h, wd, a, s); break;
+    case 6: launch_blur_r<6>(h, wd, a, s); break;
+    case 7: launch_blur_r<7>(h, wd, a, s); break;
+    default: launch_blur_r<8>(h, wd, a, s); break;
   }
 }
 
@@ -345,30 +391,47 @@ __global__ void __launch_bounds__(256) k_adj_rho_blur(const WorldDev* __restrict
 //   X_bar_i += sum_c grad_X w [rho_s_bar(c) - k_rep grad rho_bar(c) . Ftot_bar_i]
 // and the elastic-force adjoint d_bar_i = kappa/dt Ftot_bar_i for the PBD.
 // ---------------------------------------------------------------------------
-// Bead i: adds its a4 / a6-gradient terms to X_bar, returns Ftot_bar_i.
-__device__ __forceinline__ float2 adj_bead_b_one(const WorldDev& w, const AdjDev& a, int i) {
+// Bead i at p with Ftot_bar fb: its a4 / a6-gradient terms (gx, gy) of X_bar.
+// The central differences of neighbouring stencil cells share their cells:
+// rho_bar is read once per cell of the 6 x 6 window (without its corners).
+__device__ __forceinline__ float2 adj_bead_b_terms(const WorldDev& w, const AdjDev& a, const float4 p,
+                                                   const float2 fb) {
   const int W = w.W, H = w.H;
-  const float4 p = w.pos[i];
   const Stencil s = make_stencil(p, W, H);
-  const float2 fb = a.fbt[i];
+  const int cx = cell_x(p), cy = cell_y(p);
+  int col[6], row[6];
+#pragma unroll
+  for (int c = 0; c < 6; ++c) {
+    col[c] = wrap_once(cx - 2 + c, W);
+    row[c] = wrap_once(cy - 2 + c, H) * W;
+  }
+  float r[6][6];
+#pragma unroll
+  for (int b = 0; b < 6; ++b)
+#pragma unroll
+    for (int c = 0; c < 6; ++c)
+      if ((b > 0 && b < 5) || (c > 0 && c < 5)) r[b][c] = w.rho_b[row[b] + col[c]];
   float gx = 0.0f, gy = 0.0f;
 #pragma unroll
   for (int b = 0; b < 4; ++b) {
-    const int row = s.iy[b];
-    const int rowm = wrap_once(cell_y(p) - 2 + b, H) * W, rowp = wrap_once(cell_y(p) + b, H) * W;
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      const int col = s.ix[c];
-      const int colm = wrap_once(cell_x(p) - 2 + c, W), colp = wrap_once(cell_x(p) + c, W);
-      const float grx = 0.5f * (w.rho_b[row + colp] - w.rho_b[row + colm]);
-      const float gry = 0.5f * (w.rho_b[rowp + col] - w.rho_b[rowm + col]);
-      const float q = a.rsb[row + col] - w.k_rep * (grx * fb.x + gry * fb.y);
+      const float grx = 0.5f * (r[b + 1][c + 2] - r[b + 1][c]);
+      const float gry = 0.5f * (r[b + 2][c + 1] - r[b][c + 1]);
+      const float q = a.rsb[row[b + 1] + col[c + 1]] - w.k_rep * (grx * fb.x + gry * fb.y);
       gx = fmaf(s.dx[c] * s.wy[b], q, gx);
       gy = fmaf(s.wx[c] * s.dy[b], q, gy);
     }
   }
+  return make_float2(gx, gy);
+}
+
+// Bead i: adds those terms to X_bar, returns Ftot_bar_i.
+__device__ __forceinline__ float2 adj_bead_b_one(const WorldDev& w, const AdjDev& a, int i) {
+  const float2 fb = a.fbt[i];
+  const float2 g = adj_bead_b_terms(w, a, w.pos[i], fb);
   const float2 xb = a.adjX[i];
-  a.adjX[i] = make_float2(xb.x + gx, xb.y + gy);
+  a.adjX[i] = make_float2(xb.x + g.x, xb.y + g.y);
   return fb;
 }
 
@@ -383,8 +446,9 @@ __global__ void __launch_bounds__(256) k_adj_bead_b(const WorldDev* __restrict__
 }
 
 // ---------------------------------------------------------------------------
-// a3 + a1 transposed, one block of two warps per filament (each thread
-// holds at most one edge of a filament of up to 64 beads per loop trip).  The forward Jacobi PBD is
+// a3 + a1 transposed.  A filament of at most 64 beads is one warp's, in
+// registers (k_adj_pbd_regs); a longer one a block's, in shared memory
+// (k_adj_pbd).  The forward Jacobi PBD is
 // recomputed from (X^n, theta^n) keeping, per iteration, the frames before
 // and after the bending pass and the corrections before the position pass;
 // then the iterations are reversed:
@@ -406,7 +470,7 @@ __global__ void __launch_bounds__(256) k_adj_bead_b(const WorldDev* __restrict__
 // of the position pass; the reverse runs odd edges, even edges, odd joints,
 // even joints, each colour's constraints independent of one another.
 // ---------------------------------------------------------------------------
-constexpr int kAdjPbdThreads = 64;  // threads per filament
+constexpr int kAdjPbdThreads = 128; // threads of a long filament's block
 constexpr int kAdjPbdPerBead = 12;   // floats of working arrays per bead slot
 constexpr int kAdjTapePerPass = 4;   // Jacobi, per pass: theta before and after the bend pass, d (x, y)
 constexpr int kAdjTapePerPassRB = 7; // red-black, per pass: theta x 3, d (x, y) before each edge colour
@@ -795,6 +859,278 @@ __global__ void __launch_bounds__(kAdjPbdThreads) k_adj_pbd(const WorldDev* __re
   }
 }
 
+// ---------------------------------------------------------------------------
+// The same for a filament of at most 64 beads in one warp: lane l holds
+// beads, edges and joints 2l and 2l + 1 and reads its neighbours' by
+// shuffles, as the forward's pbd_regs.  The tape keeps what the reverse reads
+// again, all of the lane's own: per pass the joints' C, the angles after the
+// bending pass and the edge vectors of the position pass (8 floats a lane).
+// With few filaments the kernel is bound by latency: the block form spent it
+// on its seven barriers a pass (64 filaments of 48 beads, 4 passes: 14.5 us;
+// this form 10.9 us).
+// ---------------------------------------------------------------------------
+constexpr int kAdjTapeRegs = 8;
+constexpr int kAdjRegsWarps = 4;   // most filaments per block
+
+// The adjoints of a bead's out and in unit vectors from its normal's (see
+// k_adj_pbd).
+__device__ __forceinline__ void adj_normal(float2 nb, float2 out, bool ho, float2 in, bool hi, float2& ob, float2& ib) {
+  ob = make_float2(0.0f, 0.0f);
+  ib = make_float2(0.0f, 0.0f);
+  const float tbx = nb.y, tby = -nb.x;
+  const float sx = out.x + in.x, sy = out.y + in.y;
+  const float ns = sqrtf(sx * sx + sy * sy);
+  if (ns >= 1e-3f) {
+    const float tx = sx / ns, ty = sy / ns;
+    const float dot = tbx * tx + tby * ty;
+    const float2 sb = make_float2((tbx - dot * tx) / ns, (tby - dot * ty) / ns);
+    if (ho) ob = sb;
+    if (hi) ib = sb;
+  } else if (ho) {
+    ob = make_float2(tbx, tby);
+  } else {
+    ib = make_float2(tbx, tby);
+  }
+}
+
+template <bool kRB>
+__global__ void __launch_bounds__(32 * kAdjRegsWarps) k_adj_pbd_regs(const WorldDev* __restrict__ wd, AdjDev a,
+                                                                     const int2* __restrict__ items, int n_items,
+                                                                     int n_pbd) {
+  constexpr unsigned kAll = 0xffffffffu;
+  extern __shared__ __align__(16) float smem[];
+  const WorldDev& w = *wd;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int item = blockIdx.x * (blockDim.x >> 5) + warp;
+  if (item >= n_items) return;   // warp-uniform; no block barrier
+  float* tape = smem + (size_t)warp * n_pbd * kAdjTapeRegs * 32 + lane;
+  const int f = items[item].y;
+  const int b0 = w.fil_off[f];
+  const int B = w.fil_off[f + 1] - b0;
+  const int nE = B - 1, nJ = B - 2;
+  const int e0 = b0 - f, j0 = b0 - 2 * f;
+  const int i0 = 2 * lane, i1 = i0 + 1;
+  const bool hb0 = i0 < B, hb1 = i1 < B, he0 = i0 < nE, he1 = i1 < nE, hj0 = i0 < nJ, hj1 = i1 < nJ;
+  const long long t = a.setup ? a.t_step : *w.t;
+  const float4* __restrict__ P = a.xt ? a.xt : w.pos;   // the PBD's start: X~ with direct forcing
+  const float4 z4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  const float2 z2 = make_float2(0.0f, 0.0f);
+  const float4 P0 = hb0 ? P[b0 + i0] : z4, P1 = hb1 ? P[b0 + i1] : z4;
+  float th0 = he0 ? a.theta_n[e0 + i0] : 0.0f, th1 = he1 ? a.theta_n[e0 + i1] : 0.0f;
+  const float L0 = he0 ? rest_length(w, e0 + i0, t) : 1.0f, L1 = he1 ? rest_length(w, e0 + i1, t) : 1.0f;
+  const float thr0 = hj0 ? drive_angle(w.drive[j0 + i0], t) : 0.0f;
+  const float thr1 = hj1 ? drive_angle(w.drive[j0 + i1], t) : 0.0f;
+  float thb0 = he0 ? a.adjTh[e0 + i0] : 0.0f, thb1 = he1 ? a.adjTh[e0 + i1] : 0.0f;
+  float2 X0 = hb0 ? a.adjX[b0 + i0] : z2, X1 = hb1 ? a.adjX[b0 + i1] : z2;
+  // d_bar: direct forcing, from the bead velocities' adjoint; penalty, a4 and
+  // the a6 gradient of the bead first, d_bar = kappa/dt Ftot_bar
+  float2 d0 = z2, d1 = z2;
+  if (a.xt) {
+    if (hb0) d0 = a.dbar[b0 + i0];
+    if (hb1) d1 = a.dbar[b0 + i1];
+  } else {
+    if (hb0) {
+      const float2 fb = a.fbt[b0 + i0];
+      const float2 g = adj_bead_b_terms(w, a, P0, fb);
+      X0 = make_float2(X0.x + g.x, X0.y + g.y);
+      d0 = make_float2(w.kappa_dt * fb.x, w.kappa_dt * fb.y);
+    }
+    if (hb1) {
+      const float2 fb = a.fbt[b0 + i1];
+      const float2 g = adj_bead_b_terms(w, a, P1, fb);
+      X1 = make_float2(X1.x + g.x, X1.y + g.y);
+      d1 = make_float2(w.kappa_dt * fb.x, w.kappa_dt * fb.y);
+    }
+  }
+  float4 Pn;   // bead 2l + 2
+  Pn.x = __shfl_down_sync(kAll, P0.x, 1);
+  Pn.y = __shfl_down_sync(kAll, P0.y, 1);
+  Pn.z = __shfl_down_sync(kAll, P0.z, 1);
+  Pn.w = __shfl_down_sync(kAll, P0.w, 1);
+  const float2 v0 = edge_vec(P0, P1, w.W, w.H), v1 = edge_vec(P1, Pn, w.W, w.H);
+  const float hb = 0.5f * w.k_bend, hs = 0.5f * w.k_st, ksh = w.k_sh;
+  const float orient = w.orient;
+  const float ko = orient * hs * ksh;
+  // ---- forward recompute with tape ----
+  float2 dl0 = z2, dl1 = z2;
+  for (int it = 0; it < n_pbd; ++it) {
+    float* tp = tape + it * kAdjTapeRegs * 32;
+    const float C0 = hj0 ? th1 - th0 - thr0 : 0.0f;
+    if (kRB) {
+      th0 += hb * C0;
+      th1 -= hb * C0;
+    }
+    const float thn = __shfl_down_sync(kAll, th0, 1);
+    const float C1 = hj1 ? thn - th1 - thr1 : 0.0f;
+    float Cm = __shfl_up_sync(kAll, C1, 1);
+    if (lane == 0) Cm = 0.0f;
+    if (kRB) {
+      th1 += hb * C1;
+      th0 -= hb * Cm;
+    } else {
+      if (he0) th0 += hb * (C0 - Cm);
+      if (he1) th1 += hb * (C1 - C0);
+    }
+    tp[0] = C0;
+    tp[32] = C1;
+    tp[64] = th0;
+    tp[96] = th1;
+    float2 x0 = make_float2(v0.x + (dl1.x - dl0.x), v0.y + (dl1.y - dl0.y));
+    float2 D0 = z2, D1 = z2;
+    if (he0) adj_edge_forward(x0.x, x0.y, L0, th0, hs, ksh, ko, D0.x, D0.y);
+    if (kRB) {
+      dl0 = make_float2(dl0.x + D0.x, dl0.y + D0.y);
+      dl1 = make_float2(dl1.x - D0.x, dl1.y - D0.y);
+    }
+    const float2 dln = make_float2(__shfl_down_sync(kAll, dl0.x, 1), __shfl_down_sync(kAll, dl0.y, 1));
+    const float2 x1 = make_float2(v1.x + (dln.x - dl1.x), v1.y + (dln.y - dl1.y));
+    if (he1) adj_edge_forward(x1.x, x1.y, L1, th1, hs, ksh, ko, D1.x, D1.y);
+    tp[128] = x0.x;
+    tp[160] = x0.y;
+    tp[192] = x1.x;
+    tp[224] = x1.y;
+    float2 Dm = make_float2(__shfl_up_sync(kAll, D1.x, 1), __shfl_up_sync(kAll, D1.y, 1));
+    if (lane == 0) Dm = z2;
+    if (kRB) {
+      dl1 = make_float2(dl1.x + D1.x, dl1.y + D1.y);
+      dl0 = make_float2(dl0.x - Dm.x, dl0.y - Dm.y);
+    } else {
+      dl0 = make_float2(dl0.x + (D0.x - Dm.x), dl0.y + (D0.y - Dm.y));
+      dl1 = make_float2(dl1.x + (D1.x - D0.x), dl1.y + (D1.y - D0.y));
+    }
+  }
+  // ---- reverse ----
+  float2 vb0 = z2, vb1 = z2;   // adjoints of the edge vectors
+  if (w.layers == 2) {
+    const float r0 = he0 ? rsqrtf(v0.x * v0.x + v0.y * v0.y) : 0.0f;
+    const float r1 = he1 ? rsqrtf(v1.x * v1.x + v1.y * v1.y) : 0.0f;
+    const float2 u0 = make_float2(v0.x * r0, v0.y * r0), u1 = make_float2(v1.x * r1, v1.y * r1);
+    float2 um = make_float2(__shfl_up_sync(kAll, u1.x, 1), __shfl_up_sync(kAll, u1.y, 1));
+    if (lane == 0) um = z2;
+    float2 ob0 = z2, ib0 = z2, ob1 = z2, ib1 = z2;
+    if (hb0) adj_normal(a.nbar[b0 + i0], u0, he0, um, lane > 0, ob0, ib0);
+    if (hb1) adj_normal(a.nbar[b0 + i1], u1, he1, u0, true, ob1, ib1);
+    const float2 ibn = make_float2(__shfl_down_sync(kAll, ib0.x, 1), __shfl_down_sync(kAll, ib0.y, 1));
+    if (he0) {
+      const float2 ub = make_float2(ob0.x + ib1.x, ob0.y + ib1.y);
+      const float dot = ub.x * u0.x + ub.y * u0.y;
+      vb0 = make_float2((ub.x - dot * u0.x) * r0, (ub.y - dot * u0.y) * r0);
+    }
+    if (he1) {
+      const float2 ub = make_float2(ob1.x + ibn.x, ob1.y + ibn.y);
+      const float dot = ub.x * u1.x + ub.y * u1.y;
+      vb1 = make_float2((ub.x - dot * u1.x) * r1, (ub.y - dot * u1.y) * r1);
+    }
+  }
+  float gL0 = 0.0f, gL1 = 0.0f, tr0 = 0.0f, tr1 = 0.0f;   // L_rest and theta_rest adjoints of this step
+  float hbb = 0.0f, hsb = 0.0f, kshb = 0.0f;
+  // edge 2l + 1's reverse and its beads' d_bar
+  auto odd_edge = [&](const float* tp, float2& xb1) {
+    const float2 dn = make_float2(__shfl_down_sync(kAll, d0.x, 1), __shfl_down_sync(kAll, d0.y, 1));
+    xb1 = z2;
+    if (he1) {
+      float th_new;
+      adj_edge_reverse(tp[192], tp[224], L1, tp[96], d1.x - dn.x, d1.y - dn.y, thb1, hs, ksh, ko, orient, xb1.x, xb1.y,
+                       th_new, hsb, kshb, gL1);
+      thb1 = th_new;
+      vb1 = make_float2(vb1.x + xb1.x, vb1.y + xb1.y);
+    }
+  };
+  auto even_edge = [&](const float* tp, float2& xb0) {
+    xb0 = z2;
+    if (he0) {
+      float th_new;
+      adj_edge_reverse(tp[128], tp[160], L0, tp[64], d0.x - d1.x, d0.y - d1.y, thb0, hs, ksh, ko, orient, xb0.x, xb0.y,
+                       th_new, hsb, kshb, gL0);
+      thb0 = th_new;
+      vb0 = make_float2(vb0.x + xb0.x, vb0.y + xb0.y);
+    }
+  };
+  auto from_left = [&](float2 v) {   // edge 2l - 1's value, zero at the first bead
+    const float2 m = make_float2(__shfl_up_sync(kAll, v.x, 1), __shfl_up_sync(kAll, v.y, 1));
+    return lane == 0 ? z2 : m;
+  };
+  for (int it = n_pbd - 1; it >= 0; --it) {
+    const float* tp = tape + it * kAdjTapeRegs * 32;
+    float2 xb0, xb1;
+    // position pass: D_bar_e = d_bar_e - d_bar_{e+1}; x = v0 + d_{e+1} - d_e,
+    // so d_bar_i += x_bar_{i-1} - x_bar_i (red-black: odd edges, then even ones)
+    odd_edge(tp, xb1);
+    if (!kRB) even_edge(tp, xb0);
+    const float2 xm = from_left(xb1);
+    if (kRB) {
+      d0 = make_float2(d0.x + xm.x, d0.y + xm.y);
+      d1 = make_float2(d1.x - xb1.x, d1.y - xb1.y);
+      even_edge(tp, xb0);
+      d0 = make_float2(d0.x - xb0.x, d0.y - xb0.y);
+      d1 = make_float2(d1.x + xb0.x, d1.y + xb0.y);
+    } else {
+      d0 = make_float2(d0.x + (xm.x - xb0.x), d0.y + (xm.y - xb0.y));
+      d1 = make_float2(d1.x + (xb0.x - xb1.x), d1.y + (xb0.y - xb1.y));
+    }
+    // bending pass: C_bar_j = hb (theta_bar_j - theta_bar_{j+1}); d theta_e /
+    // d hb = C_e - C_{e-1} (red-black: odd joints, then even ones)
+    const float thbn = __shfl_down_sync(kAll, thb0, 1);
+    const float dt1 = hj1 ? thb1 - thbn : 0.0f;
+    hbb += tp[32] * dt1;
+    const float Cb1 = hb * dt1;
+    float Cbm = __shfl_up_sync(kAll, Cb1, 1);
+    if (lane == 0) Cbm = 0.0f;
+    if (kRB) {
+      thb1 -= Cb1;
+      thb0 += Cbm;
+    }
+    const float dt0 = hj0 ? thb0 - thb1 : 0.0f;
+    hbb += tp[0] * dt0;
+    const float Cb0 = hb * dt0;
+    if (kRB) {
+      thb0 -= Cb0;
+      thb1 += Cb0;
+    } else {
+      thb0 += Cbm - Cb0;
+      thb1 += Cb0 - Cb1;
+    }
+    tr0 -= Cb0;
+    tr1 -= Cb1;
+  }
+  // outputs (with a rest-length drive L(t) = L0 (1 + A s(t)): dL(t)/dL0 = L(t)/L0)
+  auto edge_out = [&](int e, float thb, float gL) {
+    a.adjTh[e] = thb;
+    const float dLdL0 = w.ldrive ? 1.0f + w.ldrive[e].y * drive_sin(w.ldrive[e].z, w.ldrive[e].w, t) : 1.0f;
+    a.gL[e] += gL * dLdL0;
+  };
+  if (he0) edge_out(e0 + i0, thb0, gL0);
+  if (he1) edge_out(e0 + i1, thb1, gL1);
+  if (hj0) a.gth0[j0 + i0] += tr0;
+  if (hj1) a.gth0[j0 + i1] += tr1;
+  // X_bar is final for this step: its largest |dt X_bar| bounds the next
+  // reversed step's u_bar (slot par ^ 1; every lane takes part)
+  const float2 vm = from_left(vb1);
+  float xm = 0.0f;
+  auto bead_out = [&](int i, float2 X, float gx, float gy) {
+    X.x += gx;
+    X.y += gy;
+    a.adjX[i] = X;
+    if (a.xtb) a.xtb[i] = make_float2(gx, gy);
+    xm = fmaxf(xm, w.dt * fmaxf(fabsf(X.x), fabsf(X.y)));
+  };
+  if (hb0) bead_out(b0 + i0, X0, vm.x - vb0.x, vm.y - vb0.y);
+  if (hb1) bead_out(b0 + i1, X1, vb0.x - vb1.x, vb0.y - vb1.y);
+  warp_max_abs(&a.amax[a.par ^ 1], xm);
+  // k_bend = 2 hb, k_stretch = 2 hs, k_shear = ksh: the filament's sums in a
+  // fixed order, added to its own accumulator
+  for (int o = 16; o > 0; o >>= 1) {
+    hbb += __shfl_xor_sync(kAll, hbb, o);
+    hsb += __shfl_xor_sync(kAll, hsb, o);
+    kshb += __shfl_xor_sync(kAll, kshb, o);
+  }
+  if (lane == 0) {
+    a.gkf[3 * f] += 0.5f * hbb;
+    a.gkf[3 * f + 1] += 0.5f * hsb;
+    a.gkf[3 * f + 2] += kshb;
+  }
+}
+
 // The stiffness gradients: the per-filament sums added over filaments in
 // index order (one block).
 __global__ void __launch_bounds__(256) k_adj_gk_reduce(const float* __restrict__ gkf, int n_fil, float* gk) {
@@ -880,7 +1216,16 @@ static int blocks(int n) { return (n + 255) / 256; }
 // then spread over several times more SMs
 constexpr int kAdjBeadThreads = 64;
 static int bead_blocks(int n) { return (n + kAdjBeadThreads - 1) / kAdjBeadThreads; }
-static int blur_blocks(const WorldDev& h) { return h.ntx * ((h.H + kBlurRows - 1) / kBlurRows); }
+
+// Filaments per block of k_adj_pbd_regs: one while the launch has fewer than
+// two per SM (they spread over the SMs), and no more than 48 KB of tape holds.
+static size_t adj_regs_smem(int n_pbd) { return (size_t)n_pbd * kAdjTapeRegs * 32 * sizeof(float); }
+static int adj_regs_warps(int n, int n_pbd) {
+  const size_t per = adj_regs_smem(n_pbd);
+  int wpb = n < 304 ? 1 : kAdjRegsWarps;
+  while (wpb > 1 && wpb * per > 48 * 1024) wpb /= 2;
+  return wpb;
+}
 
 // One reversed step.  Penalty coupling: a8, a7, a6/a4 gathers, a5, a6
 // gradient/a4, then a3/a1.  Direct forcing (m != NULL): a7, the MDF passes
@@ -889,13 +1234,19 @@ void launch_adj_step(const Plan& p, const WorldDev& h, AdjDev a, const AdjMdf* m
   const WorldDev* wd = p.d_worlds;
   const int HW = h.H * h.W;
   auto pbd = [&](const AdjDev& ap) {
-    if (!p.n_fil_items) return;
-    const int mb = (p.max_B + 3) & ~3;
-    const size_t smem = adj_pbd_smem_per_filament(mb, h.n_pbd, h.pbd_order);
-    if (h.pbd_order == 1)
-      k_adj_pbd<true><<<p.n_fil_items, kAdjPbdThreads, smem, s>>>(wd, ap, p.d_fil_items, p.n_fil_items, mb, h.n_pbd);
-    else
-      k_adj_pbd<false><<<p.n_fil_items, kAdjPbdThreads, smem, s>>>(wd, ap, p.d_fil_items, p.n_fil_items, mb, h.n_pbd);
+    if (p.n_long) {
+      const int mb = (p.max_B + 3) & ~3;
+      const size_t smem = adj_pbd_smem_per_filament(mb, h.n_pbd, h.pbd_order);
+      (h.pbd_order == 1 ? k_adj_pbd<true> : k_adj_pbd<false>)<<<p.n_long, kAdjPbdThreads, smem, s>>>(
+          wd, ap, p.d_fil_items, p.n_long, mb, h.n_pbd);
+    }
+    const int n_short = p.n_fil_items - p.n_long;
+    if (n_short) {
+      const int wpb = adj_regs_warps(n_short, h.n_pbd);
+      (h.pbd_order == 1 ? k_adj_pbd_regs<true> : k_adj_pbd_regs<false>)<<<(n_short + wpb - 1) / wpb, 32 * wpb,
+                                                                         wpb * adj_regs_smem(h.n_pbd), s>>>(
+          wd, ap, p.d_fil_items + p.n_long, n_short, h.n_pbd);
+    }
   };
   // (u_bar and Q are cleared by the caller before each step)
   if (m) {
@@ -906,15 +1257,15 @@ void launch_adj_step(const Plan& p, const WorldDev& h, AdjDev a, const AdjMdf* m
     ap.xtb = m->xtb;
     pbd(ap);
     launch_adj_mdf_moments(h, wd, a, *m, s);
-    if (h.N) k_adj_bead_a<<<bead_blocks(h.N), kAdjBeadThreads, 0, s>>>(wd, a);
-    k_adj_rho_blur<<<blur_blocks(h), 256, 0, s>>>(wd, a);
+    if (h.N) k_adj_bead_a<<<bead_blocks(4 * h.N), kAdjBeadThreads, 0, s>>>(wd, a);
+    launch_adj_rho_blur(h, wd, a, s);
     if (h.N) k_adj_bead_b<<<bead_blocks(h.N), kAdjBeadThreads, 0, s>>>(wd, a);
     return;
   }
-  if (h.N || a.setup) k_adj_spread_u<<<std::max(bead_blocks(h.N), 1), kAdjBeadThreads, 0, s>>>(wd, a);
+  if (h.N || a.setup) k_adj_spread_u<<<std::max(bead_blocks(4 * h.N), 1), kAdjBeadThreads, 0, s>>>(wd, a);
   k_adj_lbm<<<blocks(HW), 256, 0, s>>>(wd, a, src_parity);
-  if (h.N) k_adj_bead_a<<<bead_blocks(h.N), kAdjBeadThreads, 0, s>>>(wd, a);
-  k_adj_rho_blur<<<blur_blocks(h), 256, 0, s>>>(wd, a);
+  if (h.N) k_adj_bead_a<<<bead_blocks(4 * h.N), kAdjBeadThreads, 0, s>>>(wd, a);
+  launch_adj_rho_blur(h, wd, a, s);
   pbd(a);   // with a4 and the a6 gradient per bead (k_adj_bead_b's work) first
 }
 
@@ -928,6 +1279,11 @@ void adj_setup(const Plan& p, const WorldDev& h) {
   if (per > 48 * 1024) {
     cudaFuncSetAttribute(k_adj_pbd<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)per);
     cudaFuncSetAttribute(k_adj_pbd<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)per);
+  }
+  if (adj_regs_smem(h.n_pbd) > 48 * 1024) {
+    const int most = (int)adj_regs_smem(kMaxNpbd);
+    cudaFuncSetAttribute(k_adj_pbd_regs<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    cudaFuncSetAttribute(k_adj_pbd_regs<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   }
 }
 
@@ -969,29 +1325,29 @@ __device__ __forceinline__ float2 image_coords(const float4 p, float sx, float s
 
 __global__ void __launch_bounds__(256) k_splat_accum(const WorldDev* __restrict__ wd, int R, float sx, float sy,
                                                      float inv2s2, int K, unsigned long long* __restrict__ acc) {
+  // one thread per bead and image row (blocks along x: beads, y: rows)
   const WorldDev& w = *wd;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= w.N) return;
   const float2 u = image_coords(w.pos[i], sx, sy);
   const int bx = (int)floorf(u.x), by = (int)floorf(u.y);
-  for (int b = -K; b <= K; ++b) {
-    const float dy = (float)(by + b) + 0.5f - u.y;
-    const float gy = expf(-dy * dy * inv2s2);
-    const int row = ((by + b) % R + R) % R;
-    for (int a = -K; a <= K; ++a) {
-      const float dx = (float)(bx + a) + 0.5f - u.x;
-      const float g = gy * expf(-dx * dx * inv2s2);
-      const int col = ((bx + a) % R + R) % R;
-      atomicAdd(&acc[row * R + col], (unsigned long long)__double2ull_rn((double)g * kSplatScale));
-    }
+  const int b = (int)blockIdx.y - K;
+  const float dy = (float)(by + b) + 0.5f - u.y;
+  const float gy = expf(-dy * dy * inv2s2);
+  const int row = ((by + b) % R + R) % R;
+  for (int a = -K; a <= K; ++a) {
+    const float dx = (float)(bx + a) + 0.5f - u.x;
+    const float g = gy * expf(-dx * dx * inv2s2);
+    const int col = ((bx + a) % R + R) % R;
+    atomicAdd(&acc[row * R + col], (unsigned long long)__float2ull_rn(g * (float)kSplatScale));   // (a power of two: exact)
   }
 }
 
 // One block: diff = I - T per pixel and loss = mean(diff^2), summed in a fixed order.
-__global__ void __launch_bounds__(256) k_splat_loss(const unsigned long long* __restrict__ acc,
+__global__ void __launch_bounds__(1024) k_splat_loss(const unsigned long long* __restrict__ acc,
                                                     const float* __restrict__ target, int RR, float* __restrict__ diff,
                                                     float* loss) {
-  __shared__ float red[256];
+  __shared__ float red[1024];
   float sum = 0.0f;
   for (int q = threadIdx.x; q < RR; q += blockDim.x) {
     const float d = (float)((double)acc[q] / kSplatScale) - target[q];
@@ -1000,7 +1356,7 @@ __global__ void __launch_bounds__(256) k_splat_loss(const unsigned long long* __
   }
   red[threadIdx.x] = sum;
   __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
+  for (int o = 512; o > 0; o >>= 1) {
     if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
     __syncthreads();
   }
@@ -1040,8 +1396,8 @@ void launch_loss_splat(const Plan& p, const WorldDev& h, const float* target, in
   const float sx = (float)R / (float)h.W, sy = (float)R / (float)h.H;
   const float inv2s2 = 1.0f / (2.0f * sigma * sigma);
   cudaMemsetAsync(acc, 0, (size_t)R * R * sizeof(unsigned long long), s);
-  if (h.N) k_splat_accum<<<blocks(h.N), 256, 0, s>>>(p.d_worlds, R, sx, sy, inv2s2, K, acc);
-  k_splat_loss<<<1, 256, 0, s>>>(acc, target, R * R, diff, loss);
+  if (h.N) k_splat_accum<<<dim3(blocks(h.N), 2 * K + 1), 256, 0, s>>>(p.d_worlds, R, sx, sy, inv2s2, K, acc);
+  k_splat_loss<<<1, 1024, 0, s>>>(acc, target, R * R, diff, loss);
   if (h.N) k_splat_grad<<<blocks(h.N), 256, 0, s>>>(p.d_worlds, R, sx, sy, inv2s2, K, diff, gx, gy);
 }
 
