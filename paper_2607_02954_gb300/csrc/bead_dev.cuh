@@ -608,11 +608,13 @@ __device__ __forceinline__ float pbd_block(const WorldDev& w, const PbdConst& k,
       if (valid) bin_store(w, slot, b0 + i, p, fe);
     }
   }
-  if (kExt && w.observe && t >= 1) {
+  if (kExt && w.observe && t >= 1 && tid < 32) {
+    // the first warp alone, so that the rounding of its partial sums does not
+    // depend on the width of the block
     float eb = 0.0f, ep = 0.0f;
-    for (int j = tid; j < nJ; j += T) eb += sq(drive_angle(D[j], t - 1) - thr[j]);
+    for (int j = tid; j < nJ; j += 32) eb += sq(drive_angle(D[j], t - 1) - thr[j]);
     if (w.ldrive)
-      for (int e = tid; e < nE; e += T) ep += sq(drive_length(w.ldrive[e0 + e], t - 1) - Lr[e]);
+      for (int e = tid; e < nE; e += 32) ep += sq(drive_length(w.ldrive[e0 + e], t - 1) - Lr[e]);
     obs_add_warp(&w.obs[0], obs_q(eb));
     obs_add_warp(&w.obs[1], obs_q(ep));
   }

@@ -173,7 +173,8 @@ def test_long_filaments_beside_short_ones(lengths, kw):
     assert_field("theta", a.state()["theta"], t2n(st.theta), 1e-6)
     assert_field("disp", a.state()["disp"], t2n(st.D), 1e-5)
     assert_field("fel", a.field("fel"), t2n(rec["F_el"]), 1e-5)
-    other = synth.world_random(4, (40, 72), 5)
+    # beside a world whose longest filament asks for another width of block
+    other = synth.with_observables(synth.world_random(4, (40, 240), 2, lengths=[5, 200]), 4)
     batch = [World(other), World(spec), World(other)]
     step_batched(batch, 4)
     b = World(spec)
