@@ -43,8 +43,9 @@ __device__ __forceinline__ float4 advance_pos(const WorldDev& w, float4 p, float
 // (|U| > u_max or non-finite: flag the world, keep the bead),
 // X^{n+1} = wrap(X^n + dt U) in cell + fraction form, D += dt U.
 // Returns X^{n+1} (X^n when the watchdog fired).
+// d: the bead's displacement so far.
 template <bool kRecord = true>
-__device__ __forceinline__ float4 advance_tail(const WorldDev& w, int i, float4 p, float Ux, float Uy) {
+__device__ __forceinline__ float4 advance_tail(const WorldDev& w, int i, float4 p, float2 d, float Ux, float Uy) {
   if (kRecord) w.ubead[i] = make_float2(Ux, Uy);
   const float m2 = Ux * Ux + Uy * Uy;
   if (!(m2 <= w.u_max * w.u_max)) {   // also catches NaN
@@ -53,7 +54,6 @@ __device__ __forceinline__ float4 advance_tail(const WorldDev& w, int i, float4 
   }
   const float4 q = advance_pos(w, p, Ux, Uy);
   w.pos[i] = q;
-  float2 d = w.disp[i];
   d.x += w.dt * Ux;
   d.y += w.dt * Uy;
   w.disp[i] = d;
@@ -152,15 +152,23 @@ __device__ __forceinline__ void bead_energy(const WorldDev& w, int i, const floa
   }
 }
 
-template <bool kExt>
-__device__ __forceinline__ float2 bead_velocity(const WorldDev& w, int i, const float4 p, long long& q) {
-  if (kExt) bead_energy(w, i, p, q);
-  if (kExt && w.layers == 2) {
+// (the extended worlds' part: U is the velocity interpolated at p)
+__device__ __forceinline__ float2 bead_velocity_ext(const WorldDev& w, int i, const float4 p, float2 U, long long& q) {
+  bead_energy(w, i, p, q);
+  if (w.layers == 2) {
     const float2 n = w.nrm[i];
     const float2 Up = layer_velocity(w, p, n, w.layer_half), Um = layer_velocity(w, p, n, -w.layer_half);
     return make_float2(0.5f * (Up.x + Um.x), 0.5f * (Up.y + Um.y));
   }
-  return interp_u(w, p);
+  return U;
+}
+
+template <bool kExt>
+__device__ __forceinline__ float2 bead_velocity(const WorldDev& w, int i, const float4 p, long long& q) {
+  float2 U = make_float2(0.0f, 0.0f);
+  if (!(kExt && w.layers == 2)) U = interp_u(w, p);
+  if (kExt) U = bead_velocity_ext(w, i, p, U, q);
+  return U;
 }
 
 __device__ __forceinline__ float sq(float v) { return v * v; }
@@ -312,27 +320,38 @@ __device__ __forceinline__ float pbd_regs(const WorldDev& w, const PbdConst& k, 
   const int i0 = 2 * lane, i1 = i0 + 1;
   const bool hb0 = i0 < B, hb1 = i1 < B, he0 = i0 < nE, he1 = i1 < nE, hj0 = i0 < nJ, hj1 = i1 < nJ;
   const float4 z4 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+  // every load that needs only the work item first, then (kMode 1, 2) the
+  // gathers of both beads before either's arithmetic: a step of a small world
+  // is a chain of memory round trips of some 0.4 us each
   float4 P0 = hb0 ? w.pos[b0 + i0] : z4;
   float4 P1 = hb1 ? w.pos[b0 + i1] : z4;
-  // the filament's own inputs first: their loads and the drive's sines
-  // overlap the advance's gathers
+  float2 D0 = make_float2(0.0f, 0.0f), D1 = D0;
+  if (kMode == 1) {
+    if (hb0) D0 = w.disp[b0 + i0];
+    if (hb1) D1 = w.disp[b0 + i1];
+  }
   float th0 = he0 ? w.theta[e0 + i0] : 0.0f;
   float th1 = he1 ? w.theta[e0 + i1] : 0.0f;
   const float L0 = he0 ? (kExt ? rest_length(w, e0 + i0, t) : w.L_rest[e0 + i0]) : 1.0f;
   const float L1 = he1 ? (kExt ? rest_length(w, e0 + i1, t) : w.L_rest[e0 + i1]) : 1.0f;
-  const float thr0 = hj0 ? drive_angle(w.drive[j0 + i0], t) : 0.0f;
-  const float thr1 = hj1 ? drive_angle(w.drive[j0 + i1], t) : 0.0f;
+  const float4 dr0 = hj0 ? w.drive[j0 + i0] : z4, dr1 = hj1 ? w.drive[j0 + i1] : z4;
+  float2 U0 = make_float2(0.0f, 0.0f), U1 = U0;
+  if (kMode != 0 && !(kExt && w.layers == 2)) {
+    // (lanes without a bead gather at cell 0: valid, unused)
+    U0 = interp_u(w, P0);
+    U1 = interp_u(w, P1);
+  }
+  const float thr0 = hj0 ? drive_angle(dr0, t) : 0.0f;
+  const float thr1 = hj1 ? drive_angle(dr1, t) : 0.0f;
   if (kMode == 1) {
     // a8 of the previous step for the lane's beads, then this step's PBD from X^n
     long long q = 0;
-    if (hb0) {
-      const float2 U = bead_velocity<kExt>(w, b0 + i0, P0, q);
-      P0 = advance_tail<false>(w, b0 + i0, P0, U.x, U.y);
+    if (kExt) {
+      if (hb0) U0 = bead_velocity_ext(w, b0 + i0, P0, U0, q);
+      if (hb1) U1 = bead_velocity_ext(w, b0 + i1, P1, U1, q);
     }
-    if (hb1) {
-      const float2 U = bead_velocity<kExt>(w, b0 + i1, P1, q);
-      P1 = advance_tail<false>(w, b0 + i1, P1, U.x, U.y);
-    }
+    if (hb0) P0 = advance_tail<false>(w, b0 + i0, P0, D0, U0.x, U0.y);
+    if (hb1) P1 = advance_tail<false>(w, b0 + i1, P1, D1, U1.x, U1.y);
     if (kExt && w.observe && w.energy) obs_add_warp(&w.obs[2], q);
   } else if (kMode == 0 && w.rec_pos) {
     // the step's start, into the reverse mode's record
@@ -343,14 +362,12 @@ __device__ __forceinline__ float pbd_regs(const WorldDev& w, const PbdConst& k, 
   } else if (kMode == 2) {
     // direct forcing: the fluid (u* in u) carries the beads, PBD starts there
     if (hb0) {
-      const float2 U = interp_u(w, P0);
-      w.ubead[b0 + i0] = U;
-      P0 = advance_pos(w, P0, U.x, U.y);
+      w.ubead[b0 + i0] = U0;
+      P0 = advance_pos(w, P0, U0.x, U0.y);
     }
     if (hb1) {
-      const float2 U = interp_u(w, P1);
-      w.ubead[b0 + i1] = U;
-      P1 = advance_pos(w, P1, U.x, U.y);
+      w.ubead[b0 + i1] = U1;
+      P1 = advance_pos(w, P1, U1.x, U1.y);
     }
   }
   float4 Pn;   // bead 2l + 2
@@ -495,8 +512,9 @@ __device__ __forceinline__ float pbd_block(const WorldDev& w, const PbdConst& k,
     long long q = 0;
     for (int i = tid; i < B; i += T) {
       const float4 p = w.pos[b0 + i];
+      const float2 d = w.disp[b0 + i];
       const float2 U = bead_velocity<kExt>(w, b0 + i, p, q);
-      P[i] = advance_tail<false>(w, b0 + i, p, U.x, U.y);
+      P[i] = advance_tail<false>(w, b0 + i, p, d, U.x, U.y);
     }
     if (kExt && w.observe && w.energy) obs_add_warp(&w.obs[2], q);
   } else if (kMode == 2) {
@@ -637,21 +655,18 @@ extern __shared__ __align__(16) float pbd_dyn_smem[];
 // kLong: the launch has such filaments (a kernel of its own: holding both
 // forms costs the warp form registers, 150 -> 167 us at 2^22 beads).
 template <bool kExt, int kMode, bool kSingle, bool kLong>
-__device__ __forceinline__ void pbd_body(const WorldDev* __restrict__ worlds, const int2* __restrict__ items,
+__device__ __forceinline__ void pbd_body(const WorldDev* __restrict__ worlds, const int4* __restrict__ items,
                                          const PbdWork& pw, int off, int fields, unsigned blk) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int n_long = kLong ? pw.n_long : 0;
   const bool is_long = kLong && (int)blk < n_long;   // block-uniform
   const int item = is_long ? (int)blk : n_long + ((int)blk - n_long) * pw.wpb + warp;
   if (!is_long && (warp >= pw.wpb || item >= pw.n_items)) return;  // warp-uniform exit; no block barrier follows
-  // a single-world launch takes its item from the block index (the world
-  // stays in the table: its fields reach the arithmetic exactly as in a batch)
-  const int2 it = kSingle && !kLong ? make_int2(0, item) : items[item];
-  const WorldDev& w = worlds[it.x];
+  const int4 it = items[item];
+  // (a single-world launch's descriptor need not wait for the item)
+  const WorldDev& w = worlds[kSingle ? 0 : it.x];
   if ((kMode == 2) != (w.ib == 1)) return;   // direct-forcing worlds run their PBD after the steric spread
-  const int f = it.y;
-  const int b0 = w.fil_off[f];
-  const int B = w.fil_off[f + 1] - b0;
+  const int f = it.y, b0 = it.z, B = it.w;
   const int e0 = b0 - f, j0 = b0 - 2 * f;
   const long long t = *w.t + off;
   const PbdConst k = pbd_const(w);
@@ -683,8 +698,10 @@ __device__ __forceinline__ void interp_advance_body(const WorldDev* __restrict__
   long long q = 0;
   float4 p = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   float2 U = make_float2(0.0f, 0.0f);
+  float2 d = make_float2(0.0f, 0.0f);
   if (i < w.N) {
     p = w.pos[i];
+    d = w.disp[i];
     if (kExt && w.ib == 1) {
       U = w.ubead[i];   // direct forcing: the bead's own velocity U_s
       bead_energy(w, i, p, q);
@@ -694,7 +711,7 @@ __device__ __forceinline__ void interp_advance_body(const WorldDev* __restrict__
   }
   if (kExt && w.observe && w.energy) obs_add_warp(&w.obs[2], q);
   if (i >= w.N) return;
-  advance_tail(w, i, p, U.x, U.y);
+  advance_tail(w, i, p, d, U.x, U.y);
 }
 
 }  // namespace mc

@@ -526,7 +526,7 @@ __device__ __forceinline__ void adj_edge_reverse(float x, float y, float L, floa
 
 template <bool kRB>
 __global__ void __launch_bounds__(kAdjPbdThreads) k_adj_pbd(const WorldDev* __restrict__ wd, AdjDev a,
-                                                            const int2* __restrict__ items, int n_items,
+                                                            const int4* __restrict__ items, int n_items,
                                                             int maxB, int n_pbd) {
   constexpr int kTape = kRB ? kAdjTapePerPassRB : kAdjTapePerPass;
   extern __shared__ __align__(16) float smem[];
@@ -534,9 +534,8 @@ __global__ void __launch_bounds__(kAdjPbdThreads) k_adj_pbd(const WorldDev* __re
   const int tid = threadIdx.x, lane = tid & 31;
   const int item = blockIdx.x;
   if (item >= n_items) return;   // block-uniform
-  const int f = items[item].y;
-  const int b0 = w.fil_off[f];
-  const int B = w.fil_off[f + 1] - b0;
+  const int4 it = items[item];
+  const int f = it.y, b0 = it.z, B = it.w;
   const int nE = B - 1, nJ = B - 2;
   const int e0 = b0 - f, j0 = b0 - 2 * f;
   float* s = smem;
@@ -895,7 +894,7 @@ __device__ __forceinline__ void adj_normal(float2 nb, float2 out, bool ho, float
 
 template <bool kRB>
 __global__ void __launch_bounds__(32 * kAdjRegsWarps) k_adj_pbd_regs(const WorldDev* __restrict__ wd, AdjDev a,
-                                                                     const int2* __restrict__ items, int n_items,
+                                                                     const int4* __restrict__ items, int n_items,
                                                                      int n_pbd) {
   constexpr unsigned kAll = 0xffffffffu;
   extern __shared__ __align__(16) float smem[];
@@ -904,9 +903,8 @@ __global__ void __launch_bounds__(32 * kAdjRegsWarps) k_adj_pbd_regs(const World
   const int item = blockIdx.x * (blockDim.x >> 5) + warp;
   if (item >= n_items) return;   // warp-uniform; no block barrier
   float* tape = smem + (size_t)warp * n_pbd * kAdjTapeRegs * 32 + lane;
-  const int f = items[item].y;
-  const int b0 = w.fil_off[f];
-  const int B = w.fil_off[f + 1] - b0;
+  const int4 it = items[item];
+  const int f = it.y, b0 = it.z, B = it.w;
   const int nE = B - 1, nJ = B - 2;
   const int e0 = b0 - f, j0 = b0 - 2 * f;
   const int i0 = 2 * lane, i1 = i0 + 1;

@@ -9,9 +9,11 @@ namespace mc {
 
 // a1 + a3 + a2, one warp per filament of at most 64 beads (in registers), one
 // block per longer one (in dynamic shared memory): see pbd_body.
-template <bool kExt, int kMode, bool kSingle, bool kLong>
-__global__ void __launch_bounds__(256, 4) k_pbd(const WorldDev* __restrict__ worlds,
-                                             const int2* __restrict__ items, const PbdWork pw, int off,
+// kRoomy: twice the registers, for launches whose filaments are all resident
+// at half the warps per SM (more of a filament's loads are in flight at once).
+template <bool kExt, int kMode, bool kSingle, bool kLong, bool kRoomy>
+__global__ void __launch_bounds__(256, kRoomy ? 2 : 4) k_pbd(const WorldDev* __restrict__ worlds,
+                                             const int4* __restrict__ items, const PbdWork pw, int off,
                                              int fields) {
   pdl_trigger();
   pdl_wait();
@@ -211,9 +213,11 @@ static void launch_pbd_kernel(const Plan& p, cudaStream_t s, int off, int fields
   if (p.n_fil_items == 0) return;
   const PbdLaunch l = pbd_launch(p);
   const bool one = p.n_worlds == 1;
-  auto kern = p.n_long ? (one ? k_pbd<kExt, kMode, true, true> : k_pbd<kExt, kMode, false, true>)
-                       : (one ? k_pbd<kExt, kMode, true, false> : k_pbd<kExt, kMode, false, false>);
-  launch_pdl(kern, l.grid, l.block, l.smem, s, (const WorldDev*)p.d_worlds, (const int2*)p.d_fil_items, l.pw, off,
+  const bool roomy = !p.n_long && p.n_fil_items <= 16 * num_sms();
+  auto kern = p.n_long ? (one ? k_pbd<kExt, kMode, true, true, false> : k_pbd<kExt, kMode, false, true, false>)
+              : roomy  ? (one ? k_pbd<kExt, kMode, true, false, true> : k_pbd<kExt, kMode, false, false, true>)
+                       : (one ? k_pbd<kExt, kMode, true, false, false> : k_pbd<kExt, kMode, false, false, false>);
+  launch_pdl(kern, l.grid, l.block, l.smem, s, (const WorldDev*)p.d_worlds, (const int4*)p.d_fil_items, l.pw, off,
              fields);
 }
 
@@ -243,10 +247,10 @@ void kernel_setup() {
     steric_setup(num_sms());
     persistent_setup();
     const int most = 227 * 1024;
-    for (auto f : {k_pbd<false, 0, false, true>, k_pbd<true, 0, false, true>, k_pbd<false, 1, false, true>,
-                   k_pbd<true, 1, false, true>, k_pbd<true, 2, false, true>, k_pbd<false, 0, true, true>,
-                   k_pbd<true, 0, true, true>, k_pbd<false, 1, true, true>, k_pbd<true, 1, true, true>,
-                   k_pbd<true, 2, true, true>})
+    for (auto f : {k_pbd<false, 0, false, true, false>, k_pbd<true, 0, false, true, false>, k_pbd<false, 1, false, true, false>,
+                   k_pbd<true, 1, false, true, false>, k_pbd<true, 2, false, true, false>, k_pbd<false, 0, true, true, false>,
+                   k_pbd<true, 0, true, true, false>, k_pbd<false, 1, true, true, false>, k_pbd<true, 1, true, true, false>,
+                   k_pbd<true, 2, true, true, false>})
       cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
   });
 }

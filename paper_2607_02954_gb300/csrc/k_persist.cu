@@ -83,7 +83,7 @@ union PersistSmem {
 struct PersistArgs {
   const WorldDev* worlds;
   int n_worlds;
-  const int2* fil_items;
+  const int4* fil_items;
   int n_pbd_blocks, n_fil_items;
   const int2* bead_items;
   int n_bead_items;

@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_force_spread(const WorldDev* 
   const TileBox tb = tile_box(w, it.y);
   float2* __restrict__ F_out = w.F;
   const int W = w.W;
-  const int k = force_tile<R, NT>(sm, w, (tb.y0 / kTile) * w.ntx + tb.x0 / kTile, tb, store_fields, off, true);
+  const int k = force_tile<R, NT>(sm, w, tb, store_fields, off, true, []() {});
   __syncthreads();
   force_fold<NT>(sm.wk, tb, w.ntx, w.nty);
   const float inv = pow2f(-k);
@@ -159,13 +159,12 @@ __global__ void __launch_bounds__(kThreads, 4) k_force_lbm_ws(const WorldDev* __
     const WorldDev& w = kSingle ? w1 : worlds[it.x];
     const TileBox tb = tile_box(w, it.y);
     if (force_group) {
-      prefetch_populations<kWsForce>(w, tb, off);
       const int tile = (tb.y0 / kTile) * w.ntx + tb.x0 / kTile;
       int k = 40;
       if (!kSingle && w.tile_rho_max[tile] == 0.0f) {
         tile_clear<kWsForce>(sm.f.wk);   // no bead reaches the tile: F = 0 (see k_force_lbm)
       } else {
-        k = force_tile<R, kWsForce>(sm.f, w, tile, tb, 0, off, fields);
+        k = force_tile<R, kWsForce>(sm.f, w, tb, 0, off, fields, [&]() { prefetch_populations<kWsForce>(w, tb, off); });
       }
       force_sync<kWsForce>();
       force_fold<kWsForce>(sm.f.wk, tb, w.ntx, w.nty);
@@ -323,8 +322,7 @@ __global__ void __launch_bounds__(kThreads) k_mdf_pass(const WorldDev* __restric
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const float2* __restrict__ u_in = (pass & 1) ? w.u2 : w.u;
   float2* __restrict__ u_out = (pass & 1) ? w.u : w.u2;
-  if (warp == 0)
-    build_segments(w, step_counts(w, *w.t), tb.x0 - 2, tb.x0 + tb.tw, tb.y0 - 2, tb.y0 + tb.th, sm.sg);
+  if (warp == 0) build_segments<true>(w, 0, tb.x0 - 2, tb.x0 + tb.tw, tb.y0 - 2, tb.y0 + tb.th, sm.sg);
   // the velocity and density windows, rows y0 - 3 .. y0 + th + 2 and
   // columns x0 - 4 .. x0 + tw + 3, periodic (W, H >= 8: one wrap at most),
   // in 16-byte chunks (2 velocities or 4 densities; x0 and W are multiples

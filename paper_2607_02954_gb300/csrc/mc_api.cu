@@ -154,7 +154,8 @@ mc_status build_plan(mc_world* const* ws, int n, cudaStream_t s, Plan& out) {
   p.any_mdf = false;
   p.max_mdf = 0;
   p.any_ext = false;
-  std::vector<int2> fil_long, fil, bead, tile, cell;
+  std::vector<int4> fil_long, fil;
+  std::vector<int2> bead, tile, cell;
   std::vector<WorldDev> table(n);
   for (int k = 0; k < n; ++k) {
     const mc_world* w = ws[k];
@@ -167,7 +168,8 @@ mc_status build_plan(mc_world* const* ws, int n, cudaStream_t s, Plan& out) {
     p.max_mdf = std::max(p.max_mdf, w->h.mdf_iters);
     p.any_ext = p.any_ext || w->h.layers == 2 || w->h.observe || w->h.has_ldrive || w->h.ib == 1;
     for (int f = 0; f < w->h.n_fil; ++f)
-      (w->fil_off[f + 1] - w->fil_off[f] > 64 ? fil_long : fil).push_back(make_int2(k, f));
+      (w->fil_off[f + 1] - w->fil_off[f] > 64 ? fil_long : fil)
+          .push_back(make_int4(k, f, w->fil_off[f], w->fil_off[f + 1] - w->fil_off[f]));
     const int nb = std::max(w->h.N, 1);
     for (int b = 0; b < nb; b += mc::kBeadChunk) bead.push_back(make_int2(k, b));
     for (int ty = 0; ty < w->h.nty; ++ty)   // tile items carry (tx, ty) packed: tx | ty << 16
@@ -179,14 +181,14 @@ mc_status build_plan(mc_world* const* ws, int n, cudaStream_t s, Plan& out) {
   fil.insert(fil.begin(), fil_long.begin(), fil_long.end());
   Layout L;
   const size_t o_w = L.take<WorldDev>(n);
-  const size_t o_f = L.take<int2>(fil.size());
+  const size_t o_f = L.take<int4>(fil.size());
   const size_t o_b = L.take<int2>(bead.size());
   const size_t o_t = L.take<int2>(tile.size());
   const size_t o_c = L.take<int2>(cell.size());
   const size_t o_bar = L.take<unsigned>(4);
   std::vector<char> host(L.off);
   std::memcpy(host.data() + o_w, table.data(), n * sizeof(WorldDev));
-  if (!fil.empty()) std::memcpy(host.data() + o_f, fil.data(), fil.size() * sizeof(int2));
+  if (!fil.empty()) std::memcpy(host.data() + o_f, fil.data(), fil.size() * sizeof(int4));
   std::memcpy(host.data() + o_b, bead.data(), bead.size() * sizeof(int2));
   if (!tile.empty()) std::memcpy(host.data() + o_t, tile.data(), tile.size() * sizeof(int2));
   std::memcpy(host.data() + o_c, cell.data(), cell.size() * sizeof(int2));
@@ -196,7 +198,7 @@ mc_status build_plan(mc_world* const* ws, int n, cudaStream_t s, Plan& out) {
   if (e != cudaSuccess) return cuda_fail(e, "plan upload");
   // pageable source: the copy is staged before cudaMemcpyAsync returns
   p.d_worlds = at<WorldDev>(p.d_mem, o_w);
-  p.d_fil_items = at<int2>(p.d_mem, o_f);
+  p.d_fil_items = at<int4>(p.d_mem, o_f);
   p.d_bead_items = at<int2>(p.d_mem, o_b);
   p.d_tile_items = at<int2>(p.d_mem, o_t);
   p.d_cell_items = at<int2>(p.d_mem, o_c);

@@ -201,7 +201,7 @@ struct Plan {
   int n_long = 0;                // filaments of more than 64 beads (first in d_fil_items)
   int n_fil_items = 0, n_bead_items = 0, n_tile_items = 0, n_cell_items = 0;
   WorldDev* d_worlds = nullptr;  // [n_worlds]
-  int2* d_fil_items = nullptr;   // (world, filament)
+  int4* d_fil_items = nullptr;   // (world, filament, first bead, beads)
   int2* d_bead_items = nullptr;  // (world, first bead)
   int2* d_tile_items = nullptr;  // (world, tx | ty << 16), row-major over the tiles
   int2* d_cell_items = nullptr;  // (world, first cell)

@@ -150,7 +150,7 @@ size_t footprint(int H, int W, int n_fil, int N, bool ldrive, bool energy, int l
   h.has_energy = energy;
   h.layers = layers;
   // arena plus this world's share of a plan (work items and table entry)
-  const size_t items = (size_t)n_fil + (N / mc::kBeadChunk + 1) + h.n_tiles + (size_t)H * W / mc::kCellChunk + 1 +
+  const size_t items = 2 * (size_t)n_fil + (N / mc::kBeadChunk + 1) + h.n_tiles + (size_t)H * W / mc::kCellChunk + 1 +
                        h.n_chunks;
   return mc::world_layout(h, nullptr).total + items * sizeof(int2) + sizeof(mc::WorldDev) + 4096;
 }

@@ -56,10 +56,16 @@ struct Segments {
 
 // Builds the list for the box [x_lo, x_hi] x [y_lo, y_hi] (inclusive,
 // unwrapped coordinates; at most 8 bins a side: tile + 2 R + 3 <= 51 cells)
-// with one warp; lane l handles bins l and l + 32, so all counts load in one
-// round trip.
-__device__ void build_segments(const WorldDev& w, const int* counts, int x_lo, int x_hi, int y_lo, int y_hi,
-                               Segments& sg) {
+// with one warp; lane l handles bins l and l + 32.  With kBoth the counts of
+// both parities load beside the step counter that chooses between them: one
+// round trip in all (force + LBM at 2^22 beads: 351 -> 337 us).  The deposit,
+// whose blocks clear the other parity's counts meanwhile, loads the step's
+// own after the counter (with both, 86 -> 102 us there).
+template <bool kBoth>
+__device__ void build_segments(const WorldDev& w, int off, int x_lo, int x_hi, int y_lo, int y_hi, Segments& sg) {
+  const long long t = *w.t + off;
+  const int* c0 = kBoth ? w.bin_cnt : step_counts(w, t);
+  const int* c1 = w.bin_cnt + (w.n_bins + 1);
   const int lane = threadIdx.x & 31;
   const int nbx = w.nbx, nby = w.nby, cap = w.slot_cap;
   int bx0 = floor_div(x_lo, kBin), bx1 = floor_div(x_hi, kBin);
@@ -68,16 +74,23 @@ __device__ void build_segments(const WorldDev& w, const int* counts, int x_lo, i
   if (by1 - by0 + 1 >= nby) { by0 = 0; by1 = nby - 1; }
   const int ncol = bx1 - bx0 + 1, nrow = by1 - by0 + 1;
   const int cc = lane & 7, rr = lane >> 3;
-  int bin[2] = {0, 0}, n[2] = {0, 0};
+  int bin[2] = {0, 0}, n[2] = {0, 0}, m[2] = {0, 0};
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int r = rr + 4 * h;
     if (cc < ncol && r < nrow) {
       bin[h] = wrap_once(by0 + r, nby) * nbx + wrap_once(bx0 + cc, nbx);
-      n[h] = counts[bin[h]];
+      n[h] = c0[bin[h]];
+      if (kBoth) m[h] = c1[bin[h]];
     }
   }
-  const int over = counts[w.n_bins];
+  int over = c0[w.n_bins];
+  const int over1 = kBoth ? c1[w.n_bins] : 0;
+  if (kBoth && (t & 1)) {
+    n[0] = m[0];
+    n[1] = m[1];
+    over = over1;
+  }
   int covered = n[0] + n[1], most = max(n[0], n[1]);
   int incl0 = min(n[0], cap), incl1 = min(n[1], cap);
 #pragma unroll
@@ -380,10 +393,9 @@ __device__ __forceinline__ void deposit_x_body(const WorldDev* __restrict__ worl
   d.full_y = w.nty == 1;
   d.cx0 = d.full_x ? 0 : d.x0;                  // region column origin
   d.oxe = d.full_x ? 4 : R + 4;                 // accumulator column of region column 0
-  const long long t = *w.t + off;
-  if (warp == 0)
-    build_segments(w, step_counts(w, t), d.x0 - d.wR - 2, d.x0 + d.tw + d.wR, d.y0 - 2, d.y0 + d.th, sm.sg);
+  if (warp == 0) build_segments<false>(w, off, d.x0 - d.wR - 2, d.x0 + d.tw + d.wR, d.y0 - 2, d.y0 + d.th, sm.sg);
   if (warp == 2) {
+    const long long t = *w.t + off;
     int* next = step_counts(w, t + 1);
     const int bx = d.x0 / kBin + (lane & 3), by = d.y0 / kBin + (lane >> 2);
     if (lane < 16 && bx < w.nbx && by < w.nby) next[by * w.nbx + bx] = 0;
@@ -443,7 +455,7 @@ template <int R>
 struct TileIn {
   float xb[Geo<R>::kLoadRows * kWin];   // rho_x window
   Segments sg;
-  float nbmax[9];                       // largest rho_s of the 3x3 tiles around
+  int k;                                // exponent of the spread's fixed point
   float tap_s[Geo<R>::kTaps];
 };
 
@@ -563,17 +575,25 @@ __device__ __forceinline__ void tile_stage_window(TileIn<R>& in, const WorldDev&
 template <int R>
 __device__ __forceinline__ void tile_stage_meta(TileIn<R>& in, const WorldDev& w, const TileBox& tb, int off) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (warp == 0)
-    build_segments(w, step_counts(w, *w.t + off), tb.x0 - 2, tb.x0 + tb.tw, tb.y0 - 2, tb.y0 + tb.th, in.sg);
+  if (warp == 0) build_segments<true>(w, off, tb.x0 - 2, tb.x0 + tb.tw, tb.y0 - 2, tb.y0 + tb.th, in.sg);
   if (warp == 1 && lane < Geo<R>::kTaps) in.tap_s[lane] = padded_tap<R>(w, w.R, lane);
   // bound of the cell sums of weight * |F_el + F_s|:
   //   |F_s| <= k_rep/2 max|rho_bar(c+1) - rho_bar(c-1)| <= k_rep/2 max rho_bar
   //        <= k_rep/2 max rho_s over the 3x3 tiles around this one,
   // times max rho_s of this tile (the sum of the spread weights of a cell)
-  if (warp == 2 && lane < 9) {
-    const int tx = tb.x0 / kTile, ty = tb.y0 / kTile;
-    const int ty2 = wrap_once(ty + lane / 3 - 1, w.nty), tx2 = wrap_once(tx + lane % 3 - 1, w.ntx);
-    in.nbmax[lane] = w.tile_rho_max[ty2 * w.ntx + tx2];
+  if (warp == 2) {
+    float v = 0.0f;   // (bounds are non-negative)
+    if (lane < 9) {
+      const int tx = tb.x0 / kTile, ty = tb.y0 / kTile;
+      const int ty2 = wrap_once(ty + lane / 3 - 1, w.nty), tx2 = wrap_once(tx + lane % 3 - 1, w.ntx);
+      v = w.tile_rho_max[ty2 * w.ntx + tx2];
+    }
+    const long long t = *w.t + off;
+    const unsigned f0 = w.fel_max[0], f1 = w.fel_max[1];
+    const float rho_max = __shfl_sync(0xffffffffu, v, 4);   // this tile's
+    for (int o = 8; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    if (lane == 0)
+      in.k = fix_exponent((__uint_as_float((t & 1) ? f1 : f0) + 0.5f * w.k_rep * v) * rho_max * 1.0001f + 1e-30f);
   }
 }
 
@@ -681,27 +701,26 @@ __device__ __forceinline__ void tile_beads(TileWork<NT>& wk, const WorldDev& w, 
   }
 }
 
-// The y pass of a5 and a6 for one tile.  Returns k: after the caller
+// The y pass of a5 and a6 for one tile.  pull() runs once the tile's own
+// loads are under way (the fused kernel starts its population reads there:
+// they wait for the step counter, and nothing before needs it).  Returns k: after the caller
 // synchronises the block, accx/accy hold the tile's F 2^k (before folding,
 // see force_fold).
-template <int R, int NT>
-__device__ __forceinline__ int force_tile(ForceSmem<R, NT>& sm, const WorldDev& w, int tile, const TileBox& tb,
-                                          int store_fields, int off, bool keep_fs) {
+template <int R, int NT, class Pull>
+__device__ __forceinline__ int force_tile(ForceSmem<R, NT>& sm, const WorldDev& w, const TileBox& tb,
+                                          int store_fields, int off, bool keep_fs, Pull pull) {
   constexpr int kCap = TileWork<NT>::kCap;
   TileIn<R>& in = sm.in;
   TileWork<NT>& wk = sm.wk;
   tile_stage_window<R, NT>(in, w, tb);
   tile_stage_meta(in, w, tb, off);
   tile_clear<NT>(wk);
+  pull();
   force_sync<NT>();
   const int total = in.sg.pre[kSegs];
   force_list<NT>(in.sg, wk, w, 0, min(kCap, total), tb);
   cp_async_wait_all();   // the window
-  const float fmax_el = __uint_as_float(w.fel_max[(*w.t + off) & 1]);
-  const float rho_max = w.tile_rho_max[tile];
-  float rho_nb = in.nbmax[0];
-  for (int k2 = 1; k2 < 9; ++k2) rho_nb = fmaxf(rho_nb, in.nbmax[k2]);
-  const int k = fix_exponent((fmax_el + 0.5f * w.k_rep * rho_nb) * rho_max * 1.0001f + 1e-30f);
+  const int k = in.k;
   const float scale = pow2f(k);
   force_sync<NT>();
   // (only the beads' gradients and the rho_bar field read the y pass)
@@ -763,37 +782,56 @@ __device__ __forceinline__ void prefetch_populations(const WorldDev& w, const Ti
 }
 
 // a7 on the tile's cells with F = acc 2^-k from shared memory.  Each warp
-// collides rows warp, warp + NT / 32, ...; the first row's populations are pulled
-// before the barrier that completes the spread (pulling one row ahead in the
-// loop measured slower: register pressure).
+// collides rows warp, warp + NT / 32, ...  A warp's first row is pulled in
+// begin(): by 32 warps, one row each, as soon as the tile's own loads are
+// under way, so that the collision's memory round trip overlaps the force
+// phase; by fewer warps, whose blocks overlap one another instead, only
+// before the barrier that completes the spread (pulling earlier, or one row
+// ahead in the loop, measured slower there: register pressure).
 template <int NT>
-__device__ __forceinline__ void tile_lbm(TileWork<NT>& wk, const WorldDev& w, const TileBox& tb, int k, int off) {
-  const int W = w.W, H = w.H, HW = H * W;
-  const long long t = *w.t + off;
-  const float* __restrict__ src = w.g[t & 1];
-  float* __restrict__ dst = w.g[(t + 1) & 1];
-  float2* __restrict__ u_out = w.u;
-  const LbmConst kc{w.om_p, w.om_m, w.src_p, w.src_m};
-  const float inv = pow2f(-k);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const bool active = lane < tb.tw && warp < tb.th;
-  const int x = tb.x0 + lane;
-  const int xm = x == 0 ? W - 1 : x - 1, xp = x == W - 1 ? 0 : x + 1;
+struct TileLbm {
+  const float* src;
+  float* dst;
+  int x, xm, xp, y, warp, lane;
+  bool active;
   LbmPull q;
-  int y = tb.y0 + warp;
-  if (active) lbm_pull(src, HW, y * W, (y == 0 ? H - 1 : y - 1) * W, (y == H - 1 ? 0 : y + 1) * W, x, xm, xp, q);
-  __syncthreads();
-  force_fold<NT>(wk, tb, w.ntx, w.nty);
-  if (!active) return;
-  for (int ly = warp; ly < tb.th; ly += NT / 32) {
-    if (ly != warp)
-      lbm_pull(src, HW, y * W, (y == 0 ? H - 1 : y - 1) * W, (y == H - 1 ? 0 : y + 1) * W, x, xm, xp, q);
-    const int s = (ly + 3) * kAx + lane + 3;
-    const float2 F = make_float2((float)wk.accx[s] * inv, (float)wk.accy[s] * inv);
-    u_out[(size_t)y * W + x] = lbm_collide(q, dst, HW, y * W + x, F, kc);
-    y += NT / 32;
+
+  __device__ __forceinline__ void begin(const WorldDev& w, const TileBox& tb, int off) {
+    const long long t = *w.t + off;
+    src = w.g[t & 1];
+    dst = w.g[(t + 1) & 1];
+    const int W = w.W;
+    lane = threadIdx.x & 31;
+    warp = threadIdx.x >> 5;
+    active = lane < tb.tw && warp < tb.th;
+    x = tb.x0 + lane;
+    xm = x == 0 ? W - 1 : x - 1;
+    xp = x == W - 1 ? 0 : x + 1;
+    y = tb.y0 + warp;
+    if (active) pull(w);
   }
-}
+  __device__ __forceinline__ void pull(const WorldDev& w) {
+    const int W = w.W, H = w.H;
+    lbm_pull(src, H * W, y * W, (y == 0 ? H - 1 : y - 1) * W, (y == H - 1 ? 0 : y + 1) * W, x, xm, xp, q);
+  }
+  // after the spread: synchronises the block, folds, collides
+  __device__ __forceinline__ void finish(TileWork<NT>& wk, const WorldDev& w, const TileBox& tb, int k) {
+    float2* __restrict__ u_out = w.u;
+    const int W = w.W, HW = w.H * W;
+    const LbmConst kc{w.om_p, w.om_m, w.src_p, w.src_m};
+    const float inv = pow2f(-k);
+    __syncthreads();
+    force_fold<NT>(wk, tb, w.ntx, w.nty);
+    if (!active) return;
+    for (int ly = warp; ly < tb.th; ly += NT / 32) {
+      if (ly != warp) pull(w);
+      const int s = (ly + 3) * kAx + lane + 3;
+      const float2 F = make_float2((float)wk.accx[s] * inv, (float)wk.accy[s] * inv);
+      u_out[(size_t)y * W + x] = lbm_collide(q, dst, HW, y * W + x, F, kc);
+      y += NT / 32;
+    }
+  }
+};
 
 // y pass of a5 + a6 + a7 on one tile: the force density goes from shared
 // memory straight into the collision (the same arithmetic as k_force_spread
@@ -808,20 +846,27 @@ __device__ __forceinline__ void force_lbm_body(const WorldDev* __restrict__ worl
   const WorldDev& w = kSingle ? w1 : worlds[it.x];
   const TileBox tb = tile_box(w, it.y);
   const bool layered = w.layers == 2;
-  if (!layered) prefetch_populations<NT>(w, tb, off);
   const int tile = (tb.y0 / kTile) * w.ntx + tb.x0 / kTile;
   int k = 40;
+  TileLbm<NT> lbm;
+  constexpr bool kEarly = NT == 1024;
   if (!kSingle && !layered && w.tile_rho_max[tile] == 0.0f) {
     // no bead's stencil reaches this tile's cells (the deposit's bound is 0
     // exactly then), so it owns no bead and the spread has no term on it:
     // F = 0, as the force pass would give.  Sparse batched worlds have many
     // such tiles.
     tile_clear<NT>(sm.wk);
+    lbm.begin(w, tb, off);
   } else {
-    k = force_tile<R, NT>(sm, w, tile, tb, 0, off, fields || layered);
+    k = force_tile<R, NT>(sm, w, tb, 0, off, fields || layered, [&]() {
+      if (layered) return;
+      if (kEarly) lbm.begin(w, tb, off);
+      else prefetch_populations<NT>(w, tb, off);
+    });
+    if (!kEarly && !layered) lbm.begin(w, tb, off);
   }
   // two-layer worlds: F_s only; their layer spread and collision follow in their own kernels
-  if (!layered) tile_lbm<NT>(sm.wk, w, tb, k, off);
+  if (!layered) lbm.finish(sm.wk, w, tb, k);
 }
 
 }  // namespace mc
