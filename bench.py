@@ -50,9 +50,14 @@ GRAPH_STEPS = 16   # mc_step replays graphs of 16 steps: PBD, then 15 x (previou
 
 
 def mdf_launches(steps: int, m: int) -> int:
-    """Kernels of direct-forcing steps (always the unfused sequence): PBD (returns), bins, deposit,
-    steric spread, moments, predicted PBD, m passes (one tile kernel each), LBM, advance."""
-    return steps * (8 + m)
+    """Kernels of a run of direct-forcing steps, in 16-step graphs and a leftover run: per step bins (with
+    the previous advance), deposit, steric spread + moments, predicted PBD and m passes (one tile kernel
+    each, the last with the LBM), and a run's last advance; without passes the unfused sequence (PBD, which
+    returns, bins, deposit, spread, moments, predicted PBD, LBM, advance)."""
+    if m == 0:
+        return 8 * steps
+    r = steps % GRAPH_STEPS
+    return steps * (4 + m) + steps // GRAPH_STEPS + (1 if r else 0)
 
 
 def graph_launches(steps: int) -> int:

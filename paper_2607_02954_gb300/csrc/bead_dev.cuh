@@ -336,10 +336,14 @@ __device__ __forceinline__ float pbd_regs(const WorldDev& w, const PbdConst& k, 
   const float L1 = he1 ? (kExt ? rest_length(w, e0 + i1, t) : w.L_rest[e0 + i1]) : 1.0f;
   const float4 dr0 = hj0 ? w.drive[j0 + i0] : z4, dr1 = hj1 ? w.drive[j0 + i1] : z4;
   float2 U0 = make_float2(0.0f, 0.0f), U1 = U0;
-  if (kMode != 0 && !(kExt && w.layers == 2)) {
+  if (kMode == 1 && !(kExt && w.layers == 2)) {
     // (lanes without a bead gather at cell 0: valid, unused)
     U0 = interp_u(w, P0);
     U1 = interp_u(w, P1);
+  } else if (kMode == 2) {
+    const float2* u = mdf_u(w, 0);   // u*
+    U0 = interp_field(u, w.W, w.H, P0);
+    U1 = interp_field(u, w.W, w.H, P1);
   }
   const float thr0 = hj0 ? drive_angle(dr0, t) : 0.0f;
   const float thr1 = hj1 ? drive_angle(dr1, t) : 0.0f;
@@ -360,7 +364,7 @@ __device__ __forceinline__ float pbd_regs(const WorldDev& w, const PbdConst& k, 
     if (he0) w.rec_theta[e0 + i0] = th0;
     if (he1) w.rec_theta[e0 + i1] = th1;
   } else if (kMode == 2) {
-    // direct forcing: the fluid (u* in u) carries the beads, PBD starts there
+    // direct forcing: the fluid (u*) carries the beads, PBD starts there
     if (hb0) {
       w.ubead[b0 + i0] = U0;
       P0 = advance_pos(w, P0, U0.x, U0.y);
@@ -518,10 +522,10 @@ __device__ __forceinline__ float pbd_block(const WorldDev& w, const PbdConst& k,
     }
     if (kExt && w.observe && w.energy) obs_add_warp(&w.obs[2], q);
   } else if (kMode == 2) {
-    // direct forcing: the positions the fluid (u* in u) carries the beads to
+    // direct forcing: the positions the fluid (u*) carries the beads to
     for (int i = tid; i < B; i += T) {
       const float4 p = w.pos[b0 + i];
-      const float2 U = interp_u(w, p);
+      const float2 U = interp_field(mdf_u(w, 0), w.W, w.H, p);
       w.ubead[b0 + i] = U;
       P[i] = advance_pos(w, p, U.x, U.y);
     }

@@ -165,7 +165,7 @@ __global__ void k_cells_out(const float4* __restrict__ pos, int N, int W, int* c
 // Warps (filaments) per block: at most the configuration's, and few enough
 // that a small launch still spreads over every SM (each warp's filament is a
 // serial chain; warps sharing an SM's schedulers only delay one another).
-static int num_sms() {
+int num_sms() {
   // first asked by kernel_setup, outside any stream capture
   static const int sms = [] {
     int dev = 0, n = 0;
@@ -230,7 +230,7 @@ void launch_pbd(const Plan& p, cudaStream_t s) {
 
 // The PBD of direct-forcing worlds (from the positions the fluid carries
 // the beads to; the others return at once).
-void launch_pbd_mdf(const Plan& p, cudaStream_t s) { launch_pbd_kernel<true, 2>(p, s, 0, 1); }
+void launch_pbd_mdf(const Plan& p, cudaStream_t s, int off) { launch_pbd_kernel<true, 2>(p, s, off, 1); }
 
 // a8 of the previous step fused with this step's a1-a3 (plans without
 // direct-forcing worlds), off steps after the worlds' counters.

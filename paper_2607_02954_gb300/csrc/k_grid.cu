@@ -183,6 +183,10 @@ void launch_lbm(const Plan& p, cudaStream_t s, int layered_only, int off) {
 // arithmetic, one kernel and one position round trip fewer), and the worlds'
 // counters move by n at the end.
 void enqueue_steps(const Plan& p, int n, cudaStream_t s) {
+  if (p.fuse_mdf) {
+    enqueue_mdf_steps(p, n, s);
+    return;
+  }
   if (p.any_mdf || n < 2) {
     for (int k = 0; k < n; ++k) enqueue_step(p, s);
     return;

@@ -59,7 +59,7 @@ namespace mc {
 // LBM 53.7 -> 31.3; 512^2 with 1024 beads a tile: 17.1 -> 15.9 and, with 512
 // threads, 22.4 -> 18.9; 128^2: force + LBM 7.9 -> 7.3.  A tile's sums are
 // integers or per-cell, so the width changes no result.
-static int tile_threads(const Plan& p, int sms, int regs, bool beads_only) {
+int tile_threads(const Plan& p, int sms, int regs, bool beads_only) {
   const long long room = (long long)sms * (65536 / (regs * 256));   // blocks of 256 resident at once
   const long long tiles = p.n_tile_items;
   for (int nt : {1024, 512})
@@ -77,11 +77,13 @@ __global__ void __launch_bounds__(NT, 2048 / NT) k_deposit_x(const WorldDev* __r
   deposit_x_body<R, kSingle, NT>(worlds, items, store_fields, off, w1, blockIdx.x, sm);
 }
 
-// y pass of a5 + a6: writes F.
+// y pass of a5 + a6: writes F.  moments: direct-forcing worlds also get u* =
+// (sum_i c_i f_i + F/2) / rho and rho of the tile's cells (the fluid before
+// the filament's forcing), F taken from shared memory.
 template <int R, int NT>
 __global__ void __launch_bounds__(NT, 1024 / NT) k_force_spread(const WorldDev* __restrict__ worlds,
                                                            const int2* __restrict__ items, int store_fields,
-                                                           int off) {
+                                                           int off, int moments) {
   pdl_trigger();
   pdl_wait();
   __shared__ __align__(16) ForceSmem<R, NT> sm;
@@ -90,7 +92,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_force_spread(const WorldDev* 
   const TileBox tb = tile_box(w, it.y);
   float2* __restrict__ F_out = w.F;
   const int W = w.W;
-  const int k = force_tile<R, NT>(sm, w, tb, store_fields, off, true, []() {});
+  const int k = force_tile<R, NT>(sm, w, tb, store_fields, off, true,
+                                  [&]() { if (moments && w.ib == 1) prefetch_populations<NT>(w, tb, off); });
   __syncthreads();
   force_fold<NT>(sm.wk, tb, w.ntx, w.nty);
   const float inv = pow2f(-k);
@@ -98,10 +101,22 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_force_spread(const WorldDev* 
   // a direct-forcing world's F holds the step's total force (steric spread
   // plus MDF passes): a re-run for the density fields leaves it
   if (store_fields && w.ib == 1) return;
+  const bool mom = moments && w.ib == 1;
+  const int x = tb.x0 + lane, H = w.H, HW = H * W;
+  const int xm = x == 0 ? W - 1 : x - 1, xp = x == W - 1 ? 0 : x + 1;
+  const float* src = mom ? w.g[(*w.t + off) & 1] : nullptr;
+  float2* __restrict__ u_out = mom ? mdf_u(w, 0) : nullptr;
   for (int ly = threadIdx.x >> 5; ly < tb.th; ly += NT / 32) {
     if (lane < tb.tw) {
-      const int s = (ly + 3) * kAx + lane + 3;
-      F_out[(size_t)(tb.y0 + ly) * W + tb.x0 + lane] = make_float2((float)sm.wk.accx[s] * inv, (float)sm.wk.accy[s] * inv);
+      const int s = (ly + 3) * kAx + lane + 3, y = tb.y0 + ly;
+      const float2 F = make_float2((float)sm.wk.accx[s] * inv, (float)sm.wk.accy[s] * inv);
+      const size_t c = (size_t)y * W + x;
+      F_out[c] = F;
+      if (mom) {
+        LbmPull q;
+        lbm_pull(src, HW, y * W, (y == 0 ? H - 1 : y - 1) * W, (y == H - 1 ? 0 : y + 1) * W, x, xm, xp, q);
+        u_out[c] = lbm_moments(q, F, w.mrho[c]);
+      }
     }
   }
 }
@@ -206,228 +221,6 @@ __global__ void __launch_bounds__(kThreads, 4) k_force_lbm_ws(const WorldDev* __
   if (force_group && done > 0) ws_bar_sync(kWsEmpty);   // the last F has been read
 }
 
-// One MDF pass of the direct-forcing worlds on one tile, Jacobi in u.  Every
-// bead whose stencil reaches the tile gets
-//   dF_i = 2 I[rho](X_i) (U_s,i - I[u](X_i))
-// from the pass's input velocity (u for even passes, u2 for odd ones) and
-// rho, both staged with a 3-cell halo; then the tile's cells get
-// F += S[dF] and u' = u + S[dF] / (2 rho) in the other velocity buffer, and
-// the tile that holds a bead adds its dF to F_el.  A bead near a tile edge
-// is evaluated by each tile its stencil reaches, from the same inputs in the
-// same order, so every tile uses the same dF bitwise.  The spread is in
-// int32 fixed point with the scale from the largest |dF| component among
-// the tile's beads times the tile's largest rho_s (the sum of the spread
-// weights of a cell): bitwise independent of order.  The dF of a tile's
-// beads are kept in shared memory when they fit one staging pass, and are
-// evaluated again in a second sweep otherwise.
-constexpr int kMwy = kTile + 6;   // window rows: the tile and 3 cells a side
-constexpr int kMwx = kTile + 8;   // window columns: the tile and 4 cells a side (16-byte chunks)
-
-constexpr int kMdfCap = 640;      // bead records staged per pass
-
-struct MdfSmem {
-  float4 sp[kMdfCap];   // staged bead records
-  float2 su[kMdfCap];   // their U_s
-  float2 df[kMdfCap];   // their dF (one-pass tiles)
-  int si[kMdfCap];      // their bead indices
-  float2 uw[kMwy * kMwx];   // input velocity window
-  float rw[kMwy * kMwx];    // density window
-  int accx[kAx * kAx];    // spread accumulators
-  int accy[kAx * kAx];
-  int list[kMdfCap];
-  int s_cnt;
-  Segments sg;
-  float red[kWarps];
-};
-
-// dF of the staged bead v whose tile-relative cell is (rx, ry) in [-2, tw] x
-// [-2, th]: its stencil cells sit at window rows ry + 2 .. ry + 5 and
-// columns rx + 3 .. rx + 6.
-__device__ __forceinline__ float2 mdf_bead_force(const MdfSmem& sm, int v, int rx, int ry) {
-  const float4 p = sm.sp[v];
-  float wx[4], wy[4];
-  peskin4(p.x, wx);
-  peskin4(p.y, wy);
-  float Ux = 0.0f, Uy = 0.0f, r = 0.0f;
-#pragma unroll
-  for (int b = 0; b < 4; ++b) {
-    const int row = (ry + 2 + b) * kMwx + rx + 3;
-    float ax = 0.0f, ay = 0.0f, ar = 0.0f;
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const float2 v2 = sm.uw[row + a];
-      ax = fmaf(wx[a], v2.x, ax);
-      ay = fmaf(wx[a], v2.y, ay);
-      ar = fmaf(wx[a], sm.rw[row + a], ar);
-    }
-    Ux = fmaf(wy[b], ax, Ux);
-    Uy = fmaf(wy[b], ay, Uy);
-    r = fmaf(wy[b], ar, r);
-  }
-  const float2 Us = sm.su[v];
-  return make_float2(2.0f * r * (Us.x - Ux), 2.0f * r * (Us.y - Uy));
-}
-
-// Stages chunk c0 of the tile's bead segments and lists the beads whose
-// stencil reaches the tile (the block synchronises inside).
-__device__ __forceinline__ int mdf_stage_chunk(MdfSmem& sm, const WorldDev& w, const TileBox& tb, int c0, int total) {
-  const int tid = threadIdx.x;
-  const int W = w.W, H = w.H, ntx = w.ntx, nty = w.nty;
-  const int n = min(kMdfCap, total - c0);
-  for (int v = tid; v < n; v += kThreads) {
-    const int slot = seg_slot(c0 + v, sm.sg);
-    cp_async16(&sm.sp[v], &w.bpos[slot]);
-    cp_async8(&sm.su[v], &w.sus[slot]);
-    cp_async4(&sm.si[v], reinterpret_cast<const int*>(&w.brec[slot]) + 2);   // the record's id
-  }
-  cp_async_wait_all();
-  if (tid == 0) sm.s_cnt = 0;
-  __syncthreads();
-  for (int v0 = 0; v0 < n; v0 += kThreads) {
-    const int v = v0 + tid;
-    bool keep = false;
-    int rx = 0, ry = 0;
-    if (v < n) {
-      const float4 p = sm.sp[v];
-      rx = cell_x(p) - tb.x0;
-      ry = cell_y(p) - tb.y0;
-      keep = true;
-      if (ntx > 1) {
-        rx = image_lo(rx, W, 2);
-        keep = rx <= tb.tw;
-      }
-      if (nty > 1) {
-        ry = image_lo(ry, H, 2);
-        keep = keep && ry <= tb.th;
-      }
-    }
-    const int at = list_place(keep, &sm.s_cnt);
-    if (keep) sm.list[at] = pack_code(v, rx, ry);
-  }
-  __syncthreads();
-  return sm.s_cnt;
-}
-
-__global__ void __launch_bounds__(kThreads) k_mdf_pass(const WorldDev* __restrict__ worlds,
-                                                       const int2* __restrict__ items, int pass) {
-  pdl_trigger();
-  pdl_wait();
-  __shared__ __align__(16) MdfSmem sm;
-  const int2 it = items[blockIdx.x];
-  const WorldDev& w = worlds[it.x];
-  if (w.ib != 1 || pass >= w.mdf_iters) return;
-  const TileBox tb = tile_box(w, it.y);
-  const int W = w.W, H = w.H, ntx = w.ntx, nty = w.nty;
-  const int tile = (tb.y0 / kTile) * ntx + tb.x0 / kTile;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const float2* __restrict__ u_in = (pass & 1) ? w.u2 : w.u;
-  float2* __restrict__ u_out = (pass & 1) ? w.u : w.u2;
-  if (warp == 0) build_segments<true>(w, 0, tb.x0 - 2, tb.x0 + tb.tw, tb.y0 - 2, tb.y0 + tb.th, sm.sg);
-  // the velocity and density windows, rows y0 - 3 .. y0 + th + 2 and
-  // columns x0 - 4 .. x0 + tw + 3, periodic (W, H >= 8: one wrap at most),
-  // in 16-byte chunks (2 velocities or 4 densities; x0 and W are multiples
-  // of 8, so a chunk never straddles the periodic edge)
-  const bool full = tb.tw == kTile;   // full tile: constant divisors
-  const int nu = full ? kMwx / 2 : (tb.tw + 8) >> 1, nr = full ? kMwx / 4 : (tb.tw + 8) >> 2, wh = tb.th + 6;
-  for (int c = tid; c < wh * nu; c += kThreads) {
-    const int i = full ? c / (kMwx / 2) : c / nu, j = 2 * (c - i * nu);
-    const size_t g = (size_t)wrap_once(tb.y0 - 3 + i, H) * W + wrap_once(tb.x0 - 4 + j, W);
-    cp_async16(&sm.uw[i * kMwx + j], &u_in[g]);
-  }
-  for (int c = tid; c < wh * nr; c += kThreads) {
-    const int i = full ? c / (kMwx / 4) : c / nr, j = 4 * (c - i * nr);
-    const size_t g = (size_t)wrap_once(tb.y0 - 3 + i, H) * W + wrap_once(tb.x0 - 4 + j, W);
-    cp_async16(&sm.rw[i * kMwx + j], &w.mrho[g]);
-  }
-  for (int c = tid; c < kAx * kAx / 4; c += kThreads) {
-    reinterpret_cast<int4*>(sm.accx)[c] = make_int4(0, 0, 0, 0);
-    reinterpret_cast<int4*>(sm.accy)[c] = make_int4(0, 0, 0, 0);
-  }
-  __syncthreads();   // segments visible (the windows land with the first chunk's wait)
-  const int total = sm.sg.pre[kSegs];
-  const bool one_pass = total <= kMdfCap;
-  // sweep 1: dF of every listed bead and their largest component
-  float m = 0.0f;
-  for (int c0 = 0; c0 < total; c0 += kMdfCap) {
-    if (c0 > 0) __syncthreads();   // the previous chunk is no longer read
-    const int cnt = mdf_stage_chunk(sm, w, tb, c0, total);
-    for (int q = tid; q < cnt; q += kThreads) {
-      const int code = sm.list[q];
-      const int v = code_slot(code);
-      const float2 dF = mdf_bead_force(sm, v, code_rx(code), code_ry(code));
-      if (one_pass) sm.df[v] = dF;
-      m = fmaxf(m, fmaxf(fabsf(dF.x), fabsf(dF.y)));
-    }
-  }
-  if (total == 0) cp_async_wait_all();
-  m = block_max<kThreads>(m, sm.red);   // also orders the df writes before sweep 2
-  const int k = fix_exponent(m * w.tile_rho_max[tile] * 1.0001f + 1e-30f);
-  const float scale = pow2f(k);
-  // sweep 2: the spread, and F_el += dF on the bead's own tile
-  float2* __restrict__ fel = w.fel;
-  for (int c0 = 0; c0 < total; c0 += kMdfCap) {
-    int cnt = sm.s_cnt;
-    if (!one_pass) {
-      __syncthreads();
-      cnt = mdf_stage_chunk(sm, w, tb, c0, total);
-    }
-    for (int q = tid; q < cnt; q += kThreads) {
-      const int code = sm.list[q];
-      const int v = code_slot(code), rx = code_rx(code), ry = code_ry(code);
-      const float2 dF = one_pass ? sm.df[v] : mdf_bead_force(sm, v, rx, ry);
-      if (rx >= 0 && rx < tb.tw && ry >= 0 && ry < tb.th) {
-        // the bead's own tile is its one writer in this pass: the adds
-        // need no return value and leave the same bits in any order
-        const int i = sm.si[v];
-        atomicAdd(&fel[i].x, dF.x);
-        atomicAdd(&fel[i].y, dF.y);
-      }
-      const float4 p = sm.sp[v];
-      float wx[4], wy[4];
-      peskin4(p.x, wx);
-      peskin4(p.y, wy);
-      const float Fx = dF.x * scale, Fy = dF.y * scale;
-      int* bx = sm.accx + (ry + 2) * kAx + rx + 2;
-      int* by = sm.accy + (ry + 2) * kAx + rx + 2;
-#pragma unroll
-      for (int b = 0; b < 4; ++b) {
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-          const float g = wx[a] * wy[b];
-          atomicAdd(bx + b * kAx + a, __float2int_rn(g * Fx));
-          atomicAdd(by + b * kAx + a, __float2int_rn(g * Fy));
-        }
-      }
-    }
-  }
-  __syncthreads();
-  force_fold<kThreads>(sm, tb, ntx, nty);
-  const float inv = pow2f(-k);
-  // the warp's rows warp, warp + 8, ...: every F load in flight at once
-  float2* __restrict__ Fg = w.F;
-  constexpr int kRows = kTile / kWarps;
-  float2 Fv[kRows];
-#pragma unroll
-  for (int r = 0; r < kRows; ++r) {
-    const int ly = warp + r * kWarps;
-    if (ly < tb.th && lane < tb.tw) Fv[r] = Fg[(size_t)(tb.y0 + ly) * W + tb.x0 + lane];
-  }
-#pragma unroll
-  for (int r = 0; r < kRows; ++r) {
-    const int ly = warp + r * kWarps;
-    if (ly < tb.th && lane < tb.tw) {
-      const int sidx = (ly + 3) * kAx + lane + 3;
-      const int widx = (ly + 3) * kMwx + lane + 4;
-      const size_t c = (size_t)(tb.y0 + ly) * W + tb.x0 + lane;
-      const float Gx = (float)sm.accx[sidx] * inv, Gy = (float)sm.accy[sidx] * inv;
-      Fg[c] = make_float2(Fv[r].x + Gx, Fv[r].y + Gy);
-      const float ih = __frcp_rn(2.0f * sm.rw[widx]);   // 1 / (2 rho), correctly rounded
-      const float2 u = sm.uw[widx];
-      u_out[c] = make_float2(fmaf(Gx, ih, u.x), fmaf(Gy, ih, u.y));
-    }
-  }
-}
-
 namespace {
 
 // Blocks of the warp-specialised force + LBM kernel: as many as fit on every
@@ -457,8 +250,8 @@ void launch_deposit(const Plan& p, cudaStream_t s, int store_fields, int off) {
 }
 
 template <int R, int NT>
-void launch_spread(const Plan& p, cudaStream_t s, int store_fields, int off) {
-  k_force_spread<R, NT><<<p.n_tile_items, NT, 0, s>>>(p.d_worlds, p.d_tile_items, store_fields, off);
+void launch_spread(const Plan& p, cudaStream_t s, int store_fields, int off, int moments) {
+  k_force_spread<R, NT><<<p.n_tile_items, NT, 0, s>>>(p.d_worlds, p.d_tile_items, store_fields, off, moments);
 }
 
 template <int R, int NT>
@@ -469,15 +262,15 @@ void launch_fused(const Plan& p, cudaStream_t s, int off, int fields) {
 
 template <int R>
 void launch_steric(const Plan& p, cudaStream_t s, int which, int store_fields, int off, int fields) {
-  const int nt = tile_threads(p, g_sms, which == 0 ? 32 : 64, which != 2);
+  const int nt = tile_threads(p, g_sms, which == 0 ? 32 : 64, which == 0 || (which == 1 && !fields));
   if (which == 0) {
     if (nt == 1024) launch_deposit<R, 1024>(p, s, store_fields, off);
     else if (nt == 512) launch_deposit<R, 512>(p, s, store_fields, off);
     else launch_deposit<R, 256>(p, s, store_fields, off);
   } else if (which == 1) {
-    if (nt == 1024) launch_spread<R, 1024>(p, s, store_fields, off);
-    else if (nt == 512) launch_spread<R, 512>(p, s, store_fields, off);
-    else launch_spread<R, 256>(p, s, store_fields, off);
+    if (nt == 1024) launch_spread<R, 1024>(p, s, store_fields, off, fields);
+    else if (nt == 512) launch_spread<R, 512>(p, s, store_fields, off, fields);
+    else launch_spread<R, 256>(p, s, store_fields, off, fields);
   } else if (p.cfg.force_ws && !p.any_layered) {
     const int grid = std::min(p.n_tile_items, ws_grid<R>());
     if (p.n_worlds == 1)
@@ -527,13 +320,11 @@ void launch_deposit_x(const Plan& p, cudaStream_t s, int store_fields, int off) 
 
 // Two-layer worlds get F from their layer points after the tile pass.
 void launch_force_spread(const Plan& p, cudaStream_t s, int store_fields, int off) {
-  dispatch_steric(p, s, 1, store_fields, off);
+  dispatch_steric(p, s, 1, store_fields, off, 0);
   launch_layer_spread(p, s);
 }
 
-void launch_mdf_pass(const Plan& p, cudaStream_t s, int pass) {
-  if (p.n_tile_items) k_mdf_pass<<<p.n_tile_items, kThreads, 0, s>>>(p.d_worlds, p.d_tile_items, pass);
-}
+void launch_force_moments(const Plan& p, cudaStream_t s, int off) { dispatch_steric(p, s, 1, 0, off, 1); }
 
 void launch_force_lbm(const Plan& p, cudaStream_t s, int off, int fields) {
   dispatch_steric(p, s, 2, 0, off, fields);

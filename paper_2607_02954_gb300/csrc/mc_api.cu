@@ -177,6 +177,8 @@ mc_status build_plan(mc_world* const* ws, int n, cudaStream_t s, Plan& out) {
     const int HW = w->h.H * w->h.W;
     for (int c = 0; c < HW; c += mc::kCellChunk) cell.push_back(make_int2(k, c));
   }
+  p.fuse_mdf = n > 0 && p.max_mdf > 0;
+  for (int k = 0; k < n; ++k) p.fuse_mdf = p.fuse_mdf && ws[k]->h.ib == 1 && ws[k]->h.mdf_iters == p.max_mdf;
   p.n_long = (int)fil_long.size();
   fil.insert(fil.begin(), fil_long.begin(), fil_long.end());
   Layout L;

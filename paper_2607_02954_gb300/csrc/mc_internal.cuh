@@ -90,7 +90,7 @@ struct WorldDev {
   int ib, mdf_iters;      // coupling (0 penalty, 1 direct forcing) and MDF passes per step
   float* mrho;            // [H * W] fluid density of the step (ib == 1)
   int* bead_slot;         // [N] slot of each bead in bpos and brec (ib == 1 or layers == 2, else nullptr)
-  float2* u2;             // [H * W] second velocity buffer: MDF passes alternate u -> u2 -> u (ib == 1)
+  float2* u2;             // [H * W] second velocity buffer of the MDF passes (ib == 1, see mdf_u)
   float2* sus;            // [n_bins slot_cap + N] U_s by slot (ib == 1)
   float2* nrm;            // [N] filament unit normal at each bead (layers == 2)
   unsigned long long* facc;  // [2 H W] fixed-point spread of the layer points (layers == 2)
@@ -196,6 +196,7 @@ struct Plan {
   bool any_layered = false;      // some world is a two-layer filament world
   bool any_mdf = false;          // some world couples by direct forcing (ib == 1)
   int max_mdf = 0;               // most MDF passes of a world
+  bool fuse_mdf = false;         // every world couples by direct forcing, with the same number of passes >= 1
   bool any_ext = false;          // some world has two layers, observables, a rest-length drive or direct forcing
   long long beads = 0;           // of all worlds
   int n_long = 0;                // filaments of more than 64 beads (first in d_fil_items)
@@ -245,10 +246,16 @@ void launch_interp_advance(const Plan& p, cudaStream_t s, int inc = 1);   // inc
 // direct forcing (ib == 1 worlds; the others return at once): bins and a
 // zero F_el before the steric spread, then u*, the predicted PBD and the
 // MDF passes after it
-void launch_mdf_bins(const Plan& p, cudaStream_t s);
+void launch_mdf_bins(const Plan& p, cudaStream_t s, int off = 0);
 void launch_mdf(const Plan& p, cudaStream_t s);
+// n steps of a plan of direct-forcing worlds with one number of passes (at
+// least one), fused
+void enqueue_mdf_steps(const Plan& p, int n, cudaStream_t s);
+void launch_force_moments(const Plan& p, cudaStream_t s, int off);   // k_steric.cu: the spread and u*, rho
+int tile_threads(const Plan& p, int sms, int regs, bool beads_only);   // k_steric.cu
+int num_sms();
 cudaError_t launch_mdf_recorded(const Plan& p, const WorldDev& h, float2* mu, cudaStream_t s);   // one world, passes' inputs kept
-void launch_mdf_pass(const Plan& p, cudaStream_t s, int pass);   // k_steric.cu: one MDF pass (tile kernel)
+void launch_mdf_pass(const Plan& p, cudaStream_t s, int pass, int off, int fields, int fuse);   // one MDF pass (tile kernel)
 void enqueue_step(const Plan& p, cudaStream_t s);
 void enqueue_steps(const Plan& p, int n, cudaStream_t s);   // n steps, fused bead stages where possible
 // fields = 0: a step within a run, whose per-bead fields for read-out (F_el,
@@ -405,6 +412,19 @@ __device__ __forceinline__ void lbm_pull(const float* __restrict__ src, int HW, 
   q.d[8] = src[8 * HW + rp + xm];   // ( 1,-1) from (x-1, y+1)
 }
 
+// The velocity (sum_i c_i f_i + F/2) / rho and density of a cell from its
+// pulled populations.
+__device__ __forceinline__ float2 lbm_moments(const LbmPull& q, float2 F, float& rho_out) {
+  const float* d = q.d;
+  const float drho = ((d[0] + (d[1] + d[3])) + (d[2] + d[4])) + ((d[5] + d[7]) + (d[6] + d[8]));
+  const float rho = 1.0f + drho;
+  const float jx = (d[1] - d[3]) + (d[5] - d[7]) + (d[8] - d[6]);
+  const float jy = (d[2] - d[4]) + (d[5] - d[7]) + (d[6] - d[8]);
+  const float inv = __frcp_rn(rho);
+  rho_out = rho;
+  return make_float2((jx + 0.5f * F.x) * inv, (jy + 0.5f * F.y) * inv);
+}
+
 // Collision of cell c from its pulled populations: stores the post-collision
 // populations of c in `dst` and returns u.
 __device__ __forceinline__ float2 lbm_collide(const LbmPull& q, float* __restrict__ dst, int HW, int c, float2 F,
@@ -493,6 +513,13 @@ __device__ __forceinline__ long long obs_q(float v) { return __float2ll_rn(v * k
 __device__ __forceinline__ void obs_add_warp(unsigned long long* acc, long long q) {
   for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
   if ((threadIdx.x & 31) == 0 && q != 0) atomicAdd(acc, (unsigned long long)q);
+}
+
+// Input velocity of MDF pass k of a direct-forcing world (u* for pass 0); the
+// passes alternate two buffers so that the last one's output, and with it the
+// collision's velocity, goes to u.
+__host__ __device__ __forceinline__ float2* mdf_u(const WorldDev& w, int k) {
+  return ((k + w.mdf_iters) & 1) ? w.u2 : w.u;
 }
 
 // A world's bin counts of step t (see WorldDev).

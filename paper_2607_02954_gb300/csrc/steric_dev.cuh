@@ -152,12 +152,6 @@ __device__ __forceinline__ int list_place(bool keep, int* s_cnt) {
   return base + __popc(m & ((1u << lane) - 1u));
 }
 
-// list code: staged slot v (10 bits), rx + 16 and ry + 16 (11 bits each)
-__device__ __forceinline__ int pack_code(int v, int rx, int ry) { return v | ((rx + 16) << 10) | ((ry + 16) << 21); }
-__device__ __forceinline__ int code_slot(int c) { return c & 1023; }
-__device__ __forceinline__ int code_rx(int c) { return ((c >> 10) & 2047) - 16; }
-__device__ __forceinline__ int code_ry(int c) { return (c >> 21) - 16; }
-
 template <int NT, typename T>
 __device__ __forceinline__ T block_max(T v, T* red) {
   for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));

@@ -183,3 +183,55 @@ def test_long_filaments_beside_short_ones(lengths, kw):
     for k in want:
         assert np.array_equal(want[k], got[k]), k
     assert b.observables() == batch[1].observables()
+
+
+@pytest.mark.parametrize("m", [0, 1, 2, 3, 4])
+@pytest.mark.parametrize("steps", [1, 2, 5, 18])
+def test_direct_forcing_runs_alone_batched_and_mixed(m, steps):
+    """The fused sequence of a direct-forcing world (odd and even numbers of
+    passes), the unfused one it takes beside a penalty world, and single steps:
+    bitwise the same, read-outs included."""
+    p = dict(ib=1, mdf_iters=m)
+    spec = synth.world_random(21, (72, 136), 9)
+    spec.params = synth.Params(**p)
+    spec = synth.with_observables(spec, 5)
+    dense = crowded(17, n_fil=60)
+    dense.params.ib, dense.params.mdf_iters = 1, m
+    penalty = synth.world_random(22, 64, 4)
+    for sp in (spec, dense):
+        a, s, b, c = (World(sp) for _ in range(4))
+        a.step(steps)
+        for _ in range(steps):
+            s.step(1)
+        step_batched([b, World(sp)], steps)        # a batch of the same coupling
+        step_batched([c, World(penalty)], steps)   # a mixed one
+        want = a.state(fluid=True)
+        for other in (s, b, c):
+            got = other.state(fluid=True)
+            for k in want:
+                assert np.array_equal(want[k], got[k]), k
+            for f in ("fel", "fs", "ubead", "u", "force", "bin", "bin_off", "rho_s", "rho_bar"):
+                assert np.array_equal(a.field(f), other.field(f)), f
+            assert a.observables() == other.observables()
+
+
+@pytest.mark.parametrize("H,W,n_fil", [(64, 96, 20), (256, 512, 500), (520, 1288, 2000)])
+def test_direct_forcing_tile_widths(H, W, n_fil):
+    """One step of direct forcing with tile blocks of 1024, 512 and 256
+    threads, some tiles holding more beads than one list, against the oracle."""
+    rng = np.random.default_rng(H)
+    B = 40
+    x = np.concatenate([rng.uniform(0, W) + np.arange(B) for _ in range(n_fil)]) % W
+    y = np.repeat(rng.uniform(0, H / 2, n_fil), B)
+    x, y = x.astype(np.float32), y.astype(np.float32)
+    x[x >= W] = 0
+    J = n_fil * (B - 2)
+    spec = synth._world("mdf", H, W, [B] * n_fil, x, y, np.zeros(n_fil * (B - 1), np.float32), rng.normal(0, 0.1, J),
+                        np.zeros(J), np.zeros(J), np.zeros(J), params=synth.Params(ib=1, mdf_iters=2, k_rep=0.01))
+    ow = O.World(spec)
+    st, rec = O.step(ow, ow.initial_state(), record=True)
+    w = World(spec)
+    w.step(1)
+    assert_field("u", w.field("u"), np.moveaxis(t2n(rec["u"]), 0, -1), 1e-5)
+    assert_field("force", w.field("force"), np.moveaxis(t2n(rec["F"]), 0, -1), 1e-5)
+    assert_field("ubead", w.field("ubead"), t2n(rec["U"]), 1e-5)
