@@ -250,16 +250,19 @@ __device__ __forceinline__ float2 bead_normal(float2 out, bool has_out, float2 i
 // the others a negative one of their own); bin_place returns the lane's slot.
 // Every lane calls both; two claims can be in flight before their places.
 struct BinClaim {
-  int bin, base;
+  int base, lo, hi;   // the group's first place; the bin's slots
   unsigned peers;
 };
 
-__device__ __forceinline__ BinClaim bin_claim(int* counts, bool valid, int bin) {
+__device__ __forceinline__ BinClaim bin_claim(const WorldDev& w, int* counts, bool valid, int bin) {
   const int lane = threadIdx.x & 31;
   BinClaim c;
-  c.bin = valid ? bin : -1 - lane;
-  c.peers = __match_any_sync(0xffffffffu, c.bin);
-  c.base = 0;
+  c.peers = __match_any_sync(0xffffffffu, valid ? bin : -1 - lane);
+  c.base = c.lo = c.hi = 0;
+  if (valid) {
+    c.lo = w.bin_base[bin];
+    c.hi = w.bin_base[bin + 1];
+  }
   if (valid && (__ffs(c.peers) - 1) == lane) c.base = atomicAdd(&counts[bin], __popc(c.peers));
   return c;
 }
@@ -268,8 +271,8 @@ __device__ __forceinline__ int bin_place(const WorldDev& w, int* counts, bool va
   const int lane = threadIdx.x & 31;
   const int at = __shfl_sync(0xffffffffu, c.base, __ffs(c.peers) - 1) + __popc(c.peers & ((1u << lane) - 1u));
   if (!valid) return -1;
-  if (at < w.slot_cap) return c.bin * w.slot_cap + at;
-  return w.n_bins * w.slot_cap + atomicAdd(&counts[w.n_bins], 1);   // the bin's slots are full
+  if (c.lo + at < c.hi) return c.lo + at;
+  return w.slot_end + atomicAdd(&counts[w.n_bins], 1);   // the bin's slots are full
 }
 
 // The bin of the bead at P.
@@ -465,7 +468,7 @@ __device__ __forceinline__ float pbd_regs(const WorldDev& w, const PbdConst& k, 
     if (hb0) fe0 = bead_out_force(w, k, b0 + i0, bin0, dlx0, dly0, fields, fmax);
     if (hb1) fe1 = bead_out_force(w, k, b0 + i1, bin1, dlx1, dly1, fields, fmax);
     int* counts = step_counts(w, t);
-    const BinClaim c0 = bin_claim(counts, hb0, bin0), c1 = bin_claim(counts, hb1, bin1);
+    const BinClaim c0 = bin_claim(w, counts, hb0, bin0), c1 = bin_claim(w, counts, hb1, bin1);
     const int s0 = bin_place(w, counts, hb0, c0), s1 = bin_place(w, counts, hb1, c1);
     if (hb0) bin_store(w, s0, b0 + i0, P0, fe0);
     if (hb1) bin_store(w, s1, b0 + i1, P1, fe1);
@@ -623,7 +626,7 @@ __device__ __forceinline__ float pbd_block(const WorldDev& w, const PbdConst& k,
       const bool valid = i < B;
       const float4 p = valid ? P[i] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
       const int bin = bead_bin_of(p, k.nbx);
-      const BinClaim c = bin_claim(counts, valid, bin);
+      const BinClaim c = bin_claim(w, counts, valid, bin);
       float2 fe = make_float2(0.0f, 0.0f);
       if (valid) fe = bead_out_force(w, k, b0 + i, bin, dlx[i], dly[i], fields, fmax);
       const int slot = bin_place(w, counts, valid, c);

@@ -1202,6 +1202,7 @@ __global__ void __launch_bounds__(256) k_set_counter(const __grid_constant__ Wor
   if (i == 0) {
     *w.t = v;
     w.fel_max[v & 1] = 0u;
+    *w.cnt_valid = 0;   // the counts in place are not those of step v - 1
   }
   if (i <= w.n_bins) step_counts(w, v)[i] = 0;
 }

@@ -7,13 +7,19 @@
 namespace mc {
 
 // ---------------------------------------------------------------------------
-// Sorted read-outs of a step's bins: the exclusive prefix sum of the bin
-// counts, in blocks of kScanChunk bins (k_scan_sums adds up each block,
-// k_scan_apply offsets each block by the sum of the earlier ones and scans
-// it), then the records in bin order (k_sort_records).  A step does not run
-// them: its tile kernels read each bin's slots directly.  They serve the
-// field read-outs and saved images, and k_unsort_records puts a loaded
-// image's records back into slots.
+// Prefix sums over a world's bins, in blocks of kScanChunk bins (k_scan_sums
+// adds up each block, k_scan_apply offsets each block by the sum of the
+// earlier ones and scans it; worlds of one block need no sums).
+//   kSrc 0  the bin counts of step (counter + off): the exclusive offsets of
+//           the sorted read-outs (bin_off), and in bin_cursor each bin's first
+//           place after its slots' records
+//   kSrc 1  the room for the counts of the last completed step: bin_base, the
+//           slots of the coming steps (left alone while no counts are in place)
+//   kSrc 2  the room for the position histogram in bin_cursor: bin_base
+// The layout is by far cheaper than the sort it replaces: once in
+// kLayoutSteps steps, and no record moves.  The sorted read-outs
+// (k_sort_records) serve fields and saved images; k_unsort_records puts a
+// loaded image's records back into slots.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ int block_sum_256(int v, int* red) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -30,33 +36,51 @@ __device__ __forceinline__ int block_sum_256(int v, int* red) {
   return r;
 }
 
-__global__ void __launch_bounds__(256) k_scan_sums(const __grid_constant__ WorldDev w, int off) {
-  __shared__ int red[9];
-  const int* counts = step_counts(w, *w.t + off);
-  const int base = (int)blockIdx.x * kScanChunk;
-  const int end = min(base + kScanChunk, w.n_bins);
-  int s = 0;
-  for (int k = base + threadIdx.x; k < end; k += blockDim.x) s += counts[k];
-  s = block_sum_256(s, red);
-  if (threadIdx.x == 0) w.chunk_sum[blockIdx.x] = s;
+template <int kSrc>
+__device__ __forceinline__ int scan_value(const WorldDev& w, const int* counts, int k) {
+  if (kSrc == 0) return counts[k];
+  return slot_room(kSrc == 1 ? counts[k] : w.bin_cursor[k]);
 }
 
-// The offsets, and in bin_cursor each bin's first place after its slots'
-// records (where k_sort_records appends the beads that found them full).
-__global__ void __launch_bounds__(256) k_scan_apply(const __grid_constant__ WorldDev w, int off) {
+template <int kSrc>
+__global__ void __launch_bounds__(256) k_scan_sums(const WorldDev* __restrict__ worlds,
+                                                   const int2* __restrict__ items, int off) {
+  pdl_trigger();
+  pdl_wait();
+  __shared__ int red[9];
+  const int2 it = items[blockIdx.x];
+  const WorldDev& w = worlds[it.x];
+  if (kSrc == 1 && !*w.cnt_valid) return;
+  const int* counts = step_counts(w, *w.t + off);
+  const int base = it.y * kScanChunk;
+  const int end = min(base + kScanChunk, w.n_bins);
+  int s = 0;
+  for (int k = base + threadIdx.x; k < end; k += blockDim.x) s += scan_value<kSrc>(w, counts, k);
+  s = block_sum_256(s, red);
+  if (threadIdx.x == 0) w.chunk_sum[it.y] = s;
+}
+
+template <int kSrc>
+__global__ void __launch_bounds__(256) k_scan_apply(const WorldDev* __restrict__ worlds,
+                                                    const int2* __restrict__ items, int off) {
+  pdl_trigger();
+  pdl_wait();
   __shared__ int red[9];
   __shared__ int warp_tot[8];
+  const int2 it = items[blockIdx.x];
+  const WorldDev& w = worlds[it.x];
+  if (kSrc == 1 && !*w.cnt_valid) return;
   const int* counts = step_counts(w, *w.t + off);
   int pre = 0;
-  for (int k = threadIdx.x; k < (int)blockIdx.x; k += blockDim.x) pre += w.chunk_sum[k];
+  for (int k = threadIdx.x; k < it.y; k += blockDim.x) pre += w.chunk_sum[k];
   pre = block_sum_256(pre, red);
   const int n = w.n_bins;
-  const int base = (int)blockIdx.x * kScanChunk + threadIdx.x * 4;
+  const int base = it.y * kScanChunk + threadIdx.x * 4;
   int v[4];
   int tsum = 0;
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
-    v[j] = base + j < n ? counts[base + j] : 0;
+    v[j] = base + j < n ? scan_value<kSrc>(w, counts, base + j) : 0;
     tsum += v[j];
   }
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -71,16 +95,28 @@ __global__ void __launch_bounds__(256) k_scan_apply(const __grid_constant__ Worl
   int wbase = 0;
   for (int k = 0; k < wid; ++k) wbase += warp_tot[k];
   int run = pre + wbase + incl - tsum;
+  int* out = kSrc == 0 ? w.bin_off : w.bin_base;
+  // (slot numbers stay below slot_end whatever the counts)
+  auto within = [&](int r) { return kSrc == 0 || (unsigned)r <= (unsigned)w.slot_end ? r : w.slot_end; };
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     const int k = base + j;
     if (k < n) {
-      w.bin_off[k] = run;
-      w.bin_cursor[k] = run + min(v[j], w.slot_cap);
+      out[k] = within(run);
+      if (kSrc == 0) w.bin_cursor[k] = run + min(v[j], w.bin_base[k + 1] - w.bin_base[k]);
       run += v[j];
-      if (k == n - 1) w.bin_off[n] = run;
+      if (k == n - 1) out[n] = within(run);
     }
   }
+}
+
+// Histogram of the beads' bins from their positions, into bin_cursor (zeroed
+// before).
+__global__ void __launch_bounds__(256) k_bin_histogram(const __grid_constant__ WorldDev w) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= w.N) return;
+  const float4 p = w.pos[i];
+  atomicAdd(&w.bin_cursor[(cell_y(p) / kBin) * w.nbx + cell_x(p) / kBin], 1);
 }
 
 // One warp per bin copies its slots; the last block appends the beads that
@@ -90,7 +126,7 @@ __global__ void __launch_bounds__(256) k_sort_records(const __grid_constant__ Wo
   if (blockIdx.x == gridDim.x - 1) {
     const int n = counts[w.n_bins];
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
-      const int src = w.n_bins * w.slot_cap + k;
+      const int src = w.slot_end + k;
       const float4 p = w.bpos[src];
       const int bin = (cell_y(p) / kBin) * w.nbx + cell_x(p) / kBin;
       const int dst = atomicAdd(&w.bin_cursor[bin], 1);
@@ -101,10 +137,10 @@ __global__ void __launch_bounds__(256) k_sort_records(const __grid_constant__ Wo
   }
   const int bin = (int)blockIdx.x * 8 + (threadIdx.x >> 5);
   if (bin >= w.n_bins) return;
-  const int n = min(counts[bin], w.slot_cap), dst = w.bin_off[bin];
+  const int lo = w.bin_base[bin], n = min(counts[bin], w.bin_base[bin + 1] - lo), dst = w.bin_off[bin];
   for (int k = threadIdx.x & 31; k < n; k += 32) {
-    w.spos[dst + k] = w.bpos[bin * w.slot_cap + k];
-    w.srec[dst + k] = w.brec[bin * w.slot_cap + k];
+    w.spos[dst + k] = w.bpos[lo + k];
+    w.srec[dst + k] = w.brec[lo + k];
   }
 }
 
@@ -116,7 +152,9 @@ __global__ void __launch_bounds__(256) k_unsort_records(const __grid_constant__ 
   const float4 p = w.spos[k];
   const int bin = (cell_y(p) / kBin) * w.nbx + cell_x(p) / kBin;
   const int at = atomicAdd(&counts[bin], 1);
-  const int slot = at < w.slot_cap ? bin * w.slot_cap + at : w.n_bins * w.slot_cap + atomicAdd(&counts[w.n_bins], 1);
+  const int lo = w.bin_base[bin];
+  const int slot = lo + at < w.bin_base[bin + 1] ? lo + at : w.slot_end + atomicAdd(&counts[w.n_bins], 1);
+  if (k == 0) *w.cnt_valid = 1;
   const float4 rec = w.srec[k];
   w.bpos[slot] = p;
   w.brec[slot] = rec;
@@ -158,11 +196,25 @@ __global__ void __launch_bounds__(kCellChunk) k_lbm(const WorldDev* __restrict__
 // ---------------------------------------------------------------------------
 // Launchers and the step sequence.
 // ---------------------------------------------------------------------------
-void launch_sorted_offsets(const Plan& p, cudaStream_t s, int off) {
-  const WorldDev& w = p.h_world0;
-  if (w.n_chunks > 1) k_scan_sums<<<w.n_chunks, 256, 0, s>>>(w, off);
-  k_scan_apply<<<w.n_chunks, 256, 0, s>>>(w, off);
+template <int kSrc>
+static void launch_scan(const Plan& p, cudaStream_t s, int off) {
+  if (!p.n_scan_items) return;
+  const WorldDev* ws = p.d_worlds;
+  const int2* items = p.d_scan_items;
+  if (!p.one_chunk) launch_pdl(k_scan_sums<kSrc>, p.n_scan_items, 256, 0, s, ws, items, off);
+  launch_pdl(k_scan_apply<kSrc>, p.n_scan_items, 256, 0, s, ws, items, off);
 }
+
+void launch_slot_layout(const Plan& p, cudaStream_t s) { launch_scan<1>(p, s, -1); }
+
+void launch_slot_layout_from_positions(const Plan& p, cudaStream_t s) {
+  const WorldDev& w = p.h_world0;
+  cudaMemsetAsync(w.bin_cursor, 0, (size_t)w.n_bins * sizeof(int), s);
+  if (w.N) k_bin_histogram<<<(w.N + 255) / 256, 256, 0, s>>>(w);
+  launch_scan<2>(p, s, 0);
+}
+
+void launch_sorted_offsets(const Plan& p, cudaStream_t s, int off) { launch_scan<0>(p, s, off); }
 
 void launch_sorted_records(const Plan& p, cudaStream_t s, int off) {
   const WorldDev& w = p.h_world0;

@@ -37,7 +37,7 @@ namespace {
 // lane of the warp calls.
 __device__ __forceinline__ void mdf_bin_bead(const WorldDev& w, int* counts, bool valid, int i, const float4 p) {
   const int bin = bead_bin_of(p, w.nbx);
-  const BinClaim c = bin_claim(counts, valid, bin);
+  const BinClaim c = bin_claim(w, counts, valid, bin);
   if (valid) {
     w.bead_bin[i] = bin;
     w.fel[i] = make_float2(0.0f, 0.0f);

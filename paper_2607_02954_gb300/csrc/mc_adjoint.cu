@@ -367,6 +367,7 @@ mc_status mc_rollout_forward_stored(mc_world* w, int n_steps, void* stream) {
     for (int q = 0; q < n_steps; ++q) {
       st = mdf_recorded_step(w, seg, ss, q, n_steps, t0, s);
       if (st != MC_OK) return st;
+      if (q % mc::kLayoutSteps == 0) mc::launch_slot_layout(w->plan, s);
     }
     w->t += n_steps;
     st = save_state(h, (int)(w->t & 1), tape + sl.bytes, sl, s);   // the final state
@@ -385,6 +386,7 @@ mc_status mc_rollout_forward_stored(mc_world* w, int n_steps, void* stream) {
     p.d_worlds = d_desc + q;
     p.h_world0 = desc[q];
     run_recorded_step(p, s);
+    if (q % mc::kLayoutSteps == 0) mc::launch_slot_layout(w->plan, s);
   }
   MC_ACUDA(cudaGetLastError());
   w->t += n_steps;
@@ -537,6 +539,8 @@ mc_status sweep(mc_world* w, mc::AdjDev a, const mc::AdjMdf* mdf, float* const a
       } else {
         run_recorded_step(step_plan(b, q, (int)((tk + q) & 1), false), rs);   // fields straight into the record
       }
+      // the slots follow the beads from the segment's first step on
+      if (q % mc::kLayoutSteps == 0) mc::launch_slot_layout(w->plan, rs);
     }
     MC_ACUDA(cudaGetLastError());
     return MC_OK;

@@ -155,7 +155,7 @@ mc_status build_plan(mc_world* const* ws, int n, cudaStream_t s, Plan& out) {
   p.max_mdf = 0;
   p.any_ext = false;
   std::vector<int4> fil_long, fil;
-  std::vector<int2> bead, tile, cell;
+  std::vector<int2> bead, tile, cell, scan;
   std::vector<WorldDev> table(n);
   for (int k = 0; k < n; ++k) {
     const mc_world* w = ws[k];
@@ -174,6 +174,8 @@ mc_status build_plan(mc_world* const* ws, int n, cudaStream_t s, Plan& out) {
     for (int b = 0; b < nb; b += mc::kBeadChunk) bead.push_back(make_int2(k, b));
     for (int ty = 0; ty < w->h.nty; ++ty)   // tile items carry (tx, ty) packed: tx | ty << 16
       for (int tx = 0; tx < w->h.ntx; ++tx) tile.push_back(make_int2(k, tx | (ty << 16)));
+    p.one_chunk = p.one_chunk && w->h.n_chunks <= 1;
+    for (int c = 0; c < w->h.n_chunks; ++c) scan.push_back(make_int2(k, c));
     const int HW = w->h.H * w->h.W;
     for (int c = 0; c < HW; c += mc::kCellChunk) cell.push_back(make_int2(k, c));
   }
@@ -187,6 +189,7 @@ mc_status build_plan(mc_world* const* ws, int n, cudaStream_t s, Plan& out) {
   const size_t o_b = L.take<int2>(bead.size());
   const size_t o_t = L.take<int2>(tile.size());
   const size_t o_c = L.take<int2>(cell.size());
+  const size_t o_s = L.take<int2>(scan.size());
   const size_t o_bar = L.take<unsigned>(4);
   std::vector<char> host(L.off);
   std::memcpy(host.data() + o_w, table.data(), n * sizeof(WorldDev));
@@ -194,6 +197,7 @@ mc_status build_plan(mc_world* const* ws, int n, cudaStream_t s, Plan& out) {
   std::memcpy(host.data() + o_b, bead.data(), bead.size() * sizeof(int2));
   if (!tile.empty()) std::memcpy(host.data() + o_t, tile.data(), tile.size() * sizeof(int2));
   std::memcpy(host.data() + o_c, cell.data(), cell.size() * sizeof(int2));
+  std::memcpy(host.data() + o_s, scan.data(), scan.size() * sizeof(int2));
   cudaError_t e = cudaMallocAsync(&p.d_mem, L.off, s);
   if (e != cudaSuccess) return fail(MC_ERR_OOM, std::string("plan allocation: ") + cudaGetErrorString(e));
   e = cudaMemcpyAsync(p.d_mem, host.data(), L.off, cudaMemcpyHostToDevice, s);
@@ -204,11 +208,14 @@ mc_status build_plan(mc_world* const* ws, int n, cudaStream_t s, Plan& out) {
   p.d_bead_items = at<int2>(p.d_mem, o_b);
   p.d_tile_items = at<int2>(p.d_mem, o_t);
   p.d_cell_items = at<int2>(p.d_mem, o_c);
+  p.d_scan_items = at<int2>(p.d_mem, o_s);
   p.d_persist_bar = at<unsigned>(p.d_mem, o_bar);
   p.n_fil_items = (int)fil.size();
   p.n_bead_items = (int)bead.size();
   p.n_tile_items = (int)tile.size();
   p.n_cell_items = (int)cell.size();
+  p.n_scan_items = (int)scan.size();
+  p.since_layout = mc::kLayoutSteps;   // the worlds' slots may be old: laid out before the plan's first step
   if (n == 1) p.h_world0 = table[0];
   out = p;
   return MC_OK;
@@ -222,10 +229,23 @@ cudaStream_t capture_stream() {
   return cs;
 }
 
+// Lays the slots out before a run of n steps outside the graph when the plan
+// has run kLayoutSteps steps on the present layout.
+void lay_out_slots(Plan& p, int n, cudaStream_t s) {
+  if (p.since_layout >= mc::kLayoutSteps) {
+    mc::launch_slot_layout(p, s);
+    p.since_layout = 0;
+  }
+  p.since_layout += n;
+}
+
 mc_status run_steps(Plan& p, int n, cudaStream_t s) {
   if (p.cfg.persistent && mc::persistent_supported(p)) {
     // one cooperative launch for the whole run
-    if (n > 0) MC_CUDA(mc::launch_persistent(p, n, s));
+    if (n > 0) {
+      lay_out_slots(p, n, s);
+      MC_CUDA(mc::launch_persistent(p, n, s));
+    }
     MC_CUDA(cudaGetLastError());
     return MC_OK;
   }
@@ -233,6 +253,7 @@ mc_status run_steps(Plan& p, int n, cudaStream_t s) {
     if (!p.graph) {
       cudaStream_t cs = capture_stream();
       MC_CUDA(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
+      mc::launch_slot_layout(p, cs);
       mc::enqueue_steps(p, kGraphSteps, cs);
       cudaGraph_t g = nullptr;
       MC_CUDA(cudaStreamEndCapture(cs, &g));
@@ -244,9 +265,13 @@ mc_status run_steps(Plan& p, int n, cudaStream_t s) {
     while (n >= p.graph_steps) {
       MC_CUDA(cudaGraphLaunch(p.graph, s));
       n -= p.graph_steps;
+      p.since_layout = p.graph_steps;
     }
   }
-  if (n > 0) mc::enqueue_steps(p, n, s);
+  if (n > 0) {
+    lay_out_slots(p, n, s);
+    mc::enqueue_steps(p, n, s);
+  }
   MC_CUDA(cudaGetLastError());
   return MC_OK;
 }
@@ -320,12 +345,11 @@ void world_sizes(WorldDev& h, int H, int W, int n_fil, int N) {
   h.nty = (H + kTile - 1) / kTile;
   h.n_tiles = h.ntx * h.nty;
   h.n_chunks = (h.n_bins + kScanChunk - 1) / kScanChunk;
-  // slots of a bin: twice the mean count and some more, at least 32 (beads
-  // of a chain are about a cell apart, so a chain crossing a bin leaves 8 to
-  // 11 in it); slot numbers stay below 2^31
-  const long long mean = ((long long)N + h.n_bins - 1) / h.n_bins;
-  const long long room = (0x7fffffffLL - N) / h.n_bins;
-  h.slot_cap = (int)std::min(std::max(32LL, (2 * mean + 24 + 7) & ~7LL), room);
+  // the most that slot_room can ask for over all bins; no slots where the
+  // numbers would pass 2^31 (some 9e8 beads: all of them then share the list
+  // of beads beyond their bin's slots)
+  const long long most = (long long)N + N / 4 + 24LL * h.n_bins;
+  h.slot_end = most + N <= 0x7fffffffLL ? (int)most : 0;
 }
 
 // Places every array of a world inside one arena (256-byte aligned slices).
@@ -377,8 +401,10 @@ ArenaSize world_layout(WorldDev& h, void* A) {
   ArenaSize sz;
   sz.image = L.off;
   const size_t o_cnt = L.take<int>(2 * ((size_t)h.n_bins + 1));
+  const size_t o_cv = L.take<int>(1);
   sz.zero = L.off;
-  const size_t slots = (size_t)h.n_bins * h.slot_cap + N;
+  const size_t o_bb2 = L.take<int>((size_t)h.n_bins + 1);
+  const size_t slots = (size_t)h.slot_end + N;
   const size_t o_bp = L.take<float4>(slots);
   const size_t o_br = L.take<float4>(slots);
   const size_t o_ls = L.take<int>(h.layers == 2 ? N : 0);
@@ -422,6 +448,8 @@ ArenaSize world_layout(WorldDev& h, void* A) {
   h.mrho = df ? at<float>(A, o_mr) : nullptr;
   h.bead_slot = df ? at<int>(A, o_bs) : h.layers == 2 ? at<int>(A, o_ls) : nullptr;
   h.bin_cnt = at<int>(A, o_cnt);
+  h.cnt_valid = at<int>(A, o_cv);
+  h.bin_base = at<int>(A, o_bb2);
   h.bpos = at<float4>(A, o_bp);
   h.brec = at<float4>(A, o_br);
   h.u2 = df ? at<float2>(A, o_u2) : nullptr;
@@ -671,6 +699,7 @@ mc_status mc_world_create(const mc_world_desc* d, void* stream, mc_world** out) 
   st = build_plan(&self, 1, s, w->plan);
   if (st != MC_OK) return fail_free(st);
 #undef MC_CUDA_W
+  mc::launch_slot_layout_from_positions(w->plan, s);
   *out = w;
   return MC_OK;
 }
@@ -797,6 +826,7 @@ mc_status mc_world_load(const void* buf, size_t bytes, void* stream, mc_world** 
     delete w;
     return st;
   }
+  mc::launch_slot_layout_from_positions(w->plan, w->stream);
   mc::launch_slots_from_sorted(w->plan, w->stream);
   *out = w;
   return MC_OK;

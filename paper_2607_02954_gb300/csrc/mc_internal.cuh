@@ -64,15 +64,20 @@ struct WorldDev {
   int* chunk_sum;         // [n_chunks] sorted read-out
   float4* spos;           // [N] sorted read-out: positions in bin order
   float4* srec;           // [N] sorted read-out: the records in bin order
-  // The step's binned beads: bin b holds bin_cnt[par][b] beads, the first
-  // slot_cap of them in slots b slot_cap .. of bpos and brec; beads beyond
-  // that (bin_cnt[par][n_bins] of them in all) follow at n_bins slot_cap.
+  // The step's binned beads: bin b holds bin_cnt[par][b] beads, as many of
+  // them as fit in its slots bin_base[b] .. bin_base[b + 1] of bpos and brec;
+  // the others (bin_cnt[par][n_bins] of them in all) follow at slot_end.
   // The counts alternate by step parity par: the deposit of a step zeroes
-  // the other parity's for the next step.
-  int slot_cap;
+  // the other parity's for the next step.  The slots are laid out again every
+  // few steps, between steps, from the last step's counts (slot_room), and at
+  // first from the initial positions: beads move by a fraction of a cell a
+  // step, so hardly any bin outgrows its slots in between.
+  int slot_end;
+  int* bin_base;          // [n_bins + 1]
   int* bin_cnt;           // [2][n_bins + 1], the last entry of each: beads that found their bin's slots full
-  float4* bpos;           // [n_bins slot_cap + N] positions
-  float4* brec;           // [n_bins slot_cap + N] F_el (x, y), bead id (int bits), 0
+  int* cnt_valid;         // 1: the counts of step t - 1 are in place
+  float4* bpos;           // [slot_end + N] positions
+  float4* brec;           // [slot_end + N] F_el (x, y), bead id (int bits), 0
   float* g[2];            // [9 * H * W] post-collision population deviations (ping-pong)
   float2* F;              // [H * W]
   float2* u;              // [H * W]
@@ -91,7 +96,7 @@ struct WorldDev {
   float* mrho;            // [H * W] fluid density of the step (ib == 1)
   int* bead_slot;         // [N] slot of each bead in bpos and brec (ib == 1 or layers == 2, else nullptr)
   float2* u2;             // [H * W] second velocity buffer of the MDF passes (ib == 1, see mdf_u)
-  float2* sus;            // [n_bins slot_cap + N] U_s by slot (ib == 1)
+  float2* sus;            // [slot_end + N] U_s by slot (ib == 1)
   float2* nrm;            // [N] filament unit normal at each bead (layers == 2)
   unsigned long long* facc;  // [2 H W] fixed-point spread of the layer points (layers == 2)
   const float4* ldrive;   // [E] (L0, amp, freq, phase) rest-length drive, or nullptr (static L_rest)
@@ -200,12 +205,15 @@ struct Plan {
   bool any_ext = false;          // some world has two layers, observables, a rest-length drive or direct forcing
   long long beads = 0;           // of all worlds
   int n_long = 0;                // filaments of more than 64 beads (first in d_fil_items)
-  int n_fil_items = 0, n_bead_items = 0, n_tile_items = 0, n_cell_items = 0;
+  int n_fil_items = 0, n_bead_items = 0, n_tile_items = 0, n_cell_items = 0, n_scan_items = 0;
   WorldDev* d_worlds = nullptr;  // [n_worlds]
   int4* d_fil_items = nullptr;   // (world, filament, first bead, beads)
   int2* d_bead_items = nullptr;  // (world, first bead)
   int2* d_tile_items = nullptr;  // (world, tx | ty << 16), row-major over the tiles
   int2* d_cell_items = nullptr;  // (world, first cell)
+  int2* d_scan_items = nullptr;  // (world, scan block)
+  bool one_chunk = true;         // every world's bins fit one scan block (no block sums to add)
+  int since_layout = 0;          // steps run since the slots were laid out
   void* d_mem = nullptr;
   unsigned* d_persist_bar = nullptr;   // [3] barrier words and status of the persistent step
   cudaGraphExec_t graph = nullptr;
@@ -226,6 +234,11 @@ void steric_setup(int sms);   // host set-up of the tile kernels (k_steric.cu), 
 // last advance: its kernels take `off`, the step's distance from the counter
 // (0 in a step of its own, -1 to re-run a stage of the completed step).
 void launch_pbd(const Plan& p, cudaStream_t s);
+// the slots of every world of the plan laid out from the last step's counts
+void launch_slot_layout(const Plan& p, cudaStream_t s);
+// ... and from the positions (single-world plans: a new or loaded world)
+void launch_slot_layout_from_positions(const Plan& p, cudaStream_t s);
+constexpr int kLayoutSteps = 16;   // at most so many steps between layouts
 // sorted read-outs (off as above): the bin offsets, then the records in bin order
 void launch_sorted_offsets(const Plan& p, cudaStream_t s, int off);
 void launch_sorted_records(const Plan& p, cudaStream_t s, int off);
@@ -521,6 +534,10 @@ __device__ __forceinline__ void obs_add_warp(unsigned long long* acc, long long 
 __host__ __device__ __forceinline__ float2* mdf_u(const WorldDev& w, int k) {
   return ((k + w.mdf_iters) & 1) ? w.u2 : w.u;
 }
+
+// Slots for a bin that holds n beads (all of them together: at most
+// slot_end = 5 N / 4 + 24 n_bins).
+__device__ __forceinline__ int slot_room(int n) { return (n + n / 4 + 16 + 7) & ~7; }
 
 // A world's bin counts of step t (see WorldDev).
 __device__ __forceinline__ int* step_counts(const WorldDev& w, long long t) {

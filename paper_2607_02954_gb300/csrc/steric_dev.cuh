@@ -67,21 +67,24 @@ __device__ void build_segments(const WorldDev& w, int off, int x_lo, int x_hi, i
   const int* c0 = kBoth ? w.bin_cnt : step_counts(w, t);
   const int* c1 = w.bin_cnt + (w.n_bins + 1);
   const int lane = threadIdx.x & 31;
-  const int nbx = w.nbx, nby = w.nby, cap = w.slot_cap;
+  const int nbx = w.nbx, nby = w.nby;
+  const int* base = w.bin_base;
   int bx0 = floor_div(x_lo, kBin), bx1 = floor_div(x_hi, kBin);
   int by0 = floor_div(y_lo, kBin), by1 = floor_div(y_hi, kBin);
   if (bx1 - bx0 + 1 >= nbx) { bx0 = 0; bx1 = nbx - 1; }
   if (by1 - by0 + 1 >= nby) { by0 = 0; by1 = nby - 1; }
   const int ncol = bx1 - bx0 + 1, nrow = by1 - by0 + 1;
   const int cc = lane & 7, rr = lane >> 3;
-  int bin[2] = {0, 0}, n[2] = {0, 0}, m[2] = {0, 0};
+  int lo[2] = {0, 0}, hi[2] = {0, 0}, n[2] = {0, 0}, m[2] = {0, 0};
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     const int r = rr + 4 * h;
     if (cc < ncol && r < nrow) {
-      bin[h] = wrap_once(by0 + r, nby) * nbx + wrap_once(bx0 + cc, nbx);
-      n[h] = c0[bin[h]];
-      if (kBoth) m[h] = c1[bin[h]];
+      const int bin = wrap_once(by0 + r, nby) * nbx + wrap_once(bx0 + cc, nbx);
+      lo[h] = base[bin];
+      hi[h] = base[bin + 1];
+      n[h] = c0[bin];
+      if (kBoth) m[h] = c1[bin];
     }
   }
   int over = c0[w.n_bins];
@@ -92,7 +95,7 @@ __device__ void build_segments(const WorldDev& w, int off, int x_lo, int x_hi, i
     over = over1;
   }
   int covered = n[0] + n[1], most = max(n[0], n[1]);
-  int incl0 = min(n[0], cap), incl1 = min(n[1], cap);
+  int incl0 = min(n[0], hi[0] - lo[0]), incl1 = min(n[1], hi[1] - lo[1]);
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const int y0 = __shfl_up_sync(0xffffffffu, incl0, o), y1 = __shfl_up_sync(0xffffffffu, incl1, o);
@@ -102,8 +105,8 @@ __device__ void build_segments(const WorldDev& w, int off, int x_lo, int x_hi, i
     }
   }
   incl1 += __shfl_sync(0xffffffffu, incl0, 31);
-  sg.start[lane] = bin[0] * cap;
-  sg.start[lane + 32] = bin[1] * cap;
+  sg.start[lane] = lo[0];
+  sg.start[lane + 32] = lo[1];
   sg.pre[lane + 1] = incl0;
   sg.pre[lane + 33] = incl1;
   for (int o = 16; o > 0; o >>= 1) {
@@ -112,7 +115,7 @@ __device__ void build_segments(const WorldDev& w, int off, int x_lo, int x_hi, i
   }
   if (lane == 31) {
     sg.pre[0] = 0;
-    sg.start[kSegs - 1] = w.n_bins * cap;
+    sg.start[kSegs - 1] = w.slot_end;
     sg.pre[kSegs] = incl1 + over;
     sg.covered = covered;
     sg.most = most;
@@ -395,6 +398,7 @@ __device__ __forceinline__ void deposit_x_body(const WorldDev* __restrict__ worl
     if (lane < 16 && bx < w.nbx && by < w.nby) next[by * w.nbx + bx] = 0;
     if (lane == 16 && d.tile == 0) {
       next[w.n_bins] = 0;
+      if (off >= 0) *w.cnt_valid = 1;   // (not when a completed step's stage is re-run)
       w.fel_max[(t + 1) & 1] = 0u;
     }
   }
