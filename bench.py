@@ -45,33 +45,29 @@ if ROOT not in sys.path:
 # the stages one step runs, with their mc_step_stage ids
 STAGES = [("pbd", 0), ("deposit_x", 3), ("force_lbm", 7), ("interp_advance", 6)]
 KERNELS_PER_STEP = 4
-GRAPH_STEPS = 16   # mc_step replays graphs of 16 steps: PBD, then 15 x (previous advance + PBD), 16 x (deposit,
-                   # force + LBM), and the last advance = 49 kernels
+GRAPH_STEPS = 16   # mc_step replays graphs of 16 steps
 
 
-def mdf_launches(steps: int, m: int) -> int:
-    """Kernels of a run of direct-forcing steps, in 16-step graphs and a leftover run: per step bins (with
-    the previous advance), deposit, steric spread + moments, predicted PBD and m passes (one tile kernel
-    each, the last with the LBM), and a run's last advance; without passes the unfused sequence (PBD, which
-    returns, bins, deposit, spread, moments, predicted PBD, LBM, advance)."""
+def layout_kernels(specs) -> int:
+    """Kernels of a layout of the bins' slots: one when every world's bins fit one 1024-bin scan block, else
+    two.  Each 16-step graph begins with a layout, and so does the leftover run after graphs."""
+    return 1 if all((sp.H // 8) * (sp.W // 8) <= 1024 for sp in specs) else 2
+
+
+def run_launches(steps: int, cfg: dict, specs, m=None) -> int:
+    """Kernels of a run of `steps` steps: 16-step graphs (a layout, then per step PBD or the previous advance
+    + PBD, deposit, force + LBM, and a last advance), then the leftover run likewise; with m >= 1
+    direct-forcing passes a step is bins (with the previous advance), deposit, steric spread + moments,
+    predicted PBD and m passes (one tile kernel each, the last with the LBM), without passes the unfused
+    sequence of eight.  The persistent step is one cooperative launch per run."""
+    lay = layout_kernels(specs)
+    if cfg.get("persistent"):
+        return 1 + lay
+    r = steps % GRAPH_STEPS
+    runs = steps // GRAPH_STEPS + (1 if r else 0)
     if m == 0:
-        return 8 * steps
-    r = steps % GRAPH_STEPS
-    return steps * (4 + m) + steps // GRAPH_STEPS + (1 if r else 0)
-
-
-def graph_launches(steps: int) -> int:
-    """Kernels of a run of `steps` steps: 16-step graphs, then the leftover r steps in the same fused
-    order (r PBDs, r x (deposit, force + LBM), one advance)."""
-    per = 3   # PBD, deposit, force + LBM per step, plus the last advance
-    r = steps % GRAPH_STEPS
-    return (steps // GRAPH_STEPS) * (GRAPH_STEPS * per + 1) + (per * r + 1 if r else 0)
-
-
-def run_launches(steps: int, cfg: dict) -> int:
-    """Kernels of a run of `steps` steps in a launch configuration: the persistent step is one cooperative
-    launch per run; otherwise the graph sequence above."""
-    return 1 if cfg.get("persistent") else graph_launches(steps)
+        return 8 * steps + runs * lay
+    return (3 if m is None else 4 + m) * steps + runs * (1 + lay)
 
 
 # k_force_lbm, the dominant kernel: per cell read f 36 + rho_x 4, write f' 36 + u 8;
@@ -424,7 +420,7 @@ def bench_batched(args, steps=None):
                                 "description": "single direct steps, world after world"},
             "batched_over_plain_graph": batched / plain_graph, "batched_over_plain": batched / plain,
             "launch_config": tuned, "config_ms_per_step": configs,
-            "gpu_launches": run_launches(steps, tuned),
+            "gpu_launches": run_launches(steps, tuned, specs),
             "clocks": clk.summary()}
 
 
@@ -710,8 +706,7 @@ def main():
                    "l2": "state 1.8 GB > L2: no flush needed" if C >= 4096 * 4096 else "state may fit in L2; per-step timing includes no flush"},
         "e2e": {"value": e2e_val, "unit": "particle-steps/s", "steps": e2e_steps,
                 "h2d_bytes_per_step": h2d / e2e_steps, "d2h_bytes_per_step": d2h / e2e_steps},
-        "gpu_launches": (mdf_launches(args.steps, args.mdf_iters) if mdf
-                         else run_launches(args.steps, tuned)),
+        "gpu_launches": run_launches(args.steps, tuned, [spec], args.mdf_iters if mdf else None),
         "launch_config": tuned,
         "roofline": None if mdf else {
             "bound": "hbm", "kernel": "k_force_lbm", "achieved": top_gbs, "peak": hbm_peak, "unit": "GB/s",

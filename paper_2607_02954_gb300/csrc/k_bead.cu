@@ -93,42 +93,65 @@ __constant__ int kCy[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
 // The stored state is post-collision (the LBM pulls on read).  Given
 // pre-collision populations f0, store g_i(c) = f0_i(c + c_i) so that pulling
 // g_i(c - c_i) returns f0_i(c).
-__global__ void k_unstream_in(const float* __restrict__ f0, float* __restrict__ g, int H, int W) {
+// (A thread moves a cell's nine populations: a thread each, found by division,
+// took 595 us for 4096^2; 173 us so, 1.2 GB.)
+__global__ void __launch_bounds__(256) k_unstream_in(const float* __restrict__ f0, float* __restrict__ g, int H, int W) {
   pdl_trigger();
   pdl_wait();
-  const int HW = H * W;
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= 9 * HW) return;
-  const int i = idx / HW, c = idx - i * HW;
-  const int y = c / W, x = c - y * W;
-  const int sx = wrap_once(x + kCx[i], W), sy = wrap_once(y + kCy[i], H);
-  g[idx] = f0[i * HW + sy * W + sx];
+  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
+  if (x >= W) return;
+  const size_t HW = (size_t)H * W, c = (size_t)y * W + x;
+#pragma unroll
+  for (int i = 0; i < 9; ++i)
+    g[i * HW + c] = f0[i * HW + (size_t)wrap_once(y + kCy[i], H) * W + wrap_once(x + kCx[i], W)];
 }
 
-__global__ void k_stream_out(const float* __restrict__ g, float* __restrict__ out, int H, int W) {
+__global__ void __launch_bounds__(256) k_stream_out(const float* __restrict__ g, float* __restrict__ out, int H, int W) {
   pdl_trigger();
   pdl_wait();
-  const int HW = H * W;
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= 9 * HW) return;
-  const int i = idx / HW, c = idx - i * HW;
-  const int y = c / W, x = c - y * W;
-  const int sx = wrap_once(x - kCx[i], W), sy = wrap_once(y - kCy[i], H);
-  out[idx] = g[i * HW + sy * W + sx];
+  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
+  if (x >= W) return;
+  const size_t HW = (size_t)H * W, c = (size_t)y * W + x;
+#pragma unroll
+  for (int i = 0; i < 9; ++i)
+    out[i * HW + c] = g[i * HW + (size_t)wrap_once(y - kCy[i], H) * W + wrap_once(x - kCx[i], W)];
+}
+
+// The bead state into device memory (any pointer may be null; nothing is
+// assumed of their alignment beyond a float's).
+__global__ void __launch_bounds__(256) k_state_out(const float4* __restrict__ pos, const float2* __restrict__ disp_in,
+                                                   const float* __restrict__ theta_in, int N, int E, float* x,
+                                                   float* y, float* theta, float* disp) {
+  pdl_trigger();
+  pdl_wait();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < N) {
+    if (x || y) {
+      const float4 p = pos[i];
+      if (x) x[i] = (float)cell_x(p) + p.x;
+      if (y) y[i] = (float)cell_y(p) + p.y;
+    }
+    if (disp) {
+      const float2 d = disp_in[i];
+      disp[2 * (size_t)i] = d.x;
+      disp[2 * (size_t)i + 1] = d.y;
+    }
+  }
+  if (theta && i < E) theta[i] = theta_in[i];
 }
 
 // A world's set-up from its raw inputs: each position wrapped into the box
 // in double precision (fmod is exact) and split into cell index + fraction,
-// the creation positions, the drive records (theta0, A, freq, phase) and the
-// rest-length drive records (L0 = L_rest, amp, freq, phase).
-__global__ void k_world_init(WorldDev h, const float* x, const float* y, const float* t0, const float* amp,
-                             const float* frq, const float* phs, const float* la, const float* lf,
-                             const float* lp) {
+// the creation positions, the edge angles and rest lengths, the drive records
+// (theta0, A, freq, phase), the rest-length drive records (L0 = L_rest, amp,
+// freq, phase), the filament offsets and the step counter.
+__global__ void __launch_bounds__(256) k_world_init(const __grid_constant__ WorldDev h, const WorldRaw r) {
   pdl_trigger();
   pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) *h.t = r.t0;
   if (i < h.N) {
-    const double xd = fmod((double)x[i], (double)h.W), yd = fmod((double)y[i], (double)h.H);
+    const double xd = fmod((double)r.x[i], (double)h.W), yd = fmod((double)r.y[i], (double)h.H);
     float xw = (float)(xd < 0 ? xd + h.W : xd), yw = (float)(yd < 0 ? yd + h.H : yd);
     if (xw >= (float)h.W) xw = 0.0f;
     if (yw >= (float)h.H) yw = 0.0f;
@@ -136,8 +159,14 @@ __global__ void k_world_init(WorldDev h, const float* x, const float* y, const f
     h.pos0[i] = make_float2(xw, yw);
     h.pos[i] = make_float4(xw - cx, yw - cy, __int_as_float((int)cx), __int_as_float((int)cy));
   }
-  if (i < h.J) const_cast<float4*>(h.drive)[i] = make_float4(t0[i], amp[i], frq[i], phs[i]);
-  if (la && i < h.E) const_cast<float4*>(h.ldrive)[i] = make_float4(h.L_rest[i], la[i], lf[i], lp[i]);
+  if (i < h.J) const_cast<float4*>(h.drive)[i] = make_float4(r.theta0[i], r.amp[i], r.freq[i], r.phase[i]);
+  if (i < h.E) {
+    const float L = r.L_rest[i];
+    h.theta[i] = r.theta[i];
+    const_cast<float*>(h.L_rest)[i] = L;
+    if (r.len_amp) const_cast<float4*>(h.ldrive)[i] = make_float4(L, r.len_amp[i], r.len_freq[i], r.len_phase[i]);
+  }
+  if (r.fil_off && i <= h.n_fil) const_cast<int*>(h.fil_off)[i] = r.fil_off[i];
 }
 
 __global__ void k_positions_out(const float4* __restrict__ pos, int N, float* x, float* y) {
@@ -269,24 +298,27 @@ void launch_interp_advance(const Plan& p, cudaStream_t s, int inc) {
 }
 
 void launch_unstream_in(const float* f0dev, float* g_dst, int H, int W, cudaStream_t s) {
-  const int n = 9 * H * W;
-  k_unstream_in<<<(n + 255) / 256, 256, 0, s>>>(f0dev, g_dst, H, W);
+  const int nt = W < 256 ? (W + 31) & ~31 : 256;
+  k_unstream_in<<<dim3((W + nt - 1) / nt, H), nt, 0, s>>>(f0dev, g_dst, H, W);
 }
 
 void launch_stream_out(const float* g_src, float* out, int H, int W, cudaStream_t s) {
-  const int n = 9 * H * W;
-  k_stream_out<<<(n + 255) / 256, 256, 0, s>>>(g_src, out, H, W);
+  const int nt = W < 256 ? (W + 31) & ~31 : 256;
+  k_stream_out<<<dim3((W + nt - 1) / nt, H), nt, 0, s>>>(g_src, out, H, W);
 }
 
-void launch_world_init(const WorldDev& w, const float* const raw[9], cudaStream_t s) {
-  if (w.N == 0) return;
-  k_world_init<<<(w.N + 255) / 256, 256, 0, s>>>(w, raw[0], raw[1], raw[2], raw[3], raw[4], raw[5], raw[6], raw[7],
-                                                 raw[8]);
+void launch_world_init(const WorldDev& w, const WorldRaw& raw, cudaStream_t s) {
+  k_world_init<<<w.N / 256 + 1, 256, 0, s>>>(w, raw);   // (N >= E, J, 2 n_fil)
 }
 
 void launch_positions_out(const WorldDev& w, float* x, float* y, cudaStream_t s) {
   if (w.N == 0) return;
   k_positions_out<<<(w.N + 255) / 256, 256, 0, s>>>(w.pos, w.N, x, y);
+}
+
+void launch_state_out(const WorldDev& w, float* x, float* y, float* theta, float* disp, cudaStream_t s) {
+  if (w.N == 0 || !(x || y || theta || disp)) return;
+  k_state_out<<<(w.N + 255) / 256, 256, 0, s>>>(w.pos, w.disp, w.theta, w.N, w.E, x, y, theta, disp);
 }
 
 void launch_cells_out(const WorldDev& w, int* cell, cudaStream_t s) {

@@ -119,6 +119,40 @@ __global__ void __launch_bounds__(256) k_bin_histogram(const __grid_constant__ W
   atomicAdd(&w.bin_cursor[(cell_y(p) / kBin) * w.nbx + cell_x(p) / kBin], 1);
 }
 
+// The slots of a small world from its positions, in one block: the histogram
+// in shared memory, then the scan of its room.
+constexpr int kSmallBins = 8192, kSmallBeads = 1 << 15;
+__global__ void __launch_bounds__(1024) k_layout_small(const __grid_constant__ WorldDev w) {
+  __shared__ int hist[kSmallBins];
+  __shared__ int warp_tot[32];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  for (int k = tid; k < w.n_bins; k += 1024) hist[k] = 0;
+  __syncthreads();
+  for (int i = tid; i < w.N; i += 1024) {
+    const float4 p = w.pos[i];
+    atomicAdd(&hist[(cell_y(p) / kBin) * w.nbx + cell_x(p) / kBin], 1);
+  }
+  __syncthreads();
+  const int per = (w.n_bins + 1023) / 1024, lo = min(tid * per, w.n_bins), hi = min(lo + per, w.n_bins);
+  int sum = 0;
+  for (int k = lo; k < hi; ++k) sum += slot_room(hist[k]);
+  int incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  if (lane == 31) warp_tot[wid] = incl;
+  __syncthreads();
+  int run = incl - sum;
+  for (int k = 0; k < wid; ++k) run += warp_tot[k];
+  for (int k = lo; k < hi; ++k) {
+    w.bin_base[k] = run;
+    run += slot_room(hist[k]);
+    if (k == w.n_bins - 1) w.bin_base[k + 1] = run;
+  }
+}
+
 // One warp per bin copies its slots; the last block appends the beads that
 // found their slots full.
 __global__ void __launch_bounds__(256) k_sort_records(const __grid_constant__ WorldDev w, int off) {
@@ -207,8 +241,15 @@ static void launch_scan(const Plan& p, cudaStream_t s, int off) {
 
 void launch_slot_layout(const Plan& p, cudaStream_t s) { launch_scan<1>(p, s, -1); }
 
+bool launch_slot_layout_small(const WorldDev& w, cudaStream_t s) {
+  if (w.n_bins > kSmallBins || w.N > kSmallBeads) return false;
+  k_layout_small<<<1, 1024, 0, s>>>(w);
+  return true;
+}
+
 void launch_slot_layout_from_positions(const Plan& p, cudaStream_t s) {
   const WorldDev& w = p.h_world0;
+  if (launch_slot_layout_small(w, s)) return;
   cudaMemsetAsync(w.bin_cursor, 0, (size_t)w.n_bins * sizeof(int), s);
   if (w.N) k_bin_histogram<<<(w.N + 255) / 256, 256, 0, s>>>(w);
   launch_scan<2>(p, s, 0);

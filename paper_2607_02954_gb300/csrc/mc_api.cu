@@ -530,7 +530,8 @@ mc_status mc_params_default(mc_params* p) {
   return MC_OK;
 }
 
-mc_status mc_world_create(const mc_world_desc* d, void* stream, mc_world** out) {
+namespace {
+mc_status create_world(const mc_world_desc* d, void* stream, mc_world** out, bool bare) {
   if (!d || !out) return fail(MC_ERR_INVALID_ARG, "desc or out is NULL");
   *out = nullptr;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -640,39 +641,69 @@ mc_status mc_world_create(const mc_world_desc* d, void* stream, mc_world** out) 
   auto up = [&](void* dst, const void* src, size_t n, cudaMemcpyKind k) {
     return n ? cudaMemcpyAsync(dst, src, n, k, s) : cudaSuccess;
   };
-  MC_CUDA_W(up((void*)h.fil_off, fo.data(), fo.size() * sizeof(int), cudaMemcpyHostToDevice));
-  MC_CUDA_W(up(h.theta, d->theta, E * sizeof(float), kind));
-  MC_CUDA_W(up((void*)h.L_rest, d->L_rest, E * sizeof(float), kind));
   if (h.has_energy) MC_CUDA_W(up((void*)h.energy, d->energy, HW * sizeof(float), kind));
   // raw per-bead, per-joint and per-edge inputs on the device for the set-up
-  // kernel (positions wrapped and split into cell + fraction, drive records)
-  const float* raw[9] = {d->x, d->y, d->theta0, d->drive_amp, d->drive_freq, d->drive_phase,
-                         n_len == 3 ? d->len_amp : nullptr, n_len == 3 ? d->len_freq : nullptr,
-                         n_len == 3 ? d->len_phase : nullptr};
-  const size_t cnt[9] = {(size_t)N, (size_t)N, (size_t)J, (size_t)J, (size_t)J, (size_t)J,
-                         (size_t)E, (size_t)E, (size_t)E};
-  float* staging = nullptr;
+  // kernel: the caller's device arrays, or one staging buffer for the host
+  // arrays, filled by one copy of a packed image while that is small (a
+  // world's creation is then a handful of calls), array by array else
+  const float* src[11] = {d->x, d->y, d->theta, d->L_rest, d->theta0, d->drive_amp, d->drive_freq, d->drive_phase,
+                          n_len == 3 ? d->len_amp : nullptr, n_len == 3 ? d->len_freq : nullptr,
+                          n_len == 3 ? d->len_phase : nullptr};
+  const size_t cnt[11] = {(size_t)N, (size_t)N, (size_t)E, (size_t)E, (size_t)J, (size_t)J,
+                          (size_t)J, (size_t)J, (size_t)E, (size_t)E, (size_t)E};
+  const float* raw[11];
+  std::copy(src, src + 11, raw);
+  mc::WorldRaw wr{};
+  void* staging = nullptr;
   if (on_host) {
     size_t tot = 0;
-    for (int k = 0; k < 9; ++k) tot += raw[k] ? cnt[k] : 0;
-    if (tot) MC_CUDA_W(cudaMallocAsync((void**)&staging, tot * sizeof(float), s));
+    for (int k = 0; k < 11; ++k) tot += src[k] ? cnt[k] * sizeof(float) : 0;
+    const size_t fo_at = tot;
+    tot += fo.size() * sizeof(int);
+    MC_CUDA_W(cudaMallocAsync(&staging, tot, s));
+    char* dev = static_cast<char*>(staging);
+    constexpr size_t kPack = size_t(1) << 20;
+    std::vector<char> image(tot <= kPack ? tot : 0);
+    cudaError_t e2 = cudaSuccess;
     size_t off = 0;
-    for (int k = 0; k < 9; ++k) {
-      if (!raw[k] || !cnt[k]) continue;
-      const cudaError_t e2 = up(staging + off, raw[k], cnt[k] * sizeof(float), cudaMemcpyHostToDevice);
-      if (e2 != cudaSuccess) {
-        cudaFreeAsync(staging, s);
-        return fail_free(cuda_fail(e2, "input upload"));
-      }
-      raw[k] = staging + off;
-      off += cnt[k];
+    for (int k = 0; k < 11; ++k) {
+      if (!src[k] || !cnt[k]) continue;
+      const size_t bytes = cnt[k] * sizeof(float);
+      if (!image.empty()) std::memcpy(image.data() + off, src[k], bytes);
+      else if (e2 == cudaSuccess) e2 = up(dev + off, src[k], bytes, cudaMemcpyHostToDevice);
+      raw[k] = reinterpret_cast<const float*>(dev + off);
+      off += bytes;
     }
+    if (!image.empty()) {
+      std::memcpy(image.data() + fo_at, fo.data(), fo.size() * sizeof(int));
+      e2 = up(dev, image.data(), tot, cudaMemcpyHostToDevice);   // (pageable: staged before the call returns)
+    } else if (e2 == cudaSuccess) {
+      e2 = up(dev + fo_at, fo.data(), fo.size() * sizeof(int), cudaMemcpyHostToDevice);
+    }
+    wr.fil_off = reinterpret_cast<const int*>(dev + fo_at);
+    if (e2 != cudaSuccess) {
+      cudaFreeAsync(staging, s);
+      return fail_free(cuda_fail(e2, "input upload"));
+    }
+  } else {
+    MC_CUDA_W(up((void*)h.fil_off, fo.data(), fo.size() * sizeof(int), cudaMemcpyHostToDevice));
   }
-  mc::launch_world_init(h, raw, s);
+  wr.x = raw[0];
+  wr.y = raw[1];
+  wr.theta = raw[2];
+  wr.L_rest = raw[3];
+  wr.theta0 = raw[4];
+  wr.amp = raw[5];
+  wr.freq = raw[6];
+  wr.phase = raw[7];
+  wr.len_amp = raw[8];
+  wr.len_freq = raw[9];
+  wr.len_phase = raw[10];
+  wr.t0 = d->t0;
+  mc::launch_world_init(h, wr, s);
   if (staging) cudaFreeAsync(staging, s);
   MC_CUDA_W(cudaGetLastError());
   const long long t0 = d->t0;
-  MC_CUDA_W(up(h.t, &t0, sizeof(long long), cudaMemcpyHostToDevice));
   if (d->f0) {
     // stage f0 in the buffer the first step writes, then store its
     // post-collision image in the buffer the first step reads
@@ -695,13 +726,20 @@ mc_status mc_world_create(const mc_world_desc* d, void* stream, mc_world** out) 
     }
     if (pinned) MC_CUDA_W(cudaStreamSynchronize(s));
   }
-  mc_world* self = w;
-  st = build_plan(&self, 1, s, w->plan);
-  if (st != MC_OK) return fail_free(st);
+  if (!(bare && mc::launch_slot_layout_small(h, s))) {
+    mc_world* self = w;
+    st = build_plan(&self, 1, s, w->plan);
+    if (st != MC_OK) return fail_free(st);
+    mc::launch_slot_layout_from_positions(w->plan, s);
+  }
 #undef MC_CUDA_W
-  mc::launch_slot_layout_from_positions(w->plan, s);
   *out = w;
   return MC_OK;
+}
+}  // namespace
+
+mc_status mc_world_create(const mc_world_desc* d, void* stream, mc_world** out) {
+  return create_world(d, stream, out, false);
 }
 
 // ---- checkpoint / resume --------------------------------------------------
@@ -983,19 +1021,21 @@ mc_status mc_world_get_state(const mc_world* w, float* x, float* y, float* theta
   void* scratch = nullptr;
   if (need) MC_CUDA(cudaMallocAsync(&scratch, need * sizeof(float), s));
   float* sp = static_cast<float*>(scratch);
-  if (x || y) {
-    dx = host ? sp : x;
-    dy = host ? sp + h.N : y;
+  if (!host) {
+    mc::launch_state_out(h, x, y, theta, disp, s);   // one kernel for all of them
+    theta = disp = nullptr;
+  } else if (x || y) {
+    dx = sp;
+    dy = sp + h.N;
     mc::launch_positions_out(h, x ? dx : nullptr, y ? dy : nullptr, s);
-    if (host) {
+    {
       if (x && h.N) MC_CUDA(cudaMemcpyAsync(x, dx, h.N * sizeof(float), cudaMemcpyDeviceToHost, s));
       if (y && h.N) MC_CUDA(cudaMemcpyAsync(y, dy, h.N * sizeof(float), cudaMemcpyDeviceToHost, s));
     }
-    if (host) sp += 2 * (size_t)h.N;
+    sp += 2 * (size_t)h.N;
   }
-  const cudaMemcpyKind dk = host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
-  if (theta && h.E) MC_CUDA(cudaMemcpyAsync(theta, h.theta, h.E * sizeof(float), dk, s));
-  if (disp && h.N) MC_CUDA(cudaMemcpyAsync(disp, h.disp, h.N * sizeof(float2), dk, s));
+  if (theta && h.E) MC_CUDA(cudaMemcpyAsync(theta, h.theta, h.E * sizeof(float), cudaMemcpyDeviceToHost, s));
+  if (disp && h.N) MC_CUDA(cudaMemcpyAsync(disp, h.disp, h.N * sizeof(float2), cudaMemcpyDeviceToHost, s));
   if (fdev) {
     df = host ? sp : fdev;
     mc::launch_stream_out(h.g[w->t & 1], df, h.H, h.W, s);
@@ -1119,6 +1159,10 @@ mc_status mc_world_clear_flags(mc_world* w, void* stream) {
 }  // extern "C"
 
 namespace mc {
+mc_status world_create_bare(const mc_world_desc* d, cudaStream_t s, mc_world** out) {
+  kernel_setup();
+  return create_world(d, s, out, true);
+}
 const WorldDev& world_dev(const mc_world* w) { return w->h; }
 void set_last_error(const char* msg) { g_last_error = msg; }
 }  // namespace mc

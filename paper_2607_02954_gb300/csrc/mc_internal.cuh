@@ -316,10 +316,18 @@ void launch_set_counter(const WorldDev& h, long long t, cudaStream_t s);
 void launch_unstream_in(const float* f0dev, float* g_dst, int H, int W, cudaStream_t s);
 void launch_stream_out(const float* g_src, float* out, int H, int W, cudaStream_t s);
 void launch_positions_out(const WorldDev& w, float* x, float* y, cudaStream_t s);
-// positions, creation positions, drive and rest-length drive records from the
-// raw device arrays x, y [N], theta0, amp, freq, phase [J], len_amp,
-// len_freq, len_phase [E] (the last three may be null)
-void launch_world_init(const WorldDev& w, const float* const raw[9], cudaStream_t s);
+// A world's raw inputs in device memory: x, y [N], theta, L_rest [E], theta0,
+// amp, freq, phase [J], len_amp, len_freq, len_phase [E] (these three may be
+// null), fil_off [n_fil + 1] (may be null: copied separately), the counter.
+struct WorldRaw {
+  const float *x, *y, *theta, *L_rest, *theta0, *amp, *freq, *phase, *len_amp, *len_freq, *len_phase;
+  const int* fil_off;
+  long long t0;
+};
+void launch_world_init(const WorldDev& w, const WorldRaw& raw, cudaStream_t s);
+void launch_state_out(const WorldDev& w, float* x, float* y, float* theta, float* disp, cudaStream_t s);
+// slots from the positions by one block, without a plan; false: too large for it
+bool launch_slot_layout_small(const WorldDev& w, cudaStream_t s);
 void launch_cells_out(const WorldDev& w, int* cell, cudaStream_t s);
 
 // --- world life cycle and plans (host, mc_api.cu) -------------------------
@@ -344,6 +352,10 @@ mc_world* world_clone(const mc_world* w, cudaStream_t s);
 // `automatic`, only for plans large enough to repay the measurement and only
 // when the tuner is enabled.
 mc_status plan_tune(mc_world* const* ws, int n, Plan& p, cudaStream_t s, bool automatic);
+
+// mc_world_create for worlds stepped only within other plans (the server's):
+// small ones get no plan of their own
+mc_status world_create_bare(const mc_world_desc* d, cudaStream_t s, mc_world** out);
 
 // --- host accessors for code outside the ABI translation unit ------------
 const WorldDev& world_dev(const mc_world* w);

@@ -264,7 +264,7 @@ void scheduler(mc_server* s) {
       d.p = r.p;
       d.mem_kind = MC_MEM_HOST;
       mc_world* w = nullptr;
-      const mc_status st = mc_world_create(&d, s->adm_stream, &w);
+      const mc_status st = mc::world_create_bare(&d, s->adm_stream, &w);
       const int64_t t = now_ns();
       if (st != MC_OK) {
         {
