@@ -45,10 +45,11 @@ __device__ __forceinline__ float4 advance_pos(const WorldDev& w, float4 p, float
 // Returns X^{n+1} (X^n when the watchdog fired).
 // d: the bead's displacement so far.
 template <bool kRecord = true>
-__device__ __forceinline__ float4 advance_tail(const WorldDev& w, int i, float4 p, float2 d, float Ux, float Uy) {
+__device__ __forceinline__ float4 advance_tail(const WorldDev& w, float u_max, int i, float4 p, float2 d, float Ux,
+                                               float Uy) {
   if (kRecord) w.ubead[i] = make_float2(Ux, Uy);
   const float m2 = Ux * Ux + Uy * Uy;
-  if (!(m2 <= w.u_max * w.u_max)) {   // also catches NaN
+  if (!(m2 <= u_max * u_max)) {   // also catches NaN
     atomicOr(w.flags, kFlagUnstable);
     return p;
   }
@@ -175,7 +176,7 @@ __device__ __forceinline__ float sq(float v) { return v * v; }
 
 // Constants of the PBD passes, read once per warp.
 struct PbdConst {
-  float hb, hs, ksh, ko, kappa_dt, dt;
+  float hb, hs, ksh, ko, kappa_dt, dt, u_max;
   int n_pbd, order, W, H, nbx;
 };
 
@@ -187,6 +188,7 @@ __device__ __forceinline__ PbdConst pbd_const(const WorldDev& w) {
   k.ko = w.orient * k.hs * k.ksh;
   k.kappa_dt = w.kappa_dt;
   k.dt = w.dt;
+  k.u_max = w.u_max;
   k.n_pbd = w.n_pbd;
   k.order = w.pbd_order;
   k.W = w.W;
@@ -207,16 +209,17 @@ __device__ __forceinline__ void pbd_edge_terms(float x, float y, float L, float 
 }
 
 // Position pass of one edge (Eqs. 2-4) with current edge vector (x, y),
-// rest length L and frame angle th: the correction (ddx, ddy) of its first
-// bead (the second gets the opposite), and the frame's turn toward the edge.
-__device__ __forceinline__ void edge_correction(float x, float y, float L, float& th, const PbdConst& k, float& ddx,
-                                                float& ddy) {
+// rest length L (iL = 1 / L) and frame angle th: the correction (ddx, ddy) of
+// its first bead (the second gets the opposite), and the frame's turn toward
+// the edge.
+__device__ __forceinline__ void edge_correction(float x, float y, float L, float iL, float& th, const PbdConst& k,
+                                                float& ddx, float& ddy) {
   float sc, sn, cs;
   pbd_edge_terms(x, y, L, th, sc, sn, cs);
   const float csx = sc * x, csy = sc * y;
   ddx = k.hs * (csx + k.ksh * (x - L * cs - csx));
   ddy = k.hs * (csy + k.ksh * (y - L * sn - csy));
-  th += k.ko * (cs * y - sn * x) * __frcp_rn(L);   // frame turns toward the edge (orient)
+  th += k.ko * (cs * y - sn * x) * iL;   // frame turns toward the edge (orient)
 }
 
 // Unit normal of the filament at a bead (two-layer coupling): t is the
@@ -314,7 +317,11 @@ __device__ __forceinline__ float2 bead_out_force(const WorldDev& w, const PbdCon
 // Jacobi PBD of a filament of at most 64 beads in registers: lane l holds
 // beads, edges and joints 2l and 2l + 1, and reads its neighbours' values by
 // warp shuffles.  The same arithmetic, in the same order, as pbd_block.
-template <bool kExt, int kMode>
+// kEarly: the beads claim their places in the bins, which depend on the
+// positions alone, before the passes, so that the atomics' round trip
+// overlaps them (a warp alone on its scheduler waited some 2,300 cycles of
+// 10,500 for them; with many warps the registers it holds cost more).
+template <bool kExt, int kMode, bool kEarly>
 __device__ __forceinline__ float pbd_regs(const WorldDev& w, const PbdConst& k, int b0, int B, int e0, int j0,
                                           long long t, int fields) {
   constexpr unsigned kAll = 0xffffffffu;
@@ -338,6 +345,7 @@ __device__ __forceinline__ float pbd_regs(const WorldDev& w, const PbdConst& k, 
   const float L0 = he0 ? (kExt ? rest_length(w, e0 + i0, t) : w.L_rest[e0 + i0]) : 1.0f;
   const float L1 = he1 ? (kExt ? rest_length(w, e0 + i1, t) : w.L_rest[e0 + i1]) : 1.0f;
   const float4 dr0 = hj0 ? w.drive[j0 + i0] : z4, dr1 = hj1 ? w.drive[j0 + i1] : z4;
+  const float iL0 = __frcp_rn(L0), iL1 = __frcp_rn(L1);
   float2 U0 = make_float2(0.0f, 0.0f), U1 = U0;
   if (kMode == 1 && !(kExt && w.layers == 2)) {
     // (lanes without a bead gather at cell 0: valid, unused)
@@ -357,8 +365,8 @@ __device__ __forceinline__ float pbd_regs(const WorldDev& w, const PbdConst& k, 
       if (hb0) U0 = bead_velocity_ext(w, b0 + i0, P0, U0, q);
       if (hb1) U1 = bead_velocity_ext(w, b0 + i1, P1, U1, q);
     }
-    if (hb0) P0 = advance_tail<false>(w, b0 + i0, P0, D0, U0.x, U0.y);
-    if (hb1) P1 = advance_tail<false>(w, b0 + i1, P1, D1, U1.x, U1.y);
+    if (hb0) P0 = advance_tail<false>(w, k.u_max, b0 + i0, P0, D0, U0.x, U0.y);
+    if (hb1) P1 = advance_tail<false>(w, k.u_max, b0 + i1, P1, D1, U1.x, U1.y);
     if (kExt && w.observe && w.energy) obs_add_warp(&w.obs[2], q);
   } else if (kMode == 0 && w.rec_pos) {
     // the step's start, into the reverse mode's record
@@ -394,6 +402,13 @@ __device__ __forceinline__ float pbd_regs(const WorldDev& w, const PbdConst& k, 
     if (hb0) w.nrm[b0 + i0] = bead_normal(u0, he0, um, lane > 0);
     if (hb1) w.nrm[b0 + i1] = bead_normal(u1, he1, u0, true);
   }
+  int* counts = nullptr;
+  BinClaim c0, c1;
+  if (kMode != 2 && kEarly) {
+    counts = step_counts(w, t);
+    c0 = bin_claim(w, counts, hb0, bead_bin_of(P0, k.nbx));
+    c1 = bin_claim(w, counts, hb1, bead_bin_of(P1, k.nbx));
+  }
   float dlx0 = 0.0f, dly0 = 0.0f, dlx1 = 0.0f, dly1 = 0.0f;
   if (k.order == 1) {
     for (int iter = 0; iter < k.n_pbd; ++iter) {
@@ -413,7 +428,7 @@ __device__ __forceinline__ float pbd_regs(const WorldDev& w, const PbdConst& k, 
       // position pass (Eqs. 2-4), edge 2l first, then edge 2l + 1
       float ddx0 = 0.0f, ddy0 = 0.0f;
       if (he0) {
-        edge_correction(v0.x + (dlx1 - dlx0), v0.y + (dly1 - dly0), L0, th0, k, ddx0, ddy0);
+        edge_correction(v0.x + (dlx1 - dlx0), v0.y + (dly1 - dly0), L0, iL0, th0, k, ddx0, ddy0);
         dlx0 += ddx0;
         dly0 += ddy0;
         dlx1 -= ddx0;
@@ -422,7 +437,7 @@ __device__ __forceinline__ float pbd_regs(const WorldDev& w, const PbdConst& k, 
       const float dlxn = __shfl_down_sync(kAll, dlx0, 1), dlyn = __shfl_down_sync(kAll, dly0, 1);
       float ddx1 = 0.0f, ddy1 = 0.0f;
       if (he1) {
-        edge_correction(v1.x + (dlxn - dlx1), v1.y + (dlyn - dly1), L1, th1, k, ddx1, ddy1);
+        edge_correction(v1.x + (dlxn - dlx1), v1.y + (dlyn - dly1), L1, iL1, th1, k, ddx1, ddy1);
         dlx1 += ddx1;
         dly1 += ddy1;
       }
@@ -444,8 +459,8 @@ __device__ __forceinline__ float pbd_regs(const WorldDev& w, const PbdConst& k, 
     // position pass (Eqs. 2-4) on the updated frames
     const float dlxn = __shfl_down_sync(kAll, dlx0, 1), dlyn = __shfl_down_sync(kAll, dly0, 1);
     float ddx0 = 0.0f, ddy0 = 0.0f, ddx1 = 0.0f, ddy1 = 0.0f;
-    if (he0) edge_correction(v0.x + (dlx1 - dlx0), v0.y + (dly1 - dly0), L0, th0, k, ddx0, ddy0);
-    if (he1) edge_correction(v1.x + (dlxn - dlx1), v1.y + (dlyn - dly1), L1, th1, k, ddx1, ddy1);
+    if (he0) edge_correction(v0.x + (dlx1 - dlx0), v0.y + (dly1 - dly0), L0, iL0, th0, k, ddx0, ddy0);
+    if (he1) edge_correction(v1.x + (dlxn - dlx1), v1.y + (dlyn - dly1), L1, iL1, th1, k, ddx1, ddy1);
     const float ddxm = __shfl_up_sync(kAll, ddx1, 1), ddym = __shfl_up_sync(kAll, ddy1, 1);
     if (hb0) {
       dlx0 += ddx0 - (lane > 0 ? ddxm : 0.0f);
@@ -467,8 +482,11 @@ __device__ __forceinline__ float pbd_regs(const WorldDev& w, const PbdConst& k, 
     float2 fe0 = make_float2(0.0f, 0.0f), fe1 = fe0;
     if (hb0) fe0 = bead_out_force(w, k, b0 + i0, bin0, dlx0, dly0, fields, fmax);
     if (hb1) fe1 = bead_out_force(w, k, b0 + i1, bin1, dlx1, dly1, fields, fmax);
-    int* counts = step_counts(w, t);
-    const BinClaim c0 = bin_claim(w, counts, hb0, bin0), c1 = bin_claim(w, counts, hb1, bin1);
+    if (!kEarly) {
+      counts = step_counts(w, t);
+      c0 = bin_claim(w, counts, hb0, bin0);
+      c1 = bin_claim(w, counts, hb1, bin1);
+    }
     const int s0 = bin_place(w, counts, hb0, c0), s1 = bin_place(w, counts, hb1, c1);
     if (hb0) bin_store(w, s0, b0 + i0, P0, fe0);
     if (hb1) bin_store(w, s1, b0 + i1, P1, fe1);
@@ -521,7 +539,7 @@ __device__ __forceinline__ float pbd_block(const WorldDev& w, const PbdConst& k,
       const float4 p = w.pos[b0 + i];
       const float2 d = w.disp[b0 + i];
       const float2 U = bead_velocity<kExt>(w, b0 + i, p, q);
-      P[i] = advance_tail<false>(w, b0 + i, p, d, U.x, U.y);
+      P[i] = advance_tail<false>(w, k.u_max, b0 + i, p, d, U.x, U.y);
     }
     if (kExt && w.observe && w.energy) obs_add_warp(&w.obs[2], q);
   } else if (kMode == 2) {
@@ -581,7 +599,7 @@ __device__ __forceinline__ float pbd_block(const WorldDev& w, const PbdConst& k,
       for (int c = 0; c < 2; ++c) {
         for (int e = 2 * tid + c; e < nE; e += 2 * T) {
           float the = th[e], ddxe, ddye;
-          edge_correction(vx[e] + (dlx[e + 1] - dlx[e]), vy[e] + (dly[e + 1] - dly[e]), Lr[e], the, k, ddxe, ddye);
+          edge_correction(vx[e] + (dlx[e + 1] - dlx[e]), vy[e] + (dly[e + 1] - dly[e]), Lr[e], __frcp_rn(Lr[e]), the, k, ddxe, ddye);
           th[e] = the;
           dlx[e] += ddxe;
           dly[e] += ddye;
@@ -603,7 +621,7 @@ __device__ __forceinline__ float pbd_block(const WorldDev& w, const PbdConst& k,
     __syncthreads();
     for (int e = tid; e < nE; e += T) {
       float the = th[e];
-      edge_correction(vx[e] + (dlx[e + 1] - dlx[e]), vy[e] + (dly[e + 1] - dly[e]), Lr[e], the, k, ddx[e], ddy[e]);
+      edge_correction(vx[e] + (dlx[e + 1] - dlx[e]), vy[e] + (dly[e + 1] - dly[e]), Lr[e], __frcp_rn(Lr[e]), the, k, ddx[e], ddy[e]);
       th[e] = the;
     }
     __syncthreads();
@@ -661,7 +679,7 @@ extern __shared__ __align__(16) float pbd_dyn_smem[];
 
 // kLong: the launch has such filaments (a kernel of its own: holding both
 // forms costs the warp form registers, 150 -> 167 us at 2^22 beads).
-template <bool kExt, int kMode, bool kSingle, bool kLong>
+template <bool kExt, int kMode, bool kSingle, bool kLong, bool kEarly>
 __device__ __forceinline__ void pbd_body(const WorldDev* __restrict__ worlds, const int4* __restrict__ items,
                                          const PbdWork& pw, int off, int fields, unsigned blk) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -679,7 +697,7 @@ __device__ __forceinline__ void pbd_body(const WorldDev* __restrict__ worlds, co
   const PbdConst k = pbd_const(w);
   float fmax;
   if (kLong && is_long) fmax = pbd_block<kExt, kMode>(w, k, b0, B, e0, j0, t, fields, pbd_dyn_smem, pw.maxB);
-  else fmax = pbd_regs<kExt, kMode>(w, k, b0, B, e0, j0, t, fields);
+  else fmax = pbd_regs<kExt, kMode, kEarly>(w, k, b0, B, e0, j0, t, fields);
   if (kMode == 2) return;
   // largest |F_el| component of the world this step (bounds the spread's
   // fixed-point scale); non-negative floats order like their bit patterns
@@ -706,6 +724,7 @@ __device__ __forceinline__ void interp_advance_body(const WorldDev* __restrict__
   float4 p = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   float2 U = make_float2(0.0f, 0.0f);
   float2 d = make_float2(0.0f, 0.0f);
+  const float u_max = w.u_max;
   if (i < w.N) {
     p = w.pos[i];
     d = w.disp[i];
@@ -718,7 +737,7 @@ __device__ __forceinline__ void interp_advance_body(const WorldDev* __restrict__
   }
   if (kExt && w.observe && w.energy) obs_add_warp(&w.obs[2], q);
   if (i >= w.N) return;
-  advance_tail(w, i, p, d, U.x, U.y);
+  advance_tail(w, u_max, i, p, d, U.x, U.y);
 }
 
 }  // namespace mc

@@ -920,6 +920,10 @@ __global__ void __launch_bounds__(32 * kAdjRegsWarps) k_adj_pbd_regs(const World
   const float thr1 = hj1 ? drive_angle(w.drive[j0 + i1], t) : 0.0f;
   float thb0 = he0 ? a.adjTh[e0 + i0] : 0.0f, thb1 = he1 ? a.adjTh[e0 + i1] : 0.0f;
   float2 X0 = hb0 ? a.adjX[b0 + i0] : z2, X1 = hb1 ? a.adjX[b0 + i1] : z2;
+  // the accumulators this step adds to at its end
+  const float gLo0 = he0 ? a.gL[e0 + i0] : 0.0f, gLo1 = he1 ? a.gL[e0 + i1] : 0.0f;
+  const float gto0 = hj0 ? a.gth0[j0 + i0] : 0.0f, gto1 = hj1 ? a.gth0[j0 + i1] : 0.0f;
+  const float gko = lane < 3 ? a.gkf[3 * f + lane] : 0.0f;
   // d_bar: direct forcing, from the bead velocities' adjoint; penalty, a4 and
   // the a6 gradient of the bead first, d_bar = kappa/dt Ftot_bar
   float2 d0 = z2, d1 = z2;
@@ -1092,15 +1096,15 @@ __global__ void __launch_bounds__(32 * kAdjRegsWarps) k_adj_pbd_regs(const World
     tr1 -= Cb1;
   }
   // outputs (with a rest-length drive L(t) = L0 (1 + A s(t)): dL(t)/dL0 = L(t)/L0)
-  auto edge_out = [&](int e, float thb, float gL) {
+  auto edge_out = [&](int e, float thb, float gL, float old) {
     a.adjTh[e] = thb;
     const float dLdL0 = w.ldrive ? 1.0f + w.ldrive[e].y * drive_sin(w.ldrive[e].z, w.ldrive[e].w, t) : 1.0f;
-    a.gL[e] += gL * dLdL0;
+    a.gL[e] = old + gL * dLdL0;
   };
-  if (he0) edge_out(e0 + i0, thb0, gL0);
-  if (he1) edge_out(e0 + i1, thb1, gL1);
-  if (hj0) a.gth0[j0 + i0] += tr0;
-  if (hj1) a.gth0[j0 + i1] += tr1;
+  if (he0) edge_out(e0 + i0, thb0, gL0, gLo0);
+  if (he1) edge_out(e0 + i1, thb1, gL1, gLo1);
+  if (hj0) a.gth0[j0 + i0] = gto0 + tr0;
+  if (hj1) a.gth0[j0 + i1] = gto1 + tr1;
   // X_bar is final for this step: its largest |dt X_bar| bounds the next
   // reversed step's u_bar (slot par ^ 1; every lane takes part)
   const float2 vm = from_left(vb1);
@@ -1122,11 +1126,7 @@ __global__ void __launch_bounds__(32 * kAdjRegsWarps) k_adj_pbd_regs(const World
     hsb += __shfl_xor_sync(kAll, hsb, o);
     kshb += __shfl_xor_sync(kAll, kshb, o);
   }
-  if (lane == 0) {
-    a.gkf[3 * f] += 0.5f * hbb;
-    a.gkf[3 * f + 1] += 0.5f * hsb;
-    a.gkf[3 * f + 2] += kshb;
-  }
+  if (lane < 3) a.gkf[3 * f + lane] = gko + (lane == 0 ? 0.5f * hbb : lane == 1 ? 0.5f * hsb : kshb);
 }
 
 // The stiffness gradients: the per-filament sums added over filaments in

@@ -17,7 +17,7 @@ __global__ void __launch_bounds__(256, kRoomy ? 2 : 4) k_pbd(const WorldDev* __r
                                              int fields) {
   pdl_trigger();
   pdl_wait();
-  pbd_body<kExt, kMode, kSingle, kLong>(worlds, items, pw, off, fields, blockIdx.x);
+  pbd_body<kExt, kMode, kSingle, kLong, kRoomy>(worlds, items, pw, off, fields, blockIdx.x);
 }
 
 // Spread of half of F_el + F_s at each layer point of every bead of

@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(kBeadChunk) k_mdf_advance_bins(const WorldDev*
     bead_energy(w, i, p, q);
   }
   if (w.observe && w.energy) obs_add_warp(&w.obs[2], q);
-  if (valid) p = advance_tail<false>(w, i, p, d, U.x, U.y);
+  if (valid) p = advance_tail<false>(w, w.u_max, i, p, d, U.x, U.y);
   mdf_bin_bead(w, step_counts(w, *w.t + off), valid, i, p);
 }
 

@@ -110,8 +110,8 @@ __global__ void __launch_bounds__(256, kBlocks) k_step_persistent(const PersistA
     // a1-a3 with the binning (fused with the previous step's a8 after the first step)
     const int fields = s == a.n_steps - 1;
     for (unsigned b = blockIdx.x; b < (unsigned)a.n_pbd_blocks; b += gridDim.x) {
-      if (s == 0) pbd_body<kExt, 0, false, false>(a.worlds, a.fil_items, pw, s, fields, b);
-      else pbd_body<kExt, 1, false, false>(a.worlds, a.fil_items, pw, s, fields, b);
+      if (s == 0) pbd_body<kExt, 0, false, false, false>(a.worlds, a.fil_items, pw, s, fields, b);
+      else pbd_body<kExt, 1, false, false, false>(a.worlds, a.fil_items, pw, s, fields, b);
     }
     if (!(ok = barrier())) break;
     // a4 + x pass of a5
