@@ -196,9 +196,12 @@ __device__ __forceinline__ float padded_tap(const WorldDev& w, int wR, int m) {
 // most 1/4, so a cell sum is below the largest bin count near the tile.
 // That bound leaves at least 24 fractional bits up to about one bead per
 // cell.  It is loose (a bead adds 1/16 to a cell on average), so a denser
-// tile (k < 24) deposits twice: the first pass measures the largest sum of
-// the accumulator (plus the rounding its terms can hide), which gives a
-// tight scale for the second.
+// tile (k < 24) first takes a bound from the beads' cells (deposit_bound: at
+// most 2.25 times an even density's sums, so two bits at the most; the sums
+// keep 26 fractional bits at four beads a cell, and turn into floats of 24).
+// With a folded axis it deposits twice instead: the first pass measures the
+// largest sum of the accumulator (plus the rounding its terms can hide),
+// which gives a tight scale for the second.
 // ---------------------------------------------------------------------------
 
 // Geometry of one deposit tile.
@@ -269,6 +272,43 @@ __device__ __forceinline__ void deposit_accumulate(int* acc, const WorldDev& w, 
     }
     __syncthreads();
   }
+}
+
+// A bound of the tile's cell sums from the beads' cells alone (acc zeroed
+// before, and holding the counts after): a bead of cell X adds at most
+// m_a m_b / 16, m = 1, 2, 2, 1, to the cells X - 1 .. X + 2 of each axis
+// (Peskin's kernel is at most 1/2 within a cell and 1/4 beyond), so a cell's
+// sum is at most the weighted count of the 4 x 4 cells around it.  One atomic
+// a bead instead of sixteen.  Not for folded axes.
+template <int R, int NT>
+__device__ __forceinline__ float deposit_bound(int* acc, const WorldDev& w, const DepTile& d, const Segments& sg,
+                                               int* red) {
+  using G = Geo<R>;
+  const int tid = threadIdx.x, total = sg.pre[kSegs];
+  const float4* __restrict__ bpos = w.bpos;
+  for (int v = tid; v < total; v += NT) {
+    const float4 p = bpos[seg_slot(v, sg)];
+    const int rx = image_lo(cell_x(p) - d.cx0, d.W, d.wR + 2), ry = image_lo(cell_y(p) - d.y0, d.H, 2);
+    if (rx <= d.tw + d.wR && ry <= d.th) atomicAdd(acc + (ry + 3) * G::kDX + rx + d.oxe, 1);
+  }
+  __syncthreads();
+  int most = 0;
+  for (int c = tid; c < G::kDY * G::kDX; c += NT) {
+    const int i = c / G::kDX, j = c - i * G::kDX;
+    int s = 0;
+#pragma unroll
+    for (int a = -2; a < 2; ++a) {
+      if (i + a < 0 || i + a >= G::kDY) continue;
+      const int* r = acc + (i + a) * G::kDX + j;
+      int t = 2 * r[0];
+      if (j >= 2) t += r[-2];
+      if (j >= 1) t += 2 * r[-1];
+      if (j + 1 < G::kDX) t += r[1];
+      s += (a == -1 || a == 0) ? 2 * t : t;
+    }
+    most = max(most, s);
+  }
+  return (float)block_max<NT>(most, red) * 0.0625f;
 }
 
 // The x pass of the accumulated sums at scale 2^k, rho_s when asked for,
@@ -421,8 +461,14 @@ __device__ __forceinline__ void deposit_x_body(const WorldDev* __restrict__ worl
     return;
   }
   int k = fix_exponent((float)sg.most + 1.0f);
+  const bool counted = k < 24 && !d.full_x && !d.full_y;
+  if (counted) {
+    k = fix_exponent(deposit_bound<R, NT>(acc, w, d, sg, reinterpret_cast<int*>(red)) * 1.0001f);
+    for (int c = tid; c < G::kDY * G::kDX / 4; c += NT) reinterpret_cast<int4*>(acc)[c] = make_int4(0, 0, 0, 0);
+    __syncthreads();
+  }
   deposit_accumulate<R, NT>(acc, w, d, k, sg);
-  if (k < 24) {
+  if (k < 24 && !counted) {
     // dense tile: the largest accumulated sum plus the rounding of its terms
     // (half a unit per bead of the covering bins, at most one term per cell
     // each) bounds every sum; deposit again at the scale that bound gives

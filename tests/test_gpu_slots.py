@@ -280,3 +280,31 @@ def test_a_crowd_that_outgrows_its_bins_slots(kw):
         w.step(20)
     for k, v in a.state(fluid=True).items():
         assert np.array_equal(v, c.state(fluid=True)[k]), k
+
+
+@pytest.mark.parametrize("H,W,n_fil", [(32, 96, 110), (64, 64, 64), (96, 128, 700), (256, 256, 4096)])
+@pytest.mark.parametrize("sigma", [0.5, 1.0, 2.0])
+def test_dense_tiles_deposit(H, W, n_fil, sigma):
+    """Tiles of a bead a cell and more, whose fixed-point scale comes from the
+    beads' cells (or, with an axis that one tile covers, from a first deposit):
+    the density and its filter against the oracle at 1e-6 of their scale (sums
+    of 32-bit weights: 2^-24 each, some tens of terms)."""
+    rng = np.random.default_rng(n_fil)
+    B = 32
+    x = np.concatenate([rng.uniform(0, W) + np.arange(B) * 0.9 for _ in range(n_fil)]) % W
+    y = np.repeat(rng.uniform(0, H, n_fil), B) + rng.uniform(-0.3, 0.3, n_fil * B)
+    x, y = np.mod(x, W).astype(np.float32), np.mod(y, H).astype(np.float32)
+    x[x >= W] = 0
+    y[y >= H] = 0
+    J = n_fil * (B - 2)
+    spec = synth._world("dense", H, W, [B] * n_fil, x, y, np.zeros(n_fil * (B - 1), np.float32), np.zeros(J),
+                        np.zeros(J), np.zeros(J), np.zeros(J), params=synth.Params(k_rep=1e-3, sigma=sigma))
+    ow = O.World(spec)
+    _, rec = O.step(ow, ow.initial_state(), record=True)
+    w = World(spec)
+    w.step(1)
+    assert_field("rho_s", w.field("rho_s"), t2n(rec["rho_s"]), 1e-6)
+    assert_field("rho_bar", w.field("rho_bar"), t2n(rec["rho_bar"]), 1e-6)
+    b = World(spec)
+    step_batched([b, World(synth.world_random(4, (40, 72), 5))], 1)
+    assert np.array_equal(w.field("rho_s"), b.field("rho_s"))
