@@ -275,7 +275,9 @@ __device__ __forceinline__ int bin_place(const WorldDev& w, int* counts, bool va
   const int at = __shfl_sync(0xffffffffu, c.base, __ffs(c.peers) - 1) + __popc(c.peers & ((1u << lane) - 1u));
   if (!valid) return -1;
   if (c.lo + at < c.hi) return c.lo + at;
-  return w.slot_end + atomicAdd(&counts[w.n_bins], 1);   // the bin's slots are full
+  // the bin's slots are full (never more beads than N, unless a run that timed
+  // out left counts behind)
+  return w.slot_end + min(atomicAdd(&counts[w.n_bins], 1), w.N - 1);
 }
 
 // The bin of the bead at P.

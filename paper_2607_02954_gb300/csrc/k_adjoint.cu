@@ -1195,16 +1195,26 @@ __global__ void __launch_bounds__(1024) k_loss_polyline(const WorldDev* __restri
   if (threadIdx.x == 0) *loss = red[0];
 }
 
-// The step counter moves to v; the slots step v accumulates into (its bin
-// counts, its F_el maximum) start at zero, the other parity's stay.
+// The step counter moves to v.  The slots that step v accumulates into (its
+// bin counts, its F_el maximum) start at zero; counts that the last completed
+// step left there go over to the other parity, where the read-outs look for
+// them (one of the two is zero between steps).
 __global__ void __launch_bounds__(256) k_set_counter(const __grid_constant__ WorldDev w, long long v) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i == 0) {
     *w.t = v;
+    const unsigned f = w.fel_max[v & 1];
+    if (f) w.fel_max[(v + 1) & 1] = f;
     w.fel_max[v & 1] = 0u;
-    *w.cnt_valid = 0;   // the counts in place are not those of step v - 1
+    *w.cnt_valid = 0;   // they are not step v - 1's
   }
-  if (i <= w.n_bins) step_counts(w, v)[i] = 0;
+  if (i <= w.n_bins) {
+    int* now = step_counts(w, v);
+    if (now[i]) {
+      step_counts(w, v + 1)[i] = now[i];
+      now[i] = 0;
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------

@@ -110,13 +110,19 @@ __global__ void __launch_bounds__(256) k_scan_apply(const WorldDev* __restrict__
   }
 }
 
+// The bin of the bead at p, or -1 (a loaded image is taken as it is).
+__device__ __forceinline__ int checked_bin(const WorldDev& w, const float4& p) {
+  const unsigned bx = (unsigned)cell_x(p) / kBin, by = (unsigned)cell_y(p) / kBin;
+  return bx < (unsigned)w.nbx && by < (unsigned)w.nby ? (int)(by * w.nbx + bx) : -1;
+}
+
 // Histogram of the beads' bins from their positions, into bin_cursor (zeroed
 // before).
 __global__ void __launch_bounds__(256) k_bin_histogram(const __grid_constant__ WorldDev w) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= w.N) return;
-  const float4 p = w.pos[i];
-  atomicAdd(&w.bin_cursor[(cell_y(p) / kBin) * w.nbx + cell_x(p) / kBin], 1);
+  const int bin = checked_bin(w, w.pos[i]);
+  if (bin >= 0) atomicAdd(&w.bin_cursor[bin], 1);
 }
 
 // The slots of a small world from its positions, in one block: the histogram
@@ -129,8 +135,8 @@ __global__ void __launch_bounds__(1024) k_layout_small(const __grid_constant__ W
   for (int k = tid; k < w.n_bins; k += 1024) hist[k] = 0;
   __syncthreads();
   for (int i = tid; i < w.N; i += 1024) {
-    const float4 p = w.pos[i];
-    atomicAdd(&hist[(cell_y(p) / kBin) * w.nbx + cell_x(p) / kBin], 1);
+    const int bin = checked_bin(w, w.pos[i]);
+    if (bin >= 0) atomicAdd(&hist[bin], 1);
   }
   __syncthreads();
   const int per = (w.n_bins + 1023) / 1024, lo = min(tid * per, w.n_bins), hi = min(lo + per, w.n_bins);
@@ -158,12 +164,13 @@ __global__ void __launch_bounds__(1024) k_layout_small(const __grid_constant__ W
 __global__ void __launch_bounds__(256) k_sort_records(const __grid_constant__ WorldDev w, int off) {
   const int* counts = step_counts(w, *w.t + off);
   if (blockIdx.x == gridDim.x - 1) {
-    const int n = counts[w.n_bins];
+    const int n = min(counts[w.n_bins], w.N);
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
       const int src = w.slot_end + k;
       const float4 p = w.bpos[src];
       const int bin = (cell_y(p) / kBin) * w.nbx + cell_x(p) / kBin;
       const int dst = atomicAdd(&w.bin_cursor[bin], 1);
+      if (dst >= w.N) continue;   // (counts left behind by a run that timed out)
       w.spos[dst] = p;
       w.srec[dst] = w.brec[src];
     }
@@ -172,7 +179,7 @@ __global__ void __launch_bounds__(256) k_sort_records(const __grid_constant__ Wo
   const int bin = (int)blockIdx.x * 8 + (threadIdx.x >> 5);
   if (bin >= w.n_bins) return;
   const int lo = w.bin_base[bin], n = min(counts[bin], w.bin_base[bin + 1] - lo), dst = w.bin_off[bin];
-  for (int k = threadIdx.x & 31; k < n; k += 32) {
+  for (int k = threadIdx.x & 31; k < n && dst + k < w.N; k += 32) {
     w.spos[dst + k] = w.bpos[lo + k];
     w.srec[dst + k] = w.brec[lo + k];
   }
@@ -182,9 +189,10 @@ __global__ void __launch_bounds__(256) k_sort_records(const __grid_constant__ Wo
 __global__ void __launch_bounds__(256) k_unsort_records(const __grid_constant__ WorldDev w) {
   int* counts = step_counts(w, *w.t - 1);
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= w.bin_off[w.n_bins]) return;
+  if (k >= w.N || k >= w.bin_off[w.n_bins]) return;
   const float4 p = w.spos[k];
-  const int bin = (cell_y(p) / kBin) * w.nbx + cell_x(p) / kBin;
+  const int bin = checked_bin(w, p);
+  if (bin < 0) return;
   const int at = atomicAdd(&counts[bin], 1);
   const int lo = w.bin_base[bin];
   const int slot = lo + at < w.bin_base[bin + 1] ? lo + at : w.slot_end + atomicAdd(&counts[w.n_bins], 1);
@@ -192,7 +200,8 @@ __global__ void __launch_bounds__(256) k_unsort_records(const __grid_constant__ 
   const float4 rec = w.srec[k];
   w.bpos[slot] = p;
   w.brec[slot] = rec;
-  if (w.bead_slot) w.bead_slot[__float_as_int(rec.z)] = slot;
+  const unsigned id = (unsigned)__float_as_int(rec.z);
+  if (w.bead_slot && id < (unsigned)w.N) w.bead_slot[id] = slot;
 }
 
 // ---------------------------------------------------------------------------

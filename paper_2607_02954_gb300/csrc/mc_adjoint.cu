@@ -367,7 +367,7 @@ mc_status mc_rollout_forward_stored(mc_world* w, int n_steps, void* stream) {
     for (int q = 0; q < n_steps; ++q) {
       st = mdf_recorded_step(w, seg, ss, q, n_steps, t0, s);
       if (st != MC_OK) return st;
-      if (q % mc::kLayoutSteps == 0) mc::launch_slot_layout(w->plan, s);
+      if (q % mc::kLayoutSteps == mc::kLayoutSteps - 1) mc::launch_slot_layout(w->plan, s);
     }
     w->t += n_steps;
     st = save_state(h, (int)(w->t & 1), tape + sl.bytes, sl, s);   // the final state
@@ -386,7 +386,7 @@ mc_status mc_rollout_forward_stored(mc_world* w, int n_steps, void* stream) {
     p.d_worlds = d_desc + q;
     p.h_world0 = desc[q];
     run_recorded_step(p, s);
-    if (q % mc::kLayoutSteps == 0) mc::launch_slot_layout(w->plan, s);
+    if (q % mc::kLayoutSteps == mc::kLayoutSteps - 1) mc::launch_slot_layout(w->plan, s);
   }
   MC_ACUDA(cudaGetLastError());
   w->t += n_steps;
@@ -420,6 +420,7 @@ mc_status mc_rollout_rewind(mc_world* w, void* stream) {
   if (h.N) MC_ACUDA(cudaMemcpyAsync(h.disp, tape + tl.disp0, h.N * sizeof(float2), cudaMemcpyDeviceToDevice, s));
   MC_ACUDA(cudaMemcpyAsync(h.obs, tape + tl.obs0, 3 * sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s));
   mc::launch_set_counter(h, w->tape_t0, s);
+  mc::launch_slot_layout_from_positions(w->plan, s);   // the beads are back where they started
   MC_ACUDA(cudaGetLastError());
   w->t = w->tape_t0;
   return MC_OK;
@@ -530,6 +531,7 @@ mc_status sweep(mc_world* w, mc::AdjDev a, const mc::AdjMdf* mdf, float* const a
     mc_status st = load_state(h, (int)(tk & 1), tape + (size_t)k * sl.bytes, sl, rs);
     if (st != MC_OK) return st;
     mc::launch_set_counter(h, tk, rs);
+    mc::launch_slot_layout_from_positions(w->plan, rs);
     st = save_state(h, (int)(tk & 1), seg[b], sl, rs);   // the segment's first state
     if (st != MC_OK) return st;
     for (int q = 0; q < steps; ++q) {
@@ -539,8 +541,7 @@ mc_status sweep(mc_world* w, mc::AdjDev a, const mc::AdjMdf* mdf, float* const a
       } else {
         run_recorded_step(step_plan(b, q, (int)((tk + q) & 1), false), rs);   // fields straight into the record
       }
-      // the slots follow the beads from the segment's first step on
-      if (q % mc::kLayoutSteps == 0) mc::launch_slot_layout(w->plan, rs);
+      if (q % mc::kLayoutSteps == mc::kLayoutSteps - 1) mc::launch_slot_layout(w->plan, rs);
     }
     MC_ACUDA(cudaGetLastError());
     return MC_OK;

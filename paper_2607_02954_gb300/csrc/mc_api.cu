@@ -230,8 +230,15 @@ cudaStream_t capture_stream() {
 }
 
 // Lays the slots out before a run of n steps outside the graph when the plan
-// has run kLayoutSteps steps on the present layout.
+// has run kLayoutSteps steps on the present layout, and always into a capture
+// (whose replays this host does not see).
 void lay_out_slots(Plan& p, int n, cudaStream_t s) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  cudaStreamIsCapturing(s, &cs);
+  if (cs != cudaStreamCaptureStatusNone) {
+    mc::launch_slot_layout(p, s);
+    return;
+  }
   if (p.since_layout >= mc::kLayoutSteps) {
     mc::launch_slot_layout(p, s);
     p.since_layout = 0;

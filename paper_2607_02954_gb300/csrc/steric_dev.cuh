@@ -116,7 +116,7 @@ __device__ void build_segments(const WorldDev& w, int off, int x_lo, int x_hi, i
   if (lane == 31) {
     sg.pre[0] = 0;
     sg.start[kSegs - 1] = w.slot_end;
-    sg.pre[kSegs] = incl1 + over;
+    sg.pre[kSegs] = incl1 + min(over, w.N);
     sg.covered = covered;
     sg.most = most;
   }

@@ -308,3 +308,42 @@ def test_dense_tiles_deposit(H, W, n_fil, sigma):
     b = World(spec)
     step_batched([b, World(synth.world_random(4, (40, 72), 5))], 1)
     assert np.array_equal(w.field("rho_s"), b.field("rho_s"))
+
+
+@pytest.mark.parametrize("n", [3, 4])
+def test_read_outs_after_a_rewind_and_a_backward(n):
+    """The bins of the last step that ran can be read after the counter has
+    moved back, whichever parity it had, and after a reverse sweep of one
+    segment the fields are the rollout's last step's."""
+    spec = crowded(14)
+    w = World(spec)
+    w.rollout_forward(n, n)
+    want = {f: w.field(f) for f in ("bin_off", "rho_s", "rho_bar", "force")}
+    gx = torch.ones(spec.N, device="cuda")
+    w.rollout_backward(gx, gx)
+    for f, v in want.items():
+        assert np.array_equal(v, w.field(f)), f
+    w.rollout_rewind()
+    assert np.array_equal(want["bin_off"], w.field("bin_off"))
+    assert np.array_equal(want["rho_s"], w.field("rho_s"))
+
+
+def test_a_captured_step_replays_like_single_steps():
+    """One step captured by the caller into a graph of its own and replayed 40
+    times (the slots are laid out inside the capture) equals 40 single steps."""
+    spec = crowded(19)
+    a, b = World(spec), World(spec)
+    a.step(1)
+    b.step(1)
+    g = torch.cuda.CUDAGraph()
+    s = torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.graph(g, stream=s):
+        a.step(1, stream=s)
+    for _ in range(40):
+        g.replay()
+        b.step(1)
+    torch.cuda.synchronize()
+    x, y = a.state_device(), b.state_device()
+    for k in x:
+        assert torch.equal(x[k], y[k]), k
