@@ -515,7 +515,7 @@ __device__ __forceinline__ float pbd_regs(const WorldDev& w, const PbdConst& k, 
 // corrections of a pass see the state before it.  A pass over a long chain
 // is bound by the latency of its rounds: with one warp a filament of 300
 // beads took ten rounds a pass, and the fused advance + PBD of 60 filaments
-// of 2 to 300 beads 33.7 us; with a block 12.6 us.
+// of 2 to 300 beads 33.7 us; with a block 11.0 us.
 template <bool kExt, int kMode>
 __device__ __forceinline__ float pbd_block(const WorldDev& w, const PbdConst& k, int b0, int B, int e0, int j0,
                                           long long t, int fields, float* s, int maxB) {

@@ -34,7 +34,8 @@ __device__ __forceinline__ int ubar_exponent(const WorldDev& w, const AdjDev& a)
 }
 
 // (Four threads a bead, each one row of the stencil: the kernel is a chain
-// of a few loads and the atomics, bound by latency at a few thousand beads.)
+// of a few loads and the atomics, bound by latency at a few thousand beads;
+// 10,231 beads on 488 x 640: 7.1 us with one thread a bead, 5.7 us so.)
 __global__ void __launch_bounds__(256) k_adj_spread_u(const WorldDev* __restrict__ wd, AdjDev a) {
   const WorldDev& w = *wd;
   const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 2, b = threadIdx.x & 3;
@@ -213,7 +214,8 @@ __device__ __forceinline__ int q_exponent(const WorldDev& w, const AdjDev& a) {
 }
 
 // Four threads a bead: each gathers and scatters one row of the stencil, the
-// rows' sums added in a fixed order.
+// rows' sums added in a fixed order.  Latency-bound too: 10,231 beads 12.0 ->
+// 7.0 us.
 __global__ void __launch_bounds__(256) k_adj_bead_a(const WorldDev* __restrict__ wd, AdjDev a) {
   const WorldDev& w = *wd;
   const int at = (blockIdx.x * blockDim.x + threadIdx.x) >> 2, b = threadIdx.x & 3;
@@ -300,7 +302,7 @@ __global__ void __launch_bounds__(256) k_adj_bead_a(const WorldDev* __restrict__
 // ---------------------------------------------------------------------------
 // The filter half width is compiled in (the tap loops unroll).  A block's
 // strip has 8 rows while that leaves fewer than four blocks an SM, else 16
-// (less halo a cell).
+// (less halo a cell).  488 x 640: 12.6 -> 9.9 us; 256^2: 6.4 -> 6.0 us.
 template <int R, int kRows>
 __global__ void __launch_bounds__(256) k_adj_rho_blur(const WorldDev* __restrict__ wd, AdjDev a) {
   constexpr int kE = kTile + 2 * R;     // columns of the rho_bar_bar region
@@ -866,7 +868,7 @@ __global__ void __launch_bounds__(kAdjPbdThreads) k_adj_pbd(const WorldDev* __re
 // bending pass and the edge vectors of the position pass (8 floats a lane).
 // With few filaments the kernel is bound by latency: the block form spent it
 // on its seven barriers a pass (64 filaments of 48 beads, 4 passes: 14.5 us;
-// this form 10.9 us).
+// this form 9.0 us).
 // ---------------------------------------------------------------------------
 constexpr int kAdjTapeRegs = 8;
 constexpr int kAdjRegsWarps = 4;   // most filaments per block
@@ -1324,7 +1326,9 @@ void launch_set_rest(const WorldDev& h, const float* theta0, const float* L_rest
 // image coordinates u = (X R/W, Y R/H) adds exp(-|c - u|^2 / (2 s^2)) to the
 // pixels with px in floor(u_x) - K .. floor(u_x) + K (same in y, periodic),
 // K = ceil(4 s).  The image accumulates in 64-bit fixed point (2^-32 units),
-// so it does not depend on the order of the beads.
+// so it does not depend on the order of the beads.  A bead's pixel rows go
+// to blocks of their own (10,231 beads: 20.7 us with a thread a bead, 9.1 us
+// so).
 // ---------------------------------------------------------------------------
 constexpr double kSplatScale = 4294967296.0;   // 2^32
 
@@ -1352,7 +1356,8 @@ __global__ void __launch_bounds__(256) k_splat_accum(const WorldDev* __restrict_
   }
 }
 
-// One block: diff = I - T per pixel and loss = mean(diff^2), summed in a fixed order.
+// One block: diff = I - T per pixel and loss = mean(diff^2), summed in a fixed order
+// (1024 threads: 128^2 pixels 31.8 -> 15.8 us; latency).
 __global__ void __launch_bounds__(1024) k_splat_loss(const unsigned long long* __restrict__ acc,
                                                     const float* __restrict__ target, int RR, float* __restrict__ diff,
                                                     float* loss) {

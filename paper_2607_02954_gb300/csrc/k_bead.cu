@@ -11,6 +11,11 @@ namespace mc {
 // block per longer one (in dynamic shared memory): see pbd_body.
 // kRoomy: twice the registers, for launches whose filaments are all resident
 // at half the warps per SM (more of a filament's loads are in flight at once).
+// Small launches are bound by the chain of round trips (16 filaments of 32
+// beads: 7.8 us with two gathers and two claims in a row, 6.5 us so), large
+// ones by how many of them are in flight and by HBM (2^22 beads: 148 us for
+// some 0.6 GB, 139 us before it wrote the binned records, with 46 us of scan
+// and scatter after it).
 template <bool kExt, int kMode, bool kSingle, bool kLong, bool kRoomy>
 __global__ void __launch_bounds__(256, kRoomy ? 2 : 4) k_pbd(const WorldDev* __restrict__ worlds,
                                              const int4* __restrict__ items, const PbdWork pw, int off,
@@ -118,7 +123,9 @@ __global__ void __launch_bounds__(256) k_stream_out(const float* __restrict__ g,
 }
 
 // The bead state into device memory (any pointer may be null; nothing is
-// assumed of their alignment beyond a float's).
+// assumed of their alignment beyond a float's).  One kernel for all four
+// arrays: a small world's read-out is launches (2.6 us, where the positions'
+// kernel alone took 1.9 us and the other arrays a copy each).
 __global__ void __launch_bounds__(256) k_state_out(const float4* __restrict__ pos, const float2* __restrict__ disp_in,
                                                    const float* __restrict__ theta_in, int N, int E, float* x,
                                                    float* y, float* theta, float* disp) {

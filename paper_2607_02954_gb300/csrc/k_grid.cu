@@ -117,7 +117,7 @@ __device__ __forceinline__ int checked_bin(const WorldDev& w, const float4& p) {
 }
 
 // Histogram of the beads' bins from their positions, into bin_cursor (zeroed
-// before).
+// before).  Once per created or loaded world; 4 us for 2^18 beads.
 __global__ void __launch_bounds__(256) k_bin_histogram(const __grid_constant__ WorldDev w) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= w.N) return;
@@ -126,7 +126,9 @@ __global__ void __launch_bounds__(256) k_bin_histogram(const __grid_constant__ W
 }
 
 // The slots of a small world from its positions, in one block: the histogram
-// in shared memory, then the scan of its room.
+// in shared memory, then the scan of its room.  Such a world's layout is
+// launches: 3.4 us at 128^2 and 512 beads, where the clearing, histogram and
+// scan kernels take three launches.
 constexpr int kSmallBins = 8192, kSmallBeads = 1 << 15;
 __global__ void __launch_bounds__(1024) k_layout_small(const __grid_constant__ WorldDev w) {
   __shared__ int hist[kSmallBins];

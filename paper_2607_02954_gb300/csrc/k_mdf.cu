@@ -26,6 +26,12 @@
 // (k_mdf_moments, passes, k_lbm), which give the same step bitwise; there
 // every kernel returns at once for the worlds of a batch that couple by the
 // penalty force (and for a world's passes beyond its own m).
+// Bound by the latency of each tile's phases, two waves of them at 1024
+// tiles.  2^18 beads on 1024^2, us: spread with moments 29.3 (18.3 + 12.6 as
+// two kernels), last pass with the collision 35 (24 + 15.9), advance with the
+// bins 8.5 (7.5 + 4.2 + an idle PBD's 2.7); 16 steps of four passes 3251 ->
+// 3070.  A pass alone takes 24, 22 when its records were contiguous behind a
+// sort that cost 11 a step.
 #include "bead_dev.cuh"
 #include "steric_dev.cuh"
 

@@ -54,10 +54,11 @@ namespace mc {
 // of the kernel takes: 32 (deposit) or 64 (force).  A kernel that works on
 // beads alone (the deposit, the spread without the collision) also wants one
 // bead a thread of its tiles, else its barriers cost more than the idle
-// warps (128^2, 16 tiles of 32 beads: deposit 4.6 us with 256 threads, 5.4
-// with 1024).  256^2 with 4096 beads a tile: deposit 47.7 -> 24.1 us, force +
-// LBM 53.7 -> 31.3; 512^2 with 1024 beads a tile: 17.1 -> 15.9 and, with 512
-// threads, 22.4 -> 18.9; 128^2: force + LBM 7.9 -> 7.3.  A tile's sums are
+// warps (128^2, 16 tiles of 32 beads: deposit 4.7 us with 256 threads, 5.4
+// with 1024).  256^2 with 4096 beads a tile: deposit 47.7 -> 24.1 us (21.6
+// now that such tiles deposit once), force + LBM 53.7 -> 30.8; 512^2 with
+// 1024 beads a tile: 17.1 -> 15.8 and, with 512 threads, 22.4 -> 18.9;
+// 128^2: force + LBM 7.9 -> 7.1.  A tile's sums are
 // integers or per-cell, so the width changes no result.
 int tile_threads(const Plan& p, int sms, int regs, bool beads_only) {
   const long long room = (long long)sms * (65536 / (regs * 256));   // blocks of 256 resident at once
