@@ -60,11 +60,18 @@ namespace mc {
 // 1024 beads a tile: 17.1 -> 15.8 and, with 512 threads, 22.4 -> 18.9;
 // 128^2: force + LBM 7.9 -> 7.1.  A tile's sums are
 // integers or per-cell, so the width changes no result.
+// The deposit (8.5 KB of shared memory a block) takes 128 threads from four
+// tiles an SM on: sixteen tiles resident instead of eight, whose reads of
+// counter, counts and records are one dependent chain, and barriers of half
+// the warps.  7204 tiles of 13 beads: 25.9 -> 18.5 us, 16384 of 256 beads: 86
+// -> 75, 1504: 12.4 -> 11.6, 1024: 10.0 -> 9.8; fewer leave warps idle (320
+// tiles: 5.3 -> 5.5 us, 77: 5.1 -> 6.0).
 int tile_threads(const Plan& p, int sms, int regs, bool beads_only) {
   const long long room = (long long)sms * (65536 / (regs * 256));   // blocks of 256 resident at once
   const long long tiles = p.n_tile_items;
   for (int nt : {1024, 512})
     if (tiles * (nt / 256) <= room && (!beads_only || p.beads >= tiles * nt)) return nt;
+  if (regs == 32 && tiles >= 4 * (long long)sms) return 128;
   return 256;
 }
 
@@ -267,6 +274,7 @@ void launch_steric(const Plan& p, cudaStream_t s, int which, int store_fields, i
   if (which == 0) {
     if (nt == 1024) launch_deposit<R, 1024>(p, s, store_fields, off);
     else if (nt == 512) launch_deposit<R, 512>(p, s, store_fields, off);
+    else if (nt == 128) launch_deposit<R, 128>(p, s, store_fields, off);
     else launch_deposit<R, 256>(p, s, store_fields, off);
   } else if (which == 1) {
     if (nt == 1024) launch_spread<R, 1024>(p, s, store_fields, off, fields);

@@ -9,7 +9,7 @@ namespace mc {
 
 namespace {
 
-constexpr int kThreads = 256;              // threads of a tile's block (the narrowest, see tile_threads)
+constexpr int kThreads = 256;              // threads of a tile's block (the force kernels' narrowest, see tile_threads)
 constexpr int kWarps = kThreads / 32;
 constexpr int kAx = kTile + 6;             // force accumulator edge: the tile and 3 halo cells a side
 constexpr int kWin = kTile + 8;            // rho_bar window edge: the tile and 4 cells a side
@@ -333,8 +333,11 @@ __device__ __forceinline__ void deposit_xpass(const int* acc, const WorldDev& w,
 #pragma unroll
   for (int m = 0; m < G::kTaps; ++m) tp[m] = tap_s[m] * inv;
   if (!d.full_x) {
-    const int ly = tid >> 3, s = tid & 7;       // row, strip of 4 columns
-    if (ly < th && 4 * s < tw) {
+    const int s = tid & 7;                      // strip of 4 columns
+#pragma unroll
+    for (int r = 0; r < (8 * kTile + NT - 1) / NT; ++r) {
+      const int ly = (tid >> 3) + r * (NT / 8);   // row
+      if (ly >= th || 4 * s >= tw) continue;
       const int4* src = reinterpret_cast<const int4*>(acc + (ly + 3) * G::kDX + 4 * s + oxe - R);
       float v[4 * G::kL4];
 #pragma unroll
@@ -356,7 +359,7 @@ __device__ __forceinline__ void deposit_xpass(const int* acc, const WorldDev& w,
       const size_t c = (size_t)(y0 + ly) * W + x0 + 4 * s;
       *reinterpret_cast<float4*>(rho_x + c) = make_float4(o[0], o[1], o[2], o[3]);
       // the strip's own cells are v[R .. R + 3]
-      vmax = fmaxf(fmaxf(v[R], v[R + 1]), fmaxf(v[R + 2], v[R + 3]));
+      vmax = fmaxf(vmax, fmaxf(fmaxf(v[R], v[R + 1]), fmaxf(v[R + 2], v[R + 3])));
       if (store_fields)
         *reinterpret_cast<float4*>(rho_s_out + c) = make_float4(v[R] * inv, v[R + 1] * inv, v[R + 2] * inv, v[R + 3] * inv);
     }
@@ -450,8 +453,11 @@ __device__ __forceinline__ void deposit_x_body(const WorldDev* __restrict__ worl
     // no bead reaches the region: rho_s, rho_x and the tile maximum are zero
     // (what the passes below give for an empty accumulator, bitwise)
     // (tw is a multiple of 8, so each 4-column strip is whole and aligned)
-    const int ly = tid >> 3, s = tid & 7;
-    if (ly < d.th && 4 * s < d.tw) {
+    const int s = tid & 7;
+#pragma unroll
+    for (int r = 0; r < (8 * kTile + NT - 1) / NT; ++r) {
+      const int ly = (tid >> 3) + r * (NT / 8);
+      if (ly >= d.th || 4 * s >= d.tw) continue;
       const size_t c = (size_t)(d.y0 + ly) * d.W + d.x0 + 4 * s;
       const float4 z = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
       *reinterpret_cast<float4*>(w.rho_x + c) = z;

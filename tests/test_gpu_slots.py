@@ -310,6 +310,39 @@ def test_dense_tiles_deposit(H, W, n_fil, sigma):
     assert np.array_equal(w.field("rho_s"), b.field("rho_s"))
 
 
+@pytest.mark.parametrize("H,W,n_fil,sigma", [(32, 96, 40, 1.0), (40, 32, 12, 0.5), (200, 328, 60, 2.0), (256, 256, 2000, 1.0),
+                                             (800, 808, 700, 1.0)])
+def test_narrow_deposit_blocks(H, W, n_fil, sigma):
+    """A world in a batch of many tiles, whose deposit takes blocks of 128
+    threads, against the same world alone (wider blocks, but for the last) and
+    the persistent step (256 threads): bitwise the same.  Folded axes, ragged
+    and dense tiles, empty ones, other filter widths."""
+    from paper_2607_02954_gb300 import set_launch_config
+    rng = np.random.default_rng(H + W)
+    B = 24
+    x = np.concatenate([rng.uniform(0, W) + np.arange(B) * 0.9 for _ in range(n_fil)]) % W
+    y = np.repeat(rng.uniform(0, H, n_fil), B) + rng.uniform(-0.3, 0.3, n_fil * B)
+    x, y = np.mod(x, W).astype(np.float32), np.mod(y, H).astype(np.float32)
+    x[x >= W] = 0
+    y[y >= H] = 0
+    J = n_fil * (B - 2)
+    spec = synth._world("narrow", H, W, [B] * n_fil, x, y, np.zeros(n_fil * (B - 1), np.float32), np.zeros(J),
+                        np.zeros(J), np.zeros(J), np.zeros(J), params=synth.Params(k_rep=1e-3, sigma=sigma))
+    alone, persistent, batched = World(spec), World(spec), World(spec)
+    if sigma == 1.0:   # (the persistent step takes a filter half width of 4 only)
+        set_launch_config([persistent], persistent=4)
+    alone.step(3)
+    persistent.step(3)
+    sparse = [World(synth.world_random(k, (256, 288), 2)) for k in range(9)]   # 648 tiles
+    step_batched([batched] + sparse, 3)
+    want = alone.state(fluid=True)
+    for w in (persistent, batched):
+        for k, v in w.state(fluid=True).items():
+            assert np.array_equal(want[k], v), k
+        for k in ("rho_s", "rho_bar"):
+            assert np.array_equal(alone.field(k), w.field(k)), k
+
+
 @pytest.mark.parametrize("n", [3, 4])
 def test_read_outs_after_a_rewind_and_a_backward(n):
     """The bins of the last step that ran can be read after the counter has
