@@ -14,7 +14,8 @@ namespace mc {
 //           the sorted read-outs (bin_off), and in bin_cursor each bin's first
 //           place after its slots' records
 //   kSrc 1  the room for the counts of the last completed step: bin_base, the
-//           slots of the coming steps (left alone while no counts are in place)
+//           slots of the coming steps (left alone while no counts are in
+//           place); right ahead of a step only, since no record moves
 //   kSrc 2  the room for the position histogram in bin_cursor: bin_base
 // The layout is by far cheaper than the sort it replaces: once in
 // kLayoutSteps steps, and no record moves.  The sorted read-outs

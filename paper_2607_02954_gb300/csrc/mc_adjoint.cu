@@ -238,6 +238,13 @@ StoredLayout stored_layout(const mc::WorldDev& h, int n) {
   return L;
 }
 
+// The slots laid out again ahead of recorded step q when it is due: never
+// after a run's last step, whose records the read-outs find by the layout
+// they were placed in.
+void lay_out_before(const mc_world* w, int q, cudaStream_t s) {
+  if (q > 0 && q % mc::kLayoutSteps == 0) mc::launch_slot_layout(w->plan, s);
+}
+
 // One step of the penalty path in unfused stages, with p's descriptor
 // binding the step's fields to its record (bind_step).
 void run_recorded_step(const mc::Plan& p, cudaStream_t s) {
@@ -314,6 +321,7 @@ mc_status mc_rollout_forward(mc_world* w, int n_steps, int ckpt_every, void* str
   // the start's displacement and observables (the checkpoints hold the rest), for mc_rollout_rewind
   if (h.N) MC_ACUDA(cudaMemcpyAsync(tape + tl.disp0, h.disp, h.N * sizeof(float2), cudaMemcpyDeviceToDevice, s));
   MC_ACUDA(cudaMemcpyAsync(tape + tl.obs0, h.obs, 3 * sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s));
+  mc::refresh_slots(w, s);
   int done = 0;
   for (int k = 0; k < n_ck; ++k) {
     mc_status st = save_state(h, (int)(w->t & 1), tape + (size_t)k * sl.bytes, sl, s);
@@ -359,15 +367,16 @@ mc_status mc_rollout_forward_stored(mc_world* w, int n_steps, void* stream) {
   MC_ACUDA(cudaMemcpyAsync(tape + tl.obs0, h.obs, 3 * sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s));
   mc_status st = save_state(h, (int)(t0 & 1), tape, sl, s);   // the start (mc_rollout_rewind)
   if (st != MC_OK) return st;
+  mc::refresh_slots(w, s);
   if (h.ib == 1) {
     // direct forcing: the world's own buffers step, each step's record is
     // copied out after it (the same path as the sweep's recompute)
     st = save_state(h, (int)(t0 & 1), seg, sl, s);   // step 0's start state
     if (st != MC_OK) return st;
     for (int q = 0; q < n_steps; ++q) {
+      lay_out_before(w, q, s);
       st = mdf_recorded_step(w, seg, ss, q, n_steps, t0, s);
       if (st != MC_OK) return st;
-      if (q % mc::kLayoutSteps == mc::kLayoutSteps - 1) mc::launch_slot_layout(w->plan, s);
     }
     w->t += n_steps;
     st = save_state(h, (int)(w->t & 1), tape + sl.bytes, sl, s);   // the final state
@@ -385,8 +394,8 @@ mc_status mc_rollout_forward_stored(mc_world* w, int n_steps, void* stream) {
     mc::Plan p = w->plan;
     p.d_worlds = d_desc + q;
     p.h_world0 = desc[q];
+    lay_out_before(w, q, s);
     run_recorded_step(p, s);
-    if (q % mc::kLayoutSteps == mc::kLayoutSteps - 1) mc::launch_slot_layout(w->plan, s);
   }
   MC_ACUDA(cudaGetLastError());
   w->t += n_steps;
@@ -420,9 +429,9 @@ mc_status mc_rollout_rewind(mc_world* w, void* stream) {
   if (h.N) MC_ACUDA(cudaMemcpyAsync(h.disp, tape + tl.disp0, h.N * sizeof(float2), cudaMemcpyDeviceToDevice, s));
   MC_ACUDA(cudaMemcpyAsync(h.obs, tape + tl.obs0, 3 * sizeof(unsigned long long), cudaMemcpyDeviceToDevice, s));
   mc::launch_set_counter(h, w->tape_t0, s);
-  mc::launch_slot_layout_from_positions(w->plan, s);   // the beads are back where they started
   MC_ACUDA(cudaGetLastError());
   w->t = w->tape_t0;
+  w->slots_stale = true;   // the beads are back where they started
   return MC_OK;
 }
 
@@ -535,13 +544,13 @@ mc_status sweep(mc_world* w, mc::AdjDev a, const mc::AdjMdf* mdf, float* const a
     st = save_state(h, (int)(tk & 1), seg[b], sl, rs);   // the segment's first state
     if (st != MC_OK) return st;
     for (int q = 0; q < steps; ++q) {
+      lay_out_before(w, q, rs);
       if (mdf) {
         st = mdf_recorded_step(w, seg[b], ss, q, steps, tk, rs);
         if (st != MC_OK) return st;
       } else {
         run_recorded_step(step_plan(b, q, (int)((tk + q) & 1), false), rs);   // fields straight into the record
       }
-      if (q % mc::kLayoutSteps == mc::kLayoutSteps - 1) mc::launch_slot_layout(w->plan, rs);
     }
     MC_ACUDA(cudaGetLastError());
     return MC_OK;
@@ -783,6 +792,7 @@ mc_status backward(mc_world* w, const float* dL_dx, const float* dL_dy, float* d
     w->bwd_key = key;
   }
   MC_ACUDA(cudaGraphLaunch(w->bwd_exec, s));
+  if (!stored) w->slots_stale = true;   // (laid out for the first segment's re-run, the last that ran)
   // outputs (caller memory)
   if (h.J) MC_ACUDA(cudaMemcpyAsync(dL_dtheta0, a.gth0, h.J * sizeof(float), cudaMemcpyDeviceToDevice, s));
   if (dL_dL_rest && h.E)

@@ -501,6 +501,13 @@ mc_world* world_clone(const mc_world* w, cudaStream_t s) {
   return c;   // no plan of its own: a copy is only stepped within the plan it is made for
 }
 mc_status plan_run(Plan& p, int n_steps, cudaStream_t s) { return run_steps(p, n_steps, s); }
+void refresh_slots(mc_world* w, cudaStream_t s) {
+  if (!w->slots_stale) return;
+  launch_slot_layout_from_positions(w->plan, s);
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  cudaStreamIsCapturing(s, &cs);
+  w->slots_stale = cs != cudaStreamCaptureStatusNone;   // (a capture has laid nothing out yet)
+}
 void plan_free(Plan& p, cudaStream_t s) { free_plan(p, s); }
 
 }  // namespace mc
@@ -913,6 +920,7 @@ mc_status mc_step(mc_world* w, int n_steps, void* stream) {
     mc_status st = mc::plan_tune(&self, 1, w->plan, s, true);
     if (st != MC_OK) return st;
   }
+  if (n_steps > 0) mc::refresh_slots(w, s);
   mc_status st = run_steps(w->plan, n_steps, s);
   if (st == MC_OK) w->t += n_steps;
   return st;
@@ -932,6 +940,7 @@ mc_status mc_step_batched(mc_world* const* ws, int n, int n_steps, void* stream)
     st = mc::plan_tune(ws, n, *plan, s, true);
     if (st != MC_OK) return st;
   }
+  for (int k = 0; k < n; ++k) mc::refresh_slots(ws[k], s);
   st = run_steps(*plan, n_steps, s);
   if (st == MC_OK)
     for (int k = 0; k < n; ++k) ws[k]->t += n_steps;
@@ -998,7 +1007,10 @@ mc_status mc_step_stage(mc_world* w, int stage, void* stream) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   const Plan& p = w->plan;
   switch (stage) {
-    case 0: mc::launch_pbd(p, s); break;
+    case 0:
+      mc::refresh_slots(w, s);
+      mc::launch_pbd(p, s);
+      break;
     case 1: mc::launch_sorted_offsets(p, s, 0); break;
     case 2: mc::launch_sorted_records(p, s, 0); break;
     case 3: mc::launch_deposit_x(p, s, 0); break;

@@ -69,9 +69,11 @@ struct WorldDev {
   // the others (bin_cnt[par][n_bins] of them in all) follow at slot_end.
   // The counts alternate by step parity par: the deposit of a step zeroes
   // the other parity's for the next step.  The slots are laid out again every
-  // few steps, between steps, from the last step's counts (slot_room), and at
-  // first from the initial positions: beads move by a fraction of a cell a
-  // step, so hardly any bin outgrows its slots in between.
+  // few steps, from the last step's counts (slot_room), and at first from the
+  // initial positions: beads move by a fraction of a cell a step, so hardly
+  // any bin outgrows its slots in between.  A layout moves no record, so it
+  // is always the launch ahead of a step: until then the read-outs find the
+  // last step's records by bin_base.
   int slot_end;
   int* bin_base;          // [n_bins + 1]
   int* bin_cnt;           // [2][n_bins + 1], the last entry of each: beads that found their bin's slots full
@@ -340,6 +342,10 @@ struct ArenaSize {
 ArenaSize world_layout(WorldDev& h, void* arena);
 mc_status plan_build(mc_world* const* ws, int n, cudaStream_t s, Plan& out);
 mc_status plan_run(Plan& p, int n_steps, cudaStream_t s);
+// Ahead of a world's next step (and never earlier: the read-outs need the
+// layout of the last one): its slots laid out from the positions when a
+// rewind or a reverse sweep has moved the beads at once.
+void refresh_slots(mc_world* w, cudaStream_t s);
 void plan_free(Plan& p, cudaStream_t s);
 void plan_set_cfg(Plan& p, const LaunchCfg& c);   // drops the captured graph when the configuration changes
 // A device copy of a world (same state, its own arena; no plan of its own)
@@ -634,6 +640,7 @@ struct mc_world {
   std::vector<int> fil_off;
   mc::Plan plan;                  // single-world plan
   mc_params params{};
+  bool slots_stale = false;       // the beads have jumped since the slots were laid out (see refresh_slots)
   // reverse-mode state (mc_rollout_forward / mc_rollout_backward)
   void* tape = nullptr;           // checkpoints + final state
   size_t tape_bytes = 0;

@@ -361,6 +361,86 @@ def test_read_outs_after_a_rewind_and_a_backward(n):
     assert np.array_equal(want["rho_s"], w.field("rho_s"))
 
 
+def room(counts):
+    """Slots that bins of these bead counts are given."""
+    return (counts + counts // 4 + 16 + 7) // 8 * 8
+
+
+def drifting(seed, **kw):
+    """A crowd carried across bins by a uniform flow (beads further apart with
+    direct forcing, whose passes overshoot where several share a cell)."""
+    spec = synth.world_random(seed, (72, 64), 12) if kw.get("ib") else crowded(seed, n_fil=40, at=(20.0, 20.0))
+    for k, v in kw.items():
+        setattr(spec.params, k, v)
+    cx = np.array([0, 1, 0, -1, 0, 1, -1, -1, 1])[:, None, None]
+    cy = np.array([0, 0, 1, 0, -1, 1, 1, -1, -1])[:, None, None]
+    wt = np.array([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4)[:, None, None]
+    ux, uy = 0.3, 0.1
+    cu = cx * ux + cy * uy
+    spec.f0 = np.broadcast_to(wt * (3 * cu + 4.5 * cu * cu - 1.5 * (ux * ux + uy * uy)),
+                              (9, spec.H, spec.W)).astype(np.float32)
+    return spec
+
+
+def read_outs(w, names=("bin", "bin_off", "rho_s", "rho_bar", "force", "fs", "fel")):
+    """The fields of the last step (and the beads of each bin in order)."""
+    out = {f: w.field(f) for f in names}
+    off, beads = out["bin_off"], w.field("bin_beads")
+    out["bin_beads"] = np.concatenate([np.sort(beads[off[k]:off[k + 1]]) for k in range(len(off) - 1)])
+    return out
+
+
+def assert_same(got, want, what):
+    for k in got:
+        assert np.array_equal(want[k], got[k]), (what, k)
+
+
+@pytest.mark.parametrize("kw", [{}, dict(layers=2), dict(ib=1, mdf_iters=2)])
+@pytest.mark.parametrize("n,every,stored,before", [(3, 3, False, 0), (4, 4, False, 0), (16, 16, False, 0),
+                                                   (17, 17, False, 5), (32, 16, False, 0), (32, 32, False, 3),
+                                                   (16, 0, True, 0), (17, 0, True, 0), (32, 0, True, 21)])
+def test_read_outs_after_rollouts_backwards_and_rewinds(n, every, stored, before, kw):
+    """The read-outs are those of the last step that ran: after a recorded or
+    stored rollout (also one that ends where a layout of the slots is due),
+    after the reverse sweep (whose last re-run is the first segment), after a
+    rewind, and in an image saved there."""
+    spec = drifting(31, **kw)
+    if n >= 16:   # the first and the last step ask for other slots, so a layout between them and the read-out shows
+        last = np.diff(O.cell_and_bin(spec.x, spec.y, spec.H, spec.W, 8)[2])
+        moved = np.mod(spec.x + 0.3 * (n + before), spec.W), np.mod(spec.y + 0.1 * (n + before), spec.H)
+        assert (room(last) != room(np.diff(O.cell_and_bin(*moved, spec.H, spec.W, 8)[2]))).any()
+    plain, w = World(spec), World(spec)
+    plain.step(before)
+    w.step(before)
+    first = None
+    if not stored and every < n:
+        first = World(spec)
+        first.step(before + every)
+        first = read_outs(first)
+    plain.step(n)
+    end = read_outs(plain)
+    w.rollout_forward(n, every or n, stored=stored)
+    assert_same(read_outs(w), end, "forward")
+    w.rollout_rewind()
+    assert_same(read_outs(w), end, "rewind")
+    w.rollout_forward(n, every or n, stored=stored)
+    gx = torch.ones(spec.N, device="cuda")
+    w.rollout_backward(gx, gx)
+    # (what goes through the slots alone: F_el, F_s, the normals that the layer points of two layers need and the
+    # total force of direct forcing stay in the re-run's records)
+    names = ("bin", "bin_off", "rho_s", "rho_bar") + (() if kw else ("force",))
+    want = end if first is None else first
+    assert_same(read_outs(w, names), want, "backward")
+    w.rollout_rewind()
+    assert_same(read_outs(w, names), want, "rewind after backward")
+    loaded = World.load(w.save(), spec)
+    assert_same(read_outs(loaded, names), want, "load")
+    for other in (w, loaded):
+        other.step(n)
+        assert_same(read_outs(other), end, "again")
+        assert_same(other.state(fluid=True), plain.state(fluid=True), "again")
+
+
 def test_a_captured_step_replays_like_single_steps():
     """One step captured by the caller into a graph of its own and replayed 40
     times (the slots are laid out inside the capture) equals 40 single steps."""
