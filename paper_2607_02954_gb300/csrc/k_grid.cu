@@ -171,8 +171,8 @@ __global__ void __launch_bounds__(256) k_sort_records(const __grid_constant__ Wo
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
       const int src = w.slot_end + k;
       const float4 p = w.bpos[src];
-      const int bin = (cell_y(p) / kBin) * w.nbx + cell_x(p) / kBin;
-      const int dst = atomicAdd(&w.bin_cursor[bin], 1);
+      const int bin = checked_bin(w, p);
+      const int dst = bin < 0 ? w.N : atomicAdd(&w.bin_cursor[bin], 1);
       if (dst >= w.N) continue;   // (counts left behind by a run that timed out)
       w.spos[dst] = p;
       w.srec[dst] = w.brec[src];

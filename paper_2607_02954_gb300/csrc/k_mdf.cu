@@ -199,14 +199,9 @@ __device__ __forceinline__ void mdf_list(MdfSmem<NT>& sm, const WorldDev& w, con
   };
   auto list = [&](bool keep, Rec r) {
     int rx = cell_x(r.p) - tb.x0, ry = cell_y(r.p) - tb.y0;
-    if (w.ntx > 1) {
-      rx = image_lo(rx, w.W, 2);
-      keep = keep && rx <= tb.tw;
-    }
-    if (w.nty > 1) {
-      ry = image_lo(ry, w.H, 2);
-      keep = keep && ry <= tb.th;
-    }
+    if (w.ntx > 1) rx = image_lo(rx, w.W, 2);
+    if (w.nty > 1) ry = image_lo(ry, w.H, 2);
+    keep = keep && reaches(rx, 2, tb.tw) && reaches(ry, 2, tb.th);
     const int at = list_place(keep, &sm.s_cnt);
     if (keep) {
       r.p.z = __int_as_float(rx);
@@ -317,8 +312,10 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_mdf_pass(const WorldDev* __re
         // the bead's own tile is its one writer in this pass: the adds
         // need no return value and leave the same bits in any order
         const int i = sm.si[q];
-        atomicAdd(&fel[i].x, dF.x);
-        atomicAdd(&fel[i].y, dF.y);
+        if ((unsigned)i < (unsigned)w.N) {
+          atomicAdd(&fel[i].x, dF.x);
+          atomicAdd(&fel[i].y, dF.y);
+        }
       }
       float wx[4], wy[4];
       peskin4(p.x, wx);

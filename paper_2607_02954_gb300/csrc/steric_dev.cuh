@@ -141,6 +141,13 @@ __device__ __forceinline__ int image_lo(int d, int n, int lo) {
   return d;
 }
 
+// Whether r, an axis coordinate relative to the region, lies in [-lo, hi]:
+// the images that reach it (and, on an axis the region covers whole, every
+// cell).  For a record that the step's PBD stored the low side holds by
+// construction (image_lo); one unsigned comparison checks both, so that no
+// record of any bits gives an address outside the block's arrays.
+__device__ __forceinline__ bool reaches(int r, int lo, int hi) { return (unsigned)(r + lo) <= (unsigned)(hi + lo); }
+
 // The next place of the block's list for each lane that keeps its bead;
 // every lane of the warp calls this together.  The list order depends on
 // warp timing, which no result depends on (the accumulation is in integers).
@@ -220,6 +227,7 @@ __device__ __forceinline__ void deposit_accumulate(int* acc, const WorldDev& w, 
   const int W = d.W, H = d.H, wR = d.wR, x0 = d.x0, y0 = d.y0, tw = d.tw, th = d.th;
   const int cx0 = d.cx0, oxe = d.oxe, total = sg.pre[kSegs];
   const bool full_x = d.full_x, full_y = d.full_y;
+  const int lo_x = full_x ? 2 : wR + 2, hi_x = full_x ? W : tw + wR;   // (the accumulator has room for both)
   const float4* __restrict__ bpos = w.bpos;
   const float scale = pow2f(k);
   // each thread deposits the beads v = tid, tid + NT, ... of the segments
@@ -227,16 +235,9 @@ __device__ __forceinline__ void deposit_accumulate(int* acc, const WorldDev& w, 
   // a bead whose stencil misses the region adds nothing
   auto deposit = [&](const float4 p) {
     int rx = cell_x(p) - cx0, ry = cell_y(p) - y0;
-    bool keep = true;
-    if (!full_x) {
-      rx = image_lo(rx, W, wR + 2);
-      keep = rx <= tw + wR;
-    }
-    if (!full_y) {
-      ry = image_lo(ry, H, 2);
-      keep = keep && ry <= th;
-    }
-    if (!keep) return;
+    if (!full_x) rx = image_lo(rx, W, wR + 2);
+    if (!full_y) ry = image_lo(ry, H, 2);
+    if (!reaches(rx, lo_x, hi_x) || !reaches(ry, 2, th)) return;
     float wx[4], wy[4];
     peskin4(p.x, wx);
     peskin4(p.y, wy);
@@ -289,7 +290,7 @@ __device__ __forceinline__ float deposit_bound(int* acc, const WorldDev& w, cons
   for (int v = tid; v < total; v += NT) {
     const float4 p = bpos[seg_slot(v, sg)];
     const int rx = image_lo(cell_x(p) - d.cx0, d.W, d.wR + 2), ry = image_lo(cell_y(p) - d.y0, d.H, 2);
-    if (rx <= d.tw + d.wR && ry <= d.th) atomicAdd(acc + (ry + 3) * G::kDX + rx + d.oxe, 1);
+    if (reaches(rx, d.wR + 2, d.tw + d.wR) && reaches(ry, 2, d.th)) atomicAdd(acc + (ry + 3) * G::kDX + rx + d.oxe, 1);
   }
   __syncthreads();
   int most = 0;
@@ -556,14 +557,9 @@ __device__ __forceinline__ void force_list(const Segments& sg, TileWork<NT>& wk,
   const float4* __restrict__ brec = w.brec;
   auto list = [&](bool keep, float4 p, const float4 rec) {
     int rx = cell_x(p) - tb.x0, ry = cell_y(p) - tb.y0;
-    if (ntx > 1) {
-      rx = image_lo(rx, W, 2);
-      keep = keep && rx <= tb.tw;
-    }
-    if (nty > 1) {
-      ry = image_lo(ry, H, 2);
-      keep = keep && ry <= tb.th;
-    }
+    if (ntx > 1) rx = image_lo(rx, W, 2);
+    if (nty > 1) ry = image_lo(ry, H, 2);
+    keep = keep && reaches(rx, 2, tb.tw) && reaches(ry, 2, tb.th);
     const int at = list_place(keep, &wk.s_cnt);
     if (keep) {
       p.z = __int_as_float(rx);
@@ -728,8 +724,10 @@ __device__ __forceinline__ void tile_beads(TileWork<NT>& wk, const WorldDev& w, 
     }
     const float Fsx = -0.5f * k_rep * gsx, Fsy = -0.5f * k_rep * gsy;
     const float4 rec = wk.sr[q];
-    if (keep_fs && rx >= 0 && rx < tb.tw && ry >= 0 && ry < tb.th)
-      fs_out[__float_as_int(rec.z)] = make_float2(Fsx, Fsy);
+    if (keep_fs && rx >= 0 && rx < tb.tw && ry >= 0 && ry < tb.th) {
+      const unsigned id = (unsigned)__float_as_int(rec.z);
+      if (id < (unsigned)w.N) fs_out[id] = make_float2(Fsx, Fsy);
+    }
     if (layered) continue;   // two-layer worlds spread at their layer points (k_layer_spread)
     const float Fx = (rec.x + Fsx) * scale, Fy = (rec.y + Fsy) * scale;
     float ax[4], ay[4];

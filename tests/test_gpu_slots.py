@@ -441,6 +441,39 @@ def test_read_outs_after_rollouts_backwards_and_rewinds(n, every, stored, before
         assert_same(other.state(fluid=True), plain.state(fluid=True), "again")
 
 
+@pytest.mark.parametrize("before", [3, 16, 37])
+def test_steps_after_a_run_that_timed_out_stay_in_bounds(before):
+    """A persistent run that ends at its first barrier leaves its PBD's counts
+    behind, and the layout of a later step gives them slots that hold no
+    record.  The world's state is unspecified then, but its steps and read-outs
+    stay within their arrays, and other worlds are not affected."""
+    from paper_2607_02954_gb300 import _lib, set_launch_config
+    lib = _lib.load()
+    spec, other = drifting(31), synth.world_random(4, (40, 72), 5)
+    w, a, b = World(spec), World(other), World(other)
+    w.step(before)
+    set_launch_config([w], persistent=4)
+    _lib.check(lib.mc_debug_barrier_test(1, 2_000_000))   # 2 ms
+    try:
+        w.step(1)
+        with pytest.raises(_lib.MCError):
+            w.check()
+    finally:
+        _lib.check(lib.mc_debug_barrier_test(0, 1_000_000_000))
+    set_launch_config([w], persistent=0)
+    _lib.check(lib.mc_world_clear_flags(w.handle, None))
+    for _ in range(40):
+        step_batched([w, a], 1)
+        w.step(1)
+        b.step(1)
+    got = w.state(fluid=True)
+    assert np.isfinite(got["x"]).all() and (got["x"] >= 0).all() and (got["x"] <= spec.W).all()
+    for f in ("rho_s", "rho_bar", "force", "bin_off", "bin_beads"):
+        w.field(f)
+    w.save()
+    assert_same(a.state(fluid=True), b.state(fluid=True), "other world")
+
+
 def test_a_captured_step_replays_like_single_steps():
     """One step captured by the caller into a graph of its own and replayed 40
     times (the slots are laid out inside the capture) equals 40 single steps."""
