@@ -42,6 +42,7 @@ __global__ void __launch_bounds__(kBeadChunk) k_layer_spread(const WorldDev* __r
   if (i >= w.N) return;
   const int W = w.W, H = w.H;
   const int slot = w.bead_slot[i];
+  if (slot < 0) return;   // no step has binned the bead
   const float4 rec = w.brec[slot];
   const float4 p = w.bpos[slot];
   const float2 n = w.nrm[i], fe = make_float2(rec.x, rec.y), fs = w.fs[i];
@@ -165,6 +166,7 @@ __global__ void __launch_bounds__(256) k_world_init(const __grid_constant__ Worl
     const float cx = floorf(xw), cy = floorf(yw);
     h.pos0[i] = make_float2(xw, yw);
     h.pos[i] = make_float4(xw - cx, yw - cy, __int_as_float((int)cx), __int_as_float((int)cy));
+    if (h.layers == 2) h.bead_slot[i] = -1;
   }
   if (i < h.J) const_cast<float4*>(h.drive)[i] = make_float4(r.theta0[i], r.amp[i], r.freq[i], r.phase[i]);
   if (i < h.E) {

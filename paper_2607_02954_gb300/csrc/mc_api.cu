@@ -862,6 +862,7 @@ mc_status mc_world_load(const void* buf, size_t bytes, void* stream, mc_world** 
   }
   mc::world_layout(h, w->arena);
   e = cudaMemsetAsync(static_cast<char*>(w->arena) + sz.image, 0, sz.zero - sz.image, w->stream);
+  if (e == cudaSuccess && h.layers == 2) e = cudaMemsetAsync(h.bead_slot, 0xff, h.N * sizeof(int), w->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(w->arena, static_cast<const char*>(buf) + sizeof(hd) + fo_bytes, w->image_bytes,
                         cudaMemcpyHostToDevice, w->stream);

@@ -96,7 +96,8 @@ struct WorldDev {
   float layer_half;       // half distance between the layers (cells)
   int ib, mdf_iters;      // coupling (0 penalty, 1 direct forcing) and MDF passes per step
   float* mrho;            // [H * W] fluid density of the step (ib == 1)
-  int* bead_slot;         // [N] slot of each bead in bpos and brec (ib == 1 or layers == 2, else nullptr)
+  int* bead_slot;         // [N] slot of each bead in bpos and brec (ib == 1 or layers == 2, else nullptr; -1 with
+                          // two layers before the first step)
   float2* u2;             // [H * W] second velocity buffer of the MDF passes (ib == 1, see mdf_u)
   float2* sus;            // [slot_end + N] U_s by slot (ib == 1)
   float2* nrm;            // [N] filament unit normal at each bead (layers == 2)

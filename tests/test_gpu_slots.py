@@ -474,6 +474,23 @@ def test_steps_after_a_run_that_timed_out_stay_in_bounds(before):
     assert_same(a.state(fluid=True), b.state(fluid=True), "other world")
 
 
+@pytest.mark.parametrize("kw", [{}, dict(layers=2), dict(ib=1, mdf_iters=1)])
+def test_read_outs_before_the_first_step_are_zero(kw):
+    """A world that no step has binned yet, in memory that another world's
+    records may have left behind, created and loaded."""
+    spec = drifting(31, **kw)
+    old = World(spec)
+    old.step(3)
+    torch.cuda.synchronize()
+    old.close()
+    w = World(spec)
+    for v in (w, World.load(w.save(), spec)):
+        for f in ("force", "rho_s", "rho_bar", "bin_off"):
+            assert not v.field(f).any(), f
+        v.step(2)
+    assert_same(v.state(fluid=True), w.state(fluid=True), "steps")
+
+
 def test_a_captured_step_replays_like_single_steps():
     """One step captured by the caller into a graph of its own and replayed 40
     times (the slots are laid out inside the capture) equals 40 single steps."""
