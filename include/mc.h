@@ -284,8 +284,10 @@ mc_status mc_debug_barrier_test(unsigned extra_arrivals, int64_t timeout_ns);
  * in that order is exactly one mc_step(w, 1) without the graph.  Stages 4
  * (y pass + steric force + spread, writes F) and 5 (LBM, reads F) are stage 7
  * split in two kernels with F through device memory; 0, 1, 2, 3, 4, 5, 6
- * give the same step bitwise.  Any other use leaves the world in an
- * unspecified state.  The step counter advances with stage 6.  Errors:
+ * give the same step bitwise.  Between stages the fields that come from the
+ * binned beads (MC_FIELD_RHO_S, _RHO_BAR, _FORCE, _BIN_OFF, _BIN_BEADS) are
+ * those of the step in progress, and reading them does not disturb it.  Any
+ * other use leaves the world in an unspecified state.  The step counter advances with stage 6.  Errors:
  * MC_ERR_INVALID_ARG for an unknown stage or a world with ib = 1 (its
  * step has more stages; mc_step runs them). */
 mc_status mc_step_stage(mc_world* w, int stage, void* stream);

@@ -432,6 +432,7 @@ mc_status mc_rollout_rewind(mc_world* w, void* stream) {
   MC_ACUDA(cudaGetLastError());
   w->t = w->tape_t0;
   w->slots_stale = true;   // the beads are back where they started
+  w->staged = false;
   return MC_OK;
 }
 

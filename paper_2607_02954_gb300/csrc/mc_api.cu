@@ -502,6 +502,7 @@ mc_world* world_clone(const mc_world* w, cudaStream_t s) {
 }
 mc_status plan_run(Plan& p, int n_steps, cudaStream_t s) { return run_steps(p, n_steps, s); }
 void refresh_slots(mc_world* w, cudaStream_t s) {
+  w->staged = false;
   if (!w->slots_stale) return;
   launch_slot_layout_from_positions(w->plan, s);
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -774,6 +775,11 @@ struct SaveHeader {
 };
 constexpr char kSaveMagic[8] = {'M', 'C', 'W', 'O', 'R', 'L', 'D', '1'};
 
+// The step whose binned beads the read-outs take, from the step counter: the
+// last completed one, or the one in progress from its PBD on (mc_step_stage),
+// which takes the slots over.
+int binned_step(const mc_world* w) { return w->staged ? 0 : -1; }
+
 size_t save_size(const mc_world* w) {
   return sizeof(SaveHeader) + (size_t)(w->h.n_fil + 1) * sizeof(int) + w->image_bytes;
 }
@@ -806,8 +812,8 @@ mc_status mc_world_save(const mc_world* w, void* buf, size_t bytes, void* stream
   char* out = static_cast<char*>(buf);
   std::memcpy(out, &hd, sizeof(hd));
   std::memcpy(out + sizeof(hd), w->fil_off.data(), (size_t)(w->h.n_fil + 1) * sizeof(int));
-  mc::launch_sorted_offsets(w->plan, s, -1);
-  mc::launch_sorted_records(w->plan, s, -1);
+  mc::launch_sorted_offsets(w->plan, s, binned_step(w));
+  mc::launch_sorted_records(w->plan, s, binned_step(w));
   MC_CUDA(cudaGetLastError());
   MC_CUDA(cudaMemcpyAsync(out + sizeof(hd) + (size_t)(w->h.n_fil + 1) * sizeof(int), w->arena, w->image_bytes,
                           cudaMemcpyDeviceToHost, s));
@@ -1011,6 +1017,7 @@ mc_status mc_step_stage(mc_world* w, int stage, void* stream) {
     case 0:
       mc::refresh_slots(w, s);
       mc::launch_pbd(p, s);
+      w->staged = true;
       break;
     case 1: mc::launch_sorted_offsets(p, s, 0); break;
     case 2: mc::launch_sorted_records(p, s, 0); break;
@@ -1021,6 +1028,7 @@ mc_status mc_step_stage(mc_world* w, int stage, void* stream) {
     default:
       mc::launch_interp_advance(p, s);
       w->t += 1;
+      w->staged = false;
       break;
   }
   MC_CUDA(cudaGetLastError());
@@ -1077,6 +1085,7 @@ mc_status mc_world_get_field(const mc_world* w, int field, void* out, int mem_ki
   const cudaMemcpyKind dk = host ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
   const void* src = nullptr;
   size_t bytes = 0;
+  const int off = binned_step(w);
   switch (field) {
     case MC_FIELD_FEL: src = h.fel; bytes = h.N * sizeof(float2); break;
     case MC_FIELD_FS: src = h.fs; bytes = h.N * sizeof(float2); break;
@@ -1086,8 +1095,8 @@ mc_status mc_world_get_field(const mc_world* w, int field, void* out, int mem_ki
       // the step keeps these in shared memory only: re-run the steric
       // stages on the last step's binned beads with field output on (they
       // are deterministic, so rho_x, F and F_s are rewritten identically)
-      mc::launch_deposit_x(w->plan, s, field == MC_FIELD_RHO_S, -1);
-      if (field == MC_FIELD_RHO_BAR) mc::launch_force_spread(w->plan, s, 1, -1);
+      mc::launch_deposit_x(w->plan, s, field == MC_FIELD_RHO_S, off);
+      if (field == MC_FIELD_RHO_BAR) mc::launch_force_spread(w->plan, s, 1, off);
       MC_CUDA(cudaGetLastError());
       src = field == MC_FIELD_RHO_S ? (const void*)h.rho_s : (const void*)h.rho_b;
       bytes = HW * sizeof(float);
@@ -1096,7 +1105,8 @@ mc_status mc_world_get_field(const mc_world* w, int field, void* out, int mem_ki
       // the step hands F from the spread to the collision in shared memory:
       // re-run the spread on the last step's binned beads (deterministic);
       // a direct-forcing step leaves its total F in device memory
-      if (h.ib != 1) mc::launch_force_spread(w->plan, s, 0, -1);
+      if (w->staged) mc::launch_deposit_x(w->plan, s, 0, off);   // (the step's own may not have run)
+      if (h.ib != 1) mc::launch_force_spread(w->plan, s, 0, off);
       MC_CUDA(cudaGetLastError());
       src = h.F;
       bytes = HW * sizeof(float2);
@@ -1104,13 +1114,13 @@ mc_status mc_world_get_field(const mc_world* w, int field, void* out, int mem_ki
     case MC_FIELD_U: src = h.u; bytes = HW * sizeof(float2); break;
     case MC_FIELD_BIN: src = h.bead_bin; bytes = h.N * sizeof(int); break;
     case MC_FIELD_BIN_OFF:
-      mc::launch_sorted_offsets(w->plan, s, -1);
+      mc::launch_sorted_offsets(w->plan, s, off);
       MC_CUDA(cudaGetLastError());
       src = h.bin_off;
       bytes = (h.n_bins + 1) * sizeof(int); break;
     case MC_FIELD_BIN_BEADS:   // the id word of each bin-ordered record
-      mc::launch_sorted_offsets(w->plan, s, -1);
-      mc::launch_sorted_records(w->plan, s, -1);
+      mc::launch_sorted_offsets(w->plan, s, off);
+      mc::launch_sorted_records(w->plan, s, off);
       MC_CUDA(cudaGetLastError());
       if (h.N)
         MC_CUDA(cudaMemcpy2DAsync(out, sizeof(int), reinterpret_cast<const char*>(h.srec) + 2 * sizeof(float),

@@ -641,6 +641,7 @@ struct mc_world {
   std::vector<int> fil_off;
   mc::Plan plan;                  // single-world plan
   mc_params params{};
+  bool staged = false;            // mc_step_stage has run the PBD of the next step, and not yet its last stage
   bool slots_stale = false;       // the beads have jumped since the slots were laid out (see refresh_slots)
   // reverse-mode state (mc_rollout_forward / mc_rollout_backward)
   void* tape = nullptr;           // checkpoints + final state

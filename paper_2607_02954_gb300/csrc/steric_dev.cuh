@@ -406,7 +406,8 @@ struct DepositSmem {
 // control flow; the caller's block runs it whole).  It also readies the next
 // step: the other parity's counts of the tile's own bins, its overflow count
 // and its F_el-maximum slot go to zero (the previous step's; this step's
-// stay readable).
+// stay readable).  A re-run of a completed step's deposit (off < 0) clears
+// nothing: the other parity's counts may be a step's in progress.
 template <int R, bool kSingle, int NT>
 __device__ __forceinline__ void deposit_x_body(const WorldDev* __restrict__ worlds, const int2* __restrict__ items,
                                                int store_fields, int off, const WorldDev& w1, unsigned blk,
@@ -435,14 +436,14 @@ __device__ __forceinline__ void deposit_x_body(const WorldDev* __restrict__ worl
   d.cx0 = d.full_x ? 0 : d.x0;                  // region column origin
   d.oxe = d.full_x ? 4 : R + 4;                 // accumulator column of region column 0
   if (warp == 0) build_segments<false>(w, off, d.x0 - d.wR - 2, d.x0 + d.tw + d.wR, d.y0 - 2, d.y0 + d.th, sm.sg);
-  if (warp == 2) {
+  if (warp == 2 && off >= 0) {
     const long long t = *w.t + off;
     int* next = step_counts(w, t + 1);
     const int bx = d.x0 / kBin + (lane & 3), by = d.y0 / kBin + (lane >> 2);
     if (lane < 16 && bx < w.nbx && by < w.nby) next[by * w.nbx + bx] = 0;
     if (lane == 16 && d.tile == 0) {
       next[w.n_bins] = 0;
-      if (off >= 0) *w.cnt_valid = 1;   // (not when a completed step's stage is re-run)
+      *w.cnt_valid = 1;
       w.fel_max[(t + 1) & 1] = 0u;
     }
   }

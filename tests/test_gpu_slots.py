@@ -491,6 +491,26 @@ def test_read_outs_before_the_first_step_are_zero(kw):
     assert_same(v.state(fluid=True), w.state(fluid=True), "steps")
 
 
+@pytest.mark.parametrize("order", [(0, 1, 2, 3, 7, 6), (0, 3, 7, 6), (0, 1, 2, 3, 4, 5, 6)])
+def test_read_outs_between_the_stages_of_a_step(order):
+    """A read-out between two stages shows the step in progress (its PBD has
+    taken the slots over) and does not disturb it."""
+    from paper_2607_02954_gb300 import _lib
+    lib = _lib.load()
+    spec = drifting(31)
+    w, ref = World(spec), World(spec)
+    names = ("bin_off", "rho_s", "rho_bar", "force")
+    for k in range(3):
+        ref.step(1)
+        want = read_outs(ref, names)
+        for stage in order:
+            _lib.check(lib.mc_step_stage(w.handle, stage, None))
+            for f in names + ("force", "rho_s"):
+                assert np.array_equal(w.field(f), want[f]), (k, stage, f)
+            assert_same(read_outs(w, names), want, (k, stage))
+        assert_same(w.state(fluid=True), ref.state(fluid=True), k)
+
+
 def test_a_captured_step_replays_like_single_steps():
     """One step captured by the caller into a graph of its own and replayed 40
     times (the slots are laid out inside the capture) equals 40 single steps."""
