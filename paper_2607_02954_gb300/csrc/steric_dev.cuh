@@ -173,6 +173,16 @@ __device__ __forceinline__ T block_max(T v, T* red) {
   return m;
 }
 
+// The largest of the block's non-negative values.  One barrier, before the
+// result: red is not written again until the block has passed another.
+template <int NT>
+__device__ __forceinline__ int block_max_int(int v, int* red) {
+  v = __reduce_max_sync(0xffffffffu, v);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  return __reduce_max_sync(0xffffffffu, red[threadIdx.x & (NT / 32 - 1)]);
+}
+
 // The tile item of this block in a launch over the tiles of one world
 // (row-major, as the plan lists them).
 __device__ __forceinline__ int2 single_tile_item(const WorldDev& w, unsigned blk) {
@@ -203,12 +213,14 @@ __device__ __forceinline__ float padded_tap(const WorldDev& w, int wR, int m) {
 // most 1/4, so a cell sum is below the largest bin count near the tile.
 // That bound leaves at least 24 fractional bits up to about one bead per
 // cell.  It is loose (a bead adds 1/16 to a cell on average), so a denser
-// tile (k < 24) first takes a bound from the beads' cells (deposit_bound: at
-// most 2.25 times an even density's sums, so two bits at the most; the sums
-// keep 26 fractional bits at four beads a cell, and turn into floats of 24).
-// With a folded axis it deposits twice instead: the first pass measures the
-// largest sum of the accumulator (plus the rounding its terms can hide),
-// which gives a tight scale for the second.
+// tile (k < 24) takes the scale that its largest sum allows (that sum plus
+// the rounding its terms can hide): it deposits, measures, and deposits again
+// if that scale is the finer one.  The first scale of such a tile comes from
+// the beads' cells (deposit_bound, where no axis is folded): 2.25 times an
+// even density's sums, within the one bit more that a bound known to hold may
+// use (31 bits), so it is as fine as the measured one, 27 fractional bits at
+// four beads a cell, and the second deposit left out, unless the beads lie
+// where the kernel is far below its bounds.
 // ---------------------------------------------------------------------------
 
 // Geometry of one deposit tile.
@@ -309,7 +321,7 @@ __device__ __forceinline__ float deposit_bound(int* acc, const WorldDev& w, cons
     }
     most = max(most, s);
   }
-  return (float)block_max<NT>(most, red) * 0.0625f;
+  return (float)block_max_int<NT>(most, red) * 0.0625f;
 }
 
 // The x pass of the accumulated sums at scale 2^k, rho_s when asked for,
@@ -400,6 +412,7 @@ struct DepositSmem {
   float tap_s[Geo<R>::kTaps];
   Segments sg;
   float red[NT / 32];
+  int most[NT / 32];
 };
 
 // a4 + the x pass of a5 for the tile item of block `blk` (block-uniform
@@ -469,20 +482,26 @@ __device__ __forceinline__ void deposit_x_body(const WorldDev* __restrict__ worl
     return;
   }
   int k = fix_exponent((float)sg.most + 1.0f);
-  const bool counted = k < 24 && !d.full_x && !d.full_y;
-  if (counted) {
-    k = fix_exponent(deposit_bound<R, NT>(acc, w, d, sg, reinterpret_cast<int*>(red)) * 1.0001f);
+  const bool dense = k < 24;
+  if (dense && !d.full_x && !d.full_y) {
+    // b 2^k < 2^30 with b the bound; 2^31 leaves room for the rounding of the
+    // at most 16 b terms, half a unit each, from k = 16 on (1e-4 b 2^17 > 8 b)
+    k = fix_exponent(deposit_bound<R, NT>(acc, w, d, sg, sm.most) * 1.0001f);
+    if (k >= 16 && k < 40) ++k;
     for (int c = tid; c < G::kDY * G::kDX / 4; c += NT) reinterpret_cast<int4*>(acc)[c] = make_int4(0, 0, 0, 0);
     __syncthreads();
   }
   deposit_accumulate<R, NT>(acc, w, d, k, sg);
-  if (k < 24 && !counted) {
-    // dense tile: the largest accumulated sum plus the rounding of its terms
+  if (dense) {
+    // the largest accumulated sum plus the rounding of its terms
     // (half a unit per bead of the covering bins, at most one term per cell
     // each) bounds every sum; deposit again at the scale that bound gives
     int m = 0;
-    for (int c = tid; c < G::kDY * G::kDX; c += NT) m = max(m, acc[c]);
-    m = block_max<NT>(m, reinterpret_cast<int*>(red));
+    for (int c = tid; c < G::kDY * G::kDX / 4; c += NT) {
+      const int4 v = reinterpret_cast<const int4*>(acc)[c];
+      m = max(m, max(max(v.x, v.y), max(v.z, v.w)));
+    }
+    m = block_max_int<NT>(m, sm.most);
     const int k2 = fix_exponent(((float)m + 0.5f * (float)d.total) * pow2f(-k) * 1.0001f);
     if (k2 > k) {
       for (int c = tid; c < G::kDY * G::kDX / 4; c += NT) reinterpret_cast<int4*>(acc)[c] = make_int4(0, 0, 0, 0);

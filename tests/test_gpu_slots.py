@@ -511,6 +511,52 @@ def test_read_outs_between_the_stages_of_a_step(order):
         assert_same(w.state(fluid=True), ref.state(fluid=True), k)
 
 
+@pytest.mark.parametrize("at", [(20.2, 20.2), (20.5, 20.5), (20.9, 20.1), (31.4, 9.5)])
+@pytest.mark.parametrize("n_fil", [300, 700, 3000, 9000])
+def test_a_crowded_spot_leaves_its_tile_the_bits_of_the_largest_sum(at, n_fil):
+    """A crowd in a few cells and single beads elsewhere in the tile: the
+    deposit's fixed point is as fine as the largest sum M of the tile allows
+    (the largest k with M 2^k < 2^30), so a cell that t beads reach is off by
+    t halves of 2^-k, and by the rounding of their 32-bit weights (products of
+    two factors of at most 1/2, each off by 2^-25: 2^-25 a bead)."""
+    H, W, B = 96, 96, 2
+    rng = np.random.default_rng(n_fil)
+    h = rng.uniform(0, 2 * np.pi, n_fil + 12)
+    x0, y0 = (rng.uniform(8, 30, n_fil + 12) for _ in range(2))
+    x0[:n_fil] = at[0] + rng.uniform(0, 0.05, n_fil)
+    y0[:n_fil] = at[1] + rng.uniform(0, 0.05, n_fil)
+    L = np.where(np.arange(n_fil + 12) < n_fil, 0.05, 1.0)
+    x = np.stack([x0, x0 + L * np.cos(h)], 1).ravel().astype(np.float32)
+    y = np.stack([y0, y0 + L * np.sin(h)], 1).ravel().astype(np.float32)
+    e = np.zeros(0)
+    spec = synth._world("spot", H, W, [B] * len(h), x, y, h.astype(np.float32), e, e, e, e,
+                        params=synth.Params(k_rep=1e-6, kappa=1e-6))
+    ow = O.World(spec)
+    _, rec = O.step(ow, ow.initial_state(), record=True)
+    want = t2n(rec["rho_s"])
+    reach = np.zeros((H, W), int)
+    for b in range(-1, 3):
+        for a in range(-1, 3):
+            np.add.at(reach, ((np.floor(y).astype(int) + b) % H, (np.floor(x).astype(int) + a) % W), 1)
+    w = World(spec)
+    w.step(1)
+    got = w.field("rho_s").astype(np.float64)
+    checked = 0
+    for ty in range(0, H, 32):
+        for tx in range(0, W, 32):
+            # the tile and what its filter reads
+            rows, cols = np.arange(ty - 3, ty + 35) % H, np.arange(tx - 8, tx + 40) % W
+            k = 30 - np.frexp(want[np.ix_(rows, cols)].max())[1]
+            if k >= 24:
+                continue
+            t = np.s_[ty:ty + 32, tx:tx + 32]
+            few = (reach[t] > 0) & (reach[t] < 8)
+            err = np.abs(got[t] - want[t]) / reach[t].clip(min=1)
+            assert (err[few] <= 2.0 ** -(k + 1) + 2.0 ** -25).all(), (k, err[few].max() * 2.0 ** (k + 1))
+            checked += few.sum()
+    assert checked
+
+
 def test_a_captured_step_replays_like_single_steps():
     """One step captured by the caller into a graph of its own and replayed 40
     times (the slots are laid out inside the capture) equals 40 single steps."""
