@@ -173,10 +173,10 @@ __device__ __forceinline__ T block_max(T v, T* red) {
   return m;
 }
 
-// The largest of the block's non-negative values.  One barrier, before the
-// result: red is not written again until the block has passed another.
+// The largest of the block's values.  One barrier, before the result: red is
+// not written again until the block has passed another.
 template <int NT>
-__device__ __forceinline__ int block_max_int(int v, int* red) {
+__device__ __forceinline__ unsigned block_max_u(unsigned v, unsigned* red) {
   v = __reduce_max_sync(0xffffffffu, v);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
   __syncthreads();
@@ -217,10 +217,10 @@ __device__ __forceinline__ float padded_tap(const WorldDev& w, int wR, int m) {
 // the rounding its terms can hide): it deposits, measures, and deposits again
 // if that scale is the finer one.  The first scale of such a tile comes from
 // the beads' cells (deposit_bound, where no axis is folded): 2.25 times an
-// even density's sums, within the one bit more that a bound known to hold may
-// use (31 bits), so it is as fine as the measured one, 27 fractional bits at
-// four beads a cell, and the second deposit left out, unless the beads lie
-// where the kernel is far below its bounds.
+// even density's sums.  A bound known to hold may use all 32 bits of a cell
+// (kWideFrom), two more than the measured rule, so this scale is as fine as the
+// measured one unless a tile's sums are below a quarter of their bound, and
+// hardly any tile deposits twice.
 // ---------------------------------------------------------------------------
 
 // Geometry of one deposit tile.
@@ -228,6 +228,17 @@ struct DepTile {
   int W, H, wR, x0, y0, tw, th, cx0, oxe, tile, total;
   bool full_x, full_y;
 };
+
+// Sums of a tile whose scale comes from deposit_bound fill 32 bits unsigned: b
+// 2^k < 2^32 / 1.0001, and the rounding of the at most 16 b terms of a cell,
+// half a unit each, adds at most 8 b < 2^15 (k >= 20 then).  Weights of rounding
+// size may be negative and leave a sum some units below zero: the range above
+// kWideFrom, which the other sums stay below by the 1.0001, is theirs.
+// Sums that do not fit 31 bits are halved before the x pass, which reads them
+// signed: that leaves one bit more than the measured rule, so the rounding of
+// the halving (2^-k) and of the terms (2^-k / 2 each) stays below that rule's
+// (2 2^-k a term).
+constexpr unsigned kWideFrom = 0xfffe0000u;   // 2^32 - 2^17
 
 // Deposits the tile's beads at scale 2^k into acc (zeroed) and folds the
 // wrapped cells.  Ends with the block synchronised.
@@ -295,7 +306,7 @@ __device__ __forceinline__ void deposit_accumulate(int* acc, const WorldDev& w, 
 // a bead instead of sixteen.  Not for folded axes.
 template <int R, int NT>
 __device__ __forceinline__ float deposit_bound(int* acc, const WorldDev& w, const DepTile& d, const Segments& sg,
-                                               int* red) {
+                                               unsigned* red) {
   using G = Geo<R>;
   const int tid = threadIdx.x, total = sg.pre[kSegs];
   const float4* __restrict__ bpos = w.bpos;
@@ -321,7 +332,7 @@ __device__ __forceinline__ float deposit_bound(int* acc, const WorldDev& w, cons
     }
     most = max(most, s);
   }
-  return (float)block_max_int<NT>(most, red) * 0.0625f;
+  return (float)block_max_u<NT>((unsigned)most, red) * 0.0625f;
 }
 
 // The x pass of the accumulated sums at scale 2^k, rho_s when asked for,
@@ -412,7 +423,7 @@ struct DepositSmem {
   float tap_s[Geo<R>::kTaps];
   Segments sg;
   float red[NT / 32];
-  int most[NT / 32];
+  unsigned most[NT / 32];
 };
 
 // a4 + the x pass of a5 for the tile item of block `blk` (block-uniform
@@ -484,10 +495,8 @@ __device__ __forceinline__ void deposit_x_body(const WorldDev* __restrict__ worl
   int k = fix_exponent((float)sg.most + 1.0f);
   const bool dense = k < 24;
   if (dense && !d.full_x && !d.full_y) {
-    // b 2^k < 2^30 with b the bound; 2^31 leaves room for the rounding of the
-    // at most 16 b terms, half a unit each, from k = 16 on (1e-4 b 2^17 > 8 b)
     k = fix_exponent(deposit_bound<R, NT>(acc, w, d, sg, sm.most) * 1.0001f);
-    if (k >= 16 && k < 40) ++k;
+    if (k >= 18 && k <= 30) k += 2;   // (a term is at most 2^k / 4)
     for (int c = tid; c < G::kDY * G::kDX / 4; c += NT) reinterpret_cast<int4*>(acc)[c] = make_int4(0, 0, 0, 0);
     __syncthreads();
   }
@@ -496,18 +505,26 @@ __device__ __forceinline__ void deposit_x_body(const WorldDev* __restrict__ worl
     // the largest accumulated sum plus the rounding of its terms
     // (half a unit per bead of the covering bins, at most one term per cell
     // each) bounds every sum; deposit again at the scale that bound gives
-    int m = 0;
+    unsigned m = 0u;
+    auto sum = [](int v) { return (unsigned)v < kWideFrom ? (unsigned)v : 0u; };
     for (int c = tid; c < G::kDY * G::kDX / 4; c += NT) {
       const int4 v = reinterpret_cast<const int4*>(acc)[c];
-      m = max(m, max(max(v.x, v.y), max(v.z, v.w)));
+      m = max(m, max(max(sum(v.x), sum(v.y)), max(sum(v.z), sum(v.w))));
     }
-    m = block_max_int<NT>(m, sm.most);
+    m = block_max_u<NT>(m, sm.most);
     const int k2 = fix_exponent(((float)m + 0.5f * (float)d.total) * pow2f(-k) * 1.0001f);
     if (k2 > k) {
       for (int c = tid; c < G::kDY * G::kDX / 4; c += NT) reinterpret_cast<int4*>(acc)[c] = make_int4(0, 0, 0, 0);
       __syncthreads();
       k = k2;
       deposit_accumulate<R, NT>(acc, w, d, k, sg);
+    } else if (m >= 0x80000000u) {
+      for (int c = tid; c < G::kDY * G::kDX; c += NT) {
+        const int v = acc[c];
+        acc[c] = (unsigned)v < kWideFrom ? (int)(((unsigned)v + 1u) >> 1) : v / 2;
+      }
+      --k;
+      __syncthreads();
     }
   }
   deposit_xpass<R, NT>(acc, w, d, k, tap_s, red, store_fields);
