@@ -14,6 +14,7 @@
 // beads (register PBD), Gaussian half width 4 (sigma in (0.75, 1]); the
 // autotuner offers this path only for such plans.
 #include "bead_dev.cuh"
+#include "bin_dev.cuh"
 #include "steric_dev.cuh"
 
 namespace mc {
@@ -76,6 +77,7 @@ template <int R>
 union PersistSmem {
   ForceSmem<R, 256> force;
   DepositSmem<R, 256> deposit;
+  ScanSmem scan;
 };
 
 }  // namespace
@@ -89,6 +91,8 @@ struct PersistArgs {
   int n_bead_items;
   const int2* tile_items;
   int n_tile_items;
+  const int2* scan_items;
+  int n_scan_items, one_chunk;
   int n_steps;
   unsigned* bar;       // [2] barrier words, zeroed before the launch
   unsigned* status;    // set to 1 when a barrier wait ran out
@@ -107,6 +111,21 @@ __global__ void __launch_bounds__(256, kBlocks) k_step_persistent(const PersistA
   auto barrier = [&]() { return grid_barrier(a.bar, gen, target, a.timeout_ns, a.status, &s_ok); };
   bool ok = true;
   for (int s = 0; s < a.n_steps && ok; ++s) {
+    if (s > 0 && s % kLayoutSteps == 0) {
+      // the slots laid out from step s - 1's counts: a run may have any
+      // length, and beads that have left the bins of its first step would all
+      // end in the overflow list, which every tile reads (131,072 beads in a
+      // band of 64 columns of 512^2, moving 0.3 cells a step: 192 steps took
+      // 99.8 ms on the first step's layout, 29.1 so)
+      if (!a.one_chunk) {
+        for (unsigned b = blockIdx.x; b < (unsigned)a.n_scan_items; b += gridDim.x)
+          scan_sums<1>(a.worlds, a.scan_items, s - 1, b, sm.scan);
+        if (!(ok = barrier())) break;
+      }
+      for (unsigned b = blockIdx.x; b < (unsigned)a.n_scan_items; b += gridDim.x)
+        scan_apply<1>(a.worlds, a.scan_items, s - 1, b, sm.scan);
+      if (!(ok = barrier())) break;
+    }
     // a1-a3 with the binning (fused with the previous step's a8 after the first step)
     const int fields = s == a.n_steps - 1;
     for (unsigned b = blockIdx.x; b < (unsigned)a.n_pbd_blocks; b += gridDim.x) {
@@ -197,6 +216,9 @@ cudaError_t launch_persistent(const Plan& p, int n, cudaStream_t s) {
   a.n_bead_items = p.n_bead_items;
   a.tile_items = p.d_tile_items;
   a.n_tile_items = p.n_tile_items;
+  a.scan_items = p.d_scan_items;
+  a.n_scan_items = p.n_scan_items;
+  a.one_chunk = p.one_chunk;
   a.n_steps = n;
   a.bar = p.d_persist_bar;
   a.status = p.d_persist_bar + 2;

@@ -366,19 +366,21 @@ def room(counts):
     return (counts + counts // 4 + 16 + 7) // 8 * 8
 
 
+def uniform_flow(H, W, ux, uy):
+    cx = np.array([0, 1, 0, -1, 0, 1, -1, -1, 1])[:, None, None]
+    cy = np.array([0, 0, 1, 0, -1, 1, 1, -1, -1])[:, None, None]
+    wt = np.array([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4)[:, None, None]
+    cu = cx * ux + cy * uy
+    return np.broadcast_to(wt * (3 * cu + 4.5 * cu * cu - 1.5 * (ux * ux + uy * uy)), (9, H, W)).astype(np.float32)
+
+
 def drifting(seed, **kw):
     """A crowd carried across bins by a uniform flow (beads further apart with
     direct forcing, whose passes overshoot where several share a cell)."""
     spec = synth.world_random(seed, (72, 64), 12) if kw.get("ib") else crowded(seed, n_fil=40, at=(20.0, 20.0))
     for k, v in kw.items():
         setattr(spec.params, k, v)
-    cx = np.array([0, 1, 0, -1, 0, 1, -1, -1, 1])[:, None, None]
-    cy = np.array([0, 0, 1, 0, -1, 1, 1, -1, -1])[:, None, None]
-    wt = np.array([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4)[:, None, None]
-    ux, uy = 0.3, 0.1
-    cu = cx * ux + cy * uy
-    spec.f0 = np.broadcast_to(wt * (3 * cu + 4.5 * cu * cu - 1.5 * (ux * ux + uy * uy)),
-                              (9, spec.H, spec.W)).astype(np.float32)
+    spec.f0 = uniform_flow(spec.H, spec.W, 0.3, 0.1)
     return spec
 
 
@@ -555,6 +557,40 @@ def test_a_crowded_spot_leaves_its_tile_the_bits_of_the_largest_sum(at, n_fil):
             assert (err[few] <= 2.0 ** -(k + 1) + 2.0 ** -25).all(), (k, err[few].max() * 2.0 ** (k + 1))
             checked += few.sum()
     assert checked
+
+
+@pytest.mark.parametrize("n_worlds", [1, 3])
+def test_a_long_persistent_run_lays_the_slots_out_again(n_worlds):
+    """A band of beads carried out of its bins: one persistent run of 192 steps
+    equals twelve of 16 bitwise and takes about their time (every step reading
+    all the beads that have left their first bins took several times as long)."""
+    from paper_2607_02954_gb300 import set_launch_config
+    H, W, B, n_fil = 256 if n_worlds > 1 else 512, 512, 32, 4096
+    rng = np.random.default_rng(5)
+    x = (np.repeat(rng.uniform(0, 64, n_fil), B) + rng.uniform(0, 0.1, n_fil * B)).astype(np.float32)
+    y = np.mod(rng.uniform(0, H, (n_fil, 1)) + np.arange(B), H).astype(np.float32).ravel()
+    y[y >= H] = 0
+    J = n_fil * (B - 2)
+    spec = synth._world("band", H, W, [B] * n_fil, x, y, np.full(n_fil * (B - 1), np.pi / 2, np.float32), np.zeros(J),
+                        np.zeros(J), np.zeros(J), np.zeros(J), params=synth.Params(k_rep=1e-4, kappa=1e-3))
+    spec.f0 = uniform_flow(H, W, 0.3, 0.0)
+    long, short = ([World(spec) for _ in range(n_worlds)] for _ in range(2))
+    ms = []
+    for ws, runs in ((long, [16, 192]), (short, [16] + [16] * 12)):
+        set_launch_config(ws, persistent=4)
+        step_batched(ws, runs[0])
+        e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        e0.record()
+        for n in runs[1:]:
+            step_batched(ws, n)
+        e1.record()
+        torch.cuda.synchronize()
+        ms.append(e0.elapsed_time(e1))
+    print("ms of one run, of twelve:", ms)
+    for a, b in zip(long, short):
+        a.check()
+        assert_same(a.state(fluid=True), b.state(fluid=True), "state")
+    assert ms[0] < 1.5 * ms[1], ms
 
 
 def test_a_captured_step_replays_like_single_steps():
