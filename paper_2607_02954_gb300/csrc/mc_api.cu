@@ -231,7 +231,11 @@ cudaStream_t capture_stream() {
 
 // Lays the slots out before a run of n steps outside the graph when the plan
 // has run kLayoutSteps steps on the present layout, and always into a capture
-// (whose replays this host does not see).
+// (whose replays this host does not see).  A layout is looked at between runs
+// only, and such a run has fewer than kLayoutSteps steps (a persistent one lays
+// out by itself), so none serves more than 2 kLayoutSteps - 2 = 30: at the
+// watchdog's half a cell a step beads have then crossed two bins at the most,
+// and the ones that find a bin full still find the overflow list.
 void lay_out_slots(Plan& p, int n, cudaStream_t s) {
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   cudaStreamIsCapturing(s, &cs);

@@ -241,7 +241,7 @@ void launch_pbd(const Plan& p, cudaStream_t s);
 void launch_slot_layout(const Plan& p, cudaStream_t s);
 // ... and from the positions (single-world plans: a new or loaded world)
 void launch_slot_layout_from_positions(const Plan& p, cudaStream_t s);
-constexpr int kLayoutSteps = 16;   // at most so many steps between layouts
+constexpr int kLayoutSteps = 16;   // steps on one layout of the slots (up to 30 in short runs: lay_out_slots)
 // sorted read-outs (off as above): the bin offsets, then the records in bin order
 void launch_sorted_offsets(const Plan& p, cudaStream_t s, int off);
 void launch_sorted_records(const Plan& p, cudaStream_t s, int off);
