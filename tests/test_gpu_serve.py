@@ -104,6 +104,24 @@ def test_admission_respects_the_memory_budget():
     assert stats["submitted"] == 4 and stats["completed"] == 4
 
 
+@pytest.mark.parametrize("kw", [{}, dict(layers=2), dict(ib=1, mdf_iters=1)])
+def test_admission_charges_the_worlds_device_memory(kw):
+    """Two requests are admitted together only when the budget holds both
+    worlds' arenas, whatever buffers their options need."""
+    from paper_2607_02954_gb300 import Server, World
+    spec = synth.world_random(5, 512, 100)
+    spec.params = synth.Params(**kw)
+    w = World(spec)
+    arena = w.info()["device_bytes"]
+    w.close()
+    for together, budget in ((False, 2 * arena - 1), (True, int(2.1 * arena))):
+        srv = Server(hbm_budget_bytes=budget, max_slots=8, steps_per_tick=20)
+        a, b = (srv.wait(t) for t in [srv.submit(spec, 1000), srv.submit(spec, 1000)])
+        srv.close()
+        assert a["status"] == 0 and b["status"] == 0
+        assert (b["t_admit_ns"] < a["t_done_ns"]) == together, (a, b)
+
+
 def test_poll_wait_timeout_and_unknown_tickets():
     from paper_2607_02954_gb300 import Server
     from paper_2607_02954_gb300._lib import MCError
