@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(256) k_adj_rho_blur(const WorldDev* __restrict
 template <int R>
 static void launch_blur_r(const WorldDev& h, const WorldDev* wd, const AdjDev& a, cudaStream_t s) {
   const int b8 = h.ntx * ((h.H + 7) / 8);
-  if (b8 < 4 * 152) k_adj_rho_blur<R, 8><<<b8, 256, 0, s>>>(wd, a);
+  if (b8 < 4 * num_sms()) k_adj_rho_blur<R, 8><<<b8, 256, 0, s>>>(wd, a);
   else k_adj_rho_blur<R, 16><<<h.ntx * ((h.H + 15) / 16), 256, 0, s>>>(wd, a);
 }
 
@@ -1233,7 +1233,7 @@ static int bead_blocks(int n) { return (n + kAdjBeadThreads - 1) / kAdjBeadThrea
 static size_t adj_regs_smem(int n_pbd) { return (size_t)n_pbd * kAdjTapeRegs * 32 * sizeof(float); }
 static int adj_regs_warps(int n, int n_pbd) {
   const size_t per = adj_regs_smem(n_pbd);
-  int wpb = n < 304 ? 1 : kAdjRegsWarps;
+  int wpb = n < 2 * num_sms() ? 1 : kAdjRegsWarps;
   while (wpb > 1 && wpb * per > 48 * 1024) wpb /= 2;
   return wpb;
 }

@@ -192,10 +192,10 @@ struct LaunchCfg {
 struct Plan {
   int n_worlds = 0;
   // A plan of one world lets the step's kernels take each block's work item
-  // from the block index instead of the item list.  The tile kernels, the
-  // bin scatter and the scans also take the world's descriptor as a
-  // __grid_constant__ parameter, so their blocks start without a dependent
-  // load; the PBD and advance kernels keep reading it from the table (their
+  // from the block index instead of the item list.  The tile kernels also take
+  // the world's descriptor as a __grid_constant__ parameter, so their blocks
+  // start without a dependent load; the PBD, the advance and the bins' prefix
+  // sums keep reading it from the table (the bead kernels'
   // arithmetic then compiles exactly as in a batch, and a world stepped alone
   // stays bitwise equal to the same world batched, as measured).
   WorldDev h_world0{};

@@ -10,7 +10,6 @@ namespace mc {
 namespace {
 
 constexpr int kThreads = 256;              // threads of a tile's block (the force kernels' narrowest, see tile_threads)
-constexpr int kWarps = kThreads / 32;
 constexpr int kAx = kTile + 6;             // force accumulator edge: the tile and 3 halo cells a side
 constexpr int kWin = kTile + 8;            // rho_bar window edge: the tile and 4 cells a side
 __constant__ int kLbmCy[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};   // D2Q9 lattice velocities, y components
