@@ -81,7 +81,7 @@ STEP_BYTES_PER_BEAD = 32
 # dram__bytes_read.sum + dram__bytes_write.sum of one launch of the dominant
 # kernel, from an ncu capture of the workload, keyed by the fingerprint of the
 # sources the kernel is built from (reported only while they are unchanged)
-KERNEL_TRAFFIC = {("c3_22", "8a2ffe2a16cce112"): 1602457344}
+KERNEL_TRAFFIC = {("c3_22", "eed3372904107573"): 1601989120}
 KERNEL_SOURCES = ["steric_dev.cuh", "k_steric.cu", "mc_internal.cuh"]
 
 
